@@ -227,37 +227,24 @@ __device__ __forceinline__ int exp_of_key(uint64_t key) {
 }
 
 // round(x * 2^shift) to the nearest integer (ties to even) with integer
-// operations only; |result| < 2^62 is guaranteed by the caller's scaling
+// operations only; |result| < 2^62 is guaranteed by the caller's scaling.
+// Right shifts round by adding (half - 1 + the kept low bit) before the shift.
 __device__ __forceinline__ long long round_scaled(double x, int shift) {
   const uint64_t b = uint64_t(__double_as_longlong(x));
   const int E = int((b >> 52) & 0x7FF);
-  if (E == 0 && (b << 1) == 0) return 0;
-  uint64_t m = b & 0xFFFFFFFFFFFFFull;
-  int ee = E;
-  if (E == 0) ee = 1; else m |= 1ull << 52;
-  const int sh = ee - 1075 + shift;  // value = m * 2^sh
-  long long q;
-  if (sh >= 0) {
-    q = (long long)(m << sh);
-  } else if (sh <= -64) {
-    q = 0;
+  const uint64_t m = (b & 0xFFFFFFFFFFFFFull) | (uint64_t(E != 0) << 52);
+  const int r = 1075 - (E ? E : 1) - shift;  // value = m * 2^-r
+  uint64_t q;
+  if (r > 0) {
+    q = r < 64 ? (m + ((1ull << (r - 1)) - 1ull) + ((m >> r) & 1ull)) >> r : 0ull;
   } else {
-    const int r = -sh;
-    const uint64_t qq = m >> r;
-    const uint64_t rem = m & ((1ull << r) - 1ull);
-    const uint64_t half = 1ull << (r - 1);
-    q = (long long)(qq + ((rem > half || (rem == half && (qq & 1ull))) ? 1ull : 0ull));
+    q = m << -r;
   }
-  return (b >> 63) ? -q : q;
+  return (b >> 63) ? -(long long)q : (long long)q;
 }
 
 __device__ __forceinline__ int64_t map_at(const OzMap& m, int64_t i) {
   return m.in ? (i / m.in) * m.so + (i % m.in) * m.si : i * m.si;
-}
-
-// source offset of row r: ridx[r] rows of stride rm.si, else the row map
-__device__ __forceinline__ int64_t row_base(const OzMap& rm, const int* ridx, int64_t r) {
-  return ridx ? int64_t(ridx[r]) * rm.si : map_at(rm, r);
 }
 
 // |mul * kw[k] * v| as an order-preserving key
@@ -269,49 +256,23 @@ __device__ __forceinline__ uint64_t key_at(double v, int64_t k, const double* __
 
 __device__ __forceinline__ uint64_t umax64(uint64_t a, uint64_t b) { return a > b ? a : b; }
 
-// e_r: max_k |x(r,k)| < 2^e_r, x = mul * kw[k] * src[row(r) + map_k(k)]; one thread per row
-// (four loads in flight per thread on the plain-stride path)
-__global__ void k_oz_rowexp_thread(const double* __restrict__ src, OzMap rm, OzMap km, int64_t rows, int64_t K,
-                                   const double* __restrict__ kw, double mul, const int* __restrict__ ridx,
-                                   int* __restrict__ exps) {
-  const int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (r >= rows) return;
-  const double* row = src + row_base(rm, ridx, r);
-  uint64_t m = 0;
-  if (km.in == 0) {
-    const int64_t si = km.si;
-    int64_t k = 0;
-    for (; k + 4 <= K; k += 4) {
-      const double v0 = row[k * si], v1 = row[(k + 1) * si], v2 = row[(k + 2) * si], v3 = row[(k + 3) * si];
-      m = umax64(m, umax64(umax64(key_at(v0, k, kw, mul), key_at(v1, k + 1, kw, mul)),
-                           umax64(key_at(v2, k + 2, kw, mul), key_at(v3, k + 3, kw, mul))));
-    }
-    for (; k < K; ++k) m = umax64(m, key_at(row[k * si], k, kw, mul));
-  } else {
-    int64_t q = 0, rem = 0;  // k = q km.in + rem, advanced without division
-    for (int64_t k = 0; k < K; ++k) {
-      m = umax64(m, key_at(row[q * km.so + rem * km.si], k, kw, mul));
-      if (++rem == km.in) rem = 0, ++q;
-    }
-  }
-  exps[r] = exp_of_key(m);
-}
-
-// same, one block per row (few long rows); contiguous rows are read as
-// 16-byte vectors, four per thread in flight
-__global__ void k_oz_rowexp_block(const double* __restrict__ src, OzMap rm, OzMap km, int64_t K,
-                                  const double* __restrict__ kw, double mul, const int* __restrict__ ridx,
-                                  int* __restrict__ exps) {
-  __shared__ unsigned long long sh[256];
+// Row scales of few very long contiguous rows (the Coulomb spectra, K of
+// millions): blockIdx.y walks shares of one row, the shares meet in an
+// atomicMax on the row's key; k_oz_key_exps turns the keys into exponents.
+// 16-byte loads, four per thread in flight.
+__global__ void k_oz_row_keys(const double* __restrict__ src, int64_t sr, int64_t K, int64_t share,
+                              const double* __restrict__ kw, double mul, unsigned long long* __restrict__ keys) {
+  __shared__ unsigned long long sh[8];
   const int64_t r = blockIdx.x;
-  const double* row = src + row_base(rm, ridx, r);
+  const int64_t k0 = int64_t(blockIdx.y) * share, k1 = k0 + share < K ? k0 + share : K;  // share is even
+  const double* row = src + r * sr;
   uint64_t m = 0;
   const int bd = blockDim.x;
-  if (km.in == 0 && km.si == 1 && (reinterpret_cast<uintptr_t>(row) & 15) == 0) {
+  if ((reinterpret_cast<uintptr_t>(row) & 15) == 0) {
     const double2* p = reinterpret_cast<const double2*>(row);
-    const int64_t K2 = K >> 1;
-    int64_t i = threadIdx.x;
-    for (; i + 3 * bd < K2; i += 4 * bd) {
+    const int64_t i1 = k1 >> 1;
+    int64_t i = (k0 >> 1) + threadIdx.x;
+    for (; i + 3 * bd < i1; i += 4 * bd) {
       double2 t[4];
 #pragma unroll
       for (int h = 0; h < 4; ++h) t[h] = __ldg(p + i + h * bd);
@@ -321,21 +282,27 @@ __global__ void k_oz_rowexp_block(const double* __restrict__ src, OzMap rm, OzMa
         m = umax64(m, umax64(key_at(t[h].x, k, kw, mul), key_at(t[h].y, k + 1, kw, mul)));
       }
     }
-    for (; i < K2; i += bd) {
+    for (; i < i1; i += bd) {
       const double2 t = __ldg(p + i);
       m = umax64(m, umax64(key_at(t.x, 2 * i, kw, mul), key_at(t.y, 2 * i + 1, kw, mul)));
     }
-    if ((K & 1) && threadIdx.x == 0) m = umax64(m, key_at(row[K - 1], K - 1, kw, mul));
+    if ((k1 & 1) && threadIdx.x == 0) m = umax64(m, key_at(row[k1 - 1], k1 - 1, kw, mul));
   } else {
-    for (int64_t k = threadIdx.x; k < K; k += bd) m = umax64(m, key_at(row[map_at(km, k)], k, kw, mul));
+    for (int64_t k = k0 + threadIdx.x; k < k1; k += bd) m = umax64(m, key_at(row[k], k, kw, mul));
   }
-  sh[threadIdx.x] = m;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = umax64(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
   __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) sh[threadIdx.x] = sh[threadIdx.x] > sh[threadIdx.x + o] ? sh[threadIdx.x] : sh[threadIdx.x + o];
-    __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < bd / 32; ++w) m = umax64(m, sh[w]);
+    atomicMax(keys + r, (unsigned long long)m);
   }
-  if (threadIdx.x == 0) exps[r] = exp_of_key(sh[0]);
+}
+
+__global__ void k_oz_key_exps(const unsigned long long* __restrict__ keys, int64_t rows, int* __restrict__ exps) {
+  const int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (r < rows) exps[r] = exp_of_key(keys[r]);
 }
 
 // BF16 bits of a small integer d (|d| <= 2^8): 1.5 * 2^23 + d is exact in
@@ -346,20 +313,11 @@ __device__ __forceinline__ uint32_t bf16_bits_of_small(int d) {
   return __float_as_uint(__int_as_float(0x4B400000 + d) - 12582912.0f);
 }
 
-// Digits of row r and k group kg (8 values), written as 16 bytes per slice:
-// tile (row tile i, k tile j) sits at position i * kst + j of the tile array.
-template <int S>
-__device__ __forceinline__ void oz_digit_group(const double* __restrict__ src, const OzMap& rm, const OzMap& km,
-                                               int64_t rows, int64_t K, const double* __restrict__ kw, double mul,
-                                               const int* __restrict__ exps, int rt, int64_t kst,
-                                               const int* __restrict__ ridx, __nv_bfloat16* __restrict__ tiles, int r,
-                                               int64_t kg) {
-  const bool live = r < rows;
-  const int e = live ? exps[r] : 0;
-  const double* row = src + (live ? row_base(rm, ridx, r) : 0);
+// The 8 values of k group kg of a row (zero beyond K), before mul and kw.
+__device__ __forceinline__ void oz_load8(const double* __restrict__ row, bool live, int64_t sk, int64_t K, int64_t kg,
+                                         double (&v)[8]) {
   const int64_t k0 = kg * 8;
-  double v[8];
-  if (live && km.in == 0 && km.si == 1 && k0 + 8 <= K && (reinterpret_cast<uintptr_t>(row + k0) & 15) == 0) {
+  if (live && sk == 1 && k0 + 8 <= K && (reinterpret_cast<uintptr_t>(row + k0) & 15) == 0) {
     const double2* p = reinterpret_cast<const double2*>(row + k0);
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
@@ -368,89 +326,173 @@ __device__ __forceinline__ void oz_digit_group(const double* __restrict__ src, c
       v[2 * h + 1] = t.y;
     }
   } else {
-    int64_t q = 0, rem = 0;  // k0 = q km.in + rem
-    if (km.in) q = k0 / km.in, rem = k0 % km.in;
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int64_t off = km.in ? q * km.so + rem * km.si : (k0 + u) * km.si;
-      if (km.in && ++rem == km.in) rem = 0, ++q;
-      v[u] = (live && k0 + u < K) ? row[off] : 0.0;
-    }
-  }
-  long long X[8];
-  const int shift = 7 * S - e;
-#pragma unroll
-  for (int u = 0; u < 8; ++u) {
-    double x = v[u];
-    if (k0 + u < K) {
-      if (mul != 1.0) x *= mul;
-      if (kw) x *= kw[k0 + u];
-    }
-    X[u] = round_scaled(x, shift);
-  }
-  const int it = r / rt, rr = r - it * rt;
-  const int64_t jt = kg / (kBK / 8);
-  const int kc = int(kg % (kBK / 8));
-  const int64_t tile_elems = int64_t(rt) * kBK;
-  __nv_bfloat16* base = tiles + ((int64_t(it) * kst + jt) * S) * tile_elems;
-  const int inner = (rr >> 3) * (8 * kBK) + kc * 64 + (rr & 7) * 8;  // element offset in a tile
-  // Balanced digits from the least significant end (in [-64, 63]; the top one
-  // takes the rest, |d_0| <= 128), one slice at a time.  |X| < 2^(7S + 1), so
-  // once S - 4 digits are removed the remainder fits in 32 bits.
-  int Y[8];
-#pragma unroll
-  for (int u = 0; u < 8; ++u) Y[u] = int(X[u]);
-#pragma unroll
-  for (int s = S - 1; s >= 0; --s) {
-    uint32_t b[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      int dig;
-      if (s >= 4) {
-        dig = int((uint32_t(X[u]) + 64u) & 127u) - 64;
-        X[u] = (X[u] - dig) >> 7;
-        if (s == 4) Y[u] = int(X[u]);
-      } else if (s >= 1) {
-        dig = ((Y[u] + 64) & 127) - 64;
-        Y[u] = (Y[u] - dig) >> 7;
-      } else {
-        dig = Y[u];
-      }
-      b[u] = bf16_bits_of_small(dig);
-    }
-    uint4 w;
-    w.x = __byte_perm(b[0], b[1], 0x7632);
-    w.y = __byte_perm(b[2], b[3], 0x7632);
-    w.z = __byte_perm(b[4], b[5], 0x7632);
-    w.w = __byte_perm(b[6], b[7], 0x7632);
-    *reinterpret_cast<uint4*>(base + int64_t(s) * tile_elems + inner) = w;
+    for (int u = 0; u < 8; ++u) v[u] = (live && k0 + u < K) ? __ldg(row + (k0 + u) * sk) : 0.0;
   }
 }
 
-// Digits of the k groups [kg0, kg0 + ngrp) of every row (padding rows zero).
-// order 0 (k strided): 256 consecutive rows per block, one k group per
-// blockIdx.y.  order 1 (k contiguous): each warp takes 8 rows x 4
-// consecutive k groups, so it writes one 512-byte line of each slice and
-// reads 256 contiguous bytes of each of its rows; blockIdx.y walks the
-// 8-row groups.
+__device__ __forceinline__ void oz_weight8(double (&v)[8], int64_t K, int64_t kg, const double* __restrict__ kw,
+                                           double mul) {
+#pragma unroll
+  for (int u = 0; u < 8; ++u)
+    if (kg * 8 + u < K) {
+      if (mul != 1.0) v[u] *= mul;
+      if (kw) v[u] *= kw[kg * 8 + u];
+    }
+}
+
+// Digits of 8 consecutive k values of one row, 16 bytes per slice at
+// out + s * tile_elems.  With X = round(x 2^shift) the balanced digits
+// (in [-64, 63], the top one takes the rest, |d_0| <= 128) are the base-128
+// digits of X + sum_p 64 128^p less 64, so every digit is a 7-bit field of one
+// integer and no digit waits for the one below it; two fields go through
+// BF16 at once, 0x4300 | f being the pattern of 128 + f and the difference to
+// 192 exact.
 template <int S>
-__global__ void k_oz_digits(const double* __restrict__ src, OzMap rm, OzMap km, int64_t rows, int64_t K,
-                            const double* __restrict__ kw, double mul, const int* __restrict__ exps, int rt,
-                            int64_t nrt, int64_t kg0, int64_t ngrp, int64_t kst, int order,
-                            const int* __restrict__ ridx, __nv_bfloat16* __restrict__ tiles) {
-  const int64_t rows_pad = nrt * rt;
-  if (order == 0) {
-    const int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void oz_digits8(const double (&v)[8], int shift, int64_t tile_elems,
+                                           __nv_bfloat16* __restrict__ out) {
+  constexpr long long bias = 64ll * (((1ll << (7 * (S - 1))) - 1ll) / 127ll);
+  uint32_t w0[8];  // fields 0..3 (the least significant digits)
+  int w1[8];       // fields 4.. and the top digit (signed)
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const long long X = round_scaled(v[u], shift) + bias;
+    w0[u] = uint32_t(X) & 0x0FFFFFFFu;
+    w1[u] = int(X >> 28);
+  }
+  const __nv_bfloat162 c192 = __floats2bfloat162_rn(192.0f, 192.0f);
+#pragma unroll
+  for (int s = S - 1; s >= 0; --s) {
+    uint32_t r[4];
+    const int p = S - 1 - s;  // field position, 7 p bits up
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      if (s == 0) {
+        const int sh = 7 * (S - 1) - 28;
+        r[h] = __byte_perm(bf16_bits_of_small(w1[2 * h] >> sh), bf16_bits_of_small(w1[2 * h + 1] >> sh), 0x7632);
+      } else {
+        const int sh = 7 * (p & 3);
+        const uint32_t a = p < 4 ? w0[2 * h] : uint32_t(w1[2 * h]);
+        const uint32_t b = p < 4 ? w0[2 * h + 1] : uint32_t(w1[2 * h + 1]);
+        const uint32_t bu = sh <= 16 ? b << (16 - sh) : b >> (sh - 16);
+        const uint32_t t = ((a >> sh) & 0x7Fu) | (bu & 0x7F0000u) | 0x43004300u;
+        const __nv_bfloat162 d = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&t), c192);
+        r[h] = *reinterpret_cast<const uint32_t*>(&d);
+      }
+    }
+    *reinterpret_cast<uint4*>(out + int64_t(s) * tile_elems) = make_uint4(r[0], r[1], r[2], r[3]);
+  }
+}
+
+struct OzSliceArgs {
+  const double* src;
+  int64_t sr, sk;  // element (r, k) at src[row(r) sr + k sk]
+  int64_t rows, K;
+  const double* kw;
+  double mul;
+  const int* ridx;  // row(r) = ridx[r] (nullable: r)
+  int rt;
+  int64_t nrt, kst;
+  int64_t kg0, ngrp;  // window of 8-wide k groups
+  int* exps;
+  __nv_bfloat16* tiles;  // tile (row tile i, k tile j) at position i * kst + j
+};
+
+__device__ __forceinline__ const double* oz_row(const OzSliceArgs& A, int64_t r) {
+  return A.src + (A.ridx ? int64_t(A.ridx[r]) : r) * A.sr;
+}
+
+template <int S>
+__device__ __forceinline__ void oz_emit(const OzSliceArgs& A, int64_t r, int64_t kg, int e, double (&v)[8]) {
+  oz_weight8(v, A.K, kg, A.kw, A.mul);
+  const int64_t it = r / A.rt, jt = kg / (kBK / 8);
+  const int rr = int(r - it * A.rt), kc = int(kg % (kBK / 8));
+  const int64_t tile_elems = int64_t(A.rt) * kBK;
+  __nv_bfloat16* out = A.tiles + ((it * A.kst + jt) * S) * tile_elems + (rr >> 3) * (8 * kBK) + kc * 64 + (rr & 7) * 8;
+  oz_digits8<S>(v, 7 * S - e, tile_elems, out);
+}
+
+// Digits of a window of k groups for rows whose scales are in exps (padding
+// rows are written as zero).  RG 32 (rows adjacent in memory): a warp takes 32
+// rows of one k group; RG 8 (k adjacent): 8 rows x 4 k groups, so it writes one
+// 512-byte line of each slice and reads 256 contiguous bytes of each row.
+template <int S, int RG>
+__global__ void __launch_bounds__(256) k_oz_digits(OzSliceArgs A) {
+  constexpr int KG = 32 / RG;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t rows_pad = A.nrt * A.rt;
+  if (RG == 32) {
+    const int64_t r = (int64_t(blockIdx.x) * 8 + warp) * 32 + lane;
     if (r >= rows_pad) return;
-    for (int64_t g = blockIdx.y; g < ngrp; g += gridDim.y)
-      oz_digit_group<S>(src, rm, km, rows, K, kw, mul, exps, rt, kst, ridx, tiles, int(r), kg0 + g);
+    const bool live = r < A.rows;
+    const int e = live ? A.exps[r] : 0;
+    const double* row = live ? oz_row(A, r) : A.src;
+    for (int64_t g = blockIdx.y; g < A.ngrp; g += gridDim.y) {
+      double v[8];
+      oz_load8(row, live, A.sk, A.K, A.kg0 + g, v);
+      oz_emit<S>(A, r, A.kg0 + g, e, v);
+    }
   } else {
-    const int lane = threadIdx.x & 31;
-    const int64_t g = (int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 4 + (lane >> 3);
-    if (g >= ngrp) return;
-    for (int64_t g8 = blockIdx.y; g8 * 8 < rows_pad; g8 += gridDim.y)
-      oz_digit_group<S>(src, rm, km, rows, K, kw, mul, exps, rt, kst, ridx, tiles, int(g8 * 8 + (lane & 7)),
-                        kg0 + g);
+    const int64_t g = (int64_t(blockIdx.x) * 8 + warp) * KG + lane / RG;
+    if (g >= A.ngrp) return;
+    for (int64_t g8 = blockIdx.y; g8 * 8 < rows_pad; g8 += gridDim.y) {
+      const int64_t r = g8 * 8 + lane % RG;
+      const bool live = r < A.rows;
+      double v[8];
+      oz_load8(live ? oz_row(A, r) : A.src, live, A.sk, A.K, A.kg0 + g, v);
+      oz_emit<S>(A, r, A.kg0 + g, live ? A.exps[r] : 0, v);
+    }
+  }
+}
+
+// Row scales and digits of a whole operand in one launch.  A block owns RG
+// rows: it takes their maxima over all k, then reads the same values again,
+// from L1 or L2, and writes their digits: one pass over HBM.  (One thread per
+// row for the maximum and a second kernel for the digits read the operand
+// twice and left a short operand to a few serial threads.)  Blocks are small,
+// so that an SM holds many at different points of the two passes.  Bound by
+// HBM (8 B read and 2 S written per value) and the latency of the two passes;
+// measured: 250001 x 607, 8 digits, 1.89 -> 0.94 ms (3.9 TB/s); 131072 x 832,
+// 5 digits, 1.37 -> 0.65 ms; 96 gathered rows of 200 values, 50 -> 7 us.
+template <int S, int RG>
+__global__ void __launch_bounds__(512, 2) k_oz_slice(OzSliceArgs A) {
+  constexpr int KG = 32 / RG;
+  __shared__ unsigned long long key[RG];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int rl = lane % RG;
+  const int64_t r = int64_t(blockIdx.x) * RG + rl;
+  const bool live = r < A.rows;  // rows up to the tile height are padding, written as zero
+  const double* row = live ? oz_row(A, r) : A.src;
+  const int64_t g0 = int64_t(warp) * KG + lane / RG, gs = int64_t(nw) * KG;
+  double v[8];
+  uint64_t m = 0;
+  if (live)
+#pragma unroll 2
+    for (int64_t g = g0; g < A.ngrp; g += gs) {
+      oz_load8(row, true, A.sk, A.K, g, v);
+      const int64_t k0 = g * 8;
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (k0 + u < A.K) m = umax64(m, key_at(v[u], k0 + u, A.kw, A.mul));
+    }
+  if (RG == 8) {
+    m = umax64(m, __shfl_xor_sync(0xffffffffu, m, 8));
+    m = umax64(m, __shfl_xor_sync(0xffffffffu, m, 16));
+  }
+  if (nw > 1) {
+    if (threadIdx.x < RG) key[threadIdx.x] = 0ull;
+    __syncthreads();
+    if (lane < RG) atomicMax(&key[rl], (unsigned long long)m);
+    __syncthreads();
+    m = key[rl];
+  }
+  const int e = exp_of_key(m);
+  if (live && warp == 0 && lane < RG) A.exps[r] = e;
+  if (r >= A.nrt * A.rt) return;  // a 32-row block past the last (48-row) tile
+  const bool once = gs >= A.ngrp;  // every thread's only group is still in registers
+  for (int64_t g = g0; g < A.ngrp; g += gs) {
+    if (!once || !live) oz_load8(row, live, A.sk, A.K, g, v);
+    oz_emit<S>(A, r, g, e, v);
   }
 }
 
@@ -481,30 +523,81 @@ __global__ void k_oz_retile(const __nv_bfloat16* __restrict__ src, int src_rt, i
   }
 }
 
-void launch_digits(const double* src, OzMap rm, OzMap km, const double* kw, double mul, const int* ridx,
-                   const OzOperand& op, int64_t kg0, int64_t ngrp, int order, cudaStream_t s) {
-  const int64_t rows_pad = op.nrt * op.rt;
-  dim3 grid;
-  if (order == 0) {
-    grid.x = unsigned((rows_pad + 255) / 256);
-    grid.y = unsigned(std::min<int64_t>(ngrp, 65535));
-  } else {
-    grid.x = unsigned(((ngrp + 3) / 4 + 7) / 8);
-    grid.y = unsigned(std::min<int64_t>(rows_pad / 8, 65535));
-  }
-  __nv_bfloat16* t = static_cast<__nv_bfloat16*>(op.tiles);
-  if (op.S == 7)
-    k_oz_digits<7><<<grid, 256, 0, s>>>(src, rm, km, op.rows, op.K, kw, mul, op.exps, op.rt, op.nrt, kg0, ngrp,
-                                        op.kst, order, ridx, t);
-  else if (op.S == 5)
-    k_oz_digits<5><<<grid, 256, 0, s>>>(src, rm, km, op.rows, op.K, kw, mul, op.exps, op.rt, op.nrt, kg0, ngrp,
-                                        op.kst, order, ridx, t);
-  else if (op.S == 6)
-    k_oz_digits<6><<<grid, 256, 0, s>>>(src, rm, km, op.rows, op.K, kw, mul, op.exps, op.rt, op.nrt, kg0, ngrp,
-                                        op.kst, order, ridx, t);
+OzSliceArgs slice_args(const double* src, int64_t sr, int64_t sk, const double* kw, double mul, const int* ridx,
+                       const OzOperand& op, int64_t kg0, int64_t ngrp) {
+  return {src, sr, sk, op.rows, op.K, kw, mul, ridx, op.rt, op.nrt, op.kst, kg0, ngrp, op.exps,
+          static_cast<__nv_bfloat16*>(op.tiles)};
+}
+
+template <int S>
+void launch_digits_s(const OzSliceArgs& A, cudaStream_t s) {
+  const int64_t rows_pad = A.nrt * A.rt;
+  if (A.sr < A.sk)
+    k_oz_digits<S, 32><<<dim3(unsigned((rows_pad + 255) / 256), unsigned(std::min<int64_t>(A.ngrp, 65535))), 256, 0, s>>>(A);
   else
-    k_oz_digits<8><<<grid, 256, 0, s>>>(src, rm, km, op.rows, op.K, kw, mul, op.exps, op.rt, op.nrt, kg0, ngrp,
-                                        op.kst, order, ridx, t);
+    k_oz_digits<S, 8><<<dim3(unsigned((A.ngrp + 31) / 32), unsigned(std::min<int64_t>(rows_pad / 8, 65535))), 256, 0, s>>>(A);
+}
+
+void launch_digits(const OzSliceArgs& A, int S, cudaStream_t s) {
+  if (S == 5) launch_digits_s<5>(A, s);
+  else if (S == 6) launch_digits_s<6>(A, s);
+  else if (S == 7) launch_digits_s<7>(A, s);
+  else launch_digits_s<8>(A, s);
+  count_launches(1);
+}
+
+// Rows adjacent in memory (sr < sk) are taken 32 to a block when there are
+// enough of them for every SM, else 8 to a block (64-byte pieces of a
+// line, but four times the blocks); rows with k adjacent always 8 to a block.
+constexpr int64_t kWideRows = 2 * 152 * 32;
+// Warps per block: an SM holds 32 warps of this kernel, and the rows it is
+// working on have to stay in L2 between the two reads: at most about 320 KB an
+// SM (48 MB in all).  With fewer blocks than that, more warps share a row.
+constexpr int64_t kSliceBytes = 320 * 1024;
+
+template <int S>
+void launch_slice_s(const OzSliceArgs& A, cudaStream_t s) {
+  const int64_t rows_pad = A.nrt * A.rt;
+  const bool wide = A.sr < A.sk && rows_pad >= kWideRows;
+  const int rg = wide ? 32 : 8, kg = 32 / rg;
+  const int64_t blocks = (rows_pad + rg - 1) / rg;
+  int nw = 1;
+  while (nw < 16 && nw * kg < A.ngrp && (32 / nw * rg * A.K * 8 > kSliceBytes || blocks * nw < 152 * 32)) nw *= 2;
+  const unsigned grid = unsigned(blocks);
+  if (wide)
+    k_oz_slice<S, 32><<<grid, 32 * nw, 0, s>>>(A);
+  else
+    k_oz_slice<S, 8><<<grid, 32 * nw, 0, s>>>(A);
+}
+
+// Row scales, then digits, of a whole operand.  Rows of up to kFusedK values
+// with k adjacent (and every operand with rows adjacent) go through the fused
+// kernel; longer rows would fall out of L2 between its two reads (two blocks an
+// SM, 8 rows each: 80 MB at 4096 values), so their maxima are taken first by
+// blocks that share each row.
+constexpr int64_t kFusedK = 4096;
+
+void slice_operand(const OzSliceArgs& A, int S, cudaStream_t s) {
+  if (A.sr < A.sk || A.K <= kFusedK || A.ridx) {
+    if (S == 5) launch_slice_s<5>(A, s);
+    else if (S == 6) launch_slice_s<6>(A, s);
+    else if (S == 7) launch_slice_s<7>(A, s);
+    else launch_slice_s<8>(A, s);
+    count_launches(1);
+    return;
+  }
+  // the keys use the head of the operand's own tiles, which the digits overwrite afterwards
+  unsigned long long* keys = reinterpret_cast<unsigned long long*>(A.tiles);
+  cudaMemsetAsync(keys, 0, sizeof(unsigned long long) * size_t(A.rows), s);
+  // enough shares per row for about 8 waves of blocks, at least 4096 values each
+  int64_t nsh = std::max<int64_t>(1, std::min<int64_t>((int64_t(152) * 64 + A.rows - 1) / A.rows, A.K / 4096));
+  int64_t share = (A.K + nsh - 1) / nsh;
+  share += share & 1;
+  nsh = (A.K + share - 1) / share;
+  k_oz_row_keys<<<dim3(unsigned(A.rows), unsigned(nsh)), 256, 0, s>>>(A.src, A.sr, A.K, share, A.kw, A.mul, keys);
+  k_oz_key_exps<<<unsigned((A.rows + 255) / 256), 256, 0, s>>>(keys, A.rows, A.exps);
+  count_launches(2);
+  launch_digits(A, S, s);
 }
 
 // ---------------------------------------------------------------- GEMM
@@ -955,17 +1048,7 @@ void oz_free(OzOperand& op) {
 }
 
 void oz_slice(const double* src, int64_t sr, int64_t sk, const double* kw, double mul, OzOperand& op, cudaStream_t s) {
-  const bool rowwise = sr >= sk;  // k contiguous: one block per row
-  const OzMap rm = oz_stride(sr), km = oz_stride(sk);
-  if ((rowwise && op.K >= 4096) || (op.K >= 256 && op.rows <= 8192)) {
-    // few long rows: one block per row (a thread per row would stream its row alone)
-    k_oz_rowexp_block<<<unsigned(op.rows), 256, 0, s>>>(src, rm, km, op.K, kw, mul, nullptr, op.exps);
-  } else {
-    k_oz_rowexp_thread<<<unsigned((op.rows + 255) / 256), 256, 0, s>>>(src, rm, km, op.rows, op.K, kw, mul, nullptr,
-                                                                        op.exps);
-  }
-  launch_digits(src, rm, km, kw, mul, nullptr, op, 0, op.nkt * (kBK / 8), rowwise ? 1 : 0, s);
-  count_launches(2);
+  slice_operand(slice_args(src, sr, sk, kw, mul, nullptr, op, 0, op.nkt * (kBK / 8)), op.S, s);
 }
 
 void oz_retile(const OzOperand& from, OzOperand& to, cudaStream_t s) {
@@ -982,19 +1065,11 @@ void oz_retile(const OzOperand& from, OzOperand& to, cudaStream_t s) {
 void oz_slice_ex(const double* src, int64_t sr, int64_t sk, const int* ridx, OzOperand& op, int64_t kg0, int64_t kg1,
                  bool exps_ready, cudaStream_t s) {
   if (op.rows <= 0 || kg1 <= kg0) return;
-  const bool rowwise = sr >= sk;
-  const OzMap rm = oz_stride(sr), km = oz_stride(sk);
-  if (!exps_ready) {
-    // few long rows (a gathered set of rows with large K): one block per row
-    if ((rowwise && op.K >= 4096) || (op.K >= 256 && op.rows <= 8192))
-      k_oz_rowexp_block<<<unsigned(op.rows), 256, 0, s>>>(src, rm, km, op.K, nullptr, 1.0, ridx, op.exps);
-    else
-      k_oz_rowexp_thread<<<unsigned((op.rows + 255) / 256), 256, 0, s>>>(src, rm, km, op.rows, op.K, nullptr, 1.0,
-                                                                          ridx, op.exps);
-    count_launches(1);
-  }
-  launch_digits(src, rm, km, nullptr, 1.0, ridx, op, kg0, kg1 - kg0, rowwise ? 1 : 0, s);
-  count_launches(1);
+  const OzSliceArgs A = slice_args(src, sr, sk, nullptr, 1.0, ridx, op, kg0, kg1 - kg0);
+  if (exps_ready)
+    launch_digits(A, op.S, s);
+  else
+    slice_operand(A, op.S, s);  // scales need every group: callers pass the whole range
 }
 
 // S levels x BN columns of tensor memory: 5 x 48 (two CTAs per SM), 6 x 64, 7 x 48, 8 x 48
