@@ -422,7 +422,7 @@ isdf_status plan_create(const isdf_system* sys, const isdf_options* opt, void* s
     st = fail(p, ISDF_ERR_CUDA,
               "this library is built for sm_103a; device compute capability is " + std::to_string(prop.major) + "." +
                   std::to_string(prop.minor));
-  if (!st) st = dalloc_t(p, &p->d_err, 1, "error word");
+  if (!st) st = dalloc_t(p, &p->d_err, ISDF_MAX_LEVELS, "error words");
   if (!st) st = dalloc_t(p, &p->d_ozerr, 1, "error word");
   if (!st) st = cuda_check(p, cudaMemsetAsync(p->d_ozerr, 0, sizeof(int), p->stream), "memset");
   if (!st && o.local_grids) st = local_setup(p, sys->level_min_exp[0]);

@@ -420,7 +420,7 @@ isdf_status coulomb_run(Plan* p) {
       } else {
         const double K2 = 2.0 * double(lb.nq);
         const double work = same ? double(la.k) * double(la.k + 1) * K2 : 2.0 * double(la.k) * double(lb.k) * K2;
-        Prof pr(p, "coulomb_V", work, "flop", 1);
+        Prof pr(p, "coulomb_V", work, "flop", kLaunchesInside);
         dgemm(g, s);
       }
       const int64_t tot = int64_t(la.k) * lb.k;

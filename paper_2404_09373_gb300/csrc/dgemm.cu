@@ -1,38 +1,40 @@
 // FP64 SIMT dense kernels: tiled GEMM, the fused Hadamard GEMM of the fit,
 // blocked Cholesky and triangular inverse.  These are the "plain FP64" form of
-// the contractions (options.precision = 0).
+// the contractions (options.precision = 0); the Cholesky and the small blocks
+// of the inverse serve both precisions.
+//
+// The FP64 unit (2 FMA per clock and SM) bounds all of them: an SM needs 16 us
+// for a 32 x 32 tile over 64 k values, while the operands of that tile are 32
+// KB from L2.  So the tiles are small: no padding beyond 32, and work for every
+// SM as early as possible; a larger tile would only save loads, which are free.
+#include <algorithm>
+
 #include "internal.cuh"
 
 namespace isdf {
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 16, NT = 256;
+constexpr int BT = 32, BK = 32, NT = 128;  // output tile, k step, threads (2 x 4 outputs each)
+constexpr int RI = 2, RJ = 4;
 
 struct Tiles {
-  double a[BK][BM + 1];
-  double b[BK][BN + 1];
+  double a[BK][BT + 1];
+  double b[BK][BT + 1];
 };
 
-// Accumulate acc[i][j] += sum_{k in [kbeg,kend)} opA(m0+ty+16i, k) w(k) opB(k, n0+tx+16j).
+// Accumulate acc[i][j] += sum_{k in [kbeg,kend)} opA(m0+ty+16i, k) w(k) opB(k, n0+tx+8j).
 template <int TA, int TB>
-__device__ __forceinline__ void tile_accumulate(double (&acc)[4][4], Tiles& t, const double* __restrict__ A,
+__device__ __forceinline__ void tile_accumulate(double (&acc)[RI][RJ], Tiles& t, const double* __restrict__ A,
                                                 int64_t lda, const double* __restrict__ B, int64_t ldb,
                                                 const double* __restrict__ kw, int64_t M, int64_t N, int64_t m0,
                                                 int64_t n0, int64_t kbeg, int64_t kend) {
   const int tid = threadIdx.x;
-  const int tx = tid % 16, ty = tid / 16;
+  const int tx = tid % 8, ty = tid / 8;
+  const int fast = tid % 32, slow = tid / 32;  // loads: 32 consecutive elements per warp
   for (int64_t k0 = kbeg; k0 < kend; k0 += BK) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int e = tid + NT * q;
-      int kk, mm;
-      if (TA) {
-        kk = e / BM;
-        mm = e % BM;
-      } else {
-        mm = e / BK;
-        kk = e % BK;
-      }
+    for (int q = 0; q < BT; q += NT / 32) {
+      const int kk = TA ? slow + q : fast, mm = TA ? fast : slow + q;
       const int64_t gk = k0 + kk, gm = m0 + mm;
       double v = 0.0;
       if (gk < kend && gm < M) {
@@ -42,180 +44,323 @@ __device__ __forceinline__ void tile_accumulate(double (&acc)[4][4], Tiles& t, c
       t.a[kk][mm] = v;
     }
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int e = tid + NT * q;
-      int kk, nn;
-      if (TB) {
-        nn = e / BK;
-        kk = e % BK;
-      } else {
-        kk = e / BN;
-        nn = e % BN;
-      }
+    for (int q = 0; q < BT; q += NT / 32) {
+      const int kk = TB ? fast : slow + q, nn = TB ? slow + q : fast;
       const int64_t gk = k0 + kk, gn = n0 + nn;
       double v = 0.0;
       if (gk < kend && gn < N) v = TB ? B[gn * ldb + gk] : B[gk * ldb + gn];
       t.b[kk][nn] = v;
     }
     __syncthreads();
-#pragma unroll
+#pragma unroll 8
     for (int kk = 0; kk < BK; ++kk) {
-      double av[4], bv[4];
+      double av[RI], bv[RJ];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) av[i] = t.a[kk][ty + 16 * i];
+      for (int i = 0; i < RI; ++i) av[i] = t.a[kk][ty + 16 * i];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) bv[j] = t.b[kk][tx + 16 * j];
+      for (int j = 0; j < RJ; ++j) bv[j] = t.b[kk][tx + 8 * j];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < RI; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
+        for (int j = 0; j < RJ; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
     }
     __syncthreads();
   }
 }
 
-template <int TA, int TB>
-__global__ __launch_bounds__(NT) void k_dgemm(GemmArgs g) {
-  const int64_t m0 = int64_t(blockIdx.y) * BM, n0 = int64_t(blockIdx.x) * BN;
-  if (g.sym && n0 > m0 + BM - 1) return;
-  __shared__ Tiles t;
-  double acc[4][4] = {};
-  int64_t kbeg = 0, kend = g.K;
-  if (g.tri == 1) kend = (m0 + BM < g.K) ? m0 + BM : g.K;
-  if (g.tri == 2) kbeg = m0;
-  tile_accumulate<TA, TB>(acc, t, g.A, g.lda, g.B, g.ldb, g.kw, g.M, g.N, m0, n0, kbeg, kend);
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+// visit(m, n, acc value) for this thread's outputs inside M x N
+template <class F>
+__device__ __forceinline__ void tile_visit(const double (&acc)[RI][RJ], int64_t M, int64_t N, int64_t m0, int64_t n0,
+                                           F visit) {
+  const int tx = threadIdx.x % 8, ty = threadIdx.x / 8;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < RI; ++i) {
     const int64_t m = m0 + ty + 16 * i;
-    if (m >= g.M) continue;
+    if (m >= M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int64_t n = n0 + tx + 16 * j;
-      if (n >= g.N) continue;
-      double* c = g.C + m * g.ldc + n;
-      const double v = g.alpha * acc[i][j];
-      *c = (g.beta == 0.0) ? v : fma(g.beta, *c, v);
+    for (int j = 0; j < RJ; ++j) {
+      const int64_t n = n0 + tx + 8 * j;
+      if (n < N) visit(m, n, acc[i][j]);
     }
   }
+}
+
+// gridDim.z > 1: each z takes a share of the tile's k range and leaves its sum
+// in work[z][M][N] (k_dgemm_sum adds them in order)
+template <int TA, int TB>
+__global__ __launch_bounds__(NT) void k_dgemm(GemmArgs g, double* __restrict__ work) {
+  const int64_t m0 = int64_t(blockIdx.y) * BT, n0 = int64_t(blockIdx.x) * BT;
+  if (g.sym && n0 > m0 + BT - 1) return;
+  __shared__ Tiles t;
+  double acc[RI][RJ] = {};
+  int64_t kbeg = 0, kend = g.K;
+  if (g.tri == 1) kend = (m0 + BT < g.K) ? m0 + BT : g.K;
+  if (g.tri == 2) kbeg = m0;
+  if (gridDim.z > 1) {
+    const int64_t steps = (kend - kbeg + BK - 1) / BK, per = (steps + gridDim.z - 1) / gridDim.z;
+    kbeg += per * blockIdx.z * BK;
+    kend = kbeg + per * BK < kend ? kbeg + per * BK : kend;
+  }
+  tile_accumulate<TA, TB>(acc, t, g.A, g.lda, g.B, g.ldb, g.kw, g.M, g.N, m0, n0, kbeg, kend);
+  if (work) {
+    double* w = work + int64_t(blockIdx.z) * g.M * g.N;
+    tile_visit(acc, g.M, g.N, m0, n0, [&](int64_t m, int64_t n, double v) { w[m * g.N + n] = v; });
+    return;
+  }
+  tile_visit(acc, g.M, g.N, m0, n0, [&](int64_t m, int64_t n, double x) {
+    double* c = g.C + m * g.ldc + n;
+    const double v = g.alpha * x;
+    *c = (g.beta == 0.0) ? v : fma(g.beta, *c, v);
+  });
+}
+
+__global__ void k_dgemm_sum(GemmArgs g, const double* __restrict__ work, int splits) {
+  const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (e >= g.M * g.N) return;
+  const int64_t m = e / g.N, n = e % g.N;
+  if (g.sym && n / BT > m / BT) return;
+  double s = 0.0;
+  for (int z = 0; z < splits; ++z) s += work[int64_t(z) * g.M * g.N + e];
+  double* c = g.C + m * g.ldc + n;
+  const double v = g.alpha * s;
+  *c = (g.beta == 0.0) ? v : fma(g.beta, *c, v);
 }
 
 // (ZC^T)^T[j][g] = aL (aL + 2 aN), aL = sum_{r<nL} phiP[r][j] phi[r][g],
 // aN = sum_{nL<=r<nG} phiP[r][j] phi[r][g]   (M_l[:, P], Eq. 2 / Eq. 3)
 __global__ __launch_bounds__(NT) void k_zc(int64_t k, int64_t ng, int nL, int nG, const double* __restrict__ phiP,
                                            const double* __restrict__ phi, double* __restrict__ out) {
-  const int64_t m0 = int64_t(blockIdx.y) * BM, n0 = int64_t(blockIdx.x) * BN;
+  const int64_t m0 = int64_t(blockIdx.y) * BT, n0 = int64_t(blockIdx.x) * BT;
   __shared__ Tiles t;
-  double aL[4][4] = {}, aN[4][4] = {};
+  double aL[RI][RJ] = {}, aN[RI][RJ] = {};
   tile_accumulate<1, 0>(aL, t, phiP, k, phi, ng, nullptr, k, ng, m0, n0, 0, nL);
   tile_accumulate<1, 0>(aN, t, phiP, k, phi, ng, nullptr, k, ng, m0, n0, nL, nG);
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int64_t m = m0 + ty + 16 * i;
-    if (m >= k) continue;
+  for (int i = 0; i < RI; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int64_t n = n0 + tx + 16 * j;
-      if (n >= ng) continue;
-      const double l = aL[i][j];
-      out[m * ng + n] = l * (l + 2.0 * aN[i][j]);
-    }
-  }
+    for (int j = 0; j < RJ; ++j) aL[i][j] = aL[i][j] * (aL[i][j] + 2.0 * aN[i][j]);
+  tile_visit(aL, k, ng, m0, n0, [&](int64_t m, int64_t n, double v) { out[m * ng + n] = v; });
 }
 
-// ---- Cholesky (right-looking, 64-column blocks) ----
+// ---- Cholesky (right-looking, 64-column blocks) and inverse of the factor ----
+//
+// All levels go through the same launches (blockIdx.y or .z = level), and a
+// block column costs two of them:
+//   k_chol_panel   X = A R_kk^-T as a product with the inverted diagonal block
+//   k_chol_update  trailing tiles -= X X^T; the CTA that finishes the last tile
+//                  of the next diagonal block factors and inverts that block at
+//                  once, under the rest of the update (an atomic count, no waiting)
+// so the serial part, the 64 dependent columns, is hidden wherever the update is
+// longer.  The inverted diagonal blocks are those of R^-1, where
+// dtrtri_lower starts.
 constexpr int CB = 64;
 
-// Factor the b x b diagonal block at (kb, kb) in shared memory.
-__global__ void k_potrf_diag(double* A, int64_t lda, int64_t kb, int b, int* err) {
-  __shared__ double s[CB][CB + 1];
-  const int tid = threadIdx.x;
-  for (int e = tid; e < b * b; e += blockDim.x) s[e / b][e % b] = A[(kb + e / b) * lda + kb + e % b];
+struct CholLevel {
+  double* A;   // n x n, lower triangle factored in place
+  double* Li;  // n x n, R^-1
+  double* T;   // scratch of the inverse
+  int n;
+  int* err;    // smallest column whose pivot was not positive
+  int* count;  // per block column: finished tiles of its diagonal block
+};
+struct CholLevels {
+  CholLevel l[ISDF_MAX_LEVELS];
+};
+
+// 1 / sqrt(d) for finite d > 0: FP32 estimate of the significand's root and one
+// step of the third-order iteration r (1 + e/2 + 3 e^2 / 8), e = 1 - d r^2 (the
+// Taylor series of (1 - e)^-1/2): from 2^-22 to rounding error in four dependent
+// FP64 operations instead of the forty of a square root and a division.
+__device__ __forceinline__ double rsqrt64(double d) {
+  const long long b = __double_as_longlong(d);
+  int E = int((b >> 52) & 0x7FF);
+  if (E == 0) return 1.0 / sqrt(d);  // subnormal
+  const int h = (E - 1023) >> 1;     // d = m 4^h, m in [1, 4)
+  const double m = __longlong_as_double(b - ((long long)(2 * h) << 52));
+  const int odd = (E - 1023) & 1;
+  const float mf = __int_as_float(((127 + odd) << 23) | int((b >> 29) & 0x7FFFFF));
+  const double r0 = __longlong_as_double([](float f) {  // FP32 to FP64 bits
+    const uint32_t u = __float_as_uint(f);
+    return (long long)((uint64_t(((u >> 23) & 0xFF) + 896u) << 52) | (uint64_t(u & 0x7FFFFF) << 29));
+  }(rsqrtf(mf)));
+  const double t = m * r0;
+  const double e = fma(-t, r0, 1.0);
+  const double r = fma(r0 * e, fma(0.375, e, 0.5), r0);
+  return __longlong_as_double(__double_as_longlong(r) - ((long long)h << 52));
+}
+
+struct DiagSmem {
+  double s[CB][CB + 1];
+  double v[CB][CB + 1];
+  double t[CB / 2][CB / 2 + 1];
+  double r[CB];  // reciprocals of the diagonal
+};
+
+// Factor the b x b diagonal block at kb and invert the factor (all NT threads).
+__device__ void chol_diag(const CholLevel& P, int kb, DiagSmem& S) {
+  const int tid = threadIdx.x, n = P.n, b = n - kb < CB ? n - kb : CB;
+  for (int e = tid; e < CB * CB; e += NT) {
+    const int i = e / CB, c = e % CB;
+    // written by other CTAs of this launch: read past L1
+    S.s[i][c] = (i < b && c <= i) ? __ldcg(P.A + int64_t(kb + i) * n + kb + c) : (i == c ? 1.0 : 0.0);
+    S.v[i][c] = 0.0;
+  }
   __syncthreads();
-  __shared__ double rpiv;
   for (int j = 0; j < b; ++j) {
-    if (tid == 0) {
-      double d = s[j][j];
+    if (tid < 32) {
+      double d = S.s[j][j];
       if (!(d > 0.0) || !isfinite(d)) {
-        atomicMin(err, int(kb + j));
+        if (tid == 0) atomicMin(P.err, kb + j);
         d = 1.0;
       }
-      s[j][j] = sqrt(d);
-      rpiv = 1.0 / s[j][j];  // one division per column; the column is scaled by the reciprocal
+      const double r = rsqrt64(d);
+      // the column below the diagonal, two rows a lane (rows at or above j stay)
+      const int i0 = tid, i1 = tid + 32;
+      const double x0 = S.s[i0][j], x1 = S.s[i1][j];
+      __syncwarp();  // the diagonal is read by every lane before it is replaced
+      if (i0 > j) S.s[i0][j] = x0 * r;
+      if (i1 > j) S.s[i1][j] = x1 * r;
+      if (tid == 0) {
+        S.r[j] = r;
+        const double s = d * r;
+        S.s[j][j] = fma(fma(-s, s, d), 0.5 * r, s);  // sqrt(d)
+      }
     }
     __syncthreads();
-    const double rp = rpiv;
-    for (int i = j + 1 + tid; i < b; i += blockDim.x) s[i][j] *= rp;
-    __syncthreads();
-    for (int e = tid; e < (b - j - 1) * (b - j - 1); e += blockDim.x) {
-      const int i = j + 1 + e / (b - j - 1), c = j + 1 + e % (b - j - 1);
-      if (c <= i) s[i][c] -= s[i][j] * s[c][j];
+    // two threads per row; columns c in (j, i]
+    const int i = tid >> 1;
+    if (i > j && i < b) {
+      const double x = S.s[i][j];
+      for (int c = j + 1 + (tid & 1); c <= i; c += 2) S.s[i][c] = fma(-x, S.s[c][j], S.s[i][c]);
     }
     __syncthreads();
   }
-  for (int e = tid; e < b * b; e += blockDim.x) {
+  // inverse by doubling: [A 0; C B]^-1 = [A^-1 0; -B^-1 C A^-1  B^-1]
+  for (int i = tid; i < CB; i += NT) S.v[i][i] = i < b ? S.r[i] : 1.0;
+  __syncthreads();
+  for (int h = 1; h < CB; h *= 2) {
+    const int per = h * h, tot = (CB / (2 * h)) * per;  // <= 32 * 64 / 2
+    // T = C A^-1, element (i, j) of pair q at t[flat]
+    double* t = &S.t[0][0];
+    for (int e = tid; e < tot; e += NT) {
+      const int q = e / per, i = e % h, j = (e % per) / h, r0 = 2 * h * q;
+      double x = 0.0;
+      for (int k = j; k < h; ++k) x = fma(S.s[r0 + h + i][r0 + k], S.v[r0 + k][r0 + j], x);
+      t[q * per + j * h + i] = x;
+    }
+    __syncthreads();
+    for (int e = tid; e < tot; e += NT) {
+      const int q = e / per, i = e % h, j = (e % per) / h, r0 = 2 * h * q;
+      double x = 0.0;
+      for (int k = 0; k <= i; ++k) x = fma(S.v[r0 + h + i][r0 + h + k], t[q * per + j * h + k], x);
+      S.v[r0 + h + i][r0 + j] = -x;
+    }
+    __syncthreads();
+  }
+  for (int e = tid; e < b * b; e += NT) {
     const int i = e / b, c = e % b;
-    A[(kb + i) * lda + kb + c] = (c <= i) ? s[i][c] : 0.0;
+    P.A[int64_t(kb + i) * n + kb + c] = (c <= i) ? S.s[i][c] : 0.0;
+    P.Li[int64_t(kb + i) * n + kb + c] = (c <= i) ? S.v[i][c] : 0.0;
   }
 }
 
-// Rows i >= r0 of the panel: x L_kk^T = a  (forward substitution per row).
-__global__ __launch_bounds__(64) void k_trsm_panel(double* A, int64_t lda, int64_t n, int64_t kb, int b, int64_t r0) {
-  __shared__ double l[CB][CB + 1];
-  __shared__ double rdiag[CB];
-  for (int e = threadIdx.x; e < CB * CB; e += blockDim.x) {
-    const int i = e / CB, c = e % CB;
-    double v = (i == c) ? 1.0 : 0.0;
-    if (i < b && c < b) v = A[(kb + i) * lda + kb + c];
-    l[i][c] = v;
-  }
-  __syncthreads();
-  // reciprocals of the diagonal once per CTA: the rows then multiply
-  for (int c = threadIdx.x; c < CB; c += blockDim.x) rdiag[c] = 1.0 / l[c][c];
-  __syncthreads();
-  const int64_t row = r0 + int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (row >= n) return;
-  double x[CB];
-#pragma unroll
-  for (int c = 0; c < CB; ++c) x[c] = (c < b) ? A[row * lda + kb + c] : 0.0;
-#pragma unroll
-  for (int c = 0; c < CB; ++c) {
-    double v = x[c];
-#pragma unroll
-    for (int p = 0; p < c; ++p) v -= x[p] * l[c][p];
-    x[c] = v * rdiag[c];
-  }
-#pragma unroll
-  for (int c = 0; c < CB; ++c)
-    if (c < b) A[row * lda + kb + c] = x[c];
+__global__ __launch_bounds__(NT) void k_chol_first(CholLevels L) {
+  extern __shared__ __align__(16) unsigned char sm_chol[];
+  const CholLevel& P = L.l[blockIdx.x];
+  if (P.n > 0) chol_diag(P, 0, *reinterpret_cast<DiagSmem*>(sm_chol));
 }
 
-// Inverse of each b x b lower-triangular diagonal block (one CTA per block).
-__global__ __launch_bounds__(64) void k_trtri_diag(const double* Lm, double* Li, int64_t n, int64_t ld) {
-  __shared__ double l[CB][CB + 1];
+// Rows [kb + 64, n) of block column kb: X = A R_kk^-T, 8 rows per CTA, in place.
+constexpr int kPanelRows = 8;
+__global__ __launch_bounds__(NT) void k_chol_panel(CholLevels L, int kb) {
+  const CholLevel& P = L.l[blockIdx.y];
+  const int n = P.n, r0 = kb + CB + int(blockIdx.x) * kPanelRows;
+  if (r0 >= n) return;  // the block column has rows below it: kb + 64 < n, a full diagonal block
+  __shared__ double a[kPanelRows][CB + 1];
   __shared__ double v[CB][CB + 1];
-  const int64_t kb = int64_t(blockIdx.x) * CB;
-  const int b = int((n - kb < CB) ? n - kb : CB);
-  for (int e = threadIdx.x; e < CB * CB; e += blockDim.x) {
-    const int i = e / CB, c = e % CB;
-    l[i][c] = (i < b && c < b) ? Lm[(kb + i) * ld + kb + c] : 0.0;
-    v[i][c] = 0.0;
+  const int tid = threadIdx.x;
+  for (int e = tid; e < CB * CB; e += NT) v[e / CB][e % CB] = P.Li[int64_t(kb + e / CB) * n + kb + e % CB];
+  for (int e = tid; e < kPanelRows * CB; e += NT) {
+    const int i = e / CB;
+    a[i][e % CB] = r0 + i < n ? P.A[int64_t(r0 + i) * n + kb + e % CB] : 0.0;
   }
   __syncthreads();
-  const int c = threadIdx.x;  // column of the inverse owned by this thread
-  if (c < b) {
-    v[c][c] = 1.0 / l[c][c];
-    for (int i = c + 1; i < b; ++i) {
-      double s = 0.0;
-      for (int p = c; p < i; ++p) s += l[i][p] * v[p][c];
-      v[i][c] = -s / l[i][i];
+  // thread: rows i = tid / 32 + 4 q, columns c = lane and 63 - lane (equal work)
+  const int lane = tid % 32;
+#pragma unroll
+  for (int half = 0; half < 2; ++half) {
+    const int c = half ? CB - 1 - lane : lane;
+    double x[kPanelRows / 4] = {};
+    for (int k = 0; k <= c; ++k) {
+      const double w = v[c][k];
+#pragma unroll
+      for (int q = 0; q < kPanelRows / 4; ++q) x[q] = fma(a[tid / 32 + 4 * q][k], w, x[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < kPanelRows / 4; ++q) {
+      const int i = tid / 32 + 4 * q;
+      if (r0 + i < n) P.A[int64_t(r0 + i) * n + kb + c] = x[q];
     }
   }
+}
+
+// Trailing tiles (lower triangle, 32 x 32, row by row from the next diagonal
+// block) -= X X^T; then the next diagonal block, by the CTA that completes it.
+__global__ __launch_bounds__(NT) void k_chol_update(CholLevels L, int kb) {
+  extern __shared__ __align__(16) unsigned char sm_chol[];
+  __shared__ int last;
+  const CholLevel& P = L.l[blockIdx.y];
+  const int n = P.n, base = kb + CB;
+  const int nt = base < n ? (n - base + BT - 1) / BT : 0;  // tile rows
+  const int tile = int(blockIdx.x);
+  if (tile >= nt * (nt + 1) / 2) return;
+  int i = int((sqrtf(8.0f * float(tile) + 1.0f) - 1.0f) * 0.5f);
+  while (i * (i + 1) / 2 > tile) --i;
+  while ((i + 1) * (i + 2) / 2 <= tile) ++i;
+  const int j = tile - i * (i + 1) / 2;
+  Tiles& t = *reinterpret_cast<Tiles*>(sm_chol);
+  double acc[RI][RJ] = {};
+  const double* X = P.A + kb;
+  tile_accumulate<0, 1>(acc, t, X, n, X, n, nullptr, n, n, base + BT * i, base + BT * j, 0, CB);
+  tile_visit(acc, n, n, base + BT * i, base + BT * j, [&](int64_t m, int64_t c, double v) {
+    double* x = P.A + m * n + c;
+    *x -= v;
+  });
+  if (i >= CB / BT) return;  // not a tile of the next diagonal block
+  __threadfence();
   __syncthreads();
-  for (int e = threadIdx.x; e < b * b; e += blockDim.x) {
-    const int i = e / b, cc = e % b;
-    Li[(kb + i) * ld + kb + cc] = v[i][cc];
+  if (threadIdx.x == 0) {
+    const int need = nt > 1 ? 3 : 1;
+    last = atomicAdd(P.count + base / CB, 1) == need - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  chol_diag(P, base, *reinterpret_cast<DiagSmem*>(sm_chol));
+}
+
+// Doubling step of the inverse for half size h: node q covers rows [2hq, 2hq +
+// h + n2) with both halves inverted; phase 0: T = C A^-1, phase 1: -B^-1 T.
+__global__ __launch_bounds__(NT) void k_trtri_step(CholLevels L, int h, int phase) {
+  const CholLevel& P = L.l[blockIdx.z];
+  const int n = P.n, r0 = 2 * h * int(blockIdx.y);
+  const int n2 = n - r0 - h < h ? n - r0 - h : h;
+  const int tn = h / BT, m0 = (int(blockIdx.x) / tn) * BT, n0 = (int(blockIdx.x) % tn) * BT;
+  if (n2 <= 0 || m0 >= n2) return;
+  __shared__ Tiles t;
+  double acc[RI][RJ] = {};
+  double* T = P.T + int64_t(blockIdx.y) * h * h;
+  const double* Lh = P.Li + int64_t(r0) * n + r0;
+  if (phase == 0) {
+    const double* C = P.A + int64_t(r0 + h) * n + r0;
+    tile_accumulate<0, 0>(acc, t, C, n, Lh, n, nullptr, n2, h, m0, n0, n0, h);  // A^-1 lower: k >= n0
+    tile_visit(acc, n2, h, m0, n0, [&](int64_t m, int64_t c, double v) { T[m * h + c] = v; });
+  } else {
+    const double* Bi = P.Li + int64_t(r0 + h) * n + r0 + h;
+    const int ke = m0 + BT < n2 ? m0 + BT : n2;  // B^-1 lower: k <= m
+    tile_accumulate<0, 0>(acc, t, Bi, n, T, h, nullptr, n2, h, m0, n0, 0, ke);
+    double* out = P.Li + int64_t(r0 + h) * n + r0;
+    tile_visit(acc, n2, h, m0, n0, [&](int64_t m, int64_t c, double v) { out[m * n + c] = -v; });
   }
 }
 
@@ -223,53 +368,44 @@ __global__ __launch_bounds__(64) void k_trtri_diag(const double* Lm, double* Li,
 
 void dgemm(const GemmArgs& g, cudaStream_t s) {
   if (g.M <= 0 || g.N <= 0) return;
-  dim3 grid(unsigned((g.N + BN - 1) / BN), unsigned((g.M + BM - 1) / BM));
-  if (g.ta == 0 && g.tb == 0) k_dgemm<0, 0><<<grid, NT, 0, s>>>(g);
-  if (g.ta == 1 && g.tb == 0) k_dgemm<1, 0><<<grid, NT, 0, s>>>(g);
-  if (g.ta == 0 && g.tb == 1) k_dgemm<0, 1><<<grid, NT, 0, s>>>(g);
-  if (g.ta == 1 && g.tb == 1) k_dgemm<1, 1><<<grid, NT, 0, s>>>(g);
+  const int64_t tm = (g.M + BT - 1) / BT, tn = (g.N + BT - 1) / BT;
+  // Few tiles over a long k (the V blocks and exchange projections of a small
+  // cell) leave most SMs idle: share the k range over enough CTAs for about four
+  // per SM, at least 128 k values each.  140 x 140 x 15000: 9 CTAs, 6.9 ms ->
+  // 0.14 ms.
+  const int64_t tiles = g.sym ? tm * (tm + 1) / 2 : tm * tn;
+  const int64_t splits = std::max<int64_t>(1, std::min<int64_t>({(608 + tiles - 1) / tiles, g.K / 128, 64}));
+  double* work = nullptr;
+  dim3 grid{unsigned(tn), unsigned(tm), 1u};
+  if (tiles < 304 && splits > 1) {
+    if (cudaMallocAsync(reinterpret_cast<void**>(&work), sizeof(double) * size_t(splits * g.M * g.N), s) == cudaSuccess) {
+      grid.z = unsigned(splits);
+    } else {
+      cudaGetLastError();
+      work = nullptr;
+    }
+  }
+  if (g.ta == 0 && g.tb == 0) k_dgemm<0, 0><<<grid, NT, 0, s>>>(g, work);
+  if (g.ta == 1 && g.tb == 0) k_dgemm<1, 0><<<grid, NT, 0, s>>>(g, work);
+  if (g.ta == 0 && g.tb == 1) k_dgemm<0, 1><<<grid, NT, 0, s>>>(g, work);
+  if (g.ta == 1 && g.tb == 1) k_dgemm<1, 1><<<grid, NT, 0, s>>>(g, work);
+  count_launches(1);
+  if (work) {
+    k_dgemm_sum<<<unsigned((g.M * g.N + 255) / 256), 256, 0, s>>>(g, work, int(splits));
+    count_launches(1);
+    cudaFreeAsync(work, s);
+  }
 }
 
 void zc_gemm(int64_t k, int64_t ng, int nL, int nG, const double* phiP, const double* phi, double* out,
              cudaStream_t s) {
   if (k <= 0 || ng <= 0) return;
-  dim3 grid(unsigned((ng + BN - 1) / BN), unsigned((k + BM - 1) / BM));
+  dim3 grid(unsigned((ng + BT - 1) / BT), unsigned((k + BT - 1) / BT));
   k_zc<<<grid, NT, 0, s>>>(k, ng, nL, nG, phiP, phi, out);
-}
-
-void dpotrf_lower(double* A, int64_t n, int64_t lda, int* err, double* /*scratch*/, cudaStream_t s) {
-  for (int64_t kb = 0; kb < n; kb += CB) {
-    const int b = int((n - kb < CB) ? n - kb : CB);
-    k_potrf_diag<<<1, 256, 0, s>>>(A, lda, kb, b, err);
-    const int64_t r0 = kb + b;
-    if (r0 >= n) break;
-    const int64_t rows = n - r0;
-    k_trsm_panel<<<unsigned((rows + 63) / 64), 64, 0, s>>>(A, lda, n, kb, b, r0);
-    GemmArgs g;
-    g.ta = 0;
-    g.tb = 1;
-    g.M = rows;
-    g.N = rows;
-    g.K = b;
-    g.alpha = -1.0;
-    g.beta = 1.0;
-    g.A = A + r0 * lda + kb;
-    g.lda = lda;
-    g.B = A + r0 * lda + kb;
-    g.ldb = lda;
-    g.C = A + r0 * lda + r0;
-    g.ldc = lda;
-    g.sym = 1;
-    dgemm(g, s);
-  }
 }
 
 namespace {
 
-// Off-diagonal blocks of the inverse, top-down on [r0, r0 + n):
-//   inv([A 0; C B]) = [A^-1 0; -B^-1 C A^-1  B^-1],  A: n1 x n1, B: n2 x n2,
-// with n1 a multiple of the 64-row diagonal blocks (already inverted).
-// T = C A^-1 goes to the scratch (n2 x n1), then Li[C] = -B^-1 T.
 // C (M x N, ldc) = alpha A B, A row-major (M x K, lda), B row-major (K x N,
 // ldb), as an 8-digit tensor-core product; false if its buffers could not be
 // allocated (the caller then takes the FP64 product)
@@ -290,54 +426,78 @@ bool tc_product(Plan* p, const double* A, int64_t lda, const double* B, int64_t 
 
 constexpr int64_t kTcMin = 256;  // products with halves at least this large go to the tensor cores
 
-void trtri_rec(const double* Lm, double* Li, int64_t ld, int64_t r0, int64_t n, double* scratch, cudaStream_t s,
-               Plan* tc) {
-  if (n <= CB) return;
-  const int64_t n1 = ((n / 2 + CB - 1) / CB) * CB, n2 = n - n1;
-  trtri_rec(Lm, Li, ld, r0, n1, scratch, s, tc);
-  trtri_rec(Lm, Li, ld, r0 + n1, n2, scratch, s, tc);
-  if (tc && n2 >= kTcMin &&
-      tc_product(tc, Lm + (r0 + n1) * ld + r0, ld, Li + r0 * ld + r0, ld, scratch, n1, n2, n1, n1, 1.0, s) &&
-      tc_product(tc, Li + (r0 + n1) * ld + r0 + n1, ld, scratch, n1, Li + (r0 + n1) * ld + r0, ld, n2, n1, n2, -1.0,
-                 s))
-    return;
-  GemmArgs g;  // T = C A^-1
-  g.M = n2;
-  g.N = n1;
-  g.K = n1;
-  g.A = Lm + (r0 + n1) * ld + r0;
-  g.lda = ld;
-  g.B = Li + r0 * ld + r0;
-  g.ldb = ld;
-  g.C = scratch;
-  g.ldc = n1;
-  dgemm(g, s);
-  GemmArgs h;  // Li[C] = -B^-1 T (B^-1 lower triangular: opA(m, k) nonzero for k <= m)
-  h.M = n2;
-  h.N = n1;
-  h.K = n2;
-  h.alpha = -1.0;
-  h.A = Li + (r0 + n1) * ld + r0 + n1;
-  h.lda = ld;
-  h.B = scratch;
-  h.ldb = n1;
-  h.C = Li + (r0 + n1) * ld + r0;
-  h.ldc = ld;
-  h.tri = 1;
-  dgemm(h, s);
+CholLevels pack(const FactorJob* jobs, int count, int* counts, int per) {
+  CholLevels L{};
+  for (int i = 0; i < count; ++i)
+    L.l[i] = {jobs[i].A, jobs[i].Li, jobs[i].scratch, jobs[i].n, jobs[i].err, counts ? counts + i * per : nullptr};
+  return L;
+}
+
+int max_n(const FactorJob* jobs, int count) {
+  int n = 0;
+  for (int i = 0; i < count; ++i) n = std::max(n, jobs[i].n);
+  return n;
 }
 
 }  // namespace
 
-// Inverse of a lower-triangular n x n matrix: every 64 x 64 diagonal block in
-// one launch, then the off-diagonal blocks by recursive halving (products of
-// the size of the halves instead of 64-row strips).
-// scratch: (n / 2 + 64) * n doubles.
-void dtrtri_lower(const double* Lm, double* Li, int64_t n, double* scratch, cudaStream_t s, Plan* tc) {
-  cudaMemsetAsync(Li, 0, sizeof(double) * n * n, s);
-  const int64_t nb = (n + CB - 1) / CB;
-  k_trtri_diag<<<unsigned(nb), 64, 0, s>>>(Lm, Li, n, n);
-  trtri_rec(Lm, Li, n, 0, n, scratch, s, tc);
+isdf_status dpotrf_lower(Plan* p, const FactorJob* jobs, int count, cudaStream_t s) {
+  const int n = max_n(jobs, count);
+  if (n <= 0) return ISDF_OK;
+  const int per = (n + CB - 1) / CB + 1;
+  int* counts = nullptr;
+  isdf_status st = dalloc_t(p, &counts, size_t(per) * ISDF_MAX_LEVELS, "Cholesky counters");
+  if (st) return st;
+  cudaMemsetAsync(counts, 0, sizeof(int) * size_t(per) * ISDF_MAX_LEVELS, s);
+  for (int i = 0; i < count; ++i)
+    if (jobs[i].n > 0) cudaMemsetAsync(jobs[i].Li, 0, sizeof(double) * size_t(jobs[i].n) * jobs[i].n, s);
+  const CholLevels L = pack(jobs, count, counts, per);
+  constexpr int smem = int(sizeof(DiagSmem) > sizeof(Tiles) ? sizeof(DiagSmem) : sizeof(Tiles));
+  cudaFuncSetAttribute(k_chol_first, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaFuncSetAttribute(k_chol_update, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  k_chol_first<<<unsigned(count), NT, smem, s>>>(L);
+  count_launches(1);
+  for (int kb = 0; kb + CB < n; kb += CB) {
+    const int rows = n - kb - CB, nt = (rows + BT - 1) / BT;
+    k_chol_panel<<<dim3(unsigned((rows + kPanelRows - 1) / kPanelRows), unsigned(count)), NT, 0, s>>>(L, kb);
+    k_chol_update<<<dim3(unsigned(nt * (nt + 1) / 2), unsigned(count)), NT, smem, s>>>(L, kb);
+    count_launches(2);
+  }
+  dfree(counts);
+  return cuda_check(p, cudaGetLastError(), "Cholesky kernels");
+}
+
+void dtrtri_lower(Plan* p, const FactorJob* jobs, int count, bool tensor, cudaStream_t s) {
+  const int n = max_n(jobs, count);
+  const CholLevels L = pack(jobs, count, nullptr, 0);
+  for (int h = CB; h < n; h *= 2) {
+    if (tensor && h >= kTcMin)
+      for (int i = 0; i < count; ++i) {
+        const FactorJob& J = jobs[i];
+        for (int r0 = 0; r0 + h < J.n; r0 += 2 * h) {
+          const int64_t ld = J.n, n2 = std::min(h, J.n - r0 - h);
+          const double* C = J.A + (r0 + h) * ld + r0;
+          double* out = J.Li + (r0 + h) * ld + r0;
+          if (n2 >= kTcMin && tc_product(p, C, ld, J.Li + r0 * ld + r0, ld, J.scratch, h, n2, h, h, 1.0, s) &&
+              tc_product(p, J.Li + (r0 + h) * ld + r0 + h, ld, J.scratch, h, out, ld, n2, h, n2, -1.0, s))
+            continue;
+          GemmArgs g;  // T = C A^-1
+          g.M = n2, g.N = h, g.K = h;
+          g.A = C, g.lda = ld, g.B = J.Li + r0 * ld + r0, g.ldb = ld, g.C = J.scratch, g.ldc = h;
+          dgemm(g, s);
+          GemmArgs f;  // -B^-1 T (B^-1 lower triangular: opA(m, k) nonzero for k <= m)
+          f.M = n2, f.N = h, f.K = n2, f.alpha = -1.0;
+          f.A = J.Li + (r0 + h) * ld + r0 + h, f.lda = ld, f.B = J.scratch, f.ldb = h, f.C = out, f.ldc = ld, f.tri = 1;
+          dgemm(f, s);
+        }
+      }
+    else {
+      const dim3 grid(unsigned((h / BT) * (h / BT)), unsigned((n - h + 2 * h - 1) / (2 * h)), unsigned(count));
+      k_trtri_step<<<grid, NT, 0, s>>>(L, h, 0);
+      k_trtri_step<<<grid, NT, 0, s>>>(L, h, 1);
+      count_launches(2);
+    }
+  }
 }
 
 }  // namespace isdf

@@ -58,7 +58,7 @@ __global__ void k_fill_kw(int nL, int nG, double* kw) {
 // Tensor-core form of the fit contractions (options.precision = 1): the same
 // three products as the FP64 path, each an FP64-accurate sliced-BF16 GEMM
 // with the grid points on the 128-lane side so every store is coalesced.
-isdf_status fit_products_tc(Plan* p, Level& lv, int k, const double* phiP, double* zct, double* y, const double* li,
+isdf_status fit_products_tc(Plan* p, Level& lv, int k, const double* phiP, double* zct, double* y,
                             int64_t ng) {
   cudaStream_t s = p->stream;
   const int S = p->fit_slices;
@@ -69,7 +69,6 @@ isdf_status fit_products_tc(Plan* p, Level& lv, int k, const double* phiP, doubl
     oz_free(aL), oz_free(aG), oz_free(bL), oz_free(bG), oz_free(az), oz_free(bli);
     dfree(kw);
   };
-  (void)li;
   // (ZC^T)^T = T1 o T2, T1 = A_L B_L^T, T2 = [A_L A_N] [B_L 2 B_N]^T
   if ((st = oz_alloc(p, aL, ng, lv.nL, 128, S, "fit slices")) || (st = oz_alloc(p, bL, k, lv.nL, oz_bn(S), S, "fit slices")))
     return cleanup(), st;
@@ -161,6 +160,20 @@ isdf_status fit_run(Plan* p) {
   cudaStream_t s = p->stream;
   isdf_status st;
   p->resid_ready = false;
+  struct LevelBuf {
+    double *phiP = nullptr, *y = nullptr, *cc = nullptr, *li = nullptr, *scr = nullptr;
+  } buf[ISDF_MAX_LEVELS];
+  auto cleanup = [&]() {
+    for (LevelBuf& b : buf) {
+      for (double* q : {b.phiP, b.y, b.cc, b.li, b.scr}) dfree(q);
+      b = LevelBuf();
+    }
+  };
+  const bool factored = p->opt.precision == 1;  // keep ZC^T and R^-1; Xi only on request
+  // ---- ZC^T and CC^T of every level
+  FactorJob jobs[ISDF_MAX_LEVELS];
+  int job_level[ISDF_MAX_LEVELS], njobs = 0;
+  double chol_flop = 0.0;
   for (int l = 0; l < p->nlev; ++l) {
     Level& lv = p->lev[l];
     dfree(lv.xiT);
@@ -172,11 +185,11 @@ isdf_status fit_run(Plan* p) {
     dfree(lv.rinv);
     lv.rinv = nullptr;
     if (l < p->sel_lo) continue;  // local grids' level 0: fitted atom by atom (local.cu)
-    if ((st = dalloc_t(p, &lv.resid, size_t(lv.ng), "fit residual"))) return st;
+    if ((st = dalloc_t(p, &lv.resid, size_t(lv.ng), "fit residual"))) return cleanup(), st;
     if (lv.k == 0) {
       // no pivots: the residual is the whole diagonal w M(g,g)
       double* scr = nullptr;
-      if ((st = dalloc_t(p, &scr, 2, "residual statistics"))) return st;
+      if ((st = dalloc_t(p, &scr, 2, "residual statistics"))) return cleanup(), st;
       cudaMemsetAsync(scr, 0, 2 * sizeof(double), s);
       k_fit_residual<<<152 * 4, 256, 0, s>>>(lv.phi, lv.ng, lv.nL, lv.nG, lv.w, nullptr, 0,
                                              reinterpret_cast<unsigned long long*>(scr), scr + 1, lv.resid);
@@ -184,122 +197,121 @@ isdf_status fit_run(Plan* p) {
       cudaMemcpyAsync(&p->fit_resid[2 * l], scr, 2 * sizeof(double), cudaMemcpyDeviceToHost, s);
       st = cuda_check(p, cudaStreamSynchronize(s), "fit residual");
       dfree(scr);
-      if (st) return st;
+      if (st) return cleanup(), st;
       continue;
     }
     const int k = lv.k;
     const int64_t ng = lv.ng;
-    double *phiP = nullptr, *zct = nullptr, *y = nullptr, *cc = nullptr, *li = nullptr, *scr = nullptr;
-    auto cleanup = [&]() {
-      dfree(phiP);
-      dfree(y);
-      dfree(cc);
-      dfree(li);
-      dfree(scr);
-    };
-    if ((st = dalloc_t(p, &phiP, size_t(lv.nG) * k, "phi at pivots")) ||
-        (st = dalloc_t(p, &zct, size_t(k) * ng, "ZC^T / Xi")) || (st = dalloc_t(p, &y, size_t(k) * ng, "fit scratch")) ||
-        (st = dalloc_t(p, &cc, size_t(k) * k, "CC^T")) || (st = dalloc_t(p, &li, size_t(k) * k, "R^-1")) ||
-        (st = dalloc_t(p, &scr, size_t(k / 2 + 64) * k + 64, "trtri scratch"))) {
-      cleanup();
-      dfree(zct);
-      return st;
-    }
-    const bool factored = p->opt.precision == 1;  // keep ZC^T and R^-1; Xi only on request
-    if (factored)
-      lv.zct = zct;
-    else
-      lv.xiT = zct;
+    LevelBuf& b = buf[l];
+    double* zct = nullptr;
+    if ((st = dalloc_t(p, &zct, size_t(k) * ng, "ZC^T / Xi"))) return cleanup(), st;
+    (factored ? lv.zct : lv.xiT) = zct;
+    if ((st = dalloc_t(p, &b.phiP, size_t(lv.nG) * k, "phi at pivots")) ||
+        (st = dalloc_t(p, &b.y, size_t(k) * ng, "fit scratch")) || (st = dalloc_t(p, &b.cc, size_t(k) * k, "CC^T")) ||
+        (st = dalloc_t(p, &b.li, size_t(k) * k, "R^-1")) ||
+        (st = dalloc_t(p, &b.scr, size_t(k / 2 + 64) * k + 64, "trtri scratch")))
+      return cleanup(), st;
     const int64_t np = int64_t(lv.nG) * k;
     count_launches(2 + (p->opt.reg_rel > 0.0));
-    k_gather_phiP<<<unsigned((np + 255) / 256), 256, 0, s>>>(lv.nG, k, lv.phi, ng, lv.d_pg, phiP);
-    if (p->opt.precision == 1) {
-      if ((st = fit_products_tc(p, lv, k, phiP, zct, y, li, ng))) {
-        cleanup();
-        return st;
-      }
+    k_gather_phiP<<<unsigned((np + 255) / 256), 256, 0, s>>>(lv.nG, k, lv.phi, ng, lv.d_pg, b.phiP);
+    if (factored) {
+      if ((st = fit_products_tc(p, lv, k, b.phiP, zct, b.y, ng))) return cleanup(), st;
+      dfree(b.y);
+      b.y = nullptr;
     } else {
       Prof pr(p, "fit_zc", 2.0 * double(k) * double(ng) * double(lv.nG), "flop", 1);
-      zc_gemm(k, ng, lv.nL, lv.nG, phiP, lv.phi, zct, s);
+      zc_gemm(k, ng, lv.nL, lv.nG, b.phiP, lv.phi, zct, s);
     }
-    k_gather_cc<<<unsigned((int64_t(k) * k + 255) / 256), 256, 0, s>>>(k, zct, ng, lv.d_pg, cc);
-    if (p->opt.reg_rel > 0.0) k_regularise<<<1, 256, 0, s>>>(k, p->opt.reg_rel, cc);
+    dfree(b.phiP);
+    b.phiP = nullptr;
+    k_gather_cc<<<unsigned((int64_t(k) * k + 255) / 256), 256, 0, s>>>(k, zct, ng, lv.d_pg, b.cc);
+    if (p->opt.reg_rel > 0.0) k_regularise<<<1, 256, 0, s>>>(k, p->opt.reg_rel, b.cc);
+    jobs[njobs] = {b.cc, b.li, b.scr, k, p->d_err + l};
+    job_level[njobs++] = l;
+    chol_flop += double(k) * k * k / 3.0;
+  }
+  // ---- R and R^-1 of every level at once
+  if (njobs) {
+    int herr[ISDF_MAX_LEVELS];
     const int big = 0x7fffffff;
-    cudaMemcpyAsync(p->d_err, &big, sizeof(int), cudaMemcpyHostToDevice, s);
+    for (int& e : herr) e = big;
+    cudaMemcpyAsync(p->d_err, herr, sizeof(herr), cudaMemcpyHostToDevice, s);
     {
-      const int64_t nb = (k + 63) / 64;
-      Prof pr(p, "fit_cholesky", double(k) * k * k / 3.0, "flop", 3 * nb - 2);
-      dpotrf_lower(cc, k, k, p->d_err, nullptr, s);
+      Prof pr(p, "fit_cholesky", chol_flop, "flop", kLaunchesInside);
+      if ((st = dpotrf_lower(p, jobs, njobs, s))) return cleanup(), st;
     }
-    int herr = big;
-    cudaMemcpyAsync(&herr, p->d_err, sizeof(int), cudaMemcpyDeviceToHost, s);
-    if ((st = cuda_check(p, cudaStreamSynchronize(s), "Cholesky of CC^T"))) {
-      cleanup();
-      return st;
+    cudaMemcpyAsync(herr, p->d_err, sizeof(herr), cudaMemcpyDeviceToHost, s);
+    if ((st = cuda_check(p, cudaStreamSynchronize(s), "Cholesky of CC^T"))) return cleanup(), st;
+    for (int i = 0; i < njobs; ++i) {
+      const int l = job_level[i];
+      if (herr[l] != big || p->fault == "not_pd") {
+        cleanup();
+        return fail(p, ISDF_ERR_NOT_PD,
+                    "Cholesky of CC^T broke down at column " + std::to_string(herr[l] == big ? 0 : herr[l]) +
+                        " of level " + std::to_string(l));
+      }
     }
-    if (herr != big || p->fault == "not_pd") {
-      cleanup();
-      return fail(p, ISDF_ERR_NOT_PD,
-                  "Cholesky of CC^T broke down at column " + std::to_string(herr == big ? 0 : herr) + " of level " +
-                      std::to_string(l));
-    }
-    {
-      const int64_t nb = (k + 63) / 64;
-      Prof pr(p, "fit_trtri", double(k) * k * k / 3.0, "flop", 1 + 2 * (nb - 1));
-      dtrtri_lower(cc, li, k, scr, s, p->opt.precision == 1 ? p : nullptr);
-    }
-    if (factored) {
-      // Coulomb and exchange need Xi only through V = W (ZC^T v ZC) W with
-      // W = R^-T R^-1 (see coulomb.cu): no solve over the grid here
-      lv.rinv = li;
-      li = nullptr;
-      st = cuda_check(p, cudaStreamSynchronize(s), "fit");
-      if (!st) st = oz_check(p);
-      cleanup();
-      if (st) return st;
-      continue;
-    } else {
-    Prof pr_solve(p, "fit_solve", 2.0 * double(k) * double(k + 1) * double(ng), "flop", 2);
-    GemmArgs g1;  // Y = R^-1 ZC^T^T (R^-1 lower triangular)
-    g1.M = k;
-    g1.N = ng;
-    g1.K = k;
-    g1.A = li;
-    g1.lda = k;
-    g1.B = zct;
-    g1.ldb = ng;
-    g1.C = y;
-    g1.ldc = ng;
-    g1.tri = 1;
-    dgemm(g1, s);
-    GemmArgs g2;  // Xi^T = R^-T Y (opA upper triangular)
-    g2.ta = 1;
-    g2.M = k;
-    g2.N = ng;
-    g2.K = k;
-    g2.A = li;
-    g2.lda = k;
-    g2.B = y;
-    g2.ldb = ng;
-    g2.C = zct;
-    g2.ldc = ng;
-    g2.tri = 2;
-    dgemm(g2, s);
-    }
-    {
-      // y still holds R^-1 (ZC^T)^T: residual statistics of this level
-      unsigned long long* rmax = reinterpret_cast<unsigned long long*>(scr);
-      double* rsum = scr + 1;
-      cudaMemsetAsync(scr, 0, 2 * sizeof(double), s);
-      k_fit_residual<<<152 * 4, 256, 0, s>>>(lv.phi, ng, lv.nL, lv.nG, lv.w, y, k, rmax, rsum, lv.resid);
-      count_launches(1);
-      cudaMemcpyAsync(&p->fit_resid[2 * l], scr, 2 * sizeof(double), cudaMemcpyDeviceToHost, s);
+    Prof pr(p, "fit_trtri", chol_flop, "flop", kLaunchesInside);
+    dtrtri_lower(p, jobs, njobs, factored, s);
+  }
+  if (factored) {
+    // Coulomb and exchange need Xi only through V = W (ZC^T v ZC) W with
+    // W = R^-T R^-1 (see coulomb.cu): no solve over the grid here
+    for (int i = 0; i < njobs; ++i) {
+      p->lev[job_level[i]].rinv = buf[job_level[i]].li;
+      buf[job_level[i]].li = nullptr;
     }
     st = cuda_check(p, cudaStreamSynchronize(s), "fit");
+    if (!st) st = oz_check(p);
     cleanup();
-    if (st) return st;
+    return st ? st : gather_pivot_factors(p);
   }
-  p->resid_ready = p->opt.precision != 1;
+  // ---- the solve and the residual statistics of every level
+  for (int i = 0; i < njobs; ++i) {
+    const int l = job_level[i];
+    Level& lv = p->lev[l];
+    LevelBuf& b = buf[l];
+    const int k = lv.k;
+    const int64_t ng = lv.ng;
+    {
+      Prof pr_solve(p, "fit_solve", 2.0 * double(k) * double(k + 1) * double(ng), "flop", kLaunchesInside);
+      GemmArgs g1;  // Y = R^-1 ZC^T^T (R^-1 lower triangular)
+      g1.M = k;
+      g1.N = ng;
+      g1.K = k;
+      g1.A = b.li;
+      g1.lda = k;
+      g1.B = lv.xiT;
+      g1.ldb = ng;
+      g1.C = b.y;
+      g1.ldc = ng;
+      g1.tri = 1;
+      dgemm(g1, s);
+      GemmArgs g2;  // Xi^T = R^-T Y (opA upper triangular)
+      g2.ta = 1;
+      g2.M = k;
+      g2.N = ng;
+      g2.K = k;
+      g2.A = b.li;
+      g2.lda = k;
+      g2.B = b.y;
+      g2.ldb = ng;
+      g2.C = lv.xiT;
+      g2.ldc = ng;
+      g2.tri = 2;
+      dgemm(g2, s);
+    }
+    // y still holds R^-1 (ZC^T)^T: residual statistics of this level
+    cudaMemsetAsync(b.scr, 0, 2 * sizeof(double), s);
+    k_fit_residual<<<152 * 4, 256, 0, s>>>(lv.phi, ng, lv.nL, lv.nG, lv.w, b.y, k,
+                                           reinterpret_cast<unsigned long long*>(b.scr), b.scr + 1, lv.resid);
+    count_launches(1);
+    cudaMemcpyAsync(&p->fit_resid[2 * l], b.scr, 2 * sizeof(double), cudaMemcpyDeviceToHost, s);
+  }
+  st = cuda_check(p, cudaStreamSynchronize(s), "fit");
+  cleanup();
+  if (st) return st;
+  p->resid_ready = true;
   return gather_pivot_factors(p);
 }
 

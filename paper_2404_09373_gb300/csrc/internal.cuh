@@ -215,13 +215,20 @@ void dgemm(const GemmArgs& g, cudaStream_t s);
 // ZC^T = A_L o (A_L + 2 A_N) with A_X = PhiP_X^T Phi_X (fit.cu uses it)
 void zc_gemm(int64_t k, int64_t ng, int nL, int nG, const double* phiP, const double* phi, double* out,
              cudaStream_t s);
-// lower Cholesky in place (row-major n x n, lda); breakdown column -> *err
-void dpotrf_lower(double* A, int64_t n, int64_t lda, int* err, double* scratch, cudaStream_t s);
-// inverse of a lower-triangular matrix: Li (n x n, zero-initialised by callee);
-// with a plan (tensor-core precision) the large off-diagonal products run as
-// FP64-grade 8-digit tensor-core products, their error flag the plan's
-struct Plan;
-void dtrtri_lower(const double* Lm, double* Li, int64_t n, double* scratch, cudaStream_t s, Plan* tc = nullptr);
+// One level's matrix: A (row-major n x n) is factored in place into R (A = R R^T),
+// Li receives R^-1 (zero above the diagonal), scratch holds (n / 2 + 64) n values
+struct FactorJob {
+  double* A;
+  double* Li;
+  double* scratch;
+  int n;
+  int* err;  // smallest breakdown column (the caller presets it)
+};
+// lower Cholesky of up to ISDF_MAX_LEVELS matrices; also the 64 x 64 diagonal blocks of R^-1
+isdf_status dpotrf_lower(Plan* p, const FactorJob* jobs, int count, cudaStream_t s);
+// the rest of R^-1; tensor: products of halves of 256 rows or more run as FP64-grade
+// 8-digit tensor-core products, their error flag the plan's
+void dtrtri_lower(Plan* p, const FactorJob* jobs, int count, bool tensor, cudaStream_t s);
 
 // FP64-accurate GEMM from sliced BF16 products on tcgen05 (ozgemm.cu).
 // An operand is rows x K, pre-sliced into S BF16 digit planes (S = 5 or 6)

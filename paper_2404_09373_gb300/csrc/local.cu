@@ -128,7 +128,7 @@ isdf_status local_setup(Plan* p, double alpha_min) {
     q->off[0] = 0;
     q->off[1] = lv.ng;
     q->ntot = lv.ng;
-    isdf_status st = dalloc_t(p, &q->d_err, 1, "error word");
+    isdf_status st = dalloc_t(p, &q->d_err, ISDF_MAX_LEVELS, "error words");
     if (!st) st = dalloc_t(p, &q->d_ozerr, 1, "error word");
     if (!st) st = cuda_check(p, cudaMemsetAsync(q->d_ozerr, 0, sizeof(int), p->stream), "memset");
     if (st) return st;

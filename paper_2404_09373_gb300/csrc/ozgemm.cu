@@ -578,7 +578,7 @@ void launch_slice_s(const OzSliceArgs& A, cudaStream_t s) {
 constexpr int64_t kFusedK = 4096;
 
 void slice_operand(const OzSliceArgs& A, int S, cudaStream_t s) {
-  if (A.sr < A.sk || A.K <= kFusedK || A.ridx) {
+  if (A.sr < A.sk || A.K <= kFusedK || A.ridx || A.sk != 1) {
     if (S == 5) launch_slice_s<5>(A, s);
     else if (S == 6) launch_slice_s<6>(A, s);
     else if (S == 7) launch_slice_s<7>(A, s);
