@@ -75,5 +75,52 @@ __device__ __forceinline__ double f32_to_f64(float f) {
 }
 __device__ __forceinline__ double df_to_double(DF x) { return f32_to_f64(x.hi) + f32_to_f64(x.lo); }
 
+// 1 / sqrt(d) for finite d > 0: FP32 estimate of the significand's root and one
+// step of the third-order iteration r (1 + e/2 + 3 e^2 / 8), e = 1 - d r^2 (the
+// Taylor series of (1 - e)^-1/2): from 2^-22 to rounding error in four dependent
+// FP64 operations instead of the forty of a square root and a division.
+__device__ __forceinline__ double rsqrt64(double d) {
+  const long long b = __double_as_longlong(d);
+  int E = int((b >> 52) & 0x7FF);
+  if (E == 0) return 1.0 / sqrt(d);  // subnormal
+  const int h = (E - 1023) >> 1;     // d = m 4^h, m in [1, 4)
+  const double m = __longlong_as_double(b - ((long long)(2 * h) << 52));
+  const int odd = (E - 1023) & 1;
+  const float mf = __int_as_float(((127 + odd) << 23) | int((b >> 29) & 0x7FFFFF));
+  const double r0 = f32_to_f64(rsqrtf(mf));
+  const double t = m * r0;
+  const double e = fma(-t, r0, 1.0);
+  const double r = fma(r0 * e, fma(0.375, e, 0.5), r0);
+  return __longlong_as_double(__double_as_longlong(r) - ((long long)h << 52));
+}
+
+// 1 / sqrt(d) as a double-float, FP32 operations only: the same iteration with
+// the residual e = 1 - m r0^2 and its correction carried as pairs.
+__device__ __forceinline__ DF df_rsqrt(double d) {
+  const long long b = __double_as_longlong(d);
+  const int E = int((b >> 52) & 0x7FF);
+  const int h = (E - 1023) >> 1;  // d = m 4^h, m in [1, 4)
+  if (E == 0 || h < -120 || h > 120) return df_from_double(1.0 / sqrt(d));
+  const DF m = df_from_double(__longlong_as_double(b - ((long long)(2 * h) << 52)));
+  const float r = rsqrtf(m.hi);
+  const float p = __fmul_rn(m.hi, r);
+  const float pe = __fmaf_rn(m.lo, r, __fmaf_rn(m.hi, r, -p));
+  const float q = __fmul_rn(p, r);
+  const float qe = __fmaf_rn(pe, r, __fmaf_rn(p, r, -q));
+  const DF e = two_sum(__fsub_rn(1.0f, q), -qe);  // 1 - q is exact
+  const float hr = 0.5f * r, c = __fmul_rn(hr, e.hi);
+  const float cl = __fmaf_rn(hr, e.hi, -c) + __fmaf_rn(hr, e.lo, hr * (0.75f * e.hi * e.hi));
+  const DF s = two_sum(r, c);
+  const DF x = quick_two_sum(s.hi, __fadd_rn(s.lo, cl));
+  const float sc = __int_as_float((127 - h) << 23);
+  return {x.hi * sc, x.lo * sc};
+}
+
+// sqrt(d) from r = rsqrt64(d)
+__device__ __forceinline__ double sqrt_from(double d, double r) {
+  const double s = d * r;
+  return fma(fma(-s, s, d), 0.5 * r, s);
+}
+
 }  // namespace
 }  // namespace isdf

@@ -9,6 +9,7 @@
 // SM as early as possible; a larger tile would only save loads, which are free.
 #include <algorithm>
 
+#include "dfloat.cuh"
 #include "internal.cuh"
 
 namespace isdf {
@@ -167,28 +168,6 @@ struct CholLevels {
   CholLevel l[ISDF_MAX_LEVELS];
 };
 
-// 1 / sqrt(d) for finite d > 0: FP32 estimate of the significand's root and one
-// step of the third-order iteration r (1 + e/2 + 3 e^2 / 8), e = 1 - d r^2 (the
-// Taylor series of (1 - e)^-1/2): from 2^-22 to rounding error in four dependent
-// FP64 operations instead of the forty of a square root and a division.
-__device__ __forceinline__ double rsqrt64(double d) {
-  const long long b = __double_as_longlong(d);
-  int E = int((b >> 52) & 0x7FF);
-  if (E == 0) return 1.0 / sqrt(d);  // subnormal
-  const int h = (E - 1023) >> 1;     // d = m 4^h, m in [1, 4)
-  const double m = __longlong_as_double(b - ((long long)(2 * h) << 52));
-  const int odd = (E - 1023) & 1;
-  const float mf = __int_as_float(((127 + odd) << 23) | int((b >> 29) & 0x7FFFFF));
-  const double r0 = __longlong_as_double([](float f) {  // FP32 to FP64 bits
-    const uint32_t u = __float_as_uint(f);
-    return (long long)((uint64_t(((u >> 23) & 0xFF) + 896u) << 52) | (uint64_t(u & 0x7FFFFF) << 29));
-  }(rsqrtf(mf)));
-  const double t = m * r0;
-  const double e = fma(-t, r0, 1.0);
-  const double r = fma(r0 * e, fma(0.375, e, 0.5), r0);
-  return __longlong_as_double(__double_as_longlong(r) - ((long long)h << 52));
-}
-
 struct DiagSmem {
   double s[CB][CB + 1];
   double v[CB][CB + 1];
@@ -222,8 +201,7 @@ __device__ void chol_diag(const CholLevel& P, int kb, DiagSmem& S) {
       if (i1 > j) S.s[i1][j] = x1 * r;
       if (tid == 0) {
         S.r[j] = r;
-        const double s = d * r;
-        S.s[j][j] = fma(fma(-s, s, d), 0.5 * r, s);  // sqrt(d)
+        S.s[j][j] = sqrt_from(d, r);
       }
     }
     __syncthreads();

@@ -26,6 +26,7 @@
 #include <cstring>
 
 #include "dfloat.cuh"
+#include "digits.cuh"
 #include "internal.cuh"
 
 namespace isdf {
@@ -48,9 +49,8 @@ struct SelState {
   unsigned long long t0;
   // speculative blocks
   int final_;                // a stop rule ended the selection
-  int jpos;                  // this step's pivot: its position in the block's set S
-  int bsteps;                // steps taken in the current block
-  int kb[ISDF_MAX_LEVELS];   // factor columns per level when the block began
+  int bsteps;                // steps accepted in the current round of a block
+  int btried;                // steps the round tried
 };
 
 struct SelParams {
@@ -337,21 +337,58 @@ __global__ __launch_bounds__(32 * kColWarps) void k_sel_col(SelParams P, const S
 //
 // A block of the greedy loop first guesses a set S of up to s points that are
 // likely to be the next pivots (the largest local maxima of the residual on
-// the grids), computes the factor columns they would produce with
+// the grids) and computes the factor columns they would produce with
 // tensor-core products over all candidates,
-//   B[j][t] = w M(t, S_j) - sum_{k < kb} L[t,k] L[S_j,k]        (kb = columns so far)
-// and then takes ordinary greedy steps, each finishing its column from B with
-// the few columns added inside the block:
+//   B[j][t] = w M(t, S_j) - sum_{k < kb} L[t,k] L[S_j,k]        (kb = columns so far).
+// Greedy steps within S then need no other candidate: one CTA (k_blk_greedy)
+// takes up to m of them on S's own residuals, finishing each column at the
+// members of S from B with the columns added inside the block,
 //   L[t,col] = (B[pos(p)][t] - sum_{kb <= k < col} L[t,k] L[p,k]) / sqrt(d_p).
-// The pivot of every step is still the argmax over ALL candidates' exact
-// residuals (same tie rule); the block ends at the first pivot outside S.  S
-// only decides how many steps one block covers, never which point is chosen.
+// k_blk_apply then finishes the same columns at every candidate in the same
+// arithmetic and looks for the first step at which some candidate's residual
+// shows that the step was not the greedy one: its residual is above the step's
+// maximum, or inside the step's tie window with a smaller index.  The steps
+// before that one are exactly the ordinary greedy steps, the argmax over ALL
+// candidates' residuals with the same tie rule; k_blk_commit takes them over.
+// No step waits for the whole chip: three launches serve up to s steps, where
+// a cooperative launch with two grid barriers per step took 13 us a step on one
+// cell and 20 us on the 2x2x2 workload.  Per block: one cell 182 -> 75 us, 2x2x2
+// 860 -> 400 us, the digits of the new columns included.
+
+constexpr int kMaxSet = 256;  // options.select_block's limit
+
+struct StepRec {
+  double dp, dmax;  // the pivot's residual, the largest residual
+  int idx;          // pivot: index over all candidates
+  int t, pos;       // candidate in its level; row of B
+  int lev;
+};
+
+// One round of a block: tried steps, their entries in the block's earlier
+// columns, and the first step that failed.
+struct BlkRound {
+  int nsteps;
+  int jstar;  // steps [0, jstar) are accepted
+  int nl[ISDF_MAX_LEVELS];
+  int list[ISDF_MAX_LEVELS][kMaxSet];  // steps of each level in order
+  StepRec rec[kMaxSet];
+  float2 lp[kMaxSet][kMaxSet];         // lp[step][q] = L[p_step, kb + q], double-float
+};
 
 struct BlkParams {
   SelParams P;
-  const int* spos;                      // [ntot] position of a candidate in S's range of its level, -1 if not in S
-  const double* bm[ISDF_MAX_LEVELS];    // [s_l][nc_l]
-  float2* bdf[ISDF_MAX_LEVELS];         // [s][nc_l] the block's columns so far, double-float
+  const double* bm[ISDF_MAX_LEVELS];  // [s_l][nc_l]
+  float2* bdf[ISDF_MAX_LEVELS];       // [s][nc_l] the block's columns so far, double-float
+  const int* sidx;                    // S in ascending candidate order: index over all candidates
+  const int* st;                      // and position in its level
+  const int* scount;                  // per level, then in all
+  int kb[ISDF_MAX_LEVELS];            // factor columns when S was chosen
+  int kl[ISDF_MAX_LEVELS];            // factor columns now
+  int k;                              // pivots now
+  int64_t boff[ISDF_MAX_LEVELS + 1];  // blocks of kApply candidates per level
+  const int* fexp[ISDF_MAX_LEVELS];   // fixed row scales and digit planes of the factor columns
+  void* ftiles[ISDF_MAX_LEVELS];
+  int64_t fkst[ISDF_MAX_LEVELS];
 };
 
 // Order-preserving key of a residual value: its bits when positive, else 0
@@ -437,208 +474,132 @@ __device__ __forceinline__ bool is_local_max(const LmParams& Q, int64_t i) {
   return true;
 }
 
-// ordered compaction of the local maxima: per-block counts, one-block scan, scatter
-__global__ void k_lm_count(LmParams Q, int* __restrict__ counts) {
-  __shared__ int sh[32];
-  const int64_t i = int64_t(blockIdx.x) * kCompactBlock + threadIdx.x;
-  const int f = (i < Q.ntot && is_local_max(Q, i)) ? 1 : 0;
+// append the local maxima to a list (any order; k_top_s sorts what it keeps)
+__global__ void __launch_bounds__(256) k_lm_list(LmParams Q, int* __restrict__ list, int* __restrict__ n) {
+  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  const bool f = i < Q.ntot && is_local_max(Q, i);
   const unsigned b = __ballot_sync(0xffffffffu, f);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = __popc(b);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int c = 0;
-    for (int w = 0; w < kCompactBlock / 32; ++w) c += sh[w];
-    counts[blockIdx.x] = c;
-  }
-}
-
-// exclusive scan of nb counts in place; total into *total (one block of 1024)
-__global__ void k_scan_counts(int* __restrict__ counts, int64_t nb, int* __restrict__ total) {
-  __shared__ int sh[1024];
-  __shared__ int carry;
-  if (threadIdx.x == 0) carry = 0;
-  __syncthreads();
-  for (int64_t b0 = 0; b0 < nb; b0 += 1024) {
-    const int64_t b = b0 + threadIdx.x;
-    const int v = b < nb ? counts[b] : 0;
-    sh[threadIdx.x] = v;
-    __syncthreads();
-    for (int o = 1; o < 1024; o <<= 1) {
-      const int add = threadIdx.x >= o ? sh[threadIdx.x - o] : 0;
-      __syncthreads();
-      sh[threadIdx.x] += add;
-      __syncthreads();
-    }
-    if (b < nb) counts[b] = carry + sh[threadIdx.x] - v;
-    __syncthreads();
-    if (threadIdx.x == 0) carry += sh[1023];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *total = carry;
-}
-
-__global__ void k_lm_write(LmParams Q, const int* __restrict__ offs, int* __restrict__ list) {
-  __shared__ int woff[32];
-  const int64_t i = int64_t(blockIdx.x) * kCompactBlock + threadIdx.x;
-  const int f = (i < Q.ntot && is_local_max(Q, i)) ? 1 : 0;
-  const unsigned b = __ballot_sync(0xffffffffu, f);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) woff[wid] = __popc(b);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int a = 0;
-    for (int w = 0; w < kCompactBlock / 32; ++w) {
-      const int c = woff[w];
-      woff[w] = a;
-      a += c;
-    }
-  }
-  __syncthreads();
-  if (f) list[offs[blockIdx.x] + woff[wid] + __popc(b & ((1u << lane) - 1u))] = int(i);
+  if (!b) return;
+  const int lane = threadIdx.x & 31;
+  int base = 0;
+  if (lane == 0) base = atomicAdd(n, __popc(b));
+  base = __shfl_sync(0xffffffffu, base, 0);
+  if (f) list[base + __popc(b & ((1u << lane) - 1u))] = int(i);
 }
 
 // The s largest residuals of the list (ties to the smallest index), by an
-// 8-bit radix select on the bit patterns (d > 0 orders like its bits).
-// Writes S in ascending candidate order: sidx (concatenated index), sg (grid
-// index), st (position in its level), per-level counts and offsets, spos.
+// 8-bit radix select on the bit patterns (d > 0 orders like its bits), then on
+// the indices of those equal to the last one kept.  Writes S in ascending
+// candidate order: sidx (concatenated index), sg (grid index), st (position in
+// its level), per-level counts.  One CTA, bound by the latency of its passes
+// over the list: the bins are searched by one warp (a thread walking 256 bins
+// cost 4 us a pass, 39 us in all on one cell's lists; now 12).
 struct TopSOut {
   int* sidx;
   int* sg;
   int* st;
   int* scount;  // [ISDF_MAX_LEVELS + 1]: per-level counts, then the total
-  int* spos;    // [ntot]
 };
-__global__ void __launch_bounds__(1024) k_top_s(LmParams Q, const int* __restrict__ list, const int* __restrict__ nlist,
-                                                int smax, TopSOut O) {
-  __shared__ int hist[256];
-  __shared__ unsigned long long prefix, pmask;
-  __shared__ int need, take_gt;
-  __shared__ int wsum[32];
-  __shared__ int base;
-  __shared__ int lcount[ISDF_MAX_LEVELS];
-  const int n = *nlist;
-  const int tid = threadIdx.x;
-  if (tid == 0) {
-    prefix = 0ull;
-    pmask = 0ull;
-    need = n < smax ? n : smax;
-    take_gt = 0;
-    base = 0;
+constexpr int kTopKeys = 4096;  // keys kept in shared memory (longer lists are read from global memory)
+
+// Highest bin b (from the top) with count(bins > b) + above < want <= count(bins >= b) + above; one warp.
+__device__ __forceinline__ void pick_bin(const int* hist, int above, int want, int lane, int* bin, int* gt) {
+  int c[8], tot = 0;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) tot += c[q] = hist[255 - (lane * 8 + q)];
+  int pre = tot;  // inclusive prefix over lanes (lane 0: the top bins)
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int x = __shfl_up_sync(0xffffffffu, pre, o);
+    if (lane >= o) pre += x;
   }
-  if (tid < ISDF_MAX_LEVELS) lcount[tid] = 0;
-  __syncthreads();
-  const int want = need;
-  // find the threshold key T: count(key > T) < want <= count(key >= T)
-  if (want > 0 && want < n) {
-    int above = 0;  // keys above the current prefix range (already counted)
-    for (int shift = 56; shift >= 0; shift -= 8) {
-      for (int b = tid; b < 256; b += blockDim.x) hist[b] = 0;
-      __syncthreads();
-      for (int i = tid; i < n; i += blockDim.x) {
-        const unsigned long long key = (unsigned long long)__double_as_longlong(Q.d[list[i]]);
-        if ((key & pmask) == prefix) atomicAdd(&hist[(key >> shift) & 255], 1);
-      }
-      __syncthreads();
-      if (tid == 0) {
-        int acc = above, b = 255;
-        for (; b > 0; --b) {
-          if (acc + hist[b] >= want) break;
-          acc += hist[b];
-        }
-        above = acc;
-        prefix |= (unsigned long long)b << shift;
-        pmask |= 255ull << shift;
-        take_gt = acc;
-      }
-      __syncthreads();
-      above = take_gt;
+  int acc = above + pre - tot;
+  if (acc < want && want <= acc + tot) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      if (acc < want && want <= acc + c[q]) *bin = 255 - (lane * 8 + q), *gt = acc;
+      acc += c[q];
     }
-  }
-  const unsigned long long T = prefix;
-  const bool all = !(want > 0 && want < n);
-  const int n_eq_needed = all ? 0 : want - take_gt;
-  // ordered pass: keep key > T, and key == T while the equal quota lasts
-  __shared__ int eq_base;
-  if (tid == 0) eq_base = 0;
-  __syncthreads();
-  for (int i0 = 0; i0 < n; i0 += blockDim.x) {
-    const int i = i0 + tid;
-    bool gt = false, eq = false;
-    int idx = 0;
-    if (i < n) {
-      idx = list[i];
-      const unsigned long long key = (unsigned long long)__double_as_longlong(Q.d[idx]);
-      gt = all || key > T;
-      eq = !all && key == T;
-    }
-    // rank of the equals in list order
-    const unsigned be = __ballot_sync(0xffffffffu, eq);
-    const int lane = tid & 31, wid = tid >> 5;
-    if (lane == 0) wsum[wid] = __popc(be);
-    __syncthreads();
-    if (tid == 0) {
-      int a = eq_base;
-      for (int w = 0; w < 32; ++w) {
-        const int c = wsum[w];
-        wsum[w] = a;
-        a += c;
-      }
-      eq_base = a;
-    }
-    __syncthreads();
-    const int eq_rank = wsum[wid] + __popc(be & ((1u << lane) - 1u));
-    const bool sel = gt || (eq && eq_rank < n_eq_needed);
-    __syncthreads();
-    const unsigned bs = __ballot_sync(0xffffffffu, sel);
-    if (lane == 0) wsum[wid] = __popc(bs);
-    __syncthreads();
-    if (tid == 0) {
-      int a = base;
-      for (int w = 0; w < 32; ++w) {
-        const int c = wsum[w];
-        wsum[w] = a;
-        a += c;
-      }
-      base = a;
-    }
-    __syncthreads();
-    if (sel) {
-      const int pos = wsum[wid] + __popc(bs & ((1u << lane) - 1u));
-      int l = 0;
-      while (l + 1 < Q.nlev && idx >= Q.coff[l + 1]) ++l;
-      const int64_t t = idx - Q.coff[l];
-      O.sidx[pos] = idx;
-      O.st[pos] = int(t);
-      O.sg[pos] = Q.cidx[l] ? Q.cidx[l][t] : int(t);
-      atomicAdd(&lcount[l], 1);
-    }
-    __syncthreads();
-  }
-  __syncthreads();
-  if (tid == 0) {
-    int acc = 0;
-    for (int l = 0; l < Q.nlev; ++l) {
-      O.scount[l] = lcount[l];
-      acc += lcount[l];
-    }
-    O.scount[ISDF_MAX_LEVELS] = acc;
-  }
-  __syncthreads();
-  // positions within each level's range
-  const int total = base;
-  for (int j = tid; j < total; j += blockDim.x) {
-    const int idx = O.sidx[j];
-    int l = 0;
-    while (l + 1 < Q.nlev && idx >= Q.coff[l + 1]) ++l;
-    int first = 0;
-    for (int q = 0; q < l; ++q) first += lcount[q];
-    O.spos[idx] = j - first;
   }
 }
 
-__global__ void k_spos_clear(const int* __restrict__ sidx, const int* __restrict__ scount, int* __restrict__ spos) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j < scount[ISDF_MAX_LEVELS]) spos[sidx[j]] = -1;
+__global__ void __launch_bounds__(1024) k_top_s(LmParams Q, const int* __restrict__ list, const int* __restrict__ nlist,
+                                                int smax, TopSOut O) {
+  __shared__ unsigned long long skey[kTopKeys];
+  __shared__ int hist[256];
+  __shared__ int bin_sh, gt_sh, kept;
+  __shared__ int sel[kMaxSet];
+  __shared__ int lcount[ISDF_MAX_LEVELS];
+  const int n = *nlist, tid = threadIdx.x, lane = tid & 31;
+  const int want = n < smax ? n : smax;
+  if (tid == 0) kept = 0;
+  if (tid < ISDF_MAX_LEVELS) lcount[tid] = 0;
+  auto load_key = [&](int i) { return (unsigned long long)__double_as_longlong(Q.d[list[i]]); };
+  for (int i = tid; i < n && i < kTopKeys; i += 1024) skey[i] = load_key(i);
+  __syncthreads();
+  auto key = [&](int i) { return i < kTopKeys ? skey[i] : load_key(i); };
+  unsigned long long T = 0ull, mask = 0ull;
+  unsigned int tie = 0xffffffffu;  // among keys equal to T: indices up to tie
+  if (want > 0 && want < n) {
+    int above = 0;
+    for (int pass = 0; pass < 12; ++pass) {
+      // passes 0..7: the threshold key; 8..11: the largest index kept among its equals
+      const bool on_key = pass < 8;
+      const int shift = on_key ? 56 - 8 * pass : 88 - 8 * pass;
+      if (pass == 8) tie = 0u, mask = 0ull;
+      if (tid < 256) hist[tid] = 0;
+      __syncthreads();
+      for (int i = tid; i < n; i += 1024) {
+        const unsigned long long k = key(i);
+        if (on_key) {
+          if ((k & mask) == T) atomicAdd(&hist[(k >> shift) & 255], 1);
+        } else if (k == T) {
+          const unsigned int x = ~(unsigned int)list[i];  // smallest index first
+          if ((x & (unsigned int)mask) == tie) atomicAdd(&hist[(x >> shift) & 255], 1);
+        }
+      }
+      __syncthreads();
+      if (tid < 32) pick_bin(hist, above, want, lane, &bin_sh, &gt_sh);
+      __syncthreads();
+      above = gt_sh;
+      mask |= 255ull << shift;
+      if (on_key) T |= (unsigned long long)bin_sh << shift;
+      else tie |= (unsigned int)bin_sh << shift;
+      // all of the keys equal to T are wanted: no choice among them
+      if (pass == 7 && above + hist[bin_sh] == want) {
+        tie = 0u;
+        break;
+      }
+      __syncthreads();
+    }
+  } else {
+    tie = 0u;
+  }
+  __syncthreads();
+  for (int i = tid; i < n; i += 1024) {
+    const unsigned long long k = key(i);
+    const int idx = list[i];
+    if (k > T || (k == T && ~(unsigned int)idx >= tie)) sel[atomicAdd(&kept, 1)] = idx;
+  }
+  __syncthreads();
+  const int total = kept;  // = want
+  if (tid < total) {
+    const int idx = sel[tid];
+    int rank = 0;
+    for (int i = 0; i < total; ++i) rank += sel[i] < idx;
+    int l = 0;
+    while (l + 1 < Q.nlev && idx >= Q.coff[l + 1]) ++l;
+    const int64_t t = idx - Q.coff[l];
+    O.sidx[rank] = idx;
+    O.st[rank] = int(t);
+    O.sg[rank] = Q.cidx[l] ? Q.cidx[l][t] : int(t);
+    atomicAdd(&lcount[l], 1);
+  }
+  __syncthreads();
+  if (tid == 0) {
+    for (int l = 0; l < ISDF_MAX_LEVELS; ++l) O.scount[l] = l < Q.nlev ? lcount[l] : 0;
+    O.scount[ISDF_MAX_LEVELS] = total;
+  }
 }
 
 // B = w * aL (aL + 2 aN) - F over [s_l][nc]; in place in aL
@@ -670,98 +631,313 @@ __global__ void k_fac_exps(const double* __restrict__ d0c, int64_t nc, int64_t n
   exps[t] = e;
 }
 
-__global__ void k_blk_begin(SelState* st) {
+// before an ordinary step between two blocks
+__global__ void k_step_begin(SelState* st) {
   if (threadIdx.x != 0) return;
   st->done = st->final_ ? 1 : 0;
   st->skip = 1;
-  st->bsteps = 0;
   st->dmax_bits = 0ull;
   st->first = ULLONG_MAX;
-  for (int l = 0; l < ISDF_MAX_LEVELS; ++l) st->kb[l] = st->kl[l];
 }
 
-__global__ void k_blk_pick(BlkParams B, SelState* st) {
+// Largest of a warp's 64-bit keys: two 32-bit warp reductions.
+__device__ __forceinline__ unsigned long long warp_max64(unsigned long long k) {
+  const unsigned hi = unsigned(k >> 32), h = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned l = __reduce_max_sync(0xffffffffu, hi == h ? unsigned(k) : 0u);
+  return (unsigned long long)h << 32 | l;
+}
+
+// The tie threshold of a step: d >= thr and d > 0  <=>  key(d) >= tie_key.
+__device__ __forceinline__ unsigned long long tie_key(const SelParams& P, double dmax, double d0) {
+  return max(dkey(dmax - fmax(P.tie_rel * dmax, P.tie_abs * d0)), 1ull);
+}
+
+// Up to m greedy steps among the members of S, one thread per member.  A step
+// is a chain of two block syncs, the members' dots over the block's earlier
+// columns (double-float, the arithmetic of k_blk_apply) and two FP64
+// operations: the FP64 unit takes hundreds of cycles for a chain of a few
+// operations, so the reciprocal root is a double-float one, the tie window is
+// first tested against an integer bound from below (one member above it is
+// the pivot whatever the exact threshold is), and square roots and thresholds
+// of the record are left to k_blk_apply.  With `gcols` null the columns and B at
+// S x S are in shared memory ([s][nwork] each), so no step waits for L2; else
+// (more members than fit) the columns are in gcols and B is read in place.
+// (With the FP64 scalars in the chain and four syncs a step took 2.6 us.)
+__global__ void __launch_bounds__(kMaxSet) k_blk_greedy(BlkParams B, SelState* st, BlkRound* R, int m, int smax,
+                                                        float2* __restrict__ gcols) {
+  extern __shared__ double sm_greedy[];
+  __shared__ unsigned long long wmax[kMaxSet / 32];
+  __shared__ int wfirst[kMaxSet / 32], wcount[kMaxSet / 32];
+  __shared__ unsigned long long thr_sh;
+  __shared__ double dmem[kMaxSet];
   const SelParams& P = B.P;
-  if (threadIdx.x != 0 || st->done) return;
-  const unsigned long long idx = st->first;
-  if (idx == ULLONG_MAX) {
-    st->done = 1;
-    st->skip = 1;
-    st->final_ = 1;
-    return;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nwork = blockDim.x, nwarp = nwork >> 5;
+  int begin[ISDF_MAX_LEVELS + 1] = {0};  // members of level l: [begin[l], begin[l + 1])
+#pragma unroll
+  for (int l = 0; l < ISDF_MAX_LEVELS; ++l) begin[l + 1] = begin[l] + B.scount[l];
+  const int total = begin[ISDF_MAX_LEVELS];
+  int lev = 0, mfirst = 0, mlast = begin[1];  // this member's level and its range
+#pragma unroll
+  for (int l = 1; l < ISDF_MAX_LEVELS; ++l)
+    if (l < P.nlev && tid >= begin[l]) lev = l, mfirst = begin[l], mlast = begin[l + 1];
+  const bool mine = tid < total;
+  const int64_t nc = P.nc[lev];
+  const int64_t t = mine ? B.st[tid] : 0;
+  const int gidx = mine ? B.sidx[tid] : 0;
+  double* bss = sm_greedy;  // B[member p][this thread] at p * nwork + tid
+  float2* cols = gcols ? gcols : reinterpret_cast<float2*>(sm_greedy + int64_t(smax) * nwork);  // q * nwork + tid
+  double d = mine ? P.d[gidx] : 0.0;
+  if (!gcols && mine) {
+    const double* b = B.bm[lev] + t;
+#pragma unroll 8
+    for (int i = mfirst; i < mlast; ++i) bss[i * nwork + tid] = __ldcg(b + int64_t(i - mfirst) * nc);
   }
-  const int pos = B.spos[idx];
-  if (pos < 0) {  // the greedy pivot is outside S: the block ends here
-    st->done = 1;
-    st->skip = 1;
-    return;
+  unsigned long long key = mine ? dkey(d) : 0ull;
+  int nq[ISDF_MAX_LEVELS];  // columns in the block, per level (the same in every thread)
+  int nstep[ISDF_MAX_LEVELS] = {0, 0, 0, 0};
+  int mynq = 0;
+#pragma unroll
+  for (int l = 0; l < ISDF_MAX_LEVELS; ++l) {
+    nq[l] = B.kl[l] - B.kb[l];
+    if (l == lev) mynq = nq[l];
   }
-  int l = 0;
-  while (l + 1 < P.nlev && (long long)idx >= P.coff[l + 1]) ++l;
-  const long long t = (long long)idx - P.coff[l];
-  const long long g = P.cidx[l] ? P.cidx[l][t] : t;
-  const double dp = P.d[idx];
-  const int k = st->k;
-  if (k == 0) st->d0 = __longlong_as_double((long long)st->dmax_bits);
-  st->lev = l;
-  st->gp = g;
-  st->tp = t;
-  st->dp = dp;
-  st->jpos = pos;
-  st->col = st->kl[l];
-  P.piv[k] = ((long long)l << kPivShift) | g;
-  P.dval[k] = dp;
-  st->kl[l] += 1;
-  st->k = k + 1;
-  st->bsteps += 1;
-  st->skip = 0;
-  st->dmax_bits = 0ull;
-  st->first = ULLONG_MAX;
-  if (P.timeout_ns) {
-    const unsigned long long now = globaltimer();
+  if (mine)
+    for (int q = 0; q < mynq; ++q) cols[q * nwork + tid] = __ldcg(B.bdf[lev] + int64_t(q) * nc + t);
+  if (mine) dmem[tid] = d;
+  double d0 = st->d0;
+  // binary exponents: tie_rel < 2^(e_rel + 1), tie_abs d0 < 2^(e_abs + 1) 2^-1023
+  const int e_rel = int(dkey(P.tie_rel) >> 52) - 1023;
+  int e_abs = int(dkey(P.tie_abs * d0) >> 52);
+  int j = 0;
+  for (; j < m; ++j) {
+    // ---- the largest residual
+    const unsigned long long wk = warp_max64(key);
+    if (lane == 0) wmax[warp] = wk;
+    __syncthreads();
+    const unsigned long long mk = warp_max64(lane < nwarp ? wmax[lane] : 0ull);
+    const double dmax = __longlong_as_double((long long)mk);
+    const int k = B.k + j;
+    // no further pivot: the next block's set, or an ordinary step, decides what that means
+    if (k >= P.nip || mk == 0ull) break;
+    if (P.tol > 0.0 && k > 0 && dmax < P.tol * d0) break;
     if (k == 0) {
-      st->t0 = now;
-    } else if (now - st->t0 > P.timeout_ns) {
-      st->err = ISDF_ERR_TIMEOUT;
-      st->done = 1;
-      st->final_ = 1;
+      d0 = dmax;
+      e_abs = int(dkey(P.tie_abs * d0) >> 52);
+      if (tid == 0) {
+        st->d0 = dmax;
+        st->t0 = globaltimer();
+      }
+    }
+    // ---- the smallest index within the tie window (members are in index
+    // order).  A relative distance x <= 1/4 below dmax is less than x 2^54 keys;
+    // x is bounded by the power of two above it.
+    const int sh = 55 + max(e_rel, e_abs - int(mk >> 52));
+    const bool hit = key >= ((sh < 53 && (mk >> 54)) ? mk - (1ull << max(sh, 2)) : 1ull);
+    unsigned b0 = __ballot_sync(0xffffffffu, hit);
+    if (lane == 0) {
+      wfirst[warp] = b0 ? warp * 32 + __ffs(int(b0)) - 1 : INT_MAX;
+      wcount[warp] = __popc(b0);
+    }
+    __syncthreads();
+    int p = __reduce_min_sync(0xffffffffu, lane < nwarp ? wfirst[lane] : INT_MAX);
+    const int nhit = __reduce_add_sync(0xffffffffu, lane < nwarp ? unsigned(wcount[lane]) : 0u);
+    if (nhit > 1) {  // more than one member near the maximum: the exact window
+      if (tid == 0) thr_sh = tie_key(P, dmax, d0);
+      __syncthreads();
+      b0 = __ballot_sync(0xffffffffu, key >= thr_sh);
+      if (lane == 0) wfirst[warp] = b0 ? warp * 32 + __ffs(int(b0)) - 1 : INT_MAX;
+      __syncthreads();
+      p = __reduce_min_sync(0xffffffffu, lane < nwarp ? wfirst[lane] : INT_MAX);
+    }
+    int pl = 0, pfirst = 0, q = nq[0], c = nstep[0];
+#pragma unroll
+    for (int l = 1; l < ISDF_MAX_LEVELS; ++l)
+      if (l < P.nlev && p >= begin[l]) pl = l, pfirst = begin[l], q = nq[l], c = nstep[l];
+    // ---- its column at the members of its level
+    const double dp = dmem[p];
+    for (int i = tid; i < q; i += nwork) R->lp[j][i] = cols[i * nwork + p];
+    if (tid == p) {
+      StepRec& rec = R->rec[j];
+      rec.dp = dp;
+      rec.dmax = dmax;
+      rec.idx = gidx;
+      rec.t = int(t);
+      rec.pos = p - pfirst;
+      rec.lev = pl;
+      R->list[pl][c] = j;
+      key = 0ull;
+    } else if (mine && lev == pl && key) {
+      const double b = gcols ? __ldcg(B.bm[pl] + int64_t(p - pfirst) * nc + t) : bss[p * nwork + tid];
+      float ah = 0.0f, al = 0.0f;
+#pragma unroll 4
+      for (int i = 0; i < q; ++i) {
+        const float2 x = cols[i * nwork + tid], l = cols[i * nwork + p];
+        const float pr = __fmul_rn(x.x, l.x);
+        float e = __fmaf_rn(x.x, l.x, -pr);
+        e = __fmaf_rn(x.x, l.y, e);
+        e = __fmaf_rn(x.y, l.x, e);
+        const DF s = two_sum(ah, pr);
+        ah = s.hi;
+        al = __fadd_rn(al, __fadd_rn(s.lo, e));
+      }
+      const DF v = df_mul(df_sub(df_from_double(b), two_sum(ah, al)), df_rsqrt(dp));
+      cols[q * nwork + tid] = make_float2(v.hi, v.lo);
+      const double vd = df_to_double(v);
+      d = fma(-vd, vd, d);
+      key = dkey(d);
+      dmem[tid] = d;
+    }
+#pragma unroll
+    for (int l = 0; l < ISDF_MAX_LEVELS; ++l)
+      if (l == pl) ++nq[l], ++nstep[l];
+  }
+  if (tid == 0) {
+    R->nsteps = j;
+    R->jstar = j;
+#pragma unroll
+    for (int l = 0; l < ISDF_MAX_LEVELS; ++l) R->nl[l] = nstep[l];
+  }
+}
+
+// The tried columns at every candidate, and the first step that some candidate
+// shows not to be the greedy one (atomicMin into jstar; threads stop at it).
+// A candidate's entry of a step needs its entries of the level's earlier
+// columns in the block (double-float, from L1/L2), so one thread walks one
+// candidate through all steps of its level.
+constexpr int kApply = 128;
+__global__ void __launch_bounds__(kApply) k_blk_apply(BlkParams B, const SelState* st, BlkRound* R) {
+  const SelParams& P = B.P;
+  __shared__ unsigned long long dmax_s[kMaxSet], thr_s[kMaxSet];
+  __shared__ int idx_s[kMaxSet], list_s[kMaxSet], pos_s[kMaxSet], t_s[kMaxSet];
+  __shared__ DF inv_s[kMaxSet], lp_s[2][kMaxSet];
+  __shared__ double sq_s[kMaxSet];
+  const int tid = threadIdx.x;
+  int l = 0;
+  while (l + 1 < P.nlev && int64_t(blockIdx.x) >= B.boff[l + 1]) ++l;
+  const int64_t nc = P.nc[l], t = (int64_t(blockIdx.x) - B.boff[l]) * kApply + tid;
+  const bool live = t < nc;
+  const int ns = R->nsteps, nl = R->nl[l], q0 = B.kl[l] - B.kb[l];
+  for (int i = tid; i < ns; i += kApply) {
+    const StepRec& r = R->rec[i];
+    dmax_s[i] = dkey(r.dmax);
+    thr_s[i] = tie_key(P, r.dmax, st->d0);
+    idx_s[i] = r.idx;
+  }
+  for (int k = tid; k < nl; k += kApply) {
+    const int i = R->list[l][k];
+    const StepRec& r = R->rec[i];
+    list_s[k] = i;
+    pos_s[k] = r.pos;
+    t_s[k] = r.t;
+    inv_s[k] = df_rsqrt(r.dp);
+    sq_s[k] = sqrt_from(r.dp, rsqrt64(r.dp));
+  }
+  auto stage = [&](int k) {  // lp of the level's step k
+    for (int i = tid; i < q0 + k; i += kApply) {
+      const float2 c = R->lp[list_s[k]][i];
+      lp_s[k & 1][i] = {c.x, c.y};
+    }
+  };
+  __syncthreads();
+  if (nl > 0) stage(0);
+  const int64_t gi = P.coff[l] + t;
+  double d = live ? P.d[gi] : 0.0;
+  unsigned long long key = dkey(d);
+  bool on = live;
+  int from = 0;  // first step not checked yet
+  float2* bdf = B.bdf[l] + t;
+  // the residual stands still over steps [from, to]: the step maxima fall, so
+  // only the last threshold has to be looked at when it is not reached
+  auto check = [&](int to) {
+    if (!on || to < from) return;
+    if (key >= thr_s[to])
+      for (int i = from; i <= to; ++i)
+        if (key > dmax_s[i] || (key >= thr_s[i] && gi < idx_s[i])) {
+          atomicMin(&R->jstar, i);
+          on = false;
+          break;
+        }
+    from = to + 1;
+  };
+  double bnext = (on && nl > 0) ? B.bm[l][int64_t(pos_s[0]) * nc + t] : 0.0;
+  for (int k = 0; k < nl; ++k) {
+    __syncthreads();
+    const int i = list_s[k];
+    const int js = *(volatile int*)&R->jstar;
+    if (i >= js) {  // this step is lost; the ones before it still need this candidate's word
+      check(js - 1);
+      on = false;
+    }
+    if (!__syncthreads_or(on)) return;
+    if (k + 1 < nl) stage(k + 1);
+    check(i);
+    if (!on) continue;
+    const double b = bnext;
+    if (k + 1 < nl) bnext = B.bm[l][int64_t(pos_s[k + 1]) * nc + t];
+    const bool pivot = t == t_s[k];
+    const double sq = sq_s[k];
+    const DF v = pivot ? df_from_double(sq) : blk_col_df(bdf, nc, q0 + k, lp_s[k & 1], b, inv_s[k]);
+    const double vd = pivot ? sq : df_to_double(v);
+    P.fac[l][int64_t(B.kl[l] + k) * nc + t] = vd;
+    bdf[int64_t(q0 + k) * nc] = make_float2(v.hi, v.lo);
+    if (pivot) {
+      key = 0ull;  // taken: it takes no part in later steps, but its row does
+      d = 0.0;
+    } else if (key) {
+      d = fma(-vd, vd, d);
+      key = dkey(d);
     }
   }
+  if (ns > 0) check(ns - 1);
 }
 
-// column of this step from B and the block's earlier columns; residual update
-__global__ void __launch_bounds__(256) k_blk_col(BlkParams B, const SelState* st) {
-  if (st->skip) return;
-  __shared__ DF lp[256];  // L[p, kb..col) (a block has at most 256 steps)
+// Accept steps [0, jstar): residuals, the digits of the new columns (whole
+// groups of 8, from the first one touched) and the state record.
+__global__ void __launch_bounds__(kApply) k_blk_commit(BlkParams B, BlkRound* R, SelState* st) {
   const SelParams& P = B.P;
-  const int l = st->lev;
-  const int col = st->col, kb = st->kb[l];
-  const int nb = col - kb;
-  const int64_t nc = P.nc[l], tp = st->tp;
-  float2* __restrict__ bdf = B.bdf[l];
-  __shared__ double sq_sh;
-  __shared__ DF inv_sh;
-  for (int i = threadIdx.x; i < nb; i += blockDim.x) {
-    const float2 c = bdf[int64_t(i) * nc + tp];
-    lp[i] = {c.x, c.y};
+  const int tid = threadIdx.x, js = R->jstar;
+  int l = 0;
+  while (l + 1 < P.nlev && int64_t(blockIdx.x) >= B.boff[l + 1]) ++l;
+  if (blockIdx.x == 0) {
+    for (int i = tid; i < js; i += kApply) {
+      const StepRec& r = R->rec[i];
+      const long long g = P.cidx[r.lev] ? P.cidx[r.lev][r.t] : r.t;
+      P.piv[B.k + i] = ((long long)r.lev << kPivShift) | g;
+      P.dval[B.k + i] = r.dp;
+    }
+    if (tid == 0) {
+      st->bsteps = js;
+      st->btried = R->nsteps;
+      st->k = B.k + js;
+      for (int a = 0; a < P.nlev; ++a) {
+        int c = 0;
+        while (c < R->nl[a] && R->list[a][c] < js) ++c;
+        st->kl[a] = B.kl[a] + c;
+      }
+      if (js > 0) st->dp = R->rec[js - 1].dp;
+      if (js > 0 && P.timeout_ns && globaltimer() - st->t0 > P.timeout_ns) {
+        st->err = ISDF_ERR_TIMEOUT;
+        st->final_ = 1;
+      }
+    }
   }
-  if (threadIdx.x == 0) {
-    sq_sh = sqrt(st->dp);
-    inv_sh = df_from_double(1.0 / sq_sh);
+  const int64_t nc = P.nc[l], t = (int64_t(blockIdx.x) - B.boff[l]) * kApply + tid;
+  int na = 0;
+  while (na < R->nl[l] && R->list[l][na] < js) ++na;
+  if (t >= nc || na == 0) return;
+  const double* fac = P.fac[l] + t;
+  const int c0 = B.kl[l], c1 = c0 + na;
+  double d = P.d[P.coff[l] + t];
+  if (dkey(d)) {
+    for (int k = 0; k < na; ++k) {
+      const double v = fac[int64_t(c0 + k) * nc];
+      d = R->rec[R->list[l][k]].t == t ? 0.0 : fma(-v, v, d);
+      if (!dkey(d)) break;
+    }
+    P.d[P.coff[l] + t] = d;
   }
-  __syncthreads();
-  const double sq = sq_sh;
-  const DF inv = inv_sh;
-  const double* __restrict__ bcol = B.bm[l] + int64_t(st->jpos) * nc;
-  double* __restrict__ facw = P.fac[l];
-  double* __restrict__ d = P.d + P.coff[l];
-  for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < nc; t += int64_t(gridDim.x) * blockDim.x) {
-    const DF v = (t == tp) ? df_from_double(sq) : blk_col_df(bdf + t, nc, nb, lp, bcol[t], inv);
-    const double vd = (t == tp) ? sq : df_to_double(v);
-    facw[int64_t(col) * nc + t] = vd;
-    bdf[int64_t(nb) * nc + t] = make_float2(v.hi, v.lo);
-    d[t] = (t == tp) ? 0.0 : fma(-vd, vd, d[t]);
-  }
+  oz_append_row(fac, nc, c0, c1, B.fexp[l][t], t, B.fkst[l], B.ftiles[l]);
 }
 
 }  // namespace
@@ -893,241 +1069,6 @@ isdf_status select_loop(Plan* p, int nip, double tol, const double* d0full, int*
   return ISDF_OK;
 }
 
-// ---------------------------------------------------------------- persistent block steps
-//
-// All greedy steps of one speculative block in one cooperative launch (every
-// CTA resident).  Each step is two phases separated by grid barriers:
-//   B: tie rule on d_max (computed in the previous phase A): smallest index
-//      with d >= thr, atomicMin;
-//   A: every CTA derives the same pivot from the shared slots, keeps its own
-//      copy of the counters, writes its share of the new column and residual
-//      and reduces the residual's maximum for the next step; CTA 0 records
-//      the pivot.
-// The pivot's own residual is zeroed in the next phase B (other CTAs read it
-// during phase A), and that phase's search skips it.  Barriers are bounded:
-// after ~1 s of device time a CTA records an error and leaves; every CTA
-// leaves at the next barrier it reaches, so the launch always ends.
-
-struct StepSync {
-  unsigned int count;
-  unsigned int gen;
-  int abort;
-  int pad;
-  unsigned long long dmax[2];
-  unsigned long long first[2];
-};
-
-constexpr unsigned long long kBarrierNs = 1000000000ull;
-
-__device__ bool grid_sync(StepSync* sy, unsigned int nblocks) {
-  __shared__ int ok_sh;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int ok = 1;
-    volatile unsigned int* gen = &sy->gen;
-    const unsigned int g = *gen;
-    __threadfence();
-    if (atomicAdd(&sy->count, 1u) == nblocks - 1) {
-      sy->count = 0;
-      __threadfence();
-      atomicAdd(&sy->gen, 1u);
-    } else {
-      const unsigned long long t0 = globaltimer();
-      long long i = 0;
-      while (*gen == g) {
-        if (*(volatile int*)&sy->abort) { ok = 0; break; }
-        if ((++i & 1023) == 0 && globaltimer() - t0 > kBarrierNs) {
-          atomicExch(&sy->abort, 1);
-          ok = 0;
-          break;
-        }
-      }
-    }
-    __threadfence();
-    if (*(volatile int*)&sy->abort) ok = 0;
-    ok_sh = ok;
-  }
-  __syncthreads();
-  return ok_sh != 0;
-}
-
-__global__ void k_sync_init(StepSync* sy) {
-  if (threadIdx.x != 0) return;
-  sy->count = 0;
-  sy->gen = 0;
-  sy->abort = 0;
-  sy->dmax[0] = sy->dmax[1] = 0ull;
-  sy->first[0] = sy->first[1] = ULLONG_MAX;
-}
-
-__global__ void __launch_bounds__(512) k_blk_steps(BlkParams B, SelState* st, StepSync* sy, int smax) {
-  const SelParams& P = B.P;
-  __shared__ DF lpd[256];  // the pivot's entries in the block's earlier columns
-  __shared__ int kl_sh[ISDF_MAX_LEVELS];
-  __shared__ unsigned long long red[32];
-  __shared__ int stop_sh;
-  __shared__ unsigned long long thr_sh;
-  __shared__ double sq_sh;
-  __shared__ DF inv_sh;
-  const unsigned int nb = gridDim.x;
-  const int tid = threadIdx.x;
-  const int64_t gtid = int64_t(blockIdx.x) * blockDim.x + tid, gstride = int64_t(gridDim.x) * blockDim.x;
-  // private copies of the counters (identical in every CTA)
-  int k = st->k;
-  double d0 = st->d0;
-  __shared__ int kb[ISDF_MAX_LEVELS];  // columns per level when the block began
-  if (tid < ISDF_MAX_LEVELS) kl_sh[tid] = kb[tid] = st->kl[tid];
-  __syncthreads();
-  long long last = -1;  // global index of the previous step's pivot (its residual is zeroed next phase B)
-  double last_dp = st->dp;  // value of the last pivot taken (written back with the counters)
-  int bsteps = 0, reason = 0;  // reason: 0 running, 1 block end, 2 final, 3 timeout, 4 barrier failure
-  // Residual comparisons use the order-preserving integer keys of the values,
-  // and the per-step scalars are formed by one thread per CTA: the FP64 unit
-  // is left to the two operations per candidate that need it.
-  // phase 0: d_max of the current residual into slot 0
-  {
-    unsigned long long mk = 0ull;
-    for (int64_t i = gtid; i < P.ntot; i += gstride) mk = max(mk, dkey(__ldcg(P.d + i)));
-    mk = block_reduce(mk, MaxU64(), red);
-    if (tid == 0) atomicMax(&sy->dmax[0], mk);
-  }
-  if (!grid_sync(sy, nb)) reason = 4;
-  for (int j = 0; reason == 0; ++j) {
-    const int par = j & 1;
-    // ---------------- phase B
-    if (last >= 0 && gtid == 0) P.d[last] = 0.0;  // visible after the barrier
-    const double dmax = __longlong_as_double((long long)*(volatile unsigned long long*)&sy->dmax[par]);
-    if (tid == 0) {
-      const double dz = (k == 0) ? dmax : d0;
-      int stop = 0;
-      if (j >= smax)
-        stop = 1;
-      else if (k >= P.nip || !(dmax > 0.0) || dmax < P.tol * dz)
-        stop = 2;
-      stop_sh = stop;
-      // d >= thr and d > 0  <=>  key(d) >= max(key(thr), 1)
-      thr_sh = max(dkey(dmax - fmax(P.tie_rel * dmax, P.tie_abs * dz)), 1ull);
-    }
-    __syncthreads();
-    if (stop_sh) {
-      reason = stop_sh;
-      break;
-    }
-    const unsigned long long tk = thr_sh;
-    unsigned long long best = ULLONG_MAX;
-    for (int64_t i = gtid; i < P.ntot; i += gstride) {
-      if (i == last) continue;
-      if (dkey(__ldcg(P.d + i)) >= tk) {
-        best = (unsigned long long)i;
-        break;
-      }
-    }
-    best = block_reduce(best, MinOp(), red);
-    if (tid == 0 && best != ULLONG_MAX) atomicMin(&sy->first[par], best);
-    if (gtid == 0) {  // slots of the next step
-      sy->dmax[par ^ 1] = 0ull;
-      sy->first[par ^ 1] = ULLONG_MAX;
-    }
-    if (!grid_sync(sy, nb)) { reason = 4; break; }
-    // ---------------- phase A
-    const unsigned long long idx = *(volatile unsigned long long*)&sy->first[par];
-    if (idx == ULLONG_MAX) { reason = 2; break; }
-    const int pos = __ldcg(B.spos + idx);
-    if (pos < 0) { reason = 1; break; }  // greedy pivot outside S: block ends
-    int l = 0;
-    while (l + 1 < P.nlev && (long long)idx >= P.coff[l + 1]) ++l;
-    const long long tp = (long long)idx - P.coff[l];
-    const double dp = __ldcg(P.d + idx);
-    const int col = kl_sh[l];
-    const int nbk = col - kb[l];
-    const int64_t nc = P.nc[l];
-    float2* __restrict__ bdf = B.bdf[l];
-    __syncthreads();
-    for (int i = tid; i < nbk; i += blockDim.x) {
-      const float2 c = __ldcg(bdf + int64_t(i) * nc + tp);
-      lpd[i] = {c.x, c.y};
-    }
-    if (tid == 0) {
-      sq_sh = sqrt(dp);
-      inv_sh = df_from_double(1.0 / sq_sh);
-    }
-    __syncthreads();
-    if (k == 0) d0 = dmax;
-    last_dp = dp;
-    if (gtid == 0) {
-      const long long g = P.cidx[l] ? P.cidx[l][tp] : tp;
-      P.piv[k] = ((long long)l << kPivShift) | g;
-      P.dval[k] = dp;
-      if (k == 0) {
-        st->d0 = dmax;
-        st->t0 = globaltimer();
-      }
-    }
-    const double sq = sq_sh;
-    const DF inv = inv_sh;
-    const double* __restrict__ bcol = B.bm[l] + int64_t(pos) * nc;
-    double* __restrict__ facw = P.fac[l];
-    const int64_t lo = P.coff[l], hi = P.coff[l + 1];
-    unsigned long long mk = 0ull;
-    for (int64_t i = gtid; i < P.ntot; i += gstride) {
-      unsigned long long key;
-      if (i >= lo && i < hi) {
-        const int64_t t = i - lo;
-        const double di = __ldcg(P.d + i);
-        const DF v = (t == tp) ? df_from_double(sq) : blk_col_df(bdf + t, nc, nbk, lpd, bcol[t], inv);
-        const double vd = (t == tp) ? sq : df_to_double(v);
-        facw[int64_t(col) * nc + t] = vd;
-        bdf[int64_t(nbk) * nc + t] = make_float2(v.hi, v.lo);
-        if (t == tp) {
-          key = 0ull;  // written as 0 in the next phase B
-        } else {
-          const double dn = fma(-vd, vd, di);
-          P.d[i] = dn;
-          key = dkey(dn);
-        }
-      } else {
-        key = (i == (long long)idx) ? 0ull : dkey(__ldcg(P.d + i));
-      }
-      mk = max(mk, key);
-    }
-    mk = block_reduce(mk, MaxU64(), red);
-    if (tid == 0) atomicMax(&sy->dmax[par ^ 1], mk);
-    // counters advance identically in every CTA
-    __syncthreads();
-    if (tid == 0) kl_sh[l] = col + 1;
-    __syncthreads();
-    ++k;
-    ++bsteps;
-    last = (long long)idx;
-    // time budget: CTA 0's clock decides for everyone and publishes the decision
-    // before the barrier (this step's column is complete)
-    if (gtid == 0 && P.timeout_ns && globaltimer() - st->t0 > P.timeout_ns) atomicExch(&sy->abort, 2);
-    if (!grid_sync(sy, nb)) {
-      reason = (*(volatile int*)&sy->abort == 2) ? 3 : 4;
-      break;
-    }
-  }
-  // the last pivot's residual is zeroed here if no phase B followed it
-  if (last >= 0 && gtid == 0) P.d[last] = 0.0;
-  if (gtid == 0) {
-    st->k = k;
-    st->dp = last_dp;
-    for (int l = 0; l < ISDF_MAX_LEVELS; ++l) st->kl[l] = kl_sh[l];
-    st->bsteps = bsteps;
-    st->done = 1;
-    st->skip = 1;
-    if (reason == 2) st->final_ = 1;
-    if (reason == 3) {
-      st->err = ISDF_ERR_TIMEOUT;
-      st->final_ = 1;
-    }
-    if (reason == 4) {
-      st->err = ISDF_ERR_CUDA;
-      st->final_ = 1;
-    }
-  }
-}
-
 __global__ void k_scatter_pos(const int* __restrict__ cidx, int64_t nc, int* __restrict__ gpos) {
   const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (t < nc) gpos[cidx[t]] = int(t);
@@ -1173,18 +1114,6 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
   *aborted = false;
   int64_t nc[ISDF_MAX_LEVELS] = {0, 0, 0, 0};
   for (int l = 0; l < nlev; ++l) nc[l] = nc_in[l];
-  // with the cooperative block steps the factor storage of a level starts at
-  // a quarter of nip and grows between blocks (a level rarely takes more);
-  // the captured graph of the other form holds fixed arrays: full capacity
-  bool growable = false;
-  {
-    int d = 0, coop_attr = 0, spsm = 0;
-    cudaGetDevice(&d);
-    cudaDeviceGetAttribute(&coop_attr, cudaDevAttrCooperativeLaunch, d);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&spsm, k_blk_steps, 512, 0);
-    cudaGetLastError();
-    growable = coop_attr && spsm > 0;
-  }
   int* cur_cidx[ISDF_MAX_LEVELS] = {nullptr, nullptr, nullptr, nullptr};  // after compaction: owned here
   for (int l = 0; l < nlev; ++l) cur_cidx[l] = cidx[l];
   std::vector<int*> own_cidx;
@@ -1207,12 +1136,11 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
     OzOperand aL, aN, aF, bL, bN, bF;
     double *cL = nullptr, *cN = nullptr, *cF = nullptr;
     int* gpos = nullptr;
-    int sliced = 0;
   } lb[ISDF_MAX_LEVELS];
   int *counts = nullptr, *nlist = nullptr, *list = nullptr, *sidx = nullptr, *sg = nullptr, *stp = nullptr,
-      *scount = nullptr, *spos = nullptr;
-  cudaGraphExec_t exec = nullptr;
-  void* sync_mem = nullptr;
+      *scount = nullptr;
+  BlkRound* round = nullptr;
+  float2* gcols = nullptr;
   auto cleanup = [&]() {
     for (int* q : own_cidx) dfree(q);
     own_cidx.clear();
@@ -1223,9 +1151,8 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
       dfree(p->lev[l].fac);
       p->lev[l].fac = nullptr;
     }
-    dfree(counts), dfree(nlist), dfree(list), dfree(sidx), dfree(sg), dfree(stp), dfree(scount), dfree(spos);
-    dfree(sync_mem);
-    if (exec) cudaGraphExecDestroy(exec);
+    dfree(counts), dfree(nlist), dfree(list), dfree(sidx), dfree(sg), dfree(stp), dfree(scount);
+    dfree(round), dfree(gcols);
   };
   auto bail = [&](isdf_status r) {
     cleanup();
@@ -1243,9 +1170,8 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
     LevBuf& b = lb[l];
     dfree(lv.fac);
     lv.fac = nullptr;
-    lv.fac_cap = std::min<int64_t>(nip, nc[l]);
-    if (growable)
-      lv.fac_cap = std::min<int64_t>(lv.fac_cap, std::max<int64_t>(4 * int64_t(smax) + 1, nip / 4));
+    // factor storage starts at a quarter of nip and grows between blocks (a level rarely takes more)
+    lv.fac_cap = std::min<int64_t>(std::min<int64_t>(nip, nc[l]), std::max<int64_t>(4 * int64_t(smax) + 1, nip / 4));
     if ((st = dalloc_t(p, &lv.fac, size_t(std::max<int64_t>(lv.fac_cap * nc[l], 1)), "selection factor columns")))
       return bail(st);
     P.fac[l] = lv.fac;
@@ -1302,26 +1228,36 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
   P.tie_rel = p->opt.tie_rel;
   P.tie_abs = p->opt.tie_abs;
   P.timeout_ns = (unsigned long long)p->opt.timeout_ms * 1000000ull;
-  int64_t nbk = (P.ntot + kCompactBlock - 1) / kCompactBlock;
+  const int64_t nbk = (P.ntot + kCompactBlock - 1) / kCompactBlock;
+  // B and the members' columns during the greedy steps: shared memory up to 112 members, else global
+  const int gthreads = ((smax + 31) / 32) * 32;
+  const size_t gsmem = 2 * sizeof(double) * size_t(gthreads) * smax;
+  const bool gshared = gsmem <= 216 * 1024;
   if ((st = dalloc_t(p, &counts, size_t(std::max<int64_t>(nbk, 1)), "block counts")) ||
       (st = dalloc_t(p, &nlist, 1, "list size")) ||
       (st = dalloc_t(p, &list, size_t(std::max<int64_t>(P.ntot, 1)), "local maxima")) ||
       (st = dalloc_t(p, &sidx, size_t(smax), "speculative set")) || (st = dalloc_t(p, &sg, size_t(smax), "speculative set")) ||
       (st = dalloc_t(p, &stp, size_t(smax), "speculative set")) ||
       (st = dalloc_t(p, &scount, size_t(ISDF_MAX_LEVELS + 1), "speculative set")) ||
-      (st = dalloc_t(p, &spos, size_t(std::max<int64_t>(P.ntot, 1)), "speculative positions")))
+      (st = dalloc_t(p, &round, 1, "block round")) ||
+      (!gshared && (st = dalloc_t(p, &gcols, size_t(gthreads) * smax, "block columns"))))
     return bail(st);
-  cudaMemsetAsync(spos, 0xFF, sizeof(int) * size_t(std::max<int64_t>(P.ntot, 1)), s);
+  if (gshared && gsmem > 40 * 1024 &&
+      (st = cuda_check(p, cudaFuncSetAttribute(k_blk_greedy, cudaFuncAttributeMaxDynamicSharedMemorySize, int(gsmem)),
+                       "smem attribute")))
+    return bail(st);
   BlkParams BP{};
   BP.P = P;
-  BP.spos = spos;
+  BP.sidx = sidx;
+  BP.st = stp;
+  BP.scount = scount;
   for (int l = 0; l < nlev; ++l) {
     BP.bm[l] = lb[l].cL;
     // the factor product's output is free during the steps: it holds the
     // double-float copy of the block's columns (s x nc values of 8 bytes)
     BP.bdf[l] = reinterpret_cast<float2*>(lb[l].cF);
   }
-  TopSOut O{sidx, sg, stp, scount, spos};
+  TopSOut O{sidx, sg, stp, scount};
 
   SelState h{};
   h.dmax_bits = 0;
@@ -1341,33 +1277,6 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sel_col, 32 * kColWarps, smem);
   const unsigned red_blocks = unsigned(nsm) * 4;
   const unsigned col_blocks = per_sm > 0 ? unsigned(per_sm * nsm) : kColBlocks;
-  auto block_step = [&]() {
-    k_sel_max<<<red_blocks, 256, 0, s>>>(P, dst);
-    k_sel_first<<<red_blocks, 256, 0, s>>>(P, dst);
-    k_blk_pick<<<1, 32, 0, s>>>(BP, dst);
-    k_blk_col<<<unsigned(nsm) * 8, 256, 0, s>>>(BP, dst);
-  };
-  // persistent steps: one cooperative launch per block (every CTA resident)
-  StepSync* sync = nullptr;
-  int coop_dev = 0, steps_per_sm = 0;
-  cudaDeviceGetAttribute(&coop_dev, cudaDevAttrCooperativeLaunch, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&steps_per_sm, k_blk_steps, 512, 0);
-  cudaGetLastError();
-  const unsigned steps_blocks = unsigned(nsm) * unsigned(std::min(steps_per_sm, 2));
-  const bool coop = coop_dev && steps_per_sm > 0;
-  if (coop && (st = dalloc_t(p, &sync, 1, "step barrier"))) return bail(st);
-  sync_mem = sync;
-  if (!coop && s != nullptr) {
-    cudaGraph_t graph = nullptr;
-    if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-      for (int i = 0; i < smax; ++i) block_step();
-      if (cudaStreamEndCapture(s, &graph) != cudaSuccess || !graph || cudaGraphInstantiate(&exec, graph, 0) != cudaSuccess)
-        exec = nullptr;
-      if (graph) cudaGraphDestroy(graph);
-    }
-    cudaGetLastError();
-  }
-
   // ---- exact compaction of the candidates below tau (see above)
   int64_t since_compact = 0;
   auto compact = [&]() -> isdf_status {
@@ -1454,6 +1363,7 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
         cudaMemsetAsync(b.aF.tiles, 0, size_t(b.aF.nrt) * size_t(kst_keep) * kSlices * 128 * kOzBK * 2, s);
         k_fac_exps<<<unsigned((b.aF.nrt * 128 + 255) / 256), 256, 0, s>>>(d0c, nn, b.aF.nrt * 128, b.aF.exps);
         count_launches(1);
+        b.aF.K = h.kl[l];
         if (h.kl[l] > 0) oz_slice_ex(fnew, 1, nn, nullptr, b.aF, 0, (h.kl[l] + 7) / 8, true, s);
       }
       dfree(lv.fac);
@@ -1485,7 +1395,7 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
     return ISDF_OK;
   };
   // ---- factor capacity: before a block that could fill a level (at most
-  // smax block steps and one single step), that level's factor columns move
+  // smax block steps, or one single step), that level's factor columns move
   // to twice the storage and their digits are sliced again (fixed scales
   // from sqrt(d0), as at set-up)
   auto grow = [&]() -> isdf_status {
@@ -1525,7 +1435,6 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
       count_launches(1);
       b.aF.K = kl;
       if (kl > 0) oz_slice_ex(fnew, 1, nc[l], nullptr, b.aF, 0, (kl + 7) / 8, true, s);
-      b.sliced = kl;
       gst = cuda_check(p, cudaStreamSynchronize(s), "factor capacity");
       dfree(lv.fac);
       dfree(d0c);
@@ -1539,16 +1448,15 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
   };
   int64_t nblocks = 0, nplain = 0;
   std::vector<int> hcount(ISDF_MAX_LEVELS + 1);
+  int m_next = std::min(smax, 32);  // steps tried per round: a quarter more than the last one accepted, and 6
   while (true) {
-    if (growable && (st = grow())) return bail(st);
+    if ((st = grow())) return bail(st);
     // ---- 1. the speculative set S
     {
-      Prof pr(p, "select_spec", double(P.ntot) * 8.0, "byte", 4);
-      k_lm_count<<<unsigned(std::max<int64_t>(nbk, 1)), kCompactBlock, 0, s>>>(Q, counts);
-      k_scan_counts<<<1, 1024, 0, s>>>(counts, nbk, nlist);
-      k_lm_write<<<unsigned(std::max<int64_t>(nbk, 1)), kCompactBlock, 0, s>>>(Q, counts, list);
+      Prof pr(p, "select_spec", double(P.ntot) * 8.0, "byte", 2);
+      cudaMemsetAsync(nlist, 0, sizeof(int), s);
+      k_lm_list<<<unsigned(std::max<int64_t>((P.ntot + 255) / 256, 1)), 256, 0, s>>>(Q, list, nlist);
       k_top_s<<<1, 1024, 0, s>>>(Q, list, nlist, smax, O);
-      count_launches(4);
     }
     cudaMemcpyAsync(hcount.data(), scount, sizeof(int) * hcount.size(), cudaMemcpyDeviceToHost, s);
     if ((st = cuda_check(p, cudaStreamSynchronize(s), "speculative set"))) return bail(st);
@@ -1603,55 +1511,59 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
       count_launches(1);
       soff += sl;
     }
-    // ---- 3. greedy steps of this block
-    {
-      Prof pr(p, "select_steps", 0.0, "byte", coop ? 1 : 4ll * smax);
-      k_blk_begin<<<1, 32, 0, s>>>(dst);
-      if (coop) {
-        k_sync_init<<<1, 32, 0, s>>>(sync);
-        int smax_arg = smax;
-        void* args[] = {&BP, &dst, &sync, &smax_arg};
-        if ((st = cuda_check(p, cudaLaunchCooperativeKernel((const void*)k_blk_steps, dim3(steps_blocks), dim3(512), args,
-                                                            0, s),
-                             "block steps launch")))
-          return bail(st);
-        count_launches(2);
-      } else if (exec) {
-        cudaGraphLaunch(exec, s);
-        count_launches(4ll * smax);
-      } else {
-        for (int i = 0; i < smax; ++i) block_step();
-        count_launches(4ll * smax);
+    // ---- 3. greedy steps of this block, in rounds: as long as every tried step
+    // of a round is accepted there may be more in S
+    int taken = 0;
+    for (int l = 0; l < nlev; ++l) BP.kb[l] = h.kl[l];
+    while (true) {
+      int kl_before[ISDF_MAX_LEVELS];
+      for (int l = 0; l < nlev; ++l) kl_before[l] = h.kl[l];
+      const int m = std::min(m_next, smax - taken);
+      {
+        Prof pr(p, "select_steps", 0.0, "byte", 3);
+        BP.P = P;
+        BP.k = h.k;
+        BP.boff[0] = 0;
+        for (int l = 0; l < nlev; ++l) {
+          BP.kl[l] = h.kl[l];
+          BP.boff[l + 1] = BP.boff[l] + (nc[l] + kApply - 1) / kApply;
+          BP.fexp[l] = lb[l].aF.exps;
+          BP.ftiles[l] = lb[l].aF.tiles;
+          BP.fkst[l] = lb[l].aF.kst;
+        }
+        const unsigned nblk = unsigned(std::max<int64_t>(BP.boff[nlev], 1));
+        k_blk_greedy<<<1, gthreads, gshared ? gsmem : 0, s>>>(BP, dst, round, m, smax, gcols);
+        k_blk_apply<<<nblk, kApply, 0, s>>>(BP, dst, round);
+        k_blk_commit<<<nblk, kApply, 0, s>>>(BP, round, dst);
       }
-      k_spos_clear<<<unsigned((smax + 255) / 256), 256, 0, s>>>(sidx, scount, spos);
-      count_launches(2);
+      if ((st = cuda_check(p, cudaGetLastError(), "selection kernels"))) return bail(st);
+      cudaMemcpyAsync(&h, dst, sizeof(h), cudaMemcpyDeviceToHost, s);
+      if ((st = cuda_check(p, cudaStreamSynchronize(s), "block state"))) return bail(st);
+      if (p->opt.profile && !p->pend.empty() && p->pend.back().name == "select_steps") {
+        // algorithmic bytes of the round: per accepted step and candidate of its
+        // level the column of B, the block's earlier columns and the new column;
+        // the residual once
+        double bytes = 16.0 * double(P.ntot);
+        for (int l = 0; l < nlev; ++l) {
+          const double dk = h.kl[l] - kl_before[l], n = double(nc[l]);
+          bytes += 24.0 * dk * n + 8.0 * n * dk * (dk - 1.0) / 2.0;
+        }
+        p->pend.back().work = bytes;
+      }
+      taken += h.bsteps;
+      m_next = std::min(smax, std::max(12, h.bsteps + h.bsteps / 4 + 6));
+      if (h.err || h.final_ || h.k >= nip || h.bsteps < m || taken >= smax) break;
     }
     ++nblocks;
-    if ((st = cuda_check(p, cudaGetLastError(), "selection kernels"))) return bail(st);
-    int kl_before[ISDF_MAX_LEVELS];
-    for (int l = 0; l < nlev; ++l) kl_before[l] = h.kl[l];
-    cudaMemcpyAsync(&h, dst, sizeof(h), cudaMemcpyDeviceToHost, s);
-    if ((st = cuda_check(p, cudaStreamSynchronize(s), "block state"))) return bail(st);
-    if (p->opt.profile && !p->pend.empty() && p->pend.back().name == "select_steps") {
-      // algorithmic bytes of the block's steps: two passes over the residual
-      // (max, tie rule), then per candidate of the pivot's level the column of
-      // B, the block's earlier columns, the new column and the residual
-      double bytes = 0.0;
-      for (int l = 0; l < nlev; ++l) {
-        const double dk = h.kl[l] - kl_before[l], n = double(nc[l]);
-        bytes += dk * (16.0 * double(P.ntot) + 32.0 * n) + 8.0 * n * dk * (dk - 1.0) / 2.0;
-      }
-      p->pend.back().work = bytes;
-    }
     if (h.err || h.final_ || h.k >= nip) break;
-    if (tau > 0.0 && h.dp * (1.0 - 2.0 * p->opt.tie_rel) - 2.0 * p->opt.tie_abs * h.d0 < tau) {
+    if (tau > 0.0 && taken > 0 && h.dp * (1.0 - 2.0 * p->opt.tie_rel) - 2.0 * p->opt.tie_abs * h.d0 < tau) {
       *aborted = true;  // a pivot value broke the certificate: retry with a lower tau
       break;
     }
-    if (h.bsteps == 0) {
+    if (taken == 0) {
       // the greedy pivot was not in S: one ordinary step
       Prof pr(p, "select_loop", 0.0, "flop", 4);
-      k_blk_begin<<<1, 32, 0, s>>>(dst);
+      k_step_begin<<<1, 32, 0, s>>>(dst);
       k_sel_max<<<red_blocks, 256, 0, s>>>(P, dst);
       k_sel_first<<<red_blocks, 256, 0, s>>>(P, dst);
       k_sel_pick<<<1, 32, 0, s>>>(P, dst);
@@ -1666,23 +1578,18 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
       *aborted = true;
       break;
     }
-    // ---- 4. digits of the new factor columns (whole k tiles from the first changed one)
-    {
-      Prof pr(p, "select_slice", 0.0, "byte", nlev);
+    // ---- 4. digits of an ordinary step's column (a block's are written as it is accepted)
+    if (taken == 0) {
+      Prof pr(p, "select_slice", 0.0, "byte", kLaunchesInside);
       for (int l = 0; l < nlev; ++l) {
         LevBuf& b = lb[l];
-        if (h.kl[l] <= b.sliced) continue;
+        if (h.kl[l] <= BP.kl[l]) continue;
         b.aF.K = h.kl[l];
-        oz_slice_ex(p->lev[l].fac, 1, nc[l], nullptr, b.aF, b.sliced / 8, (h.kl[l] + 7) / 8, true, s);
-        b.sliced = h.kl[l];
+        oz_slice_ex(p->lev[l].fac, 1, nc[l], nullptr, b.aF, BP.kl[l] / 8, (h.kl[l] + 7) / 8, true, s);
       }
     }
-    // ---- 5. drop the candidates whose residual fell below tau (checked every
-    // other block; the graph of the non-cooperative form holds the old arrays)
-    if (tau > 0.0 && !exec && ++since_compact >= 2) {
-      if ((st = compact())) return bail(st);
-      nbk = (P.ntot + kCompactBlock - 1) / kCompactBlock;
-    }
+    // ---- 5. drop the candidates whose residual fell below tau (checked every other block)
+    if (tau > 0.0 && ++since_compact >= 2 && (st = compact())) return bail(st);
   }
   if ((st = oz_check(p))) return bail(st);
   *nfound = h.k;
