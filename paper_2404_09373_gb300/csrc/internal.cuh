@@ -273,6 +273,22 @@ void oz_slice_ex(const double* src, int64_t sr, int64_t sk, const int* ridx, OzO
 // splits > 1 needs work of splits*M*N doubles.  Error codes go to *err.
 void oz_gemm(const OzOperand& A, const OzOperand& B, double* C, int64_t ldc, int trans, double alpha, int tri, int sym,
              int splits, double* work, int* err, cudaStream_t s);
+// One level of a selection block's columns (ozgemm.cu): products q = 0 (own
+// functions), 1 (coarser functions), 2 (factor columns), each absent if its
+// operand is null or has no k tiles.  C[j][t] (j a member of the set, ld M).
+struct OzColumnJob {
+  const OzOperand* A[3] = {nullptr, nullptr, nullptr};  // candidates, 128-row tiles, 8 digits
+  OzOperand* B[3] = {nullptr, nullptr, nullptr};        // the set's rows
+  const double* src[3] = {nullptr, nullptr, nullptr};   // FP64 source of B: (row, k) at src[row + k * ld]
+  int64_t ld[3] = {0, 0, 0};
+  int64_t M = 0;
+  double* C = nullptr;
+  double w = 0.0;
+};
+// digits of the set's rows (st: candidate, sg: grid point of each member), then the columns
+void oz_set_rows(const OzColumnJob* jobs, int nlev, int smax, const int* scount, const int* st, const int* sg,
+                 cudaStream_t s);
+void oz_columns(const OzColumnJob* jobs, int nlev, const int* scount, int* err, cudaStream_t s);
 int64_t oz_tile_elems(int64_t rows, int64_t K, int rt, int S);
 // the same product with its scratch in a fixed static device array (no allocation)
 // split-K factor of a product shape: cached, else timed on these operands

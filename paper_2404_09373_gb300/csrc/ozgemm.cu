@@ -587,6 +587,84 @@ struct OzCfg {
   static_assert(smem <= 232448, "shared memory per CTA");
 };
 
+// The MMAs of one pipeline stage (32 k values).  For A digit s the products
+// with B digits t = 0..S-1-s land in levels s..S-1, i.e. tensor-memory columns
+// [s BN, S BN); the B digit tiles of a stage are contiguous, so B rows [0,
+// (S-s) BN) are exactly digits 0..S-1-s and one MMA (N up to 256, else split)
+// covers them all.  The first MMA of a chunk (s = 0) spans every level and
+// initialises the accumulators.
+template <int S, int BN>
+__device__ __forceinline__ void mma_stage(uint32_t tmem, uint32_t sA, uint32_t sB, bool first) {
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+#pragma unroll
+    for (int c0 = 0; c0 < BN * (S - s); c0 += 256) {
+      const int n = (BN * (S - s) - c0) < 256 ? (BN * (S - s) - c0) : 256;
+      const uint32_t idesc = umma_idesc(kBM, n);
+#pragma unroll
+      for (int ks = 0; ks < kBK / 16; ++ks) {
+        const uint64_t da = umma_desc(sA + s * OzCfg<S, BN>::tileA + ks * 256);
+        const uint64_t db = umma_desc(sB + (c0 / 8) * (16 * kBK) + ks * 256);
+        umma_bf16(tmem + uint32_t(s * BN + c0), da, db, idesc, (!first || s > 0 || ks > 0) ? 1u : 0u);
+      }
+    }
+  }
+}
+
+// Add one chunk's accumulators (HC columns of this warp's 32 lanes) to the
+// exact integer sums of 7 or 8 digits.  Levels 0..7 of one column and chunk
+// (512 k: levels 0..5 are exact integers below 2^24) are paired exactly in
+// 32-bit integers,
+//   P01 = L0 2^7 + L1, P23 = L2 2^7 + L3, P45 = L4 2^7 + L5  (< 2^31),
+// and levels 6, 7 (weights below 2^-42) are combined in FP32.  Per column th
+// accumulates P01 2^14 + P23 plus the part of lo = P45 2^14 + (L6 2^7 + L7)
+// above 2^28; rem keeps lo's low 28 bits (carried into th), so the value is
+// th + rem 2^-28 in units of 2^-21.  With 7 digits there is no level 7 (L7 = 0).
+template <int S, int BN, int HC>
+__device__ __forceinline__ void drain_exact(uint32_t tbase, long long (&th)[HC], uint32_t (&rem)[HC]) {
+#pragma unroll
+  for (int c0 = 0; c0 < HC; c0 += 16) {
+#pragma unroll
+    for (int pq = 0; pq < 4; ++pq) {  // level pairs (0,1) (2,3) (4,5) (6,7)
+      uint32_t ra[16], rb[16];
+      tmem_ld16(tbase + uint32_t((2 * pq) * BN + c0), ra);
+      if (2 * pq + 1 < S) {
+        tmem_ld16(tbase + uint32_t((2 * pq + 1) * BN + c0), rb);
+      } else {  // 7 digits: no level 7
+#pragma unroll
+        for (int j = 0; j < 16; ++j) rb[j] = 0u;
+      }
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        const float fa = __uint_as_float(ra[j]), fb = __uint_as_float(rb[j]);
+        if (pq < 3) {
+          const int pair = __float2int_rn(fa) * 128 + __float2int_rn(fb);  // exact, |pair| < 2^31
+          if (pq == 0) {
+            th[c0 + j] += (long long)pair * (1ll << 14);
+          } else if (pq == 1) {
+            th[c0 + j] += (long long)pair;
+          } else {
+            const long long x = (long long)pair * (1ll << 14);  // lo part of levels 4, 5
+            th[c0 + j] += x >> 28;
+            rem[c0 + j] += uint32_t(x & 0x0FFFFFFFll);
+          }
+        } else {
+          const long long x = intf_to_ll(fmaf(fa, 128.0f, fb));  // levels 6, 7
+          th[c0 + j] += x >> 28;
+          rem[c0 + j] += uint32_t(x & 0x0FFFFFFFll);
+        }
+      }
+      reg_fence16(th, rem);
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < HC; ++j) {  // rem < 3 * 2^28 here
+    th[j] += (long long)(rem[j] >> 28);
+    rem[j] &= 0x0FFFFFFFu;
+  }
+}
+
 template <int S, int BN>
 __global__ void __launch_bounds__(OzCfg<S, BN>::threads, OzCfg<S, BN>::min_blocks) k_oz_gemm(OzGemmParams P) {
   using Cfg = OzCfg<S, BN>;
@@ -717,27 +795,7 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, OzCfg<S, BN>::min_block
           asm volatile("tcgen05.fence::after_thread_sync;");
           const uint32_t sA = smem_u32(smem + st * Cfg::stage);
           const uint32_t sB = sA + Cfg::stageA;
-          // For A digit s the products with B digits t = 0..S-1-s land in
-          // levels s..S-1, i.e. tensor-memory columns [s BN, S BN); the B
-          // digit tiles of a stage are contiguous, so B rows [0, (S-s) BN) are
-          // exactly digits 0..S-1-s and one MMA (N up to 256, else split)
-          // covers them all.  The first MMA of a chunk (s = 0) spans every
-          // level and initialises the accumulators.
-#pragma unroll
-          for (int s = 0; s < S; ++s) {
-#pragma unroll
-            for (int c0 = 0; c0 < BN * (S - s); c0 += 256) {
-              const int n = (BN * (S - s) - c0) < 256 ? (BN * (S - s) - c0) : 256;
-              const uint32_t idesc = umma_idesc(kBM, n);
-#pragma unroll
-              for (int ks = 0; ks < kBK / 16; ++ks) {
-                const uint64_t da = umma_desc(sA + s * Cfg::tileA + ks * 256);
-                const uint64_t db = umma_desc(sB + (c0 / 8) * (16 * kBK) + ks * 256);
-                const uint32_t acc = (cpos > 0 || s > 0 || ks > 0) ? 1u : 0u;
-                umma_bf16(tmem + uint32_t(s * BN + c0), da, db, idesc, acc);
-              }
-            }
-          }
+          mma_stage<S, BN>(tmem, sA, sB, cpos == 0);
           umma_commit(&empty[st]);
           if (cpos == Cfg::kc - 1 || it == T.nk - 1) {
             umma_commit(acc_full);
@@ -762,14 +820,6 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, OzCfg<S, BN>::min_block
       const int64_t nchunks = (T.nk + Cfg::kc - 1) / Cfg::kc;
       const int64_t m = T.m0 + row, n0 = T.n0;
       if constexpr (Cfg::exact) {
-        // Levels 0..7 of one column and chunk (512 k: levels 0..5 are exact
-        // integers below 2^24) are paired exactly in 32-bit integers,
-        //   P01 = L0 2^7 + L1, P23 = L2 2^7 + L3, P45 = L4 2^7 + L5  (< 2^31),
-        // and levels 6, 7 (weights below 2^-42) are combined in FP32.  Per
-        // column th accumulates P01 2^14 + P23 plus the part of
-        // lo = P45 2^14 + (L6 2^7 + L7) above 2^28; rem keeps lo's low 28 bits
-        // (carried into th), so the value is th + rem 2^-28 in units of 2^-21.
-        // With 7 digits there is no level 7 (L7 = 0).
         static_assert(HC % 16 == 0, "16-column tensor-memory loads");
         long long th[HC];
         uint32_t rem[HC];
@@ -784,47 +834,7 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, OzCfg<S, BN>::min_block
           }
           ++h;
           asm volatile("tcgen05.fence::after_thread_sync;");
-#pragma unroll
-          for (int c0 = 0; c0 < HC; c0 += 16) {
-#pragma unroll
-            for (int pq = 0; pq < 4; ++pq) {  // level pairs (0,1) (2,3) (4,5) (6,7)
-              uint32_t ra[16], rb[16];
-              tmem_ld16(tbase + uint32_t((2 * pq) * BN + c0), ra);
-              if (2 * pq + 1 < S) {
-                tmem_ld16(tbase + uint32_t((2 * pq + 1) * BN + c0), rb);
-              } else {  // 7 digits: no level 7
-#pragma unroll
-                for (int j = 0; j < 16; ++j) rb[j] = 0u;
-              }
-              asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-              for (int j = 0; j < 16; ++j) {
-                const float fa = __uint_as_float(ra[j]), fb = __uint_as_float(rb[j]);
-                if (pq < 3) {
-                  const int pair = __float2int_rn(fa) * 128 + __float2int_rn(fb);  // exact, |pair| < 2^31
-                  if (pq == 0) {
-                    th[c0 + j] += (long long)pair * (1ll << 14);
-                  } else if (pq == 1) {
-                    th[c0 + j] += (long long)pair;
-                  } else {
-                    const long long x = (long long)pair * (1ll << 14);  // lo part of levels 4, 5
-                    th[c0 + j] += x >> 28;
-                    rem[c0 + j] += uint32_t(x & 0x0FFFFFFFll);
-                  }
-                } else {
-                  const long long x = intf_to_ll(fmaf(fa, 128.0f, fb));  // levels 6, 7
-                  th[c0 + j] += x >> 28;
-                  rem[c0 + j] += uint32_t(x & 0x0FFFFFFFll);
-                }
-              }
-              reg_fence16(th, rem);
-            }
-          }
-#pragma unroll
-          for (int j = 0; j < HC; ++j) {  // rem < 3 * 2^28 here
-            th[j] += (long long)(rem[j] >> 28);
-            rem[j] &= 0x0FFFFFFFu;
-          }
+          drain_exact<S, BN, HC>(tbase, th, rem);
           asm volatile("tcgen05.fence::before_thread_sync;");
           __syncwarp();
           if (lane == 0) mbar_arrive(acc_empty);
@@ -903,6 +913,314 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, OzCfg<S, BN>::min_block
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(Cfg::tcols));
+  }
+}
+
+// ---------------------------------------------------------------- speculative columns
+//
+// All columns of a selection block in one launch: for every level l and every
+// candidate t, member j of its set,
+//   C_l[j][t] = w_l aL (aL + 2 aN) - F,
+// aL, aN the products of the basis rows (own functions, coarser ones) and F that
+// of the factor rows, each an exact 8-digit product.  A tile (128 candidates x
+// 48 members of a level) runs its three k ranges through one ring of stages; the
+// epilogue turns a range's integer sums into FP64, keeps the partial result in
+// shared memory and writes the finished column once.  Separate products were
+// ten launches a block (three per level and the combination), each too short to
+// fill the chip on a small cell (18 us of fill and epilogue), and moved every
+// result through memory four more times: columns of a block on one cell 290 ->
+// 163 us, on 2x2x2 2.01 -> 1.76 ms, and one launch instead of up to 21 for the
+// digits of the set's rows.
+// Bound: the candidates' digit stream (16 bytes a value) from HBM; persistent
+// CTAs, one per SM, the levels in order (the longest k ranges first).
+struct OzColSeg {
+  const __nv_bfloat16 *A, *B;
+  const int *ea, *eb;
+  int64_t akst, bkst;
+  int nkt;
+};
+struct OzColLevel {
+  OzColSeg seg[3];
+  int64_t M, ntm;
+  double* C;
+  double w;
+};
+struct OzColParams {
+  OzColLevel l[ISDF_MAX_LEVELS];
+  int nlev;
+  const int* scount;  // members per level
+  int* err;
+  unsigned long long wait_ns;
+};
+
+struct OzColCfg : OzCfg<8, 48> {
+  static constexpr int S = 8, BN = 48;
+  static constexpr int stash = kBM * BN * 8;  // partial results, FP64
+  static constexpr int ring = nst * stage;
+  static constexpr int smem = ring + stash + 1024 + 256;  // + barriers, alignment slack
+  static_assert(smem <= 232448, "shared memory per CTA");
+};
+
+__global__ void __launch_bounds__(OzColCfg::threads, 1) k_oz_columns(const __grid_constant__ OzColParams P) {
+  using Cfg = OzColCfg;
+  constexpr int S = Cfg::S, BN = Cfg::BN;
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  double* stash = reinterpret_cast<double*>(smem + Cfg::ring);  // [BN][128]
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + Cfg::ring + Cfg::stash);
+  uint64_t* empty = full + Cfg::nst;
+  uint64_t* acc_full = empty + Cfg::nst;
+  uint64_t* acc_empty = acc_full + 1;
+  uint64_t* drain = acc_empty + 1;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+  int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  if (__syncthreads_or(threadIdx.x == 0 ? *(volatile const int*)P.err : 0)) return;
+
+  // tiles of level l: [t0[l], t0[l + 1]), N tiles fastest
+  int64_t t0[ISDF_MAX_LEVELS + 1] = {0};
+  int NT[ISDF_MAX_LEVELS], members[ISDF_MAX_LEVELS];
+#pragma unroll
+  for (int l = 0; l < ISDF_MAX_LEVELS; ++l) {
+    members[l] = l < P.nlev ? P.scount[l] : 0;
+    NT[l] = (members[l] + BN - 1) / BN;
+    t0[l + 1] = t0[l] + (l < P.nlev ? P.l[l].ntm * NT[l] : 0);
+  }
+  const int64_t ntiles = t0[ISDF_MAX_LEVELS];
+  struct Tile {
+    int l, nt, members;
+    int64_t mt;
+  };
+  auto tile_at = [&](int64_t t) {
+    Tile T{0, 0, 0, 0};
+#pragma unroll
+    for (int l = 0; l < ISDF_MAX_LEVELS; ++l)
+      if (t >= t0[l] && t < t0[l + 1]) {
+        T.l = l;
+        T.members = members[l];
+        T.mt = (t - t0[l]) / NT[l];
+        T.nt = int((t - t0[l]) - T.mt * NT[l]);
+      }
+    return T;
+  };
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < Cfg::nst; ++i) {
+      mbar_init(&full[i], 1);
+      mbar_init(&empty[i], 1);
+    }
+    mbar_init(acc_full, 1);
+    mbar_init(acc_empty, Cfg::epi);
+    mbar_init(drain, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(Cfg::tcols));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == 0) {
+    // ------------------------------------------------ producer
+    if (lane == 0) {
+      int64_t g = 0;  // stages issued so far (all tiles)
+      for (int64_t t = blockIdx.x; t < ntiles && !*(volatile int*)abort_flag; t += gridDim.x) {
+        const Tile T = tile_at(t);
+        for (int sg = 0; sg < 3 && !*(volatile int*)abort_flag; ++sg) {
+          const OzColSeg& Q = P.l[T.l].seg[sg];
+          const unsigned char* gA = reinterpret_cast<const unsigned char*>(Q.A) + T.mt * Q.akst * int64_t(Cfg::stageA);
+          const unsigned char* gB = reinterpret_cast<const unsigned char*>(Q.B) + T.nt * Q.bkst * int64_t(Cfg::stageB);
+          for (int kt = 0; kt < Q.nkt; ++kt, ++g) {
+            const int st = int(g % Cfg::nst);
+            const int64_t round = g / Cfg::nst;
+            if (round > 0 && !mbar_wait(&empty[st], uint32_t((round - 1) & 1), P.err, P.wait_ns)) {
+              set_err(P.err, 11);
+              *(volatile int*)abort_flag = 1;
+              break;
+            }
+            if (*(volatile int*)abort_flag) break;
+            unsigned char* sA = smem + st * Cfg::stage;
+            mbar_expect_tx(&full[st], Cfg::stageA + Cfg::stageB);
+            bulk_g2s(sA, gA + kt * int64_t(Cfg::stageA), Cfg::stageA, &full[st]);
+            bulk_g2s(sA + Cfg::stageA, gB + kt * int64_t(Cfg::stageB), Cfg::stageB, &full[st]);
+          }
+        }
+      }
+      if (*(volatile int*)abort_flag) {  // copies issued but never consumed must land before exit
+        const int64_t first = g > Cfg::nst ? g - Cfg::nst : 0;
+        for (int64_t it = first; it < g; ++it) mbar_wait(&full[it % Cfg::nst], uint32_t((it / Cfg::nst) & 1), nullptr);
+      }
+    }
+  } else if (warp == 1) {
+    // ------------------------------------------------ MMA issuer
+    if (lane == 0) {
+      int64_t g = 0, h = 0;  // stages consumed, accumulator chunks handed over (all tiles)
+      bool stop = false;
+      for (int64_t t = blockIdx.x; t < ntiles && !stop; t += gridDim.x) {
+        const Tile T = tile_at(t);
+        for (int sg = 0; sg < 3 && !stop; ++sg) {
+          const int nkt = P.l[T.l].seg[sg].nkt;
+          for (int kt = 0; kt < nkt; ++kt, ++g) {
+            const int st = int(g % Cfg::nst);
+            const int cpos = kt % Cfg::kc;
+            if (cpos == 0 && h > 0 && !mbar_wait(acc_empty, uint32_t((h - 1) & 1), P.err, P.wait_ns)) {
+              set_err(P.err, 12);
+              stop = true;
+            } else if (!mbar_wait(&full[st], uint32_t((g / Cfg::nst) & 1), P.err, P.wait_ns)) {
+              set_err(P.err, 13);
+              stop = true;
+            }
+            if (stop) *(volatile int*)abort_flag = 1;
+            if (stop || *(volatile int*)abort_flag) {
+              stop = true;
+              break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            const uint32_t sA = smem_u32(smem + st * Cfg::stage);
+            mma_stage<S, BN>(tmem, sA, sA + Cfg::stageA, cpos == 0);
+            umma_commit(&empty[st]);
+            if (cpos == Cfg::kc - 1 || kt == nkt - 1) {
+              umma_commit(acc_full);
+              ++h;
+            }
+          }
+        }
+      }
+      umma_commit(drain);  // all MMAs issued by this thread complete before tensor memory is freed
+      mbar_wait(drain, 0, nullptr);
+    }
+  } else {
+    // ------------------------------------------------ epilogue warps
+    constexpr int HC = BN / (Cfg::epi / 4);  // columns per thread
+    const int quarter = warp % 4;            // a warp reads tensor-memory lanes 32 (warp % 4) ..
+    const int part = (warp - 2) / 4;         // which share of the columns
+    const int row = quarter * 32 + lane;
+    const uint32_t tbase = tmem + (uint32_t(quarter * 32) << 16) + uint32_t(part * HC);
+    double* mine = stash + part * HC * kBM + row;
+    int64_t h = 0;  // accumulator chunks taken over (all tiles)
+    for (int64_t t = blockIdx.x; t < ntiles && !*(volatile int*)abort_flag; t += gridDim.x) {
+      const Tile T = tile_at(t);
+      const OzColLevel& L = P.l[T.l];
+      const int64_t m = T.mt * kBM + row;
+      const int n0 = T.nt * BN + part * HC;
+      const bool live = m < L.M;
+      const int last = L.seg[2].nkt ? 2 : L.seg[1].nkt ? 1 : 0;
+      for (int sg = 0; sg <= last; ++sg) {
+        const OzColSeg& Q = L.seg[sg];
+        const int nchunks = (Q.nkt + Cfg::kc - 1) / Cfg::kc;
+        if (nchunks == 0 && sg > 0 && sg < last) {  // no coarser functions: the M term is ready
+          for (int j = 0; j < HC; ++j) {
+            const double a = mine[j * kBM];
+            mine[j * kBM] = L.w * (a * a);
+          }
+          continue;
+        }
+        long long th[HC];
+        uint32_t rem[HC];
+#pragma unroll
+        for (int j = 0; j < HC; ++j) th[j] = 0, rem[j] = 0u;
+        for (int c = 0; c < nchunks; ++c) {
+          if (!mbar_wait(acc_full, uint32_t(h & 1), P.err, P.wait_ns)) {
+            set_err(P.err, 14);
+            *(volatile int*)abort_flag = 1;
+            break;
+          }
+          ++h;
+          asm volatile("tcgen05.fence::after_thread_sync;");
+          drain_exact<S, BN, HC>(tbase, th, rem);
+          asm volatile("tcgen05.fence::before_thread_sync;");
+          __syncwarp();
+          if (lane == 0) mbar_arrive(acc_empty);
+        }
+        if (*(volatile int*)abort_flag) break;
+        const int ea = live && nchunks ? Q.ea[m] : 0;
+#pragma unroll
+        for (int j = 0; j < HC; ++j) {
+          if (n0 + j >= T.members || !live) continue;
+          double v = nchunks ? fixed_to_double(th[j], rem[j], ea + Q.eb[n0 + j] - 14 - 21) : 0.0;  // one rounding
+          if (sg == 1) {
+            const double a = mine[j * kBM];
+            v = L.w * (a * (a + 2.0 * v));
+          } else if (sg == 2) {
+            v = mine[j * kBM] - v;
+          } else if (last == 0) {
+            v = L.w * (v * v);
+          }
+          if (sg == last)
+            L.C[int64_t(n0 + j) * L.M + m] = v;
+          else
+            mine[j * kBM] = v;
+        }
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  if (warp == 1) {
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(Cfg::tcols));
+  }
+}
+
+// Digits of the set's rows on the B side of the three products, all levels: one
+// block per member and product.  Basis rows take the scale of the same
+// candidate's row on the A side; factor rows their own maximum.
+struct OzRowsLevel {
+  const double* src[3];  // element (row, k) at src[row + k * ld]
+  int64_t ld[3];
+  int K[3];
+  const int* aexp[2];
+  int* bexp[3];
+  __nv_bfloat16* tiles[3];
+  int64_t kst[3];
+};
+struct OzRowsParams {
+  OzRowsLevel l[ISDF_MAX_LEVELS];
+  const int *scount, *st, *sg;  // members per level; candidate and grid point of each
+};
+__global__ void __launch_bounds__(256) k_oz_set_rows(const __grid_constant__ OzRowsParams P) {
+  constexpr int S = 8, BN = 48;
+  __shared__ unsigned long long key;
+  int j = int(blockIdx.x), l = 0, first = 0;
+  const int sg = int(blockIdx.y), tid = threadIdx.x;
+  while (l < ISDF_MAX_LEVELS && j >= first + P.scount[l]) first += P.scount[l], ++l;
+  if (l == ISDF_MAX_LEVELS) return;  // fewer members than the set's size
+  const OzRowsLevel& L = P.l[l];
+  const int K = L.K[sg], r = j - first;
+  const int ngrp = ((K + kBK - 1) / kBK) * (kBK / 8);
+  if (!K) return;
+  const int64_t ld = L.ld[sg];
+  const double* row = L.src[sg] + (sg == 2 ? P.st[j] : P.sg[j]);
+  double v[8];
+  int e;
+  if (sg < 2) {
+    e = L.aexp[sg][P.st[j]];
+  } else {
+    if (tid == 0) key = 0ull;
+    __syncthreads();
+    uint64_t m = 0;
+    for (int g = tid; g < ngrp; g += 256) {
+      oz_load8(row, true, ld, K, g, v);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) m = umax64(m, abs_key(v[u]));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = umax64(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((tid & 31) == 0 && m) atomicMax(&key, (unsigned long long)m);
+    __syncthreads();
+    e = exp_of_key(key);
+  }
+  if (tid == 0) L.bexp[sg][r] = e;
+  for (int g = tid; g < ngrp; g += 256) {
+    if (sg < 2 || ngrp > 256) oz_load8(row, true, ld, K, g, v);
+    __nv_bfloat16* out = L.tiles[sg] + ((r / BN * L.kst[sg] + g / (kBK / 8)) * S) * int64_t(BN * kBK) +
+                         oz_inner(r % BN, g % (kBK / 8));
+    oz_digits8<S>(v, 7 * S - e, BN * kBK, out);
   }
 }
 
@@ -1005,6 +1323,15 @@ void oz_slice_ex(const double* src, int64_t sr, int64_t sk, const int* ridx, OzO
     slice_operand(A, op.S, s);  // scales need every group: callers pass the whole range
 }
 
+// host-side fault injection (ISDF_FAULT=oz_wait): every pipeline wait gives
+// up at once, so the launch takes its error path (error code, copies and
+// MMAs in flight completed, tensor memory freed) and the call reports
+// ISDF_ERR_TIMEOUT; nothing faults or hangs
+static unsigned long long oz_wait_limit() {
+  const char* fault = std::getenv("ISDF_FAULT");
+  return (fault && std::strcmp(fault, "oz_wait") == 0) ? 0ull : kWaitNs;
+}
+
 // S levels x BN columns of tensor memory: 5 x 48 (two CTAs per SM), 6 x 64, 7 x 48, 8 x 48
 int oz_bn(int S) { return S == 6 ? 64 : 48; }
 
@@ -1029,12 +1356,7 @@ void oz_gemm(const OzOperand& A, const OzOperand& B, double* C, int64_t ldc, int
   P.alpha = alpha;
   P.work = work;
   P.err = err;
-  // host-side fault injection (ISDF_FAULT=oz_wait): every pipeline wait gives
-  // up at once, so the launch takes its error path (error code, copies and
-  // MMAs in flight completed, tensor memory freed) and the call reports
-  // ISDF_ERR_TIMEOUT; nothing faults or hangs
-  const char* fault = std::getenv("ISDF_FAULT");
-  P.wait_ns = (fault && std::strcmp(fault, "oz_wait") == 0) ? 0ull : kWaitNs;
+  P.wait_ns = oz_wait_limit();
   P.ntm = A.nrt;
   P.ntn = B.nrt;
   // Persistent CTAs pay off where a tile's epilogue is long against its
@@ -1057,6 +1379,69 @@ void oz_gemm(const OzOperand& A, const OzOperand& B, double* C, int64_t ldc, int
     k_oz_reduce<<<unsigned((tot + 255) / 256), 256, 0, s>>>(work, P.splits, A.rows, B.rows, C, P.cm, P.cn, sym);
     count_launches(1);
   }
+}
+
+void oz_set_rows(const OzColumnJob* jobs, int nlev, int smax, const int* scount, const int* st, const int* sg,
+                 cudaStream_t s) {
+  OzRowsParams P{};
+  P.scount = scount;
+  P.st = st;
+  P.sg = sg;
+  bool factor = false;
+  for (int l = 0; l < nlev; ++l) {
+    const OzColumnJob& J = jobs[l];
+    OzRowsLevel& L = P.l[l];
+    for (int q = 0; q < 3; ++q) {
+      if (!J.A[q] || J.A[q]->nkt == 0 || J.A[q]->rows == 0) continue;
+      L.src[q] = J.src[q];
+      L.ld[q] = J.ld[q];
+      L.K[q] = int(J.A[q]->K);
+      if (q < 2) L.aexp[q] = J.A[q]->exps;
+      L.bexp[q] = J.B[q]->exps;
+      L.tiles[q] = static_cast<__nv_bfloat16*>(J.B[q]->tiles);
+      L.kst[q] = J.B[q]->kst;
+      factor = factor || q == 2;
+    }
+  }
+  k_oz_set_rows<<<dim3(unsigned(smax), factor ? 3u : 2u), 256, 0, s>>>(P);
+  count_launches(1);
+}
+
+void oz_columns(const OzColumnJob* jobs, int nlev, const int* scount, int* err, cudaStream_t s) {
+  static std::atomic<int> sms[kMaxDevices];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
+    cudaGetLastError();
+    dev = 0;
+  }
+  int n = sms[dev].load(std::memory_order_acquire);
+  if (!n) {
+    cudaFuncSetAttribute(k_oz_columns, cudaFuncAttributeMaxDynamicSharedMemorySize, OzColCfg::smem);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    cudaGetLastError();
+    n = std::max(1, n);
+    sms[dev].store(n, std::memory_order_release);
+  }
+  OzColParams P{};
+  P.nlev = nlev;
+  P.scount = scount;
+  P.err = err;
+  P.wait_ns = oz_wait_limit();
+  for (int l = 0; l < nlev; ++l) {
+    const OzColumnJob& J = jobs[l];
+    OzColLevel& L = P.l[l];
+    L.M = J.M;
+    L.ntm = (J.M + kBM - 1) / kBM;
+    L.C = J.C;
+    L.w = J.w;
+    for (int q = 0; q < 3; ++q) {
+      if (!J.A[q] || J.A[q]->nkt == 0) continue;
+      L.seg[q] = {static_cast<const __nv_bfloat16*>(J.A[q]->tiles), static_cast<const __nv_bfloat16*>(J.B[q]->tiles),
+                  J.A[q]->exps, J.B[q]->exps, J.A[q]->kst, J.B[q]->kst, int(J.A[q]->nkt)};
+    }
+  }
+  k_oz_columns<<<unsigned(n), OzColCfg::threads, OzColCfg::smem, s>>>(P);
+  count_launches(1);
 }
 
 // ---------------------------------------------------------------- split-K autotuner

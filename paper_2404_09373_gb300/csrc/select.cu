@@ -51,6 +51,7 @@ struct SelState {
   int final_;                // a stop rule ended the selection
   int bsteps;                // steps accepted in the current round of a block
   int btried;                // steps the round tried
+  int members[ISDF_MAX_LEVELS];  // the block's set, per level
 };
 
 struct SelParams {
@@ -602,26 +603,6 @@ __global__ void __launch_bounds__(1024) k_top_s(LmParams Q, const int* __restric
   }
 }
 
-// B = w * aL (aL + 2 aN) - F over [s_l][nc]; in place in aL
-__global__ void k_blk_combine(double* __restrict__ aL, const double* __restrict__ aN, const double* __restrict__ F,
-                              int64_t n, double w) {
-  for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < n; e += int64_t(gridDim.x) * blockDim.x) {
-    const double a = aL[e];
-    const double b = aN ? aN[e] : 0.0;
-    double v = w * (a * (a + 2.0 * b));
-    if (F) v -= F[e];
-    aL[e] = v;
-  }
-}
-
-// per-candidate power-of-two bound of the factor rows: sum_k L[t,k]^2 <= d0(t)
-// Row scales of the speculative set's basis-value rows: those of the same
-// candidates' rows on the candidate side (the same rows, the same exact max)
-__global__ void k_gather_exps(const int* __restrict__ pos, int n, const int* __restrict__ src, int* __restrict__ dst) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r < n) dst[r] = src[pos[r]];
-}
-
 // Fixed row scales of the factor columns: |L[c][k]| <= sqrt(d0_c)
 __global__ void k_fac_exps(const double* __restrict__ d0c, int64_t nc, int64_t npad, int* __restrict__ exps) {
   const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -909,6 +890,7 @@ __global__ void __launch_bounds__(kApply) k_blk_commit(BlkParams B, BlkRound* R,
     if (tid == 0) {
       st->bsteps = js;
       st->btried = R->nsteps;
+      for (int a = 0; a < P.nlev; ++a) st->members[a] = B.scount[a];
       st->k = B.k + js;
       for (int a = 0; a < P.nlev; ++a) {
         int c = 0;
@@ -1134,7 +1116,8 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
 
   struct LevBuf {
     OzOperand aL, aN, aF, bL, bN, bF;
-    double *cL = nullptr, *cN = nullptr, *cF = nullptr;
+    double* col = nullptr;  // B of the block [s_l][nc]
+    float2* bdf = nullptr;  // the block's columns so far, double-float [s][nc]
     int* gpos = nullptr;
   } lb[ISDF_MAX_LEVELS];
   int *counts = nullptr, *nlist = nullptr, *list = nullptr, *sidx = nullptr, *sg = nullptr, *stp = nullptr,
@@ -1147,7 +1130,7 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
     for (int l = 0; l < nlev; ++l) {
       oz_free(lb[l].aL), oz_free(lb[l].aN), oz_free(lb[l].aF);
       oz_free(lb[l].bL), oz_free(lb[l].bN), oz_free(lb[l].bF);
-      dfree(lb[l].cL), dfree(lb[l].cN), dfree(lb[l].cF), dfree(lb[l].gpos);
+      dfree(lb[l].col), dfree(lb[l].bdf), dfree(lb[l].gpos);
       dfree(p->lev[l].fac);
       p->lev[l].fac = nullptr;
     }
@@ -1198,12 +1181,11 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
         (st = oz_alloc(p, b.bL, smax, std::max(lv.nL, 1), bn, kSlices, "selection slices")) ||
         (st = oz_alloc(p, b.aF, nc[l], lv.fac_cap, 128, kSlices, "selection slices")) ||
         (st = oz_alloc(p, b.bF, smax, lv.fac_cap, bn, kSlices, "selection slices")) ||
-        (st = dalloc_t(p, &b.cL, size_t(smax) * nc[l], "selection columns")) ||
-        (st = dalloc_t(p, &b.cF, size_t(smax) * nc[l], "selection columns")))
+        (st = dalloc_t(p, &b.col, size_t(smax) * nc[l], "selection columns")) ||
+        (st = dalloc_t(p, &b.bdf, size_t(smax) * nc[l], "selection columns")))
       return bail(st);
     if (lv.nN > 0 && ((st = oz_alloc(p, b.aN, nc[l], lv.nN, 128, kSlices, "selection slices")) ||
-                      (st = oz_alloc(p, b.bN, smax, lv.nN, bn, kSlices, "selection slices")) ||
-                      (st = dalloc_t(p, &b.cN, size_t(smax) * nc[l], "selection columns"))))
+                      (st = oz_alloc(p, b.bN, smax, lv.nN, bn, kSlices, "selection slices"))))
       return bail(st);
     {
       Prof pr(p, "select_slice", 8.0 * double(nc[l]) * lv.nG, "byte", 4);
@@ -1252,10 +1234,8 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
   BP.st = stp;
   BP.scount = scount;
   for (int l = 0; l < nlev; ++l) {
-    BP.bm[l] = lb[l].cL;
-    // the factor product's output is free during the steps: it holds the
-    // double-float copy of the block's columns (s x nc values of 8 bytes)
-    BP.bdf[l] = reinterpret_cast<float2*>(lb[l].cF);
+    BP.bm[l] = lb[l].col;
+    BP.bdf[l] = lb[l].bdf;
   }
   TopSOut O{sidx, sg, stp, scount};
 
@@ -1447,7 +1427,6 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
     return ISDF_OK;
   };
   int64_t nblocks = 0, nplain = 0;
-  std::vector<int> hcount(ISDF_MAX_LEVELS + 1);
   int m_next = std::min(smax, 32);  // steps tried per round: a quarter more than the last one accepted, and 6
   while (true) {
     if ((st = grow())) return bail(st);
@@ -1458,58 +1437,36 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
       k_lm_list<<<unsigned(std::max<int64_t>((P.ntot + 255) / 256, 1)), 256, 0, s>>>(Q, list, nlist);
       k_top_s<<<1, 1024, 0, s>>>(Q, list, nlist, smax, O);
     }
-    cudaMemcpyAsync(hcount.data(), scount, sizeof(int) * hcount.size(), cudaMemcpyDeviceToHost, s);
-    if ((st = cuda_check(p, cudaStreamSynchronize(s), "speculative set"))) return bail(st);
-    // ---- 2. columns of S: three products per level, then B = w M - F
-    int soff = 0;
-    for (int l = 0; l < nlev; ++l) {
-      const int sl = hcount[l];
-      if (!sl) continue;
-      Level& lv = p->lev[l];
-      LevBuf& b = lb[l];
-      const int kb = h.kl[l];
-      auto setrows = [&](OzOperand& op, int rows) {
-        op.rows = rows;
-        op.nrt = (rows + op.rt - 1) / op.rt;
-      };
+    // ---- 2. the columns of S at every candidate, B = w M - F
+    size_t gemm_event = size_t(-1);
+    {
+      OzColumnJob jobs[ISDF_MAX_LEVELS];
+      double bytes = 0.0;
+      for (int l = 0; l < nlev; ++l) {
+        if (!nc[l]) continue;
+        Level& lv = p->lev[l];
+        LevBuf& b = lb[l];
+        OzColumnJob& J = jobs[l];
+        b.aF.K = h.kl[l];
+        b.aF.nkt = (h.kl[l] + kOzBK - 1) / kOzBK;
+        J.M = nc[l];
+        J.C = b.col;
+        J.w = lv.w;
+        if (lv.nL > 0) J.A[0] = &b.aL, J.B[0] = &b.bL, J.src[0] = lv.phi, J.ld[0] = lv.ng;
+        if (lv.nN > 0) J.A[1] = &b.aN, J.B[1] = &b.bN, J.src[1] = lv.phi + int64_t(lv.nL) * lv.ng, J.ld[1] = lv.ng;
+        J.A[2] = &b.aF, J.B[2] = &b.bF, J.src[2] = lv.fac, J.ld[2] = nc[l];
+        bytes += 8.0 * double(nc[l]) * (lv.nG + h.kl[l]);
+      }
       {
-        // digits of S's rows: basis values and factor rows of the set
-        Prof pb(p, "select_sslice", 8.0 * sl * (lv.nL + lv.nN + kb), "byte", kLaunchesInside);
-        const unsigned gb = unsigned((sl + 127) / 128);
-        setrows(b.bL, sl);
-        if (lv.nL > 0) {
-          k_gather_exps<<<gb, 128, 0, s>>>(stp + soff, sl, b.aL.exps, b.bL.exps);
-          count_launches(1);
-        }
-        oz_slice_ex(lv.phi, 1, lv.ng, sg + soff, b.bL, 0, b.bL.nkt * (kOzBK / 8), lv.nL > 0, s);
-        if (lv.nN > 0) {
-          setrows(b.bN, sl);
-          k_gather_exps<<<gb, 128, 0, s>>>(stp + soff, sl, b.aN.exps, b.bN.exps);
-          count_launches(1);
-          oz_slice_ex(lv.phi + int64_t(lv.nL) * lv.ng, 1, lv.ng, sg + soff, b.bN, 0, b.bN.nkt * (kOzBK / 8), true, s);
-        }
-        if (kb > 0) {
-          setrows(b.bF, sl);
-          b.bF.K = kb;
-          b.bF.nkt = (kb + kOzBK - 1) / kOzBK;
-          oz_slice_ex(lv.fac, 1, nc[l], stp + soff, b.bF, 0, b.bF.nkt * (kOzBK / 8), false, s);
-        }
+        Prof pb(p, "select_sslice", 0.0, "byte", kLaunchesInside);
+        oz_set_rows(jobs, nlev, smax, scount, stp, sg, s);
       }
       // algorithmic traffic: the candidates' FP64 basis values and factor rows, read once per block
-      Prof pr(p, "select_gemm", 8.0 * double(nc[l]) * (lv.nL + lv.nN + kb), "byte", 3);
-      pr.e.flop = 2.0 * double(nc[l]) * double(sl) * double(lv.nL + lv.nN + kb);
-      oz_gemm(b.aL, b.bL, b.cL, nc[l], 1, 1.0, 0, 0, 1, nullptr, p->d_ozerr, s);
-      if (lv.nN > 0) oz_gemm(b.aN, b.bN, b.cN, nc[l], 1, 1.0, 0, 0, 1, nullptr, p->d_ozerr, s);
-      if (kb > 0) {
-        b.aF.K = kb;
-        b.aF.nkt = (kb + kOzBK - 1) / kOzBK;
-        oz_gemm(b.aF, b.bF, b.cF, nc[l], 1, 1.0, 0, 0, 1, nullptr, p->d_ozerr, s);
+      {
+        Prof pr(p, "select_gemm", bytes, "byte", kLaunchesInside);
+        oz_columns(jobs, nlev, scount, p->d_ozerr, s);
       }
-      const int64_t n = int64_t(sl) * nc[l];
-      k_blk_combine<<<unsigned(std::min<int64_t>((n + 255) / 256, int64_t(nsm) * 16)), 256, 0, s>>>(
-          b.cL, lv.nN > 0 ? b.cN : nullptr, kb > 0 ? b.cF : nullptr, n, lv.w);
-      count_launches(1);
-      soff += sl;
+      if (p->opt.profile) gemm_event = p->pend.size() - 1;
     }
     // ---- 3. greedy steps of this block, in rounds: as long as every tried step
     // of a round is accepted there may be more in S
@@ -1555,6 +1512,9 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
       if (h.err || h.final_ || h.k >= nip || h.bsteps < m || taken >= smax) break;
     }
     ++nblocks;
+    if (gemm_event != size_t(-1) && gemm_event < p->pend.size())
+      for (int l = 0; l < nlev; ++l)
+        p->pend[gemm_event].flop += 2.0 * double(nc[l]) * h.members[l] * double(p->lev[l].nG + BP.kb[l]);
     if (h.err || h.final_ || h.k >= nip) break;
     if (tau > 0.0 && taken > 0 && h.dp * (1.0 - 2.0 * p->opt.tie_rel) - 2.0 * p->opt.tie_abs * h.d0 < tau) {
       *aborted = true;  // a pivot value broke the certificate: retry with a lower tau
