@@ -138,80 +138,47 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
                : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-}
-
-
-// Compiler fence on 16 accumulators: the empty volatile statement reads and
-// writes them, so their updates are complete here and no later volatile
-// statement (a tensor-memory load) is moved above it.
-__device__ __forceinline__ void reg_fence16(long long (&a)[16], uint32_t (&b)[16]) {
-  asm volatile("" : "+l"(a[0]), "+l"(a[1]), "+l"(a[2]), "+l"(a[3]), "+l"(a[4]), "+l"(a[5]), "+l"(a[6]), "+l"(a[7]));
-  asm volatile("" : "+l"(a[8]), "+l"(a[9]), "+l"(a[10]), "+l"(a[11]), "+l"(a[12]), "+l"(a[13]), "+l"(a[14]),
-               "+l"(a[15]));
-  asm volatile("" : "+r"(b[0]), "+r"(b[1]), "+r"(b[2]), "+r"(b[3]), "+r"(b[4]), "+r"(b[5]), "+r"(b[6]), "+r"(b[7]),
-               "+r"(b[8]), "+r"(b[9]), "+r"(b[10]), "+r"(b[11]), "+r"(b[12]), "+r"(b[13]), "+r"(b[14]), "+r"(b[15]));
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
 }
 
 __device__ __forceinline__ void set_err(int* err, int code) { atomicCAS(err, 0, code); }
 
-// f * 2^e as a double, built with integer operations (exact; the narrow FP64
-// pipe is left alone).  Subnormal or out-of-range cases take the FP64 route.
-__device__ __forceinline__ double scaled_to_double(float f, int e) {
-  const uint32_t b = __float_as_uint(f);
-  if ((b << 1) == 0u) return __longlong_as_double((long long)(uint64_t(b >> 31) << 63));  // +-0
-  const int ef = int((b >> 23) & 0xFF);
-  const int ed = ef - 127 + 1023 + e;
-  if (ef == 0 || ef == 0xFF || ed <= 0 || ed >= 0x7FF) return ldexp(double(f), e);
-  const uint64_t bits = (uint64_t(b >> 31) << 63) | (uint64_t(ed) << 52) | (uint64_t(b & 0x7FFFFF) << 29);
-  return __longlong_as_double((long long)bits);
+// sign M 2^e as a double, |value| outside the normal range: out of line, so
+// that the epilogues' unrolled code stays short
+__device__ __noinline__ double far_double(bool neg, uint64_t M, int e) {
+  const double v = ldexp(double(M), e);
+  return neg ? -v : v;
 }
 
-// An integer-valued float (|x| < 2^62) as a 64-bit integer without the
-// 64-bit conversion instruction, which runs on the narrow FP64 unit: below
-// 2^23 a 32-bit conversion is exact, above it the value is its significand
-// shifted left.
-__device__ __forceinline__ long long intf_to_ll(float x) {
-  const uint32_t b = __float_as_uint(x);
-  const int ef = int((b >> 23) & 0xFF);
-  if (ef < 150) return (long long)__float2int_rz(x);
-  const long long m = (long long)((b & 0x7FFFFFu) | 0x800000u) << (ef - 150);
-  return (b >> 31) ? -m : m;
-}
-
-// (th + rem 2^-28) 2^e rounded once to the nearest double (ties to even),
-// from the fixed-point value with integer operations; outside the normal
-// range it takes the FP64 route.
+// (th + rem 2^-28) 2^e rounded once to the nearest double (ties to even) with
+// integer operations.  rem in [0, 2^28).
 __device__ __forceinline__ double fixed_to_double(long long th, uint32_t rem, int e) {
-  const __int128 X = ((__int128)th << 28) + (__int128)rem;  // value X 2^(e - 28)
-  if (X == 0) return 0.0;
-  const bool neg = X < 0;
-  const unsigned __int128 U = neg ? (unsigned __int128)(-X) : (unsigned __int128)X;
-  const uint64_t hi = uint64_t(U >> 64), lo = uint64_t(U);
-  const int L = hi ? 128 - __clzll((long long)hi) : 64 - __clzll((long long)lo);  // bit length
-  int E = L - 1 + e - 28;
-  uint64_t M;  // significand, 53 bits
-  if (L <= 53) {
-    M = lo << (53 - L);
-  } else {
-    const int sh = L - 53;
-    const unsigned __int128 q = U >> sh;
-    const unsigned __int128 r = U - (q << sh);
-    const unsigned __int128 half = (unsigned __int128)1 << (sh - 1);
-    M = uint64_t(q);
-    if (r > half || (r == half && (M & 1ull))) {
-      ++M;
-      if (M >> 53) M >>= 1, ++E;
-    }
+  // sign and magnitude U = hi + lo 2^-28
+  const bool neg = th < 0;
+  uint32_t lo = rem;
+  uint64_t hi = uint64_t(th);
+  if (neg) {
+    lo = (0u - rem) & 0x0FFFFFFFu;
+    hi = ~hi + (rem == 0u ? 1ull : 0ull);
   }
-  if (E < -1022 || E > 1023) return ldexp(neg ? -double(M) : double(M), E - 52);
-  const uint64_t bits = (uint64_t(neg) << 63) | (uint64_t(E + 1023) << 52) | (M & 0xFFFFFFFFFFFFFull);
-  return __longlong_as_double((long long)bits);
+  const int low = hi == 0ull;  // only the fraction is left
+  hi = low ? uint64_t(lo) : hi;
+  const uint64_t frac = low ? 0ull : uint64_t(lo) << 36;
+  if (hi == 0ull) return 0.0;
+  const int lz = __clzll((long long)hi);
+  const uint64_t top = (hi << lz) | (lz ? frac >> (64 - lz) : 0ull);
+  const uint32_t cut = uint32_t(top) & 0x7FFu;
+  const uint64_t M = top >> 11;  // 53 bits
+  // half of the last place, and what lies below it
+  const bool up = cut > 0x400u || (cut == 0x400u && ((frac << lz) != 0ull || (M & 1ull)));
+  const int E = 63 - lz + e - (low ? 28 : 0) + 1023;
+  const uint64_t R = M + (up ? 1ull : 0ull);
+  if (E < 1 || E > 2045) return far_double(neg, R, E - 1075);
+  // R's leading bit adds one to the exponent field, as does a carry out of R
+  return __longlong_as_double((long long)((uint64_t(neg) << 63) | ((uint64_t(E - 1) << 52) + R)));
 }
 
 // ---------------------------------------------------------------- slicing
@@ -225,10 +192,6 @@ __device__ __forceinline__ int exp_of_key(uint64_t key) {
   int e;
   frexp(__longlong_as_double((long long)key), &e);
   return e;
-}
-
-__device__ __forceinline__ int64_t map_at(const OzMap& m, int64_t i) {
-  return m.in ? (i / m.in) * m.so + (i % m.in) * m.si : i * m.si;
 }
 
 // |mul * kw[k] * v| as an order-preserving key
@@ -547,7 +510,7 @@ struct OzGemmParams {
   int sym;     // compute only tiles that touch the lower triangle (n <= m)
   int splits;  // split-K factor (gridDim.z)
   double* C;
-  OzMap cm, cn;  // C[map_m(m) + map_n(n)]
+  int64_t cm, cn;  // C[m cm + n cn]
   double alpha;
   double* work;  // split-K partials [z][M][N]
   int* err;
@@ -611,59 +574,75 @@ __device__ __forceinline__ void mma_stage(uint32_t tmem, uint32_t sA, uint32_t s
   }
 }
 
-// Add one chunk's accumulators (HC columns of this warp's 32 lanes) to the
-// exact integer sums of 7 or 8 digits.  Levels 0..7 of one column and chunk
-// (512 k: levels 0..5 are exact integers below 2^24) are paired exactly in
-// 32-bit integers,
-//   P01 = L0 2^7 + L1, P23 = L2 2^7 + L3, P45 = L4 2^7 + L5  (< 2^31),
-// and levels 6, 7 (weights below 2^-42) are combined in FP32.  Per column th
-// accumulates P01 2^14 + P23 plus the part of lo = P45 2^14 + (L6 2^7 + L7)
-// above 2^28; rem keeps lo's low 28 bits (carried into th), so the value is
-// th + rem 2^-28 in units of 2^-21.  With 7 digits there is no level 7 (L7 = 0).
-template <int S, int BN, int HC>
-__device__ __forceinline__ void drain_exact(uint32_t tbase, long long (&th)[HC], uint32_t (&rem)[HC]) {
+// Exact integer sums of one thread's HC columns: th in units of 2^-21 of
+// level 0, the rest a fraction of such a unit.
+//   7 or 8 digits: 28 bits in rem.  Levels 0..5 of a 512-k chunk are integers
+//     below 2^24, paired in 32 bits (L0 2^7 + L1 and so on, below 2^31); levels
+//     6 and 7 lie below 2^-42, where FP32 rounding is harmless.
+//   6 digits: 14 bits in rem.  5 digits: 7 bits, four columns to a word.  Every
+//     level's FP32 sum is an integer; levels 0 and 1 are exact for 1024 k, the
+//     deeper ones unless adversarial digits push them past 2^24.
+// Integer sums take 2 or 3 operations per level where double-float ones took 8,
+// and leave one value to round at the end.
+template <int S, int HC>
+struct OzSums {
+  static constexpr int NR = S == 5 ? HC / 4 : HC;
+  long long th[HC];
+  uint32_t rem[NR];
+  __device__ __forceinline__ void clear() {
 #pragma unroll
-  for (int c0 = 0; c0 < HC; c0 += 16) {
+    for (int j = 0; j < HC; ++j) th[j] = 0;
 #pragma unroll
-    for (int pq = 0; pq < 4; ++pq) {  // level pairs (0,1) (2,3) (4,5) (6,7)
-      uint32_t ra[16], rb[16];
-      tmem_ld16(tbase + uint32_t((2 * pq) * BN + c0), ra);
-      if (2 * pq + 1 < S) {
-        tmem_ld16(tbase + uint32_t((2 * pq + 1) * BN + c0), rb);
-      } else {  // 7 digits: no level 7
+    for (int j = 0; j < NR; ++j) rem[j] = 0u;
+  }
+  // add the accumulators of one chunk (this warp's lanes, HC columns from tbase, levels BN apart)
+  template <int BN>
+  __device__ __forceinline__ void drain(uint32_t tbase) {
 #pragma unroll
-        for (int j = 0; j < 16; ++j) rb[j] = 0u;
-      }
+    for (int c0 = 0; c0 < HC; c0 += 8) {
+      uint32_t r[S][8];
+#pragma unroll
+      for (int q = 0; q < S; ++q) tmem_ld8(tbase + uint32_t(q * BN + c0), r[q]);
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const float fa = __uint_as_float(ra[j]), fb = __uint_as_float(rb[j]);
-        if (pq < 3) {
-          const int pair = __float2int_rn(fa) * 128 + __float2int_rn(fb);  // exact, |pair| < 2^31
-          if (pq == 0) {
-            th[c0 + j] += (long long)pair * (1ll << 14);
-          } else if (pq == 1) {
-            th[c0 + j] += (long long)pair;
-          } else {
-            const long long x = (long long)pair * (1ll << 14);  // lo part of levels 4, 5
-            th[c0 + j] += x >> 28;
-            rem[c0 + j] += uint32_t(x & 0x0FFFFFFFll);
-          }
+      for (int j = 0; j < 8; ++j) {
+        const int c = c0 + j;
+        int L[S];
+#pragma unroll
+        for (int q = 0; q < S; ++q) L[q] = __float2int_rn(__uint_as_float(r[q][j]));
+        if constexpr (S >= 7) {
+          const int p01 = L[0] * 128 + L[1], p23 = L[2] * 128 + L[3], p45 = L[4] * 128 + L[5];
+          long long lo = (long long)p45 * (1 << 14) + (long long)L[6] * 128;
+          if constexpr (S == 8) lo += L[7];
+          const uint32_t f = rem[c] + (uint32_t(lo) & 0x0FFFFFFFu);
+          th[c] += (long long)p01 * (1 << 14) + (long long)p23 + (lo >> 28) + (long long)(f >> 28);
+          rem[c] = f & 0x0FFFFFFFu;
         } else {
-          const long long x = intf_to_ll(fmaf(fa, 128.0f, fb));  // levels 6, 7
-          th[c0 + j] += x >> 28;
-          rem[c0 + j] += uint32_t(x & 0x0FFFFFFFll);
+          th[c] += (long long)L[0] * (1 << 21) + (long long)L[1] * (1 << 14) + (long long)(L[2] * 128);
+          if constexpr (S == 6) {
+            const int lo = L[4] * 128 + L[5];
+            const uint32_t f = rem[c] + (uint32_t(lo) & 0x3FFFu);
+            th[c] += (long long)(L[3] + (lo >> 14) + int(f >> 14));
+            rem[c] = f & 0x3FFFu;
+          } else {
+            const int sh = 8 * (c & 3);
+            const uint32_t f = ((rem[c / 4] >> sh) & 0x7Fu) + (uint32_t(L[4]) & 0x7Fu);
+            th[c] += (long long)(L[3] + (L[4] >> 7) + int(f >> 7));
+            rem[c / 4] = (rem[c / 4] & ~(0xFFu << sh)) | ((f & 0x7Fu) << sh);
+          }
         }
       }
-      reg_fence16(th, rem);
     }
   }
-#pragma unroll
-  for (int j = 0; j < HC; ++j) {  // rem < 3 * 2^28 here
-    th[j] += (long long)(rem[j] >> 28);
-    rem[j] &= 0x0FFFFFFFu;
+  // the value times 2^e (e: the sum of the rows' exponents), rounded once
+  __device__ __forceinline__ double value(int c, int e) const {
+    uint32_t f;
+    if constexpr (S >= 7) f = rem[c];
+    else if constexpr (S == 6) f = rem[c] << 14;
+    else f = ((rem[c / 4] >> (8 * (c & 3))) & 0x7Fu) << 21;
+    return fixed_to_double(th[c], f, e - 14 - 21);
   }
-}
+};
 
 template <int S, int BN>
 __global__ void __launch_bounds__(OzCfg<S, BN>::threads, OzCfg<S, BN>::min_blocks) k_oz_gemm(OzGemmParams P) {
@@ -819,90 +798,35 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, OzCfg<S, BN>::min_block
       if (T.skip) continue;
       const int64_t nchunks = (T.nk + Cfg::kc - 1) / Cfg::kc;
       const int64_t m = T.m0 + row, n0 = T.n0;
-      if constexpr (Cfg::exact) {
-        static_assert(HC % 16 == 0, "16-column tensor-memory loads");
-        long long th[HC];
-        uint32_t rem[HC];
-#pragma unroll
-        for (int j = 0; j < HC; ++j) th[j] = 0, rem[j] = 0u;
-        const uint32_t tbase = tmem + (uint32_t(quarter * 32) << 16) + uint32_t(half * HC);
-        for (int64_t c = 0; c < nchunks; ++c) {
-          if (!mbar_wait(acc_full, uint32_t(h & 1), P.err, P.wait_ns)) {
-            set_err(P.err, 14);
-            *(volatile int*)abort_flag = 1;
-            break;
-          }
-          ++h;
-          asm volatile("tcgen05.fence::after_thread_sync;");
-          drain_exact<S, BN, HC>(tbase, th, rem);
-          asm volatile("tcgen05.fence::before_thread_sync;");
-          __syncwarp();
-          if (lane == 0) mbar_arrive(acc_empty);
+      OzSums<S, HC> sums;
+      sums.clear();
+      for (int64_t c = 0; c < nchunks; ++c) {
+        if (!mbar_wait(acc_full, uint32_t(h & 1), P.err, P.wait_ns)) {
+          set_err(P.err, 14);
+          *(volatile int*)abort_flag = 1;
+          break;
         }
-        if (m < P.M && !*(volatile int*)abort_flag) {
-          const int ea = P.ea[m];
-          const int64_t cbase = map_at(P.cm, m);
+        ++h;
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        sums.template drain<BN>(tmem + (uint32_t(quarter * 32) << 16) + uint32_t(half * HC));
+        asm volatile("tcgen05.fence::before_thread_sync;");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(acc_empty);
+      }
+      if (m < P.M && !*(volatile int*)abort_flag) {
+        const int ea = P.ea[m];
+        const int* eb = P.eb + n0 + half * HC;  // padded to whole tiles
+        const int live = int(min(int64_t(HC), P.N - n0 - half * HC));
+        const bool part = P.splits > 1;
+        double* out = part ? P.work + (int64_t(T.z) * P.M + m) * P.N + n0 + half * HC
+                           : P.C + m * P.cm + (n0 + half * HC) * P.cn;
+        const int64_t step = part ? 1 : P.cn;
 #pragma unroll
-          for (int j = 0; j < HC; ++j) {
-            const int64_t n = n0 + half * HC + j;
-            if (n >= P.N) continue;
-            double v = fixed_to_double(th[j], rem[j], ea + P.eb[n] - 14 - 21);  // one rounding
+        for (int j = 0; j < HC; ++j) {
+          if (j < live) {
+            double v = sums.value(j, ea + eb[j]);  // one rounding
             if (P.alpha != 1.0) v *= P.alpha;
-            if (P.splits > 1)
-              P.work[(int64_t(T.z) * P.M + m) * P.N + n] = v;
-            else
-              P.C[cbase + map_at(P.cn, n)] = v;
-          }
-        }
-      } else {
-        float hi[HC], lo[HC];
-#pragma unroll
-        for (int j = 0; j < HC; ++j) hi[j] = lo[j] = 0.0f;
-        for (int64_t c = 0; c < nchunks; ++c) {
-          if (!mbar_wait(acc_full, uint32_t(h & 1), P.err, P.wait_ns)) {
-            set_err(P.err, 14);
-            *(volatile int*)abort_flag = 1;
-            break;
-          }
-          ++h;
-          asm volatile("tcgen05.fence::after_thread_sync;");
-#pragma unroll
-          for (int q = 0; q < S; ++q) {
-            const float scale = __int_as_float((127 - 7 * q) << 23);  // 2^{-7q}
-#pragma unroll
-            for (int c0 = 0; c0 < HC; c0 += 16) {
-              uint32_t r[16];
-              tmem_ld16(tmem + (uint32_t(quarter * 32) << 16) + uint32_t(q * BN + half * HC + c0), r);
-              asm volatile("tcgen05.wait::ld.sync.aligned;");
-#pragma unroll
-              for (int j = 0; j < 16; ++j) {
-                const float x = __uint_as_float(r[j]) * scale;
-                const float s = hi[c0 + j] + x;
-                const float bb = s - hi[c0 + j];
-                const float e = (hi[c0 + j] - (s - bb)) + (x - bb);
-                hi[c0 + j] = s;
-                lo[c0 + j] += e;
-              }
-            }
-          }
-          asm volatile("tcgen05.fence::before_thread_sync;");
-          __syncwarp();
-          if (lane == 0) mbar_arrive(acc_empty);
-        }
-        if (m < P.M && !*(volatile int*)abort_flag) {
-          const int ea = P.ea[m];
-          const int64_t cbase = map_at(P.cm, m);
-#pragma unroll
-          for (int j = 0; j < HC; ++j) {
-            const int64_t n = n0 + half * HC + j;
-            if (n >= P.N) continue;
-            const int e = ea + P.eb[n] - 14;
-            double v = scaled_to_double(hi[j], e) + scaled_to_double(lo[j], e);  // one FP64 add
-            if (P.alpha != 1.0) v *= P.alpha;
-            if (P.splits > 1)
-              P.work[(int64_t(T.z) * P.M + m) * P.N + n] = v;
-            else
-              P.C[cbase + map_at(P.cn, n)] = v;
+            out[j * step] = v;
           }
         }
       }
@@ -1120,10 +1044,8 @@ __global__ void __launch_bounds__(OzColCfg::threads, 1) k_oz_columns(const __gri
           }
           continue;
         }
-        long long th[HC];
-        uint32_t rem[HC];
-#pragma unroll
-        for (int j = 0; j < HC; ++j) th[j] = 0, rem[j] = 0u;
+        OzSums<S, HC> sums;
+        sums.clear();
         for (int c = 0; c < nchunks; ++c) {
           if (!mbar_wait(acc_full, uint32_t(h & 1), P.err, P.wait_ns)) {
             set_err(P.err, 14);
@@ -1132,17 +1054,18 @@ __global__ void __launch_bounds__(OzColCfg::threads, 1) k_oz_columns(const __gri
           }
           ++h;
           asm volatile("tcgen05.fence::after_thread_sync;");
-          drain_exact<S, BN, HC>(tbase, th, rem);
+          sums.template drain<BN>(tbase);
           asm volatile("tcgen05.fence::before_thread_sync;");
           __syncwarp();
           if (lane == 0) mbar_arrive(acc_empty);
         }
         if (*(volatile int*)abort_flag) break;
         const int ea = live && nchunks ? Q.ea[m] : 0;
+        const int* eb = nchunks ? Q.eb + n0 : nullptr;
 #pragma unroll
         for (int j = 0; j < HC; ++j) {
           if (n0 + j >= T.members || !live) continue;
-          double v = nchunks ? fixed_to_double(th[j], rem[j], ea + Q.eb[n0 + j] - 14 - 21) : 0.0;  // one rounding
+          double v = nchunks ? sums.value(j, ea + eb[j]) : 0.0;  // one rounding
           if (sg == 1) {
             const double a = mine[j * kBM];
             v = L.w * (a * (a + 2.0 * v));
@@ -1226,14 +1149,14 @@ __global__ void __launch_bounds__(256) k_oz_set_rows(const __grid_constant__ OzR
 
 // C = sum_z work[z] (deterministic order), same store maps as the GEMM
 __global__ void k_oz_reduce(const double* __restrict__ work, int splits, int64_t M, int64_t N, double* __restrict__ C,
-                            OzMap cm, OzMap cn, int sym) {
+                            int64_t cm, int64_t cn, int sym) {
   const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (e >= M * N) return;
   const int64_t m = e / N, n = e % N;
   if (sym && n > m) return;
   double s = 0.0;
   for (int z = 0; z < splits; ++z) s += work[int64_t(z) * M * N + e];
-  C[map_at(cm, m) + map_at(cn, n)] = s;
+  C[m * cm + n * cn] = s;
 }
 
 // persistent: one wave of CTAs that loop over the tiles (a tile's epilogue
@@ -1351,8 +1274,8 @@ void oz_gemm(const OzOperand& A, const OzOperand& B, double* C, int64_t ldc, int
   P.sym = sym;
   P.splits = splits < 1 ? 1 : splits;
   P.C = C;
-  P.cm = trans ? oz_stride(1) : oz_stride(ldc);
-  P.cn = trans ? oz_stride(ldc) : oz_stride(1);
+  P.cm = trans ? 1 : ldc;
+  P.cn = trans ? ldc : 1;
   P.alpha = alpha;
   P.work = work;
   P.err = err;
