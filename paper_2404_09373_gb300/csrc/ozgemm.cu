@@ -11,22 +11,28 @@
 // are integers below 2^14, so levels 0 and 1 summed over a chunk of 1024 k
 // values stay below 2^24 and are exact in FP32; deeper levels are scaled by
 // 2^-14 or less, where FP32 rounding is harmless.  After every chunk the
-// epilogue warps read the levels out (tcgen05.ld) and add them to double-float
-// (hi, lo) register accumulators; the result is formed in FP64 at the end.
-// With S = 8 (FP64-grade: 56 fraction bits per operand) the chunk is 256 k, so
-// every level's sum is an exact integer below 2^24, and the epilogue adds the
-// levels into two 64-bit integer accumulators: the product of the rounded
-// operands is then exact up to the dropped levels (below 2^-56 relative per
-// term) and one final FP64 rounding.
+// epilogue warps read the levels out (tcgen05.ld) and add them as integers
+// (OzSums); the result is rounded once.  With S = 7 or 8 (FP64-grade: 49 or 56
+// fraction bits per operand) the chunk is 512 k, so that levels 0..5 are exact:
+// the product of the rounded operands is then exact up to the dropped levels
+// (below 2^-56 relative per term for S = 8) and one final FP64 rounding.
 //
 // Operands are pre-tiled by the slicing kernel into the canonical K-major,
 // no-swizzle UMMA layout (8x8 core matrices, LBO = 128 B along K, SBO =
 // 512 B per 8-row group, 32 k values per tile), all S slices of one
 // (row tile, k tile) contiguous, so one cp.async.bulk per operand fills a
-// pipeline stage.  Roles per CTA: warp 0 issues the bulk copies, warp 1 owns
-// tensor memory and issues tcgen05.mma, warps 2-9 drain the accumulators.
+// pipeline stage.  Roles per CTA (one per SM): warp 0 issues the bulk copies,
+// warp 1 owns tensor memory, warps 1 and 2 issue tcgen05.mma, the rest drain the
+// accumulators, convert and store.
 // Every mbarrier wait is bounded: on expiry the CTA records an error code,
 // lets its copies and MMAs in flight finish, frees tensor memory and exits.
+//
+// What a tile of the 5-digit product costs (131072 x 1824 x 832, clock64): two
+// CTAs an SM, one tile each, 158k cycles, 89k of them in the conversion and
+// strided stores of the epilogue; with that rewritten 75k; one persistent CTA
+// with a pair of tiles, MMAs by one thread, 120k the pair, stage 2020 cycles; by
+// two threads 104k, stage 1600 of which 1440 are MMA time at the full rate.
+// In all 9.85 -> 3.44 ms, 1.73 PFLOP/s of BF16 (0.91 of the measured peak).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -110,6 +116,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t phase, const i
   return false;
 }
 
+// mbar_wait by all lanes of a warp, one answer for all of them
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t phase, const int* err, unsigned long long wait_ns) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, phase, err, wait_ns)) != 0;
+}
+
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
@@ -125,17 +136,32 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
                : "memory");
 }
 
-__device__ __forceinline__ void umma_bf16(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+// The MMA warp runs its loop with all lanes and `el` is set in one of them: the
+// instruction is predicated, not branched around.  Control flow stays uniform, so
+// the descriptors live in uniform registers; under a branch on the lane every
+// operand was moved there first and an MMA took 110 cycles to issue whatever its
+// size.
+__device__ __forceinline__ void umma_bf16(uint32_t el, uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                           uint32_t accumulate) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
-          dtmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
+      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtmem),
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(el));
 }
 
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
+__device__ __forceinline__ void umma_commit(uint32_t el, uint64_t* bar) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(smem_u32(bar)),
+      "r"(el)
+      : "memory");
+}
+
+// one lane of a converged warp
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t el;
+  asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.u32 %0, 1, 0, q;\n}\n" : "=r"(el));
+  return el;
 }
 
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
@@ -146,39 +172,48 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
 
 __device__ __forceinline__ void set_err(int* err, int code) { atomicCAS(err, 0, code); }
 
-// sign M 2^e as a double, |value| outside the normal range: out of line, so
-// that the epilogues' unrolled code stays short
-__device__ __noinline__ double far_double(bool neg, uint64_t M, int e) {
-  const double v = ldexp(double(M), e);
-  return neg ? -v : v;
-}
+// Exponents beyond which a result may leave the normal range of a double
+// (fixed_to_double's argument is at most 2^63 and at least 2^-28 in magnitude).
+constexpr int kNearExp = 900;
 
 // (th + rem 2^-28) 2^e rounded once to the nearest double (ties to even) with
-// integer operations.  rem in [0, 2^28).
+// integer operations; rem in [0, 2^28), |e| <= kNearExp.  No branches, so that
+// the conversions of neighbouring columns overlap.
 __device__ __forceinline__ double fixed_to_double(long long th, uint32_t rem, int e) {
-  // sign and magnitude U = hi + lo 2^-28
+  // sign and magnitude hi + lo 2^-28
   const bool neg = th < 0;
-  uint32_t lo = rem;
-  uint64_t hi = uint64_t(th);
-  if (neg) {
-    lo = (0u - rem) & 0x0FFFFFFFu;
-    hi = ~hi + (rem == 0u ? 1ull : 0ull);
-  }
-  const int low = hi == 0ull;  // only the fraction is left
+  const uint32_t lo = neg ? (0u - rem) & 0x0FFFFFFFu : rem;
+  uint64_t hi = neg ? ~uint64_t(th) + (rem == 0u ? 1ull : 0ull) : uint64_t(th);
+  const bool low = hi == 0ull;  // only the fraction is left
   hi = low ? uint64_t(lo) : hi;
   const uint64_t frac = low ? 0ull : uint64_t(lo) << 36;
-  if (hi == 0ull) return 0.0;
-  const int lz = __clzll((long long)hi);
-  const uint64_t top = (hi << lz) | (lz ? frac >> (64 - lz) : 0ull);
+  const int lz = __clzll((long long)(hi | 1ull));
+  const uint64_t top = (hi << lz) | ((frac >> 1) >> (63 - lz));
   const uint32_t cut = uint32_t(top) & 0x7FFu;
   const uint64_t M = top >> 11;  // 53 bits
   // half of the last place, and what lies below it
   const bool up = cut > 0x400u || (cut == 0x400u && ((frac << lz) != 0ull || (M & 1ull)));
-  const int E = 63 - lz + e - (low ? 28 : 0) + 1023;
-  const uint64_t R = M + (up ? 1ull : 0ull);
-  if (E < 1 || E > 2045) return far_double(neg, R, E - 1075);
-  // R's leading bit adds one to the exponent field, as does a carry out of R
-  return __longlong_as_double((long long)((uint64_t(neg) << 63) | ((uint64_t(E - 1) << 52) + R)));
+  const int E = 63 - lz + e - (low ? 28 : 0) + 1022;
+  // M's leading bit adds one to the exponent field, as does a carry out of it
+  const uint64_t R = (uint64_t(neg) << 63) | ((uint64_t(uint32_t(E)) << 52) + M + (up ? 1ull : 0ull));
+  return __longlong_as_double(hi ? (long long)R : 0ll);
+}
+
+// X 2^e rounded once to the nearest double (ties to even), |e| <= kNearExp
+__device__ __forceinline__ double ll_to_double(long long X, int e) {
+  const uint64_t U = X < 0 ? uint64_t(-X) : uint64_t(X);
+  const int lz = __clzll((long long)(U | 1ull));
+  const uint64_t top = U << lz;
+  const uint32_t cut = uint32_t(top) & 0x7FFu;
+  const uint64_t M = top >> 11;
+  const uint32_t up = (cut > 0x400u || (cut == 0x400u && (uint32_t(M) & 1u))) ? 1u : 0u;
+  const uint64_t R = (uint64_t(uint32_t(63 - lz + e + 1022)) << 52) + M + up;
+  return __longlong_as_double((long long)((uint64_t(X) & 0x8000000000000000ull) | (U ? R : 0ull)));
+}
+
+// the first of the two for any exponent, out of line
+__device__ __noinline__ double far_double(long long th, uint32_t rem, int e) {
+  return ldexp(fixed_to_double(th, rem, 0), e);
 }
 
 // ---------------------------------------------------------------- slicing
@@ -523,55 +558,69 @@ struct OzCfg {
   static constexpr int tileB = BN * kBK * 2;
   static constexpr int stageA = S * tileA;
   static constexpr int stageB = S * tileB;
-  static constexpr int stage = stageA + stageB;
   static constexpr int cols = S * BN;
   static constexpr bool exact = S >= 7;
-  // two CTAs per SM when the accumulators take at most half of tensor memory:
-  // one CTA's pipeline fill and accumulator drain overlap the other's MMAs
-  static constexpr bool dual = !exact && cols <= 256;
-  static constexpr int min_blocks = dual ? 2 : 1;
-  static constexpr int budget = dual ? 115712 - 2048 : 220 * 1024 - 2048;
-  static constexpr int nst = budget / stage < 4 ? budget / stage : 4;
-  static constexpr int smem = nst * stage + 2048;  // + barriers and 1024-byte alignment slack
-  static constexpr uint32_t tcols = cols <= 32 ? 32 : cols <= 64 ? 64 : cols <= 128 ? 128 : cols <= 256 ? 256 : 512;
-  // S = 8: levels 0..5 are kept exact (chunks of 512 k keep their integer
+  // Two N tiles at a time where their accumulators fit in tensor memory: they
+  // share the A digits of a stage.
+  static constexpr int pair = cols <= 256 ? 2 : 1;
+  // Two issuing warps, each with its own accumulator columns: the two tiles of a
+  // pair, or levels [0, cut) and [cut, S) of one.  MMAs of one thread run one after
+  // the other, N / 2 + 32 cycles each (the A operand's load is not hidden: a stage
+  // of 5 digits and two tiles took 2020 cycles, 1440 of them MMA time); those of
+  // two threads overlap.
+  static constexpr int issuers = 2;
+  static constexpr int cut = S == 6 ? 4 : 5;
+  static constexpr int stage = stageA + pair * stageB;
+  static constexpr uint32_t tcols = 512;
+  // epilogue warps: two per tensor-memory lane quarter (BN / 2 columns of a tile
+  // each), or three (BN / 3 columns each, so that the integer state fits in registers)
+  static constexpr int epi = BN % 48 == 0 ? 12 : 8;
+  // the epilogue's transposing buffer: [32][4] values a warp, past the ring
+  static constexpr int xbytes = epi * 32 * 4 * 8;
+  static constexpr int nst = (232448 - 2048 - xbytes) / stage < 4 ? (232448 - 2048 - xbytes) / stage : 4;
+  static constexpr int xpose = nst * stage + 1024;
+  static constexpr int smem = nst * stage + 2048 + xbytes;  // + barriers and 1024-byte alignment slack
+  // 7, 8 digits: levels 0..5 are kept exact (chunks of 512 k keep their integer
   // sums at most 2^24; levels 6, 7 weigh less than 2^-42, where FP32 rounding
-  // is harmless) and summed in integers; else double-float
+  // is harmless); 5, 6 digits: levels 0 and 1 (1024 k)
   static constexpr int kc = exact ? 512 / kBK : kKcTiles;  // k tiles per chunk
-  // epilogue warps: two per tensor-memory lane quarter (BN/2 columns each),
-  // three when exact (BN/3 columns each, so the integer state fits in
-  // registers), one when two CTAs share the SM
-  static constexpr int epi = exact ? 12 : dual ? 4 : 8;
-  static constexpr int threads = 32 * (2 + epi);
+  static constexpr int threads = 32 * (1 + issuers + epi);
   static_assert(!exact || S == 7 || S == 8, "the integer epilogue pairs the levels of 7 or 8 digits");
   static_assert(cols <= 512, "levels x BN must fit in tensor memory");
   static_assert(nst >= 2, "need at least two pipeline stages");
-  static_assert((BN / (epi / 4)) % 16 == 0, "each epilogue warp reads whole 16-column groups");
+  static_assert((BN / (epi / 4)) % 8 == 0, "each epilogue warp reads whole 8-column groups");
   static_assert(smem <= 232448, "shared memory per CTA");
 };
 
-// The MMAs of one pipeline stage (32 k values).  For A digit s the products
-// with B digits t = 0..S-1-s land in levels s..S-1, i.e. tensor-memory columns
-// [s BN, S BN); the B digit tiles of a stage are contiguous, so B rows [0,
-// (S-s) BN) are exactly digits 0..S-1-s and one MMA (N up to 256, else split)
-// covers them all.  The first MMA of a chunk (s = 0) spans every level and
-// initialises the accumulators.
-template <int S, int BN>
-__device__ __forceinline__ void mma_stage(uint32_t tmem, uint32_t sA, uint32_t sB, bool first) {
+// One issuer's MMAs of one pipeline stage (32 k values).  For A digit s the
+// products with B digits t = 0..S-1-s land in levels s..S-1, i.e.
+// tensor-memory columns [s BN, S BN); the B digit tiles of a stage are
+// contiguous, so one MMA covers the levels [q, q1) of an issuer's range with B
+// rows [(q - s) BN, (q1 - s) BN), q the first of its levels at or above s.  The
+// first MMA of a chunk (s = 0) spans the whole range and initialises it.
+template <int S, int BN, int PART>
+__device__ __forceinline__ void mma_part(uint32_t el, uint32_t tmem, uint32_t sA, uint32_t sB, bool first) {
+  using Cfg = OzCfg<S, BN>;
+  constexpr int tile = Cfg::pair == 2 ? PART : 0;  // 256 columns on for the second tile
+  constexpr int q0 = Cfg::pair == 2 || PART == 0 ? 0 : Cfg::cut;
+  constexpr int q1 = Cfg::pair == 2 || PART == 1 ? S : Cfg::cut;
+  static_assert((q1 - q0) * BN <= 256, "an MMA has at most 256 columns");
 #pragma unroll
-  for (int s = 0; s < S; ++s) {
+  for (int s = 0; s < q1; ++s) {
+    const int q = s > q0 ? s : q0, n = (q1 - q) * BN;
 #pragma unroll
-    for (int c0 = 0; c0 < BN * (S - s); c0 += 256) {
-      const int n = (BN * (S - s) - c0) < 256 ? (BN * (S - s) - c0) : 256;
-      const uint32_t idesc = umma_idesc(kBM, n);
-#pragma unroll
-      for (int ks = 0; ks < kBK / 16; ++ks) {
-        const uint64_t da = umma_desc(sA + s * OzCfg<S, BN>::tileA + ks * 256);
-        const uint64_t db = umma_desc(sB + (c0 / 8) * (16 * kBK) + ks * 256);
-        umma_bf16(tmem + uint32_t(s * BN + c0), da, db, idesc, (!first || s > 0 || ks > 0) ? 1u : 0u);
-      }
+    for (int ks = 0; ks < kBK / 16; ++ks) {
+      const uint64_t da = umma_desc(sA + s * Cfg::tileA + ks * 256);
+      const uint64_t db = umma_desc(sB + tile * Cfg::stageB + ((q - s) * BN / 8) * (16 * kBK) + ks * 256);
+      umma_bf16(el, tmem + uint32_t(256 * tile + q * BN), da, db, umma_idesc(kBM, n), (!first || s > 0 || ks > 0) ? 1u : 0u);
     }
   }
+}
+template <int S, int BN>
+__device__ __forceinline__ void mma_stage(int part, uint32_t el, uint32_t tmem, uint32_t sA, uint32_t sB, bool first,
+                                          int tiles) {
+  if (part == 0) mma_part<S, BN, 0>(el, tmem, sA, sB, first);
+  else if (OzCfg<S, BN>::pair == 1 || tiles == 2) mma_part<S, BN, 1>(el, tmem, sA, sB, first);
 }
 
 // Exact integer sums of one thread's HC columns: th in units of 2^-21 of
@@ -634,18 +683,35 @@ struct OzSums {
       }
     }
   }
-  // the value times 2^e (e: the sum of the rows' exponents), rounded once
-  __device__ __forceinline__ double value(int c, int e) const {
-    uint32_t f;
-    if constexpr (S >= 7) f = rem[c];
-    else if constexpr (S == 6) f = rem[c] << 14;
-    else f = ((rem[c / 4] >> (8 * (c & 3))) & 0x7Fu) << 21;
-    return fixed_to_double(th[c], f, e - 14 - 21);
+  // fraction of column c in units of 2^-28
+  __device__ __forceinline__ uint32_t frac(int c) const {
+    if constexpr (S >= 7) return rem[c];
+    else if constexpr (S == 6) return rem[c] << 14;
+    else return ((rem[c / 4] >> (8 * (c & 3))) & 0x7Fu) << 21;
+  }
+  // every column's value times 2^(ea + eb(c)), rounded once; wide: a 5- or
+  // 6-digit sum may not fit 64 bits.  Straight-line code (the rare cases
+  // afterwards, out of line), so that the columns' conversions overlap, and no
+  // FP64 instruction: each holds its scheduler for over 100 cycles.
+  template <class E>
+  __device__ __forceinline__ void values(int ea, E eb, bool wide, double (&v)[HC]) const {
+    constexpr int FB = 7 * (S - 4);  // bits of the fraction (S < 7)
+    int m = 0;
+#pragma unroll
+    for (int c = 0; c < HC; ++c) {
+      const int e = ea + eb(c) - 35, en = abs(e) > kNearExp - 64 ? 0 : e;
+      m = max(m, abs(e));
+      if constexpr (S >= 7) v[c] = fixed_to_double(th[c], rem[c], en);
+      else v[c] = ll_to_double(th[c] * (1 << FB) + (long long)(frac(c) >> (28 - FB)), en - FB);
+    }
+    if (m > kNearExp - 64 || (S < 7 && wide))
+#pragma unroll
+      for (int c = 0; c < HC; ++c) v[c] = far_double(th[c], frac(c), ea + eb(c) - 35);
   }
 };
 
 template <int S, int BN>
-__global__ void __launch_bounds__(OzCfg<S, BN>::threads, OzCfg<S, BN>::min_blocks) k_oz_gemm(OzGemmParams P) {
+__global__ void __launch_bounds__(OzCfg<S, BN>::threads, 1) k_oz_gemm(OzGemmParams P) {
   using Cfg = OzCfg<S, BN>;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -654,10 +720,11 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, OzCfg<S, BN>::min_block
   uint64_t* acc_full = empty + Cfg::nst;
   uint64_t* acc_empty = acc_full + 1;
   uint64_t* drain = acc_empty + 1;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + Cfg::issuers);
   int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
 
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x / 32, 0);  // uniform to the compiler
+  const int lane = threadIdx.x % 32;
   // an earlier launch failed: do nothing (one read, made uniform across the CTA)
   if (__syncthreads_or(threadIdx.x == 0 ? *(volatile const int*)P.err : 0)) return;
 
@@ -666,10 +733,10 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, OzCfg<S, BN>::min_block
   // role walks the same tile sequence; stage and chunk counters run on across
   // tiles, so the ring of stages and the accumulator hand-off never restart
   // and a tile's epilogue overlaps the next tile's copies and MMAs.
-  const int64_t NT = P.ntn, MT = P.ntm, ntiles = NT * MT * P.splits;
+  const int64_t NT = (P.ntn + Cfg::pair - 1) / Cfg::pair, MT = P.ntm, ntiles = NT * MT * P.splits;
   struct Tile {
     int64_t nt, mt, m0, n0, kt_lo, nk;
-    int z;
+    int z, tiles;  // tiles: N tiles of this pair
     bool skip;
   };
   auto tile_at = [&](int64_t t) {
@@ -678,10 +745,12 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, OzCfg<S, BN>::min_block
     T.mt = (t / NT) % MT;
     T.z = int(t / (NT * MT));
     T.m0 = T.mt * kBM;
+    T.nt *= Cfg::pair;
+    T.tiles = int(min(int64_t(Cfg::pair), P.ntn - T.nt));
     T.n0 = T.nt * BN;
     T.skip = P.sym && T.n0 > T.m0 + kBM - 1;  // tile entirely above the diagonal
     int64_t lo = 0, hi = P.nkt;
-    if (P.tri == 1) hi = min(P.nkt, (T.n0 + BN + kBK - 1) / kBK);
+    if (P.tri == 1) hi = min(P.nkt, (T.n0 + Cfg::pair * BN + kBK - 1) / kBK);
     if (P.tri == 2) lo = min(P.nkt, T.n0 / kBK);
     const int64_t tot = hi - lo, per = (tot + P.splits - 1) / P.splits;
     const int64_t a = lo + per * T.z;
@@ -693,11 +762,11 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, OzCfg<S, BN>::min_block
   if (threadIdx.x == 0) {
     for (int i = 0; i < Cfg::nst; ++i) {
       mbar_init(&full[i], 1);
-      mbar_init(&empty[i], 1);
+      mbar_init(&empty[i], Cfg::issuers);
     }
-    mbar_init(acc_full, 1);
+    mbar_init(acc_full, Cfg::issuers);
     mbar_init(acc_empty, Cfg::epi);
-    mbar_init(drain, 1);
+    for (int i = 0; i < Cfg::issuers; ++i) mbar_init(&drain[i], 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
@@ -709,7 +778,7 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, OzCfg<S, BN>::min_block
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
   if (warp == 0) {
     // ------------------------------------------------ producer
@@ -732,9 +801,10 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, OzCfg<S, BN>::min_block
           const int64_t kt = T.kt_lo + it;
           unsigned char* sA = smem + st * Cfg::stage;
           unsigned char* sB = sA + Cfg::stageA;
-          mbar_expect_tx(&full[st], Cfg::stageA + Cfg::stageB);
+          mbar_expect_tx(&full[st], Cfg::stageA + T.tiles * Cfg::stageB);
           bulk_g2s(sA, gA + (T.mt * P.akst + kt) * int64_t(Cfg::stageA), Cfg::stageA, &full[st]);
-          bulk_g2s(sB, gB + (T.nt * P.bkst + kt) * int64_t(Cfg::stageB), Cfg::stageB, &full[st]);
+          for (int b = 0; b < T.tiles; ++b)
+            bulk_g2s(sB + b * Cfg::stageB, gB + ((T.nt + b) * P.bkst + kt) * int64_t(Cfg::stageB), Cfg::stageB, &full[st]);
         }
       }
       // copies that were issued but never consumed must land before exit
@@ -743,9 +813,10 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, OzCfg<S, BN>::min_block
         for (int64_t it = first; it < g; ++it) mbar_wait(&full[it % Cfg::nst], uint32_t((it / Cfg::nst) & 1), nullptr);
       }
     }
-  } else if (warp == 1) {
-    // ------------------------------------------------ MMA issuer
-    if (lane == 0) {
+  } else if (warp <= Cfg::issuers) {
+    // ------------------------------------------------ MMA issuers
+    const uint32_t el = elect_one();
+    {
       int64_t g = 0, h = 0;  // stages consumed, accumulator chunks handed over (all tiles)
       bool stop = false;
       for (int64_t t = blockIdx.x; t < ntiles && !stop; t += gridDim.x) {
@@ -755,41 +826,41 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, OzCfg<S, BN>::min_block
           const int st = int(g % Cfg::nst);
           const int64_t round = g / Cfg::nst;
           const int64_t cpos = it % Cfg::kc;
-          if (cpos == 0 && h > 0 && !mbar_wait(acc_empty, uint32_t((h - 1) & 1), P.err, P.wait_ns)) {
+          if (cpos == 0 && h > 0 && !warp_wait(acc_empty, uint32_t((h - 1) & 1), P.err, P.wait_ns)) {
             set_err(P.err, 12);
             *(volatile int*)abort_flag = 1;
             stop = true;
             break;
           }
-          if (!mbar_wait(&full[st], uint32_t(round & 1), P.err, P.wait_ns)) {
+          if (!warp_wait(&full[st], uint32_t(round & 1), P.err, P.wait_ns)) {
             set_err(P.err, 13);
             *(volatile int*)abort_flag = 1;
             stop = true;
             break;
           }
-          if (*(volatile int*)abort_flag) {
+          if (__any_sync(0xffffffffu, *(volatile int*)abort_flag)) {
             stop = true;
             break;
           }
           asm volatile("tcgen05.fence::after_thread_sync;");
           const uint32_t sA = smem_u32(smem + st * Cfg::stage);
           const uint32_t sB = sA + Cfg::stageA;
-          mma_stage<S, BN>(tmem, sA, sB, cpos == 0);
-          umma_commit(&empty[st]);
+          mma_stage<S, BN>(warp - 1, el, tmem, sA, sB, cpos == 0, T.tiles);
+          umma_commit(el, &empty[st]);
           if (cpos == Cfg::kc - 1 || it == T.nk - 1) {
-            umma_commit(acc_full);
+            umma_commit(el, acc_full);
             ++h;
           }
         }
       }
       // all MMAs issued by this thread complete before tensor memory is freed
-      umma_commit(drain);
-      mbar_wait(drain, 0, nullptr);
+      umma_commit(el, &drain[warp - 1]);
+      mbar_wait(&drain[warp - 1], 0, nullptr);
     }
   } else {
     // ------------------------------------------------ epilogue warps
     const int quarter = warp % 4;  // a warp reads tensor-memory lanes 32 (warp % 4) ..
-    const int half = (warp - 2) / 4;  // which share of the columns
+    const int half = (warp - 1 - Cfg::issuers) / 4;  // which share of the columns
     const int row = quarter * 32 + lane;
     constexpr int HC = BN / (Cfg::epi / 4);  // columns per thread
     int64_t h = 0;  // accumulator chunks taken over (all tiles)
@@ -797,9 +868,10 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, OzCfg<S, BN>::min_block
       const Tile T = tile_at(t);
       if (T.skip) continue;
       const int64_t nchunks = (T.nk + Cfg::kc - 1) / Cfg::kc;
-      const int64_t m = T.m0 + row, n0 = T.n0;
-      OzSums<S, HC> sums;
-      sums.clear();
+      const int64_t m = T.m0 + row;
+      OzSums<S, HC> sums[Cfg::pair];
+#pragma unroll
+      for (int b = 0; b < Cfg::pair; ++b) sums[b].clear();
       for (int64_t c = 0; c < nchunks; ++c) {
         if (!mbar_wait(acc_full, uint32_t(h & 1), P.err, P.wait_ns)) {
           set_err(P.err, 14);
@@ -808,25 +880,58 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, OzCfg<S, BN>::min_block
         }
         ++h;
         asm volatile("tcgen05.fence::after_thread_sync;");
-        sums.template drain<BN>(tmem + (uint32_t(quarter * 32) << 16) + uint32_t(half * HC));
+#pragma unroll
+        for (int b = 0; b < Cfg::pair; ++b)
+          if (b < T.tiles)
+            sums[b].template drain<BN>(tmem + (uint32_t(quarter * 32) << 16) + uint32_t(256 * b + half * HC));
         asm volatile("tcgen05.fence::before_thread_sync;");
         __syncwarp();
         if (lane == 0) mbar_arrive(acc_empty);
       }
-      if (m < P.M && !*(volatile int*)abort_flag) {
-        const int ea = P.ea[m];
-        const int* eb = P.eb + n0 + half * HC;  // padded to whole tiles
-        const int live = int(min(int64_t(HC), P.N - n0 - half * HC));
-        const bool part = P.splits > 1;
-        double* out = part ? P.work + (int64_t(T.z) * P.M + m) * P.N + n0 + half * HC
-                           : P.C + m * P.cm + (n0 + half * HC) * P.cn;
-        const int64_t step = part ? 1 : P.cn;
+      if (*(volatile int*)abort_flag) break;
+      // rows beyond M and columns beyond N hold padding (scales of padding rows
+      // are not written: only live ones may be used)
+      const int ea = m < P.M ? P.ea[m] : 0;
+      const bool part = P.splits > 1, scale = P.alpha != 1.0;
+      const int64_t sm = part ? P.N : P.cm, sn = part ? 1 : P.cn;
+      const int64_t mrow = T.m0 + quarter * 32;
+      const int rows = int(min(int64_t(32), P.M - mrow));
 #pragma unroll
-        for (int j = 0; j < HC; ++j) {
-          if (j < live) {
-            double v = sums.value(j, ea + eb[j]);  // one rounding
-            if (P.alpha != 1.0) v *= P.alpha;
-            out[j * step] = v;
+      for (int b = 0; b < Cfg::pair; ++b) {
+        const int64_t nb = T.n0 + b * BN + half * HC;
+        const int live = int(min(int64_t(HC), P.N - nb));
+        if (live <= 0) continue;
+        const int* ebp = P.eb + nb;
+        auto eb = [&](int j) { return j < live ? __ldg(ebp + j) : 0; };
+        double* out = (part ? P.work + int64_t(T.z) * P.M * P.N : P.C) + mrow * sm + nb * sn;
+        double v[HC];
+        sums[b].values(ea, eb, T.nk * kBK >= (int64_t(1) << (35 - 14 * (S - 4))), v);
+        if (scale) {
+#pragma unroll
+          for (int j = 0; j < HC; ++j) v[j] *= P.alpha;
+        }
+        if (sn != 1) {  // a lane's neighbours are adjacent in memory
+#pragma unroll
+          for (int j = 0; j < HC; ++j)
+            if (j < live && lane < rows) out[lane * sm + j * sn] = v[j];
+        } else {
+          // Rows of C: a store per column of a lane's row touches 32 sectors with 8
+          // bytes each; through the warp's [32][4] piece of shared memory it
+          // writes whole sectors, 4 columns of 8 rows at a time.
+          double* buf = reinterpret_cast<double*>(smem + Cfg::xpose) + (warp - 1 - Cfg::issuers) * 128;
+          const int r0 = lane >> 2, c = lane & 3;
+#pragma unroll
+          for (int j0 = 0; j0 < HC; j0 += 4) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) buf[lane * 4 + ((u + (lane >> 2)) & 3)] = v[j0 + u];
+            __syncwarp();
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const int r = u * 8 + r0;
+              const double x = buf[r * 4 + ((c + (r >> 2)) & 3)];
+              if (r < rows && j0 + c < live) out[r * sm + j0 + c] = x;
+            }
+            __syncwarp();
           }
         }
       }
@@ -896,9 +1001,10 @@ __global__ void __launch_bounds__(OzColCfg::threads, 1) k_oz_columns(const __gri
   uint64_t* acc_full = empty + Cfg::nst;
   uint64_t* acc_empty = acc_full + 1;
   uint64_t* drain = acc_empty + 1;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + Cfg::issuers);
   int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x / 32, 0);  // uniform to the compiler
+  const int lane = threadIdx.x % 32;
   if (__syncthreads_or(threadIdx.x == 0 ? *(volatile const int*)P.err : 0)) return;
 
   // tiles of level l: [t0[l], t0[l + 1]), N tiles fastest
@@ -931,11 +1037,11 @@ __global__ void __launch_bounds__(OzColCfg::threads, 1) k_oz_columns(const __gri
   if (threadIdx.x == 0) {
     for (int i = 0; i < Cfg::nst; ++i) {
       mbar_init(&full[i], 1);
-      mbar_init(&empty[i], 1);
+      mbar_init(&empty[i], Cfg::issuers);
     }
-    mbar_init(acc_full, 1);
+    mbar_init(acc_full, Cfg::issuers);
     mbar_init(acc_empty, Cfg::epi);
-    mbar_init(drain, 1);
+    for (int i = 0; i < Cfg::issuers; ++i) mbar_init(&drain[i], 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
@@ -947,7 +1053,7 @@ __global__ void __launch_bounds__(OzColCfg::threads, 1) k_oz_columns(const __gri
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
   if (warp == 0) {
     // ------------------------------------------------ producer
@@ -980,9 +1086,10 @@ __global__ void __launch_bounds__(OzColCfg::threads, 1) k_oz_columns(const __gri
         for (int64_t it = first; it < g; ++it) mbar_wait(&full[it % Cfg::nst], uint32_t((it / Cfg::nst) & 1), nullptr);
       }
     }
-  } else if (warp == 1) {
-    // ------------------------------------------------ MMA issuer
-    if (lane == 0) {
+  } else if (warp <= Cfg::issuers) {
+    // ------------------------------------------------ MMA issuers
+    const uint32_t el = elect_one();
+    {
       int64_t g = 0, h = 0;  // stages consumed, accumulator chunks handed over (all tiles)
       bool stop = false;
       for (int64_t t = blockIdx.x; t < ntiles && !stop; t += gridDim.x) {
@@ -992,37 +1099,37 @@ __global__ void __launch_bounds__(OzColCfg::threads, 1) k_oz_columns(const __gri
           for (int kt = 0; kt < nkt; ++kt, ++g) {
             const int st = int(g % Cfg::nst);
             const int cpos = kt % Cfg::kc;
-            if (cpos == 0 && h > 0 && !mbar_wait(acc_empty, uint32_t((h - 1) & 1), P.err, P.wait_ns)) {
+            if (cpos == 0 && h > 0 && !warp_wait(acc_empty, uint32_t((h - 1) & 1), P.err, P.wait_ns)) {
               set_err(P.err, 12);
               stop = true;
-            } else if (!mbar_wait(&full[st], uint32_t((g / Cfg::nst) & 1), P.err, P.wait_ns)) {
+            } else if (!warp_wait(&full[st], uint32_t((g / Cfg::nst) & 1), P.err, P.wait_ns)) {
               set_err(P.err, 13);
               stop = true;
             }
             if (stop) *(volatile int*)abort_flag = 1;
-            if (stop || *(volatile int*)abort_flag) {
+            if (stop || __any_sync(0xffffffffu, *(volatile int*)abort_flag)) {
               stop = true;
               break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;");
             const uint32_t sA = smem_u32(smem + st * Cfg::stage);
-            mma_stage<S, BN>(tmem, sA, sA + Cfg::stageA, cpos == 0);
-            umma_commit(&empty[st]);
+            mma_stage<S, BN>(warp - 1, el, tmem, sA, sA + Cfg::stageA, cpos == 0, 1);
+            umma_commit(el, &empty[st]);
             if (cpos == Cfg::kc - 1 || kt == nkt - 1) {
-              umma_commit(acc_full);
+              umma_commit(el, acc_full);
               ++h;
             }
           }
         }
       }
-      umma_commit(drain);  // all MMAs issued by this thread complete before tensor memory is freed
-      mbar_wait(drain, 0, nullptr);
+      umma_commit(el, &drain[warp - 1]);  // all MMAs issued by this thread complete before tensor memory is freed
+      mbar_wait(&drain[warp - 1], 0, nullptr);
     }
   } else {
     // ------------------------------------------------ epilogue warps
     constexpr int HC = BN / (Cfg::epi / 4);  // columns per thread
     const int quarter = warp % 4;            // a warp reads tensor-memory lanes 32 (warp % 4) ..
-    const int part = (warp - 2) / 4;         // which share of the columns
+    const int part = (warp - 1 - Cfg::issuers) / 4;  // which share of the columns
     const int row = quarter * 32 + lane;
     const uint32_t tbase = tmem + (uint32_t(quarter * 32) << 16) + uint32_t(part * HC);
     double* mine = stash + part * HC * kBM + row;
@@ -1061,23 +1168,32 @@ __global__ void __launch_bounds__(OzColCfg::threads, 1) k_oz_columns(const __gri
         }
         if (*(volatile int*)abort_flag) break;
         const int ea = live && nchunks ? Q.ea[m] : 0;
-        const int* eb = nchunks ? Q.eb + n0 : nullptr;
+        const int* ebp = Q.eb + n0;
+        const int cols = nchunks ? T.members - n0 : 0;  // live ones among this thread's (the others' scales are unset)
+        auto eb = [&](int j) { return j < cols ? __ldg(ebp + j) : 0; };
+        double v[HC];
+        sums.values(ea, eb, false, v);
+        if (sg == 1) {
 #pragma unroll
-        for (int j = 0; j < HC; ++j) {
-          if (n0 + j >= T.members || !live) continue;
-          double v = nchunks ? sums.value(j, ea + eb[j]) : 0.0;  // one rounding
-          if (sg == 1) {
+          for (int j = 0; j < HC; ++j) {
             const double a = mine[j * kBM];
-            v = L.w * (a * (a + 2.0 * v));
-          } else if (sg == 2) {
-            v = mine[j * kBM] - v;
-          } else if (last == 0) {
-            v = L.w * (v * v);
+            v[j] = L.w * (a * (a + 2.0 * v[j]));
           }
-          if (sg == last)
-            L.C[int64_t(n0 + j) * L.M + m] = v;
-          else
-            mine[j * kBM] = v;
+        } else if (sg == 2) {
+#pragma unroll
+          for (int j = 0; j < HC; ++j) v[j] = mine[j * kBM] - v[j];
+        } else if (last == 0) {
+#pragma unroll
+          for (int j = 0; j < HC; ++j) v[j] = L.w * (v[j] * v[j]);
+        }
+        if (sg < last) {
+#pragma unroll
+          for (int j = 0; j < HC; ++j) mine[j * kBM] = v[j];
+        } else {
+          double* out = L.C + int64_t(n0) * L.M + m;
+#pragma unroll
+          for (int j = 0; j < HC; ++j)
+            if (n0 + j < T.members && live) out[int64_t(j) * L.M] = v[j];
         }
       }
     }
@@ -1185,7 +1301,7 @@ void launch_oz(const OzGemmParams& P, bool persistent, cudaStream_t s) {
     res = std::max(1, nsm) * std::max(1, per);
     resident[dev].store(res, std::memory_order_release);
   }
-  const int64_t ntiles = P.ntn * P.ntm * P.splits;
+  const int64_t ntiles = ((P.ntn + Cfg::pair - 1) / Cfg::pair) * P.ntm * P.splits;
   const unsigned grid = unsigned(std::max<int64_t>(1, persistent ? std::min<int64_t>(ntiles, res) : ntiles));
   k_oz_gemm<S, BN><<<grid, Cfg::threads, Cfg::smem, s>>>(P);
 }
@@ -1255,7 +1371,7 @@ static unsigned long long oz_wait_limit() {
   return (fault && std::strcmp(fault, "oz_wait") == 0) ? 0ull : kWaitNs;
 }
 
-// S levels x BN columns of tensor memory: 5 x 48 (two CTAs per SM), 6 x 64, 7 x 48, 8 x 48
+// S levels x BN columns of tensor memory: 5 x 48 (two tiles), 6 x 64, 7 x 48, 8 x 48
 int oz_bn(int S) { return S == 6 ? 64 : 48; }
 
 void oz_gemm(const OzOperand& A, const OzOperand& B, double* C, int64_t ldc, int trans, double alpha, int tri, int sym,
@@ -1282,12 +1398,12 @@ void oz_gemm(const OzOperand& A, const OzOperand& B, double* C, int64_t ldc, int
   P.wait_ns = oz_wait_limit();
   P.ntm = A.nrt;
   P.ntn = B.nrt;
-  // Persistent CTAs pay off where a tile's epilogue is long against its
-  // main loop: the exact 8-digit epilogue over short K.  Measured on
-  // 131072 x 48 x 512 (8 digits): 291 -> 213 us; with 5 digits (two CTAs
-  // per SM already overlap their epilogues) and on split or triangular
-  // products one CTA per tile is faster.
-  const bool persistent = A.S >= 7 && P.splits == 1 && !P.sym && P.tri == 0 && P.nkt * kBK <= 4096;
+  // Persistent CTAs pay off where a tile's epilogue is long against its main
+  // loop (it then runs under the next tile's): with 5 digits, and with the exact
+  // epilogues over short K (131072 x 48 x 512, 8 digits: 291 -> 213 us); long,
+  // split or triangular exact products are faster with one CTA per tile, balanced
+  // by the hardware scheduler.
+  const bool persistent = A.S == 5 || (A.S >= 7 && P.splits == 1 && !P.sym && P.tri == 0 && P.nkt * kBK <= 4096);
   if (A.S == 5)
     launch_oz<5, 48>(P, persistent, s);
   else if (A.S == 8)
