@@ -42,36 +42,48 @@ __device__ __forceinline__ DF df_mul(DF x, DF y) {
 __device__ __forceinline__ DF df_half(DF x) { return {__fmul_rn(0.5f, x.hi), __fmul_rn(0.5f, x.lo)}; }
 
 
-// Conversions between FP64 and double-float with integer operations, so that
-// they stay off the narrow FP64 unit.  hi is x's significand rounded to 24
+// Conversions between FP64 and double-float with integer and FP32 operations, so
+// that they stay off the narrow FP64 unit.  hi is x's significand rounded to 24
 // bits (the round bit added into the exponent|significand field carries
 // correctly); lo = x - hi is the signed remainder of the low 29 bits, exact in
-// FP64 and rounded once to FP32.  Values whose hi or lo would leave FP32's
-// normal range (|x| < 2^-73 or > 2^126, zeros) take the FP64 route.
+// FP64 and rounded once to FP32.  Below 2^-73 lo, and below 2^-126 hi, run
+// into FP32's subnormals (both reached through a second power of two); only
+// values above 2^125 take the FP64 route.
 __device__ __forceinline__ DF df_from_double(double x) {
   const uint64_t b = uint64_t(__double_as_longlong(x));
   const int E = int((b >> 52) & 0x7FF);
-  if (E < 950 || E > 1148) {
+  if (E > 1148) {
     const float hi = __double2float_rn(x);
     return {hi, __double2float_rn(x - double(hi))};
   }
   const uint32_t sign = uint32_t(b >> 32) & 0x80000000u;
+  if (E < 897) {  // |x| < 2^-126
+    const float m = __uint_as_float(0x3F800000u | (uint32_t(b >> 29) & 0x7FFFFFu));
+    const float hi = E > 860 ? __fmul_rn(__fmul_rn(m, 0x1p-100f), __uint_as_float(uint32_t(E - 796) << 23)) : 0.0f;
+    return {__uint_as_float(__float_as_uint(hi) | sign), 0.0f};
+  }
   const uint32_t m29 = uint32_t(b) & 0x1FFFFFFFu;
   const uint32_t up = m29 >> 28;
   const uint32_t hb = ((uint32_t(E - 896) << 23) | (uint32_t(b >> 29) & 0x7FFFFFu)) + up;
-  const float scale = __uint_as_float(uint32_t(E - 948) << 23);  // 2^(E - 1075)
-  const float lo = __int2float_rn(int(m29) - int(up << 29)) * scale;
+  const int q = E >= 950 ? 0 : 100;  // 2^(E - 1075), in two factors below 2^-125
+  float lo = __int2float_rn(int(m29) - int(up << 29)) * __uint_as_float(uint32_t(E - 948 + q) << 23);
+  if (q) lo = __fmul_rn(lo, 0x1p-100f);
   return {__uint_as_float(hb | sign), sign ? -lo : lo};
 }
 
-// FP32 value as FP64 bits (exact; zeros, subnormals and non-finite values
-// take the conversion instruction)
+// FP32 value as FP64 bits, exact
 __device__ __forceinline__ double f32_to_f64(float f) {
-  const uint32_t b = __float_as_uint(f);
+  const uint32_t b = __float_as_uint(f), m = b & 0x7FFFFFu;
   const uint32_t ef = (b >> 23) & 0xFFu;
-  if (ef == 0u || ef == 0xFFu) return double(f);
-  const uint64_t bits = (uint64_t(b & 0x80000000u) << 32) | (uint64_t(ef + 896u) << 52) | (uint64_t(b & 0x7FFFFFu) << 29);
-  return __longlong_as_double((long long)bits);
+  const uint64_t sign = uint64_t(b & 0x80000000u) << 32;
+  uint64_t bits = (uint64_t(ef + 896u) << 52) | (uint64_t(m) << 29);
+  if (ef == 0u) {  // zero, or a subnormal: m 2^-149
+    const int lz = __clz(int(m));
+    bits = m ? (uint64_t(905u - uint32_t(lz)) << 52) + ((uint64_t(m) << (lz + 21)) & 0xFFFFFFFFFFFFFull) : 0ull;
+  } else if (ef == 0xFFu) {
+    bits = (0x7FFull << 52) | (uint64_t(m) << 29);
+  }
+  return __longlong_as_double((long long)(sign | bits));
 }
 __device__ __forceinline__ double df_to_double(DF x) { return f32_to_f64(x.hi) + f32_to_f64(x.lo); }
 
