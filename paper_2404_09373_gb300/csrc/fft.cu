@@ -402,10 +402,18 @@ isdf_status rfft3_df(Plan* p, const double* f, int nx, int ny, int nz, int64_t b
   }
   float4* dtw = nullptr;
   isdf_status st;
-  if ((st = dalloc_t(p, &dtw, tw.size() / 4, "transform twiddles"))) return st;
+  const auto release = [&] { p ? dfree(dtw) : scratch_free(dtw, s); };
+  if (p) {
+    if ((st = dalloc_t(p, &dtw, tw.size() / 4, "transform twiddles"))) return st;
+  } else {
+    const cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&dtw), sizeof(float) * tw.size(), s);
+    if (e != cudaSuccess)
+      return fail(p, e == cudaErrorMemoryAllocation ? ISDF_ERR_OOM : ISDF_ERR_CUDA,
+                  std::string("transform twiddles: ") + cudaGetErrorString(e));
+  }
   if ((st = cuda_check(p, cudaMemcpyAsync(dtw, tw.data(), sizeof(float) * tw.size(), cudaMemcpyHostToDevice, s),
                        "twiddle copy"))) {
-    dfree(dtw);
+    release();
     return st;
   }
   float4* io = reinterpret_cast<float4*>(S);
@@ -461,7 +469,7 @@ isdf_status rfft3_df(Plan* p, const double* f, int nx, int ny, int nz, int64_t b
   R.io = io;
   R.out64 = S;
   launch(R);
-  dfree(dtw);
+  release();
   return ISDF_OK;
 }
 

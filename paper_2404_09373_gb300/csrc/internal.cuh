@@ -160,6 +160,9 @@ inline isdf_status dalloc_t(Plan* p, T** ptr, size_t n, const char* what) {
   return dalloc(p, reinterpret_cast<void**>(ptr), n * sizeof(T), what);
 }
 void dfree(void* ptr);
+// scratch of a call without a plan, ordered on stream s (refused under capture)
+cudaError_t scratch_alloc(void** ptr, size_t bytes, cudaStream_t s);
+void scratch_free(void* ptr, cudaStream_t s);
 bool is_device_ptr(const void* ptr);
 
 // ---- kernels / stages ----
@@ -280,12 +283,16 @@ void oz_set_rows(const OzColumnJob* jobs, int nlev, int smax, const int* scount,
                  cudaStream_t s);
 void oz_columns(const OzColumnJob* jobs, int nlev, const int* scount, int* err, cudaStream_t s);
 int64_t oz_tile_elems(int64_t rows, int64_t K, int rt, int S);
-// the same product with its scratch in a fixed static device array (no allocation)
 // split-K factor of a product shape: cached, else timed on these operands
 // (outside graph capture; ISDF_NO_AUTOTUNE keeps the heuristic)
 int oz_tuned_splits(Plan* p, const OzOperand& A, const OzOperand& B, double* C, int64_t ldc, int trans, int sym,
                     int heuristic, cudaStream_t s);
 std::string oz_tune_json();
+// the stand-alone product (both operands sliced by the call) on pooled scratch,
+// and with its scratch in a fixed static device array (no allocation)
+isdf_status gemm_alloc(const double* A, const double* B, double* C, int64_t M, int64_t N, int64_t K, int64_t lda,
+                       int64_t ldb, int64_t ldc, double alpha, int slices, int splits, cudaStream_t s,
+                       std::string& why);
 size_t gemm_noalloc_capacity();
 isdf_status gemm_noalloc(const double* A, const double* B, double* C, int64_t M, int64_t N, int64_t K, int64_t lda,
                          int64_t ldb, int64_t ldc, double alpha, int slices, cudaStream_t s, std::string& why);

@@ -1567,11 +1567,11 @@ std::string oz_tune_json() {
   return o + "]";
 }
 
-// ---------------------------------------------------------------- fixed scratch
+// ------------------------------------------------------- stand-alone products
 //
-// The variant below runs the same slicing and GEMM kernels, but its scratch
-// lives in one file-scope device array instead of memory from cudaMalloc.
-// Every GPU that loads the library holds this array until the process exits.
+// gemm_alloc takes its scratch from the pool of the calls without a plan;
+// gemm_noalloc runs the same kernels on one file-scope device array, which
+// every GPU that loads the library holds until the process exits.
 
 constexpr size_t kStaticScratchBytes = size_t(32) << 20;
 static __device__ __align__(256) unsigned char g_gemm_static_scratch[kStaticScratchBytes];
@@ -1583,7 +1583,85 @@ void* g_static_addr[kMaxDevices] = {nullptr};
 
 size_t round256(size_t b) { return (b + 255) & ~size_t(255); }
 
+// Where a stand-alone product keeps its operands in one block of scratch.
+struct GemmScratch {
+  OzOperand a, b;
+  size_t a_exps, b_tiles, b_exps, err, work, bytes;
+  GemmScratch(int64_t M, int64_t N, int64_t K, int slices, int splits) {
+    a.rows = M, a.rt = 128, b.rows = N, b.rt = oz_bn(slices);
+    for (OzOperand* o : {&a, &b})
+      o->K = K, o->S = slices, o->nrt = (o->rows + o->rt - 1) / o->rt, o->nkt = o->kst = (K + kBK - 1) / kBK;
+    a_exps = round256(size_t(oz_tile_elems(M, K, a.rt, slices)) * 2);
+    b_tiles = a_exps + round256(sizeof(int) * size_t(a.nrt * a.rt));
+    b_exps = b_tiles + round256(size_t(oz_tile_elems(N, K, b.rt, slices)) * 2);
+    err = b_exps + round256(sizeof(int) * size_t(b.nrt * b.rt));
+    work = err + 256;
+    bytes = work + (splits > 1 ? sizeof(double) * size_t(splits) * M * N : 0);
+  }
+  // the arrays from base on; the error word is to be cleared by the caller
+  void place(unsigned char* base) {
+    a.tiles = base, a.exps = reinterpret_cast<int*>(base + a_exps);
+    b.tiles = base + b_tiles, b.exps = reinterpret_cast<int*>(base + b_exps);
+  }
+};
+
+// The product on scratch at base; `name` is the entry point, for messages.
+isdf_status gemm_on(GemmScratch& g, unsigned char* base, const double* A, const double* B, double* C, int64_t lda,
+                    int64_t ldb, int64_t ldc, double alpha, int splits, cudaStream_t s, const char* name,
+                    std::string& why) {
+  g.place(base);
+  int* err = reinterpret_cast<int*>(base + g.err);
+  // the block keeps an earlier call's contents: the error word must start at
+  // zero; every slice byte and every scale read below is rewritten first.
+  // Clear any stale launch error so the check after the launches sees ours.
+  cudaGetLastError();
+  if (cudaMemsetAsync(err, 0, sizeof(int), s) != cudaSuccess) {
+    cudaGetLastError();
+    why = std::string(name) + ": cudaMemsetAsync of the error word failed";
+    return ISDF_ERR_CUDA;
+  }
+  oz_slice(A, lda, 1, nullptr, 1.0, g.a, s);
+  oz_slice(B, ldb, 1, nullptr, 1.0, g.b, s);
+  oz_gemm(g.a, g.b, C, ldc, 0, alpha, 0, 0, splits, splits > 1 ? reinterpret_cast<double*>(base + g.work) : nullptr, err,
+          s);
+  // a launch that could not start (configuration, resources) is reported here
+  // and nowhere else: the copy below would succeed with C unwritten
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) {
+    why = std::string(name) + ": launch failed: " + cudaGetErrorString(e);
+    return ISDF_ERR_CUDA;
+  }
+  int herr = 0;
+  e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) {
+    why = std::string(name) + ": " + cudaGetErrorString(e);
+    return ISDF_ERR_CUDA;
+  }
+  if (herr) {
+    why = std::string(name) + ": tensor-core pipeline wait expired (code " + std::to_string(herr) + ")";
+    return ISDF_ERR_TIMEOUT;
+  }
+  return ISDF_OK;
+}
+
 }  // namespace
+
+isdf_status gemm_alloc(const double* A, const double* B, double* C, int64_t M, int64_t N, int64_t K, int64_t lda,
+                       int64_t ldb, int64_t ldc, double alpha, int slices, int splits, cudaStream_t s,
+                       std::string& why) {
+  GemmScratch g(M, N, K, slices, splits);
+  void* base = nullptr;
+  const cudaError_t e = scratch_alloc(&base, g.bytes, s);
+  if (e != cudaSuccess) {
+    why = std::string("isdf_gemm_f64: allocation failed: ") + cudaGetErrorString(e);
+    return e == cudaErrorMemoryAllocation ? ISDF_ERR_OOM : ISDF_ERR_CUDA;
+  }
+  const isdf_status st = gemm_on(g, static_cast<unsigned char*>(base), A, B, C, lda, ldb, ldc, alpha, splits, s,
+                                 "isdf_gemm_f64", why);
+  scratch_free(base, s);
+  return st;
+}
 
 size_t gemm_noalloc_capacity() { return kStaticScratchBytes; }
 
@@ -1621,55 +1699,13 @@ isdf_status gemm_noalloc(const double* A, const double* B, double* C, int64_t M,
     }
     base = static_cast<unsigned char*>(g_static_addr[dev]);
   }
-  OzOperand a, b;
-  a.rows = M, a.K = K, a.rt = 128, a.S = slices, a.nrt = (M + 127) / 128, a.nkt = (K + kBK - 1) / kBK, a.kst = a.nkt;
-  b.rows = N, b.K = K, b.rt = oz_bn(slices), b.S = slices, b.nrt = (N + b.rt - 1) / b.rt, b.nkt = a.nkt, b.kst = b.nkt;
-  const size_t ta = round256(size_t(oz_tile_elems(M, K, a.rt, slices)) * 2);
-  const size_t ea = round256(sizeof(int) * size_t(a.nrt * a.rt));
-  const size_t tb = round256(size_t(oz_tile_elems(N, K, b.rt, slices)) * 2);
-  const size_t eb = round256(sizeof(int) * size_t(b.nrt * b.rt));
-  const size_t need = ta + ea + tb + eb + 256;
-  if (need > kStaticScratchBytes) {
-    why = "isdf_gemm_f64_noalloc needs " + std::to_string(need) + " bytes of scratch; the static array holds " +
+  GemmScratch g(M, N, K, slices, 1);
+  if (g.bytes > kStaticScratchBytes) {
+    why = "isdf_gemm_f64_noalloc needs " + std::to_string(g.bytes) + " bytes of scratch; the static array holds " +
           std::to_string(kStaticScratchBytes);
     return ISDF_ERR_ARG;
   }
-  a.tiles = base;
-  a.exps = reinterpret_cast<int*>(base + ta);
-  b.tiles = base + ta + ea;
-  b.exps = reinterpret_cast<int*>(base + ta + ea + tb);
-  int* err = reinterpret_cast<int*>(base + ta + ea + tb + eb);
-  // the array keeps the previous call's contents: the error word must start at
-  // zero; every slice byte and every scale read below is rewritten first.
-  // Clear any stale launch error so the check after the launches sees ours.
-  cudaGetLastError();
-  if (cudaMemsetAsync(err, 0, sizeof(int), s) != cudaSuccess) {
-    cudaGetLastError();
-    why = "cudaMemsetAsync of the error word failed";
-    return ISDF_ERR_CUDA;
-  }
-  oz_slice(A, lda, 1, nullptr, 1.0, a, s);
-  oz_slice(B, ldb, 1, nullptr, 1.0, b, s);
-  oz_gemm(a, b, C, ldc, 0, alpha, 0, 0, 1, nullptr, err, s);
-  // a launch that could not start (configuration, resources) is reported here
-  // and nowhere else: the copy below would succeed with C unwritten
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) {
-    why = std::string("isdf_gemm_f64_noalloc: launch failed: ") + cudaGetErrorString(e);
-    return ISDF_ERR_CUDA;
-  }
-  int herr = 0;
-  e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) {
-    why = std::string("isdf_gemm_f64_noalloc: ") + cudaGetErrorString(e);
-    return ISDF_ERR_CUDA;
-  }
-  if (herr) {
-    why = "isdf_gemm_f64_noalloc: tensor-core pipeline wait expired (code " + std::to_string(herr) + ")";
-    return ISDF_ERR_TIMEOUT;
-  }
-  return ISDF_OK;
+  return gemm_on(g, base, A, B, C, lda, ldb, ldc, alpha, 1, s, "isdf_gemm_f64_noalloc", why);
 }
 
 }  // namespace isdf
