@@ -247,11 +247,12 @@ __device__ __forceinline__ void fft_first(const FftPass& P, float4* buf, const f
       const RealPair q = real_pair(P, l0 + li);
       const double* fa = P.in_real + q.line * P.lsi + n2;
       const bool two = q.two;
+      // all loads before the first conversion, whose branches would part them
+      double vr[R1], vi[R1];
 #pragma unroll
-      for (int t = 0; t < R1; ++t) {
-        a[t].re = df_from_double(fa[t * R2]);
-        a[t].im = two ? df_from_double(fa[P.lsi + t * R2]) : DF{0.0f, 0.0f};
-      }
+      for (int t = 0; t < R1; ++t) vr[t] = fa[t * R2], vi[t] = two ? fa[P.lsi + t * R2] : 0.0;
+#pragma unroll
+      for (int t = 0; t < R1; ++t) a[t].re = df_from_double(vr[t]), a[t].im = df_from_double(vi[t]);
     } else {
       const float4* x = P.io + line_base(P, l0 + li) + n2 * P.es;
       const int64_t step = R2 * P.es;
