@@ -33,26 +33,74 @@ __global__ void k_add(int64_t n, const double* __restrict__ a, const double* __r
   if (e < n) c[e] = a[e] + b[e];
 }
 
-// R_GG and R_LL hold their lower triangles only (symmetric GEMMs).
-__global__ void k_build_w(int64_t nip, const double* __restrict__ V, const double* __restrict__ rgg,
-                          const double* __restrict__ rgl, const double* __restrict__ rll, double* __restrict__ W) {
-  const int64_t n2 = 2 * nip;
-  const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (e >= n2 * n2) return;
-  const int64_t P = e / n2, Q = e % n2;
-  const int bp = P >= nip, bq = Q >= nip;
-  const int64_t p = P - bp * nip, q = Q - bq * nip;
-  const int64_t hi = p > q ? p : q, lo = p > q ? q : p;
-  double r;
-  if (!bp && !bq)
-    r = rgg[hi * nip + lo];
-  else if (!bp && bq)
-    r = rgl[p * nip + q];
-  else if (bp && !bq)
-    r = rgl[q * nip + p];
-  else
-    r = rll[hi * nip + lo];
-  W[e] = V[p * nip + q] * r;
+// W from V and the R products.  R_GG and R_LL hold their lower triangles only
+// (symmetric products), R_LG is R_GL^T: one block takes a 32 x 32 tile (ti, tj),
+// ti >= tj, of the pivots and its mirror image, reads the R tiles once, row by
+// row, and turns them in shared memory.  keys (nullable): the largest magnitude
+// of every row of W, as bits, for its digit planes.  Bound by memory and by the
+// FP64 unit's one product a value (0.12 ms of issue at nip = 4160).  There: one
+// thread per value read half of R along columns, 0.32 ms, and the row maxima
+// were another pass of 0.29 ms; now 0.28 ms for both.
+constexpr int kWTile = 32;
+__global__ void __launch_bounds__(256) k_build_w(int64_t nip, const double* __restrict__ V, const double* __restrict__ rgg,
+                                                 const double* __restrict__ rgl, const double* __restrict__ rll,
+                                                 double* __restrict__ W, unsigned long long* __restrict__ keys) {
+  __shared__ double gg[kWTile][kWTile + 1], ll[kWTile][kWTile + 1], gl[kWTile][kWTile + 1], lg[kWTile][kWTile + 1];
+  // tile pair of this block: ti (ti + 1) / 2 + tj
+  const int64_t b = blockIdx.x;
+  int64_t ti = int64_t((sqrt(8.0f * float(b) + 1.0f) - 1.0f) * 0.5f);
+  while (ti * (ti + 1) / 2 > b) --ti;
+  while ((ti + 1) * (ti + 2) / 2 <= b) ++ti;
+  const int64_t tj = b - ti * (ti + 1) / 2, n2 = 2 * nip;
+  const int c = threadIdx.x & 31, r0 = threadIdx.x >> 5;
+  const bool diag = ti == tj;
+#pragma unroll
+  for (int u = 0; u < kWTile; u += 8) {
+    const int r = r0 + u;
+    const int64_t p = ti * kWTile + r, q = tj * kWTile + c;          // R_*[p][q]
+    const int64_t pt = tj * kWTile + r, qt = ti * kWTile + c;        // the mirror image's rows
+    const bool in = p < nip && q < nip, low = in && p >= q;
+    gg[r][c] = low ? rgg[p * nip + q] : 0.0;
+    ll[r][c] = low ? rll[p * nip + q] : 0.0;
+    gl[r][c] = in ? rgl[p * nip + q] : 0.0;
+    lg[r][c] = pt < nip && qt < nip ? rgl[pt * nip + qt] : 0.0;
+  }
+  __syncthreads();
+  auto put = [&](int64_t p, int64_t q, double vgg, double vgl, double vlg, double vll) {
+    unsigned long long mg = 0ull, ml = 0ull;
+    if (p < nip && q < nip) {
+      const double v = V[p * nip + q];
+      const double a = v * vgg, d = v * vgl, e = v * vlg, f = v * vll;
+      W[p * n2 + q] = a;
+      W[p * n2 + nip + q] = d;
+      W[(nip + p) * n2 + q] = e;
+      W[(nip + p) * n2 + nip + q] = f;
+      auto bits = [](double x) { return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull; };
+      mg = max(bits(a), bits(d)), ml = max(bits(e), bits(f));
+    }
+    if (!keys) return;
+    auto top = [](unsigned long long k) {  // a warp's largest key, by halves
+      const unsigned hi = unsigned(k >> 32), h = __reduce_max_sync(0xffffffffu, hi);
+      const unsigned l = __reduce_max_sync(0xffffffffu, hi == h ? unsigned(k) : 0u);
+      return (unsigned long long)h << 32 | l;
+    };
+    mg = top(mg), ml = top(ml);
+    if (c == 0 && p < nip) {
+      if (mg) atomicMax(keys + p, mg);
+      if (ml) atomicMax(keys + nip + p, ml);
+    }
+  };
+#pragma unroll
+  for (int u = 0; u < kWTile; u += 8) {
+    const int r = r0 + u, h = diag && c > r ? c : r, l = diag && c > r ? r : c;
+    put(ti * kWTile + r, tj * kWTile + c, gg[h][l], gl[r][c], lg[c][r], ll[h][l]);
+  }
+  if (!diag)
+#pragma unroll
+    for (int u = 0; u < kWTile; u += 8) {
+      const int r = r0 + u;
+      put(tj * kWTile + r, ti * kWTile + c, gg[c][r], lg[r][c], gl[c][r], ll[c][r]);
+    }
 }
 
 // [X^L | X^N] as one N x 2nip matrix
@@ -87,6 +135,14 @@ __global__ void k_scatter_rows(int64_t rows, int64_t cols, const int* __restrict
   if (e >= rows * cols) return;
   const int64_t i = e / cols, c = e % cols;
   out[int64_t(perm[i]) * cols + c] = in[e];
+}
+
+// out[perm[i]][perm[j]] = in[i][j]
+__global__ void k_scatter_both(int64_t n, const int* __restrict__ perm, const double* __restrict__ in,
+                               double* __restrict__ out) {
+  const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (e >= n * n) return;
+  out[int64_t(perm[e / n]) * n + perm[e % n]] = in[e];
 }
 
 // partial[b] = sum over this block's slice of C o KC (FP64)
@@ -137,27 +193,30 @@ GemmArgs gemm(int ta, int tb, int64_t M, int64_t N, int64_t K, const double* A, 
 }
 
 // C (M x N) = A_rows B_rows^T on the tensor cores; A given as rows x K with
-// element (r, k) at a[r*sar + k*sak], B likewise.
+// element (r, k) at a[r*sar + k*sak], B likewise.  ready: the digits of A, if
+// the caller has them (freed here).  The launches are only queued: an expired
+// wait makes the later products return at once and is reported by oz_check.
 isdf_status tc_product(Plan* p, const double* a, int64_t M, int64_t sar, int64_t sak, const double* b, int64_t N,
-                       int64_t sbr, int64_t sbk, int64_t K, double* C, int64_t ldc, int sym) {
+                       int64_t sbr, int64_t sbk, int64_t K, double* C, int64_t ldc, int sym,
+                       const OzWindows* win = nullptr, OzOperand* ready = nullptr) {
   cudaStream_t s = p->stream;
   const int S = 5;
   OzOperand A, B;
   double* work = nullptr;
-  isdf_status st;
-  if ((st = oz_alloc(p, A, M, K, 128, S, "exchange slices")) || (st = oz_alloc(p, B, N, K, oz_bn(S), S, "exchange slices")))
-    return oz_free(A), oz_free(B), st;
-  oz_slice(a, sar, sak, nullptr, 1.0, A, s);
+  isdf_status st = ISDF_OK;
+  if (ready) A = *ready, *ready = OzOperand{};
+  else st = oz_alloc(p, A, M, K, 128, S, "exchange slices");
+  if (st || (st = oz_alloc(p, B, N, K, oz_bn(S), S, "exchange slices"))) return oz_free(A), oz_free(B), st;
+  if (a) oz_slice(a, sar, sak, nullptr, 1.0, A, s);
   oz_slice(b, sbr, sbk, nullptr, 1.0, B, s);
   int64_t tiles = A.nrt * B.nrt;
   int64_t splits = std::max<int64_t>(1, std::min<int64_t>((2 * 152 + tiles - 1) / tiles, A.nkt / 32 + 1));
   splits = std::min<int64_t>(splits, 16);
-  splits = oz_tuned_splits(p, A, B, C, ldc, 0, sym, int(splits), s);
+  splits = oz_tuned_splits(p, A, B, C, ldc, 0, sym, int(splits), s, win);
   if (splits > 1 && (st = dalloc_t(p, &work, size_t(splits) * M * N, "split-k partials")))
     return oz_free(A), oz_free(B), st;
-  oz_gemm(A, B, C, ldc, 0, 1.0, 0, sym, int(splits), work, p->d_ozerr, s);
-  // under graph capture the error word is read after the graph has run
-  st = p->capturing ? cuda_check(p, cudaGetLastError(), "tensor-core launch") : oz_check(p);
+  oz_gemm(A, B, C, ldc, 0, 1.0, 0, sym, int(splits), work, p->d_ozerr, s, win);
+  st = cuda_check(p, cudaGetLastError(), "tensor-core launch");
   oz_free(A);
   oz_free(B);
   dfree(work);
@@ -168,7 +227,9 @@ isdf_status tc_product(Plan* p, const double* a, int64_t M, int64_t sar, int64_t
 
 isdf_status tc_product_ex(Plan* p, const double* a, int64_t M, int64_t sar, int64_t sak, const double* b, int64_t N,
                         int64_t sbr, int64_t sbk, int64_t K, double* C, int64_t ldc) {
-  return tc_product(p, a, M, sar, sak, b, N, sbr, sbk, K, C, ldc, 0);
+  const isdf_status st = tc_product(p, a, M, sar, sak, b, N, sbr, sbk, K, C, ldc, 0);
+  // under graph capture the error word is read after the graph has run
+  return st || p->capturing ? st : oz_check(p);
 }
 
 namespace {
@@ -242,9 +303,11 @@ isdf_status exchange_run(Plan* p, const double* dC, int n, double* dK, double* d
   const int nlev = p->nlev;
   double *y2 = nullptr, *yg = nullptr, *rgg = nullptr, *rgl = nullptr, *rll = nullptr, *W = nullptr, *x2 = nullptr,
          *T = nullptr, *kc = nullptr, *kcp = nullptr, *cp = nullptr, *xlp = nullptr, *xnp = nullptr, *u = nullptr,
-         *tmp = nullptr, *part = nullptr, *dex = nullptr;
+         *kp = nullptr, *tmp = nullptr, *part = nullptr, *dex = nullptr;
+  OzOperand wd;  // the digits of W
   auto cleanup = [&]() {
-    for (double* q : {y2, yg, rgg, rgl, rll, W, x2, T, kc, kcp, cp, xlp, xnp, u, tmp, part, dex}) dfree(q);
+    for (double* q : {y2, yg, rgg, rgl, rll, W, x2, T, kp, kc, kcp, cp, xlp, xnp, u, tmp, part, dex}) dfree(q);
+    oz_free(wd);
   };
   isdf_status st;
   if (!p->d_perm) {
@@ -269,7 +332,12 @@ isdf_status exchange_run(Plan* p, const double* dC, int n, double* dK, double* d
     cleanup();
     return st;
   }
-  if (dK && ((st = dalloc_t(p, &x2, size_t(N) * n2, "[X^L X^N]")) || (st = dalloc_t(p, &T, size_t(n2) * N, "W X^T")))) {
+  if (dK && ((st = dalloc_t(p, &x2, size_t(N) * n2, "[X^L X^N]")) || (st = dalloc_t(p, &T, size_t(n2) * N, "W X^T")) ||
+             (st = dalloc_t(p, &kp, size_t(N) * N, "K by level")))) {
+    cleanup();
+    return st;
+  }
+  if (p->opt.precision == 1 && (st = oz_alloc(p, wd, n2, n2, 128, 5, "exchange slices"))) {
     cleanup();
     return st;
   }
@@ -280,14 +348,15 @@ isdf_status exchange_run(Plan* p, const double* dC, int n, double* dK, double* d
   double* yl = y2;
   double* yn = y2 + nip * n;
   // nonzero (function level x pivot level) blocks: X^L on (F_l, P_l), X^N on (F_>l, P_l)
-  double fl_y = 0.0, fl_kc = 0.0;
+  double fl_y = 0.0, fl_kc = 0.0, nzx = 0.0;  // nzx: elements of [X^L X^N] inside its nonzero blocks
   for (int l = 0; l < nlev; ++l) {
     const double k = p->lev[l].k, fL = lo.fb[l + 1] - lo.fb[l], fN = lo.fb[nlev] - lo.fb[l + 1];
     fl_y += 2.0 * k * n * (fL + fN);
     fl_kc += 2.0 * fL * n * (k + p->poff[l]);
+    nzx += fL * (k + p->poff[l]);
   }
   const double fl_r = 2.0 * nip * (nip + 1) * n * 2.0 + 2.0 * nip * nip * n;
-  const double fl = fl_y + fl_r + (dK ? 2.0 * n2 * n2 * N + 2.0 * N * N * n2 + 2.0 * N * N * n : 2.0 * n2 * n2 * n + fl_kc);
+  const double fl = fl_y + fl_r + (dK ? 2.0 * (n2 + N) * (p->opt.precision == 1 ? nzx : double(N) * n2) + 2.0 * N * N * n : 2.0 * n2 * n2 * n + fl_kc);
   {
     Prof pr(p, "exchange", fl, "flop", kLaunchesInside);
     k_gather_rows<<<unsigned((N * n + 255) / 256), 256, 0, s>>>(N, n, dperm, dC, cp);
@@ -323,22 +392,44 @@ isdf_status exchange_run(Plan* p, const double* dC, int n, double* dK, double* d
       dgemm(gemm(0, 1, nip, nip, n, yg, n, yl, n, rgl, nip), s);
       dgemm(gemm(0, 1, nip, nip, n, yl, n, yl, n, rll, nip, 1), s);
     }
-    k_build_w<<<unsigned((n2 * n2 + 255) / 256), 256, 0, s>>>(nip, p->V, rgg, rgl, rll, W);
-    count_launches(1);
+    {
+      const int64_t wt = (nip + kWTile - 1) / kWTile;
+      k_build_w<<<unsigned(wt * (wt + 1) / 2), 256, 0, s>>>(nip, p->V, rgg, rgl, rll, W,
+                                                           wd.tiles ? oz_keys_begin(wd, s) : nullptr);
+      count_launches(1);
+      if (wd.tiles) oz_slice_keyed(W, n2, wd, s);
+    }
     if (dK) {
-      k_concat<<<unsigned((N * n2 + 255) / 256), 256, 0, s>>>(N, nip, p->XL, p->XN, x2);
+      k_concat<<<unsigned((N * n2 + 255) / 256), 256, 0, s>>>(N, nip, xlp, xnp, x2);
       count_launches(1);
       if (p->opt.precision == 1) {
-        // T = W X2^T (rows of W against rows of X2), K = X2 T (rows of X2 against columns of T)
-        if ((st = tc_product(p, W, n2, n2, 1, x2, N, n2, 1, n2, T, N, 0)) ||
-            (st = tc_product(p, x2, N, n2, 1, T, N, 1, N, n2, dK, N, 0))) {
+        // T = W X2^T (rows of W against rows of X2), K = X2 T (rows of X2
+        // against columns of T), over the k tiles of X2's nonzero blocks only:
+        // about a third of the dense products on three levels (nip = 4160, 832
+        // functions: all products of a build 1.60 -> 1.12 ms)
+        OzWindows win;
+        win.n = nlev;
+        for (int l = 0; l < nlev; ++l) {
+          win.row[l] = lo.fb[l], win.row[l + 1] = lo.fb[l + 1];
+          win.lo[l][0] = p->poff[l], win.hi[l][0] = p->poff[l] + p->lev[l].k;
+          win.lo[l][1] = nip;
+          win.hi[l][1] = nip + (l == 0 && p->opt.local_grids ? p->poff[1] : p->poff[l]);
+        }
+        if ((st = tc_product(p, nullptr, n2, n2, 1, x2, N, n2, 1, n2, T, N, 0, &win, &wd))) {
+          cleanup();
+          return st;
+        }
+        win.side = 1;
+        if ((st = tc_product(p, x2, N, n2, 1, T, N, 1, N, n2, kp, N, 0, &win))) {
           cleanup();
           return st;
         }
       } else {
         dgemm(gemm(0, 1, n2, N, n2, W, n2, x2, n2, T, N), s);  // T = W X2^T
-        dgemm(gemm(0, 0, N, N, n2, x2, n2, T, N, dK, N), s);   // K = X2 T
+        dgemm(gemm(0, 0, N, N, n2, x2, n2, T, N, kp, N), s);   // K = X2 T
       }
+      k_scatter_both<<<unsigned((N * N + 255) / 256), 256, 0, s>>>(N, dperm, kp, dK);
+      count_launches(1);
       // the universal sinc grid's terms: K_FU + K_FU^T + K_UU
       if (p->opt.coarse_sinc && (st = sinc_exchange(p, dC, yl, yg, n, dK))) {
         cleanup();
@@ -355,7 +446,9 @@ isdf_status exchange_run(Plan* p, const double* dC, int n, double* dK, double* d
       if (dKC) cudaMemcpyAsync(dKC, kc, sizeof(double) * size_t(N) * n, cudaMemcpyDeviceToDevice, s);
     } else {
       // U = W [Y_L; Y_N]: rows of W against the columns i of Y2
-      if ((st = block_product(p, W, n2, n2, 1, y2, n, 1, n, n2, u, n, false, tmp))) {
+      if (p->opt.precision == 1) st = tc_product(p, nullptr, n2, n2, 1, y2, n, 1, n, n2, u, n, 0, nullptr, &wd);
+      else dgemm(gemm(0, 0, n2, n, n2, W, n2, y2, n, u, n), s);
+      if (st) {
         cleanup();
         return st;
       }

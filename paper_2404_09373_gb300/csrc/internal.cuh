@@ -264,8 +264,24 @@ void oz_slice_ex(const double* src, int64_t sr, int64_t sk, const int* ridx, OzO
 // C = alpha * A B^T (A: M x K as the 128-row side, B: N x K); trans: C[n*ldc+m];
 // tri 1/2: B-side lower/upper triangular in (n, k); sym: lower-triangle tiles only;
 // splits > 1 needs work of splits*M*N doubles.  Error codes go to *err.
+// win: k ranges outside of which an operand's rows are zero (nullptr: none known).
+struct OzWindows;
 void oz_gemm(const OzOperand& A, const OzOperand& B, double* C, int64_t ldc, int trans, double alpha, int tri, int sym,
-             int splits, double* work, int* err, cudaStream_t s);
+             int splits, double* work, int* err, cudaStream_t s, const OzWindows* win = nullptr);
+// Groups of rows of one operand (side 0: B's, 1: A's), row[g] .. row[g + 1], each
+// nonzero only for k in [lo[g][i], hi[g][i]), i = 0, 1, the first range before the
+// second.  A tile runs over the k tiles that any of its groups needs.
+struct OzWindows {
+  int n = 0;  // groups
+  int side = 0;
+  int64_t row[ISDF_MAX_LEVELS + 1] = {0};
+  int64_t lo[ISDF_MAX_LEVELS][2] = {{0}}, hi[ISDF_MAX_LEVELS][2] = {{0}};
+};
+// Rows' scales from the keys (bits of the largest magnitudes) that another kernel
+// has gathered in oz_keys_begin's array, then the digits of the whole operand
+// (k adjacent, rows sr apart).
+unsigned long long* oz_keys_begin(OzOperand& op, cudaStream_t s);
+void oz_slice_keyed(const double* src, int64_t sr, OzOperand& op, cudaStream_t s);
 // One level of a selection block's columns (ozgemm.cu): products q = 0 (own
 // functions), 1 (coarser functions), 2 (factor columns), each absent if its
 // operand is null or has no k tiles.  C[j][t] (j a member of the set, ld M).
@@ -286,7 +302,7 @@ int64_t oz_tile_elems(int64_t rows, int64_t K, int rt, int S);
 // split-K factor of a product shape: cached, else timed on these operands
 // (outside graph capture; ISDF_NO_AUTOTUNE keeps the heuristic)
 int oz_tuned_splits(Plan* p, const OzOperand& A, const OzOperand& B, double* C, int64_t ldc, int trans, int sym,
-                    int heuristic, cudaStream_t s);
+                    int heuristic, cudaStream_t s, const OzWindows* win = nullptr);
 std::string oz_tune_json();
 // the stand-alone product (both operands sliced by the call) on pooled scratch,
 // and with its scratch in a fixed static device array (no allocation)

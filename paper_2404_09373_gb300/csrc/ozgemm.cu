@@ -550,6 +550,7 @@ struct OzGemmParams {
   double* work;  // split-K partials [z][M][N]
   int* err;
   unsigned long long wait_ns;  // limit of each pipeline wait (device time)
+  OzWindows win;
 };
 
 template <int S, int BN>
@@ -735,7 +736,8 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, 1) k_oz_gemm(OzGemmPara
   // and a tile's epilogue overlaps the next tile's copies and MMAs.
   const int64_t NT = (P.ntn + Cfg::pair - 1) / Cfg::pair, MT = P.ntm, ntiles = NT * MT * P.splits;
   struct Tile {
-    int64_t nt, mt, m0, n0, kt_lo, nk;
+    int64_t nt, mt, m0, n0, kt_lo, nk;  // steps [kt_lo, kt_lo + nk) of the k tiles k_tile()
+    int64_t n1, base1, base2;           // steps below n1 are k tiles from base1 on, the others from base2 on
     int z, tiles;  // tiles: N tiles of this pair
     bool skip;
   };
@@ -752,6 +754,25 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, 1) k_oz_gemm(OzGemmPara
     int64_t lo = 0, hi = P.nkt;
     if (P.tri == 1) hi = min(P.nkt, (T.n0 + Cfg::pair * BN + kBK - 1) / kBK);
     if (P.tri == 2) lo = min(P.nkt, T.n0 / kBK);
+    T.n1 = hi, T.base1 = T.base2 = 0;
+    if (P.win.n) {
+      const int64_t r0 = P.win.side ? T.m0 : T.n0, r1 = r0 + (P.win.side ? kBM : Cfg::pair * BN);
+      int64_t a[2] = {P.nkt, P.nkt}, b[2] = {0, 0};  // k tiles of the two ranges
+#pragma unroll
+      for (int g = 0; g < ISDF_MAX_LEVELS; ++g)
+        if (g < P.win.n && P.win.row[g] < r1 && P.win.row[g + 1] > r0)
+#pragma unroll
+          for (int i = 0; i < 2; ++i)
+            if (P.win.hi[g][i] > P.win.lo[g][i]) {
+              a[i] = min(a[i], P.win.lo[g][i] / kBK);
+              b[i] = max(b[i], min(P.nkt, (P.win.hi[g][i] + kBK - 1) / kBK));
+            }
+      a[1] = max(a[1], b[0]);  // a k tile that holds the end of one and the start of the other
+      T.n1 = max(b[0] - a[0], int64_t(0));
+      T.base1 = a[0];
+      T.base2 = a[1] - T.n1;
+      hi = T.n1 + max(b[1] - a[1], int64_t(0));
+    }
     const int64_t tot = hi - lo, per = (tot + P.splits - 1) / P.splits;
     const int64_t a = lo + per * T.z;
     T.kt_lo = min(hi, a);
@@ -798,7 +819,7 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, 1) k_oz_gemm(OzGemmPara
             break;
           }
           if (*(volatile int*)abort_flag) break;
-          const int64_t kt = T.kt_lo + it;
+          const int64_t step = T.kt_lo + it, kt = step + (step < T.n1 ? T.base1 : T.base2);
           unsigned char* sA = smem + st * Cfg::stage;
           unsigned char* sB = sA + Cfg::stageA;
           mbar_expect_tx(&full[st], Cfg::stageA + T.tiles * Cfg::stageB);
@@ -1341,6 +1362,19 @@ void oz_slice(const double* src, int64_t sr, int64_t sk, const double* kw, doubl
   slice_operand(slice_args(src, sr, sk, kw, mul, nullptr, op, 0, op.nkt * (kBK / 8)), op.S, s);
 }
 
+unsigned long long* oz_keys_begin(OzOperand& op, cudaStream_t s) {
+  cudaMemsetAsync(op.tiles, 0, sizeof(unsigned long long) * size_t(op.rows), s);
+  return static_cast<unsigned long long*>(op.tiles);
+}
+
+void oz_slice_keyed(const double* src, int64_t sr, OzOperand& op, cudaStream_t s) {
+  const OzSliceArgs A = slice_args(src, sr, 1, nullptr, 1.0, nullptr, op, 0, op.nkt * (kBK / 8));
+  k_oz_key_exps<<<unsigned((op.rows + 255) / 256), 256, 0, s>>>(static_cast<unsigned long long*>(op.tiles), op.rows,
+                                                                op.exps);
+  count_launches(1);
+  launch_digits(A, op.S, s);
+}
+
 void oz_retile(const OzOperand& from, OzOperand& to, cudaStream_t s) {
   const int64_t rows_pad = to.nrt * to.rt;
   const int64_t units = (rows_pad / 8) * to.nkt * to.S;
@@ -1375,8 +1409,9 @@ static unsigned long long oz_wait_limit() {
 int oz_bn(int S) { return S == 6 ? 64 : 48; }
 
 void oz_gemm(const OzOperand& A, const OzOperand& B, double* C, int64_t ldc, int trans, double alpha, int tri, int sym,
-             int splits, double* work, int* err, cudaStream_t s) {
+             int splits, double* work, int* err, cudaStream_t s, const OzWindows* win) {
   OzGemmParams P;
+  if (win) P.win = *win;
   P.A = static_cast<const __nv_bfloat16*>(A.tiles);
   P.B = static_cast<const __nv_bfloat16*>(B.tiles);
   P.ea = A.exps;
@@ -1507,8 +1542,8 @@ std::map<TuneKey, std::pair<int, float>> g_tune;  // shape -> (splits, ms)
 }  // namespace
 
 int oz_tuned_splits(Plan* p, const OzOperand& A, const OzOperand& B, double* C, int64_t ldc, int trans, int sym,
-                    int heuristic, cudaStream_t s) {
-  const TuneKey key{A.rows, B.rows, A.nkt, A.S, sym, trans};
+                    int heuristic, cudaStream_t s, const OzWindows* win) {
+  const TuneKey key{A.rows, B.rows, A.nkt, A.S, sym | (win ? 2 << win->side : 0), trans};
   {
     std::lock_guard<std::mutex> lock(g_tune_mu);
     auto it = g_tune.find(key);
@@ -1536,7 +1571,7 @@ int oz_tuned_splits(Plan* p, const OzOperand& A, const OzOperand& B, double* C, 
     float ms = 1e30f;
     for (int rep = (c == cand.front() ? 0 : 1); rep < 2; ++rep) {  // one warm-up run before the first candidate
       cudaEventRecord(e0, s);
-      oz_gemm(A, B, C, ldc, trans, 1.0, 0, sym, c, work, err, s);
+      oz_gemm(A, B, C, ldc, trans, 1.0, 0, sym, c, work, err, s, win);
       cudaEventRecord(e1, s);
       cudaEventSynchronize(e1);
       float t = 0.0f;
@@ -1545,10 +1580,13 @@ int oz_tuned_splits(Plan* p, const OzOperand& A, const OzOperand& B, double* C, 
     if (work) cudaFreeAsync(work, s);
     if (ms < best_ms) best_ms = ms, best = c;
   }
+  int herr = 0;  // after an expired wait the products return at once: no times to keep
+  if (err) cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s);
   cudaStreamSynchronize(s);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   cudaGetLastError();
+  if (herr) return heuristic;
   std::lock_guard<std::mutex> lock(g_tune_mu);
   g_tune[key] = {best, best_ms};
   return best;
@@ -1561,7 +1599,7 @@ std::string oz_tune_json() {
     if (o.size() > 1) o += ",";
     o += "{\"M\":" + std::to_string(kv.first.M) + ",\"N\":" + std::to_string(kv.first.N) +
          ",\"k_tiles\":" + std::to_string(kv.first.nkt) + ",\"digits\":" + std::to_string(kv.first.S) +
-         ",\"sym\":" + std::to_string(kv.first.sym) + ",\"splits\":" + std::to_string(kv.second.first) +
+         ",\"sym\":" + std::to_string(kv.first.sym & 1) + ",\"splits\":" + std::to_string(kv.second.first) +
          ",\"ms\":" + std::to_string(kv.second.second) + "}";
   }
   return o + "]";
