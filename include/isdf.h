@@ -298,8 +298,9 @@ void isdf_exchange_graph_destroy(isdf_exchange_graph_t graph);
 
 /* Split-K autotuner of the tensor-core products (the launch shape the
  * library picks by measurement; not in the paper): the first product of a
- * shape outside any graph capture times every admissible split-K factor on
- * its own operands (CUDA events) and keeps the fastest for the process
+ * shape outside any graph capture that takes less than about 0.3 ms times every
+ * admissible split-K factor on its own operands (CUDA events) and keeps the
+ * fastest for the process; longer products follow a rule on their sizes
  * (setting ISDF_NO_AUTOTUNE in the environment keeps the built-in
  * heuristic).  This returns the table so far as JSON text, one object per
  * shape {M, N, k_tiles, digits, sym, splits, ms}; valid until the next call

@@ -157,24 +157,25 @@ isdf_status coulomb_block_tc(Plan* p, const double2* left, const Level& la, cons
   double* work = nullptr;
   isdf_status st;
   if ((st = oz_alloc(p, a, la.k, K2, 128, S, "Coulomb slices")) ||
-      (st = oz_alloc(p, b, lb.k, K2, oz_bn(S), S, "Coulomb slices"))) {
+      (!same && (st = oz_alloc(p, b, lb.k, K2, oz_bn(S), S, "Coulomb slices")))) {
     oz_free(a), oz_free(b);
     return st;
   }
   {
     // FP64 read twice (row scales, digits), S BF16 digits written per value
-    Prof pr(p, "coulomb_slice", double(la.k + lb.k) * double(K2) * (16.0 + 2.0 * S), "byte", 4);
+    Prof pr(p, "coulomb_slice", double(la.k + (same ? 0 : lb.k)) * double(K2) * (16.0 + 2.0 * S), "byte", 4);
     oz_slice(reinterpret_cast<const double*>(left), K2, 1, wt2, 1.0, a, s);
-    if (same)
-      oz_retile(a, b, s);  // same spectra and weights: B's digits are A's, re-tiled
-    else
-      oz_slice(reinterpret_cast<const double*>(lb.spec), K2, 1, wt2, 1.0, b, s);
+    if (!same) oz_slice(reinterpret_cast<const double*>(lb.spec), K2, 1, wt2, 1.0, b, s);
   }
-  int64_t tiles = a.nrt * b.nrt;
+  // same spectra and weights: B's digits are A's, read from A's tiles (a copy of
+  // them in B's tiles took 10 of the 2x2x2 diamond workload's 207 ms, against 4
+  // that its products lose to the smaller copies)
+  const OzOperand& rhs = same ? a : b;
+  int64_t tiles = a.nrt * ((lb.k + oz_bn(S) - 1) / oz_bn(S));
   if (same) tiles = (tiles + a.nrt) / 2;
   int64_t splits = (4 * 152 + tiles - 1) / tiles;
   splits = std::max<int64_t>(1, std::min<int64_t>(splits, std::min<int64_t>(64, a.nkt / 64 + 1)));
-  splits = oz_tuned_splits(p, a, b, Cblk, p->nip, 0, same ? 1 : 0, int(splits), s);
+  splits = oz_tuned_splits(p, a, rhs, Cblk, p->nip, 0, same ? 1 : 0, int(splits), s);
   if (splits > 1 && (st = dalloc_t(p, &work, size_t(splits) * la.k * lb.k, "split-k partials"))) {
     oz_free(a), oz_free(b);
     return st;
@@ -182,7 +183,7 @@ isdf_status coulomb_block_tc(Plan* p, const double2* left, const Level& la, cons
   {
     const double work_fl = same ? double(la.k) * double(la.k + 1) * double(K2) : 2.0 * la.k * double(lb.k) * K2;
     Prof pr(p, "coulomb_V", work_fl, "flop", kLaunchesInside);
-    oz_gemm(a, b, Cblk, p->nip, 0, 1.0, 0, same ? 1 : 0, int(splits), work, p->d_ozerr, s);
+    oz_gemm(a, rhs, Cblk, p->nip, 0, 1.0, 0, same ? 1 : 0, int(splits), work, p->d_ozerr, s);
   }
   st = oz_check(p);
   oz_free(a);
@@ -204,9 +205,9 @@ isdf_status apply_w(Plan* p) {
   const int64_t nip = p->nip;
   double* W[ISDF_MAX_LEVELS] = {nullptr, nullptr, nullptr, nullptr};
   double* T = nullptr;
-  OzOperand a, b;
+  OzOperand a, b, w[ISDF_MAX_LEVELS];  // w: the digits of W_l, for either side
   auto cleanup = [&]() {
-    for (int l = 0; l < p->nlev; ++l) dfree(W[l]);
+    for (int l = 0; l < p->nlev; ++l) dfree(W[l]), oz_free(w[l]);
     dfree(T);
     oz_free(a);
     oz_free(b);
@@ -235,12 +236,12 @@ isdf_status apply_w(Plan* p) {
   for (int l = 0; l < p->nlev; ++l) {
     const int k = p->lev[l].k;
     if (!k || !p->lev[l].rinv) continue;
-    if ((st = dalloc_t(p, &W[l], size_t(k) * k, "W"))) return cleanup(), st;
+    if ((st = dalloc_t(p, &W[l], size_t(k) * k, "W")) || (st = oz_alloc(p, w[l], k, k, 128, S, "Coulomb transform")))
+      return cleanup(), st;
     view(a, k, k);
-    view(b, k, k);
     oz_slice(p->lev[l].rinv, 1, k, nullptr, 1.0, a, s);
-    oz_slice(p->lev[l].rinv, 1, k, nullptr, 1.0, b, s);
-    oz_gemm(a, b, W[l], k, 0, 1.0, 0, 0, 1, nullptr, p->d_ozerr, s);
+    oz_gemm(a, a, W[l], k, 0, 1.0, 0, 0, 1, nullptr, p->d_ozerr, s);
+    oz_slice(W[l], k, 1, nullptr, 1.0, w[l], s);
   }
   for (int x = 0; x < p->nlev; ++x) {
     const int ka = p->lev[x].k;
@@ -253,21 +254,17 @@ isdf_status apply_w(Plan* p) {
       // T = V_Z,ab W_b   (T[m][n] = sum_j V[m][j] W_b[n][j], W_b symmetric)
       if (W[y]) {
         view(a, ka, kb);
-        view(b, kb, kb);
         oz_slice(blk, nip, 1, nullptr, 1.0, a, s);
-        oz_slice(W[y], kb, 1, nullptr, 1.0, b, s);
-        oz_gemm(a, b, T, kb, 0, 1.0, 0, 0, 1, nullptr, p->d_ozerr, s);
+        oz_gemm(a, w[y], T, kb, 0, 1.0, 0, 0, 1, nullptr, p->d_ozerr, s);
       } else {
         cudaMemcpy2DAsync(T, sizeof(double) * kb, blk, sizeof(double) * nip, sizeof(double) * kb, ka,
                           cudaMemcpyDeviceToDevice, s);
       }
       // V_ab = W_a T   (V[m][n] = sum_i W_a[m][i] T[i][n])
       if (W[x]) {
-        view(a, ka, ka);
         view(b, kb, ka);
-        oz_slice(W[x], ka, 1, nullptr, 1.0, a, s);
         oz_slice(T, 1, kb, nullptr, 1.0, b, s);
-        oz_gemm(a, b, blk, nip, 0, 1.0, 0, 0, 1, nullptr, p->d_ozerr, s);
+        oz_gemm(w[x], b, blk, nip, 0, 1.0, 0, 0, 1, nullptr, p->d_ozerr, s);
       } else {
         cudaMemcpy2DAsync(blk, sizeof(double) * nip, T, sizeof(double) * kb, sizeof(double) * kb, ka,
                           cudaMemcpyDeviceToDevice, s);

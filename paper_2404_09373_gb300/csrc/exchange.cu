@@ -192,34 +192,44 @@ GemmArgs gemm(int ta, int tb, int64_t M, int64_t N, int64_t K, const double* A, 
   return g;
 }
 
-// C (M x N) = A_rows B_rows^T on the tensor cores; A given as rows x K with
-// element (r, k) at a[r*sar + k*sak], B likewise.  ready: the digits of A, if
-// the caller has them (freed here).  The launches are only queued: an expired
-// wait makes the later products return at once and is reported by oz_check.
-isdf_status tc_product(Plan* p, const double* a, int64_t M, int64_t sar, int64_t sak, const double* b, int64_t N,
-                       int64_t sbr, int64_t sbk, int64_t K, double* C, int64_t ldc, int sym,
-                       const OzWindows* win = nullptr, OzOperand* ready = nullptr) {
+constexpr int kXS = 5;  // digits of the exchange's products
+
+// Digits of rows of K values, element (r, k) at a[r*sr + k*sk]; tile: row-tile
+// height (128: either side of a product, oz_bn: the right one only).
+isdf_status tc_slice(Plan* p, OzOperand& op, const double* a, int64_t rows, int64_t sr, int64_t sk, int64_t K, int tile) {
+  const isdf_status st = oz_alloc(p, op, rows, K, tile, kXS, "exchange slices");
+  if (!st) oz_slice(a, sr, sk, nullptr, 1.0, op, p->stream);
+  return st;
+}
+
+// C = A B^T of sliced operands.  The launches are only queued: an expired wait
+// makes the later products return at once and is reported by oz_check.
+isdf_status tc_multiply(Plan* p, const OzOperand& A, const OzOperand& B, double* C, int64_t ldc, int sym,
+                        const OzWindows* win = nullptr) {
   cudaStream_t s = p->stream;
-  const int S = 5;
-  OzOperand A, B;
   double* work = nullptr;
-  isdf_status st = ISDF_OK;
-  if (ready) A = *ready, *ready = OzOperand{};
-  else st = oz_alloc(p, A, M, K, 128, S, "exchange slices");
-  if (st || (st = oz_alloc(p, B, N, K, oz_bn(S), S, "exchange slices"))) return oz_free(A), oz_free(B), st;
-  if (a) oz_slice(a, sar, sak, nullptr, 1.0, A, s);
-  oz_slice(b, sbr, sbk, nullptr, 1.0, B, s);
-  int64_t tiles = A.nrt * B.nrt;
+  isdf_status st;
+  int64_t tiles = A.nrt * ((B.rows + oz_bn(kXS) - 1) / oz_bn(kXS));
   int64_t splits = std::max<int64_t>(1, std::min<int64_t>((2 * 152 + tiles - 1) / tiles, A.nkt / 32 + 1));
   splits = std::min<int64_t>(splits, 16);
   splits = oz_tuned_splits(p, A, B, C, ldc, 0, sym, int(splits), s, win);
-  if (splits > 1 && (st = dalloc_t(p, &work, size_t(splits) * M * N, "split-k partials")))
-    return oz_free(A), oz_free(B), st;
+  if (splits > 1 && (st = dalloc_t(p, &work, size_t(splits) * A.rows * B.rows, "split-k partials"))) return st;
   oz_gemm(A, B, C, ldc, 0, 1.0, 0, sym, int(splits), work, p->d_ozerr, s, win);
   st = cuda_check(p, cudaGetLastError(), "tensor-core launch");
+  dfree(work);
+  return st;
+}
+
+// C (M x N) = A_rows B_rows^T on the tensor cores; A given as rows x K with
+// element (r, k) at a[r*sar + k*sak], B likewise.
+isdf_status tc_product(Plan* p, const double* a, int64_t M, int64_t sar, int64_t sak, const double* b, int64_t N,
+                       int64_t sbr, int64_t sbk, int64_t K, double* C, int64_t ldc) {
+  OzOperand A, B;
+  isdf_status st;
+  if (!(st = tc_slice(p, A, a, M, sar, sak, K, 128)) && !(st = tc_slice(p, B, b, N, sbr, sbk, K, oz_bn(kXS))))
+    st = tc_multiply(p, A, B, C, ldc, 0);
   oz_free(A);
   oz_free(B);
-  dfree(work);
   return st;
 }
 
@@ -227,7 +237,7 @@ isdf_status tc_product(Plan* p, const double* a, int64_t M, int64_t sar, int64_t
 
 isdf_status tc_product_ex(Plan* p, const double* a, int64_t M, int64_t sar, int64_t sak, const double* b, int64_t N,
                         int64_t sbr, int64_t sbk, int64_t K, double* C, int64_t ldc) {
-  const isdf_status st = tc_product(p, a, M, sar, sak, b, N, sbr, sbk, K, C, ldc, 0);
+  const isdf_status st = tc_product(p, a, M, sar, sak, b, N, sbr, sbk, K, C, ldc);
   // under graph capture the error word is read after the graph has run
   return st || p->capturing ? st : oz_check(p);
 }
@@ -247,8 +257,8 @@ isdf_status block_product(Plan* p, const double* a, int64_t M, int64_t sar, int6
     return ISDF_OK;
   }
   if (p->opt.precision == 1) {
-    if (!accumulate) return tc_product(p, a, M, sar, sak, b, N, sbr, sbk, K, C, ldc, 0);
-    isdf_status st = tc_product(p, a, M, sar, sak, b, N, sbr, sbk, K, tmp, N, 0);
+    if (!accumulate) return tc_product(p, a, M, sar, sak, b, N, sbr, sbk, K, C, ldc);
+    isdf_status st = tc_product(p, a, M, sar, sak, b, N, sbr, sbk, K, tmp, N);
     if (st) return st;
     k_add2d<<<unsigned((M * N + 255) / 256), 256, 0, s>>>(M, N, tmp, C, ldc);
     count_launches(1);
@@ -304,10 +314,10 @@ isdf_status exchange_run(Plan* p, const double* dC, int n, double* dK, double* d
   double *y2 = nullptr, *yg = nullptr, *rgg = nullptr, *rgl = nullptr, *rll = nullptr, *W = nullptr, *x2 = nullptr,
          *T = nullptr, *kc = nullptr, *kcp = nullptr, *cp = nullptr, *xlp = nullptr, *xnp = nullptr, *u = nullptr,
          *kp = nullptr, *tmp = nullptr, *part = nullptr, *dex = nullptr;
-  OzOperand wd;  // the digits of W
+  OzOperand wd, od[2];  // the digits of W, of the other operands
   auto cleanup = [&]() {
     for (double* q : {y2, yg, rgg, rgl, rll, W, x2, T, kp, kc, kcp, cp, xlp, xnp, u, tmp, part, dex}) dfree(q);
-    oz_free(wd);
+    for (OzOperand* o : {&wd, &od[0], &od[1]}) oz_free(*o);
   };
   isdf_status st;
   if (!p->d_perm) {
@@ -337,7 +347,7 @@ isdf_status exchange_run(Plan* p, const double* dC, int n, double* dK, double* d
     cleanup();
     return st;
   }
-  if (p->opt.precision == 1 && (st = oz_alloc(p, wd, n2, n2, 128, 5, "exchange slices"))) {
+  if (p->opt.precision == 1 && (st = oz_alloc(p, wd, n2, n2, 128, kXS, "exchange slices"))) {
     cleanup();
     return st;
   }
@@ -381,12 +391,13 @@ isdf_status exchange_run(Plan* p, const double* dC, int n, double* dK, double* d
     k_add<<<unsigned((nip * n + 255) / 256), 256, 0, s>>>(nip * n, yl, yn, yg);
     count_launches(1);
     if (p->opt.precision == 1) {
-      if ((st = tc_product(p, yg, nip, n, 1, yg, nip, n, 1, n, rgg, nip, 1)) ||
-          (st = tc_product(p, yg, nip, n, 1, yl, nip, n, 1, n, rgl, nip, 0)) ||
-          (st = tc_product(p, yl, nip, n, 1, yl, nip, n, 1, n, rll, nip, 1))) {
+      if ((st = tc_slice(p, od[0], yg, nip, n, 1, n, 128)) || (st = tc_slice(p, od[1], yl, nip, n, 1, n, 128)) ||
+          (st = tc_multiply(p, od[0], od[0], rgg, nip, 1)) || (st = tc_multiply(p, od[0], od[1], rgl, nip, 0)) ||
+          (st = tc_multiply(p, od[1], od[1], rll, nip, 1))) {
         cleanup();
         return st;
       }
+      oz_free(od[0]), oz_free(od[1]);
     } else {
       dgemm(gemm(0, 1, nip, nip, n, yg, n, yg, n, rgg, nip, 1), s);
       dgemm(gemm(0, 1, nip, nip, n, yg, n, yl, n, rgl, nip), s);
@@ -415,12 +426,12 @@ isdf_status exchange_run(Plan* p, const double* dC, int n, double* dK, double* d
           win.lo[l][1] = nip;
           win.hi[l][1] = nip + (l == 0 && p->opt.local_grids ? p->poff[1] : p->poff[l]);
         }
-        if ((st = tc_product(p, nullptr, n2, n2, 1, x2, N, n2, 1, n2, T, N, 0, &win, &wd))) {
-          cleanup();
-          return st;
+        if (!(st = tc_slice(p, od[0], x2, N, n2, 1, n2, 128)) && !(st = tc_multiply(p, wd, od[0], T, N, 0, &win)) &&
+            !(st = tc_slice(p, od[1], T, N, 1, N, n2, oz_bn(kXS)))) {
+          win.side = 1;
+          st = tc_multiply(p, od[0], od[1], kp, N, 0, &win);
         }
-        win.side = 1;
-        if ((st = tc_product(p, x2, N, n2, 1, T, N, 1, N, n2, kp, N, 0, &win))) {
+        if (st) {
           cleanup();
           return st;
         }
@@ -436,7 +447,7 @@ isdf_status exchange_run(Plan* p, const double* dC, int n, double* dK, double* d
         return st;
       }
       if (p->opt.precision == 1) {
-        if ((st = tc_product(p, dK, N, N, 1, dC, n, 1, n, N, kc, n, 0))) {  // (K C)[mu][i]
+        if ((st = tc_product(p, dK, N, N, 1, dC, n, 1, n, N, kc, n))) {  // (K C)[mu][i]
           cleanup();
           return st;
         }
@@ -446,8 +457,9 @@ isdf_status exchange_run(Plan* p, const double* dC, int n, double* dK, double* d
       if (dKC) cudaMemcpyAsync(dKC, kc, sizeof(double) * size_t(N) * n, cudaMemcpyDeviceToDevice, s);
     } else {
       // U = W [Y_L; Y_N]: rows of W against the columns i of Y2
-      if (p->opt.precision == 1) st = tc_product(p, nullptr, n2, n2, 1, y2, n, 1, n, n2, u, n, 0, nullptr, &wd);
-      else dgemm(gemm(0, 0, n2, n, n2, W, n2, y2, n, u, n), s);
+      if (p->opt.precision == 1) {
+        if (!(st = tc_slice(p, od[0], y2, n, 1, n, n2, oz_bn(kXS)))) st = tc_multiply(p, wd, od[0], u, n, 0);
+      } else dgemm(gemm(0, 0, n2, n, n2, W, n2, y2, n, u, n), s);
       if (st) {
         cleanup();
         return st;

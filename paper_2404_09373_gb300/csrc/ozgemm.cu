@@ -426,34 +426,6 @@ __global__ void __launch_bounds__(512, 2) k_oz_slice(OzSliceArgs A) {
     oz_emit<S>(A, r, g, e, v);
   }
 }
-
-// Re-tile an operand's digit planes to another row-tile height: rows of 8
-// (one 512-byte line of a slice for 32 k values) move as whole lines, so the
-// digits are copied, not recomputed.  Rows at or beyond the source's real rows
-// are written as zeros (padding).
-__global__ void k_oz_retile(const __nv_bfloat16* __restrict__ src, int src_rt, int64_t src_kst,
-                            __nv_bfloat16* __restrict__ dst, int dst_rt, int64_t dst_kst, int S, int64_t rows,
-                            int64_t rows_pad, int64_t nkt) {
-  const int lane = threadIdx.x & 31;
-  const int64_t units = (rows_pad / 8) * nkt * S;
-  for (int64_t u = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; u < units;
-       u += (int64_t(gridDim.x) * blockDim.x) >> 5) {
-    const int s = int(u % S);
-    const int64_t kt = (u / S) % nkt, g8 = u / (int64_t(S) * nkt);
-    const int64_t r0 = g8 * 8;
-    const int64_t dt = r0 / dst_rt, drg = (r0 % dst_rt) / 8;
-    uint4* out = reinterpret_cast<uint4*>(dst + ((dt * dst_kst + kt) * S + s) * int64_t(dst_rt) * kBK + drg * 8 * kBK);
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (r0 < rows) {
-      const int64_t st = r0 / src_rt, srg = (r0 % src_rt) / 8;
-      const uint4* in =
-          reinterpret_cast<const uint4*>(src + ((st * src_kst + kt) * S + s) * int64_t(src_rt) * kBK + srg * 8 * kBK);
-      v = in[lane];
-    }
-    out[lane] = v;
-  }
-}
-
 OzSliceArgs slice_args(const double* src, int64_t sr, int64_t sk, const double* kw, double mul, const int* ridx,
                        const OzOperand& op, int64_t kg0, int64_t ngrp) {
   return {src, sr, sk, op.rows, op.K, kw, mul, ridx, op.rt, op.nrt, op.kst, kg0, ngrp, op.exps,
@@ -541,6 +513,7 @@ struct OzGemmParams {
   int64_t M, N, nkt;
   int64_t ntm, ntn;    // M tiles (of 128 rows) and N tiles (of BN rows)
   int64_t akst, bkst;  // k-tile strides of the A and B tile arrays (>= nkt)
+  int64_t bgroups;     // 8-row groups of B if its array has 128-row tiles, else 0
   int tri;     // 0 dense; 1 B-side lower (k <= n); 2 B-side upper (k >= n)
   int sym;     // compute only tiles that touch the lower triangle (n <= m)
   int splits;  // split-K factor (gridDim.z)
@@ -822,10 +795,28 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, 1) k_oz_gemm(OzGemmPara
           const int64_t step = T.kt_lo + it, kt = step + (step < T.n1 ? T.base1 : T.base2);
           unsigned char* sA = smem + st * Cfg::stage;
           unsigned char* sB = sA + Cfg::stageA;
-          mbar_expect_tx(&full[st], Cfg::stageA + T.tiles * Cfg::stageB);
+          if (!P.bgroups) {
+            mbar_expect_tx(&full[st], Cfg::stageA + T.tiles * Cfg::stageB);
+            bulk_g2s(sA, gA + (T.mt * P.akst + kt) * int64_t(Cfg::stageA), Cfg::stageA, &full[st]);
+            for (int b = 0; b < T.tiles; ++b)
+              bulk_g2s(sB + b * Cfg::stageB, gB + ((T.nt + b) * P.bkst + kt) * int64_t(Cfg::stageB), Cfg::stageB,
+                       &full[st]);
+            continue;
+          }
+          // B's rows from 128-row tiles: groups of 8 rows (512 bytes a digit) are
+          // contiguous up to the end of a tile, so a digit takes one or two copies.
+          // Groups behind the last tile are left out: their columns are not stored.
+          const int64_t g0 = T.n0 / 8, g1 = min(g0 + T.tiles * (BN / 8), P.bgroups);
+          mbar_expect_tx(&full[st], Cfg::stageA + uint32_t(g1 - g0) * (512 * S));
           bulk_g2s(sA, gA + (T.mt * P.akst + kt) * int64_t(Cfg::stageA), Cfg::stageA, &full[st]);
-          for (int b = 0; b < T.tiles; ++b)
-            bulk_g2s(sB + b * Cfg::stageB, gB + ((T.nt + b) * P.bkst + kt) * int64_t(Cfg::stageB), Cfg::stageB, &full[st]);
+          for (int64_t gb = g0; gb < g1;) {
+            const int in_b = int(gb - g0) % (BN / 8), b = int(gb - g0) / (BN / 8);
+            const int n = int(min(min(int64_t(BN / 8 - in_b), 16 - gb % 16), g1 - gb));
+            const unsigned char* from = gB + ((gb / 16) * P.bkst + kt) * int64_t(Cfg::stageA) + (gb % 16) * 512;
+            unsigned char* to = sB + b * Cfg::stageB + in_b * 512;
+            for (int d = 0; d < S; ++d) bulk_g2s(to + d * Cfg::tileB, from + d * Cfg::tileA, n * 512, &full[st]);
+            gb += n;
+          }
         }
       }
       // copies that were issued but never consumed must land before exit
@@ -1375,17 +1366,6 @@ void oz_slice_keyed(const double* src, int64_t sr, OzOperand& op, cudaStream_t s
   launch_digits(A, op.S, s);
 }
 
-void oz_retile(const OzOperand& from, OzOperand& to, cudaStream_t s) {
-  const int64_t rows_pad = to.nrt * to.rt;
-  const int64_t units = (rows_pad / 8) * to.nkt * to.S;
-  const int64_t blocks = std::min<int64_t>((units * 32 + 255) / 256, 152 * 64);
-  k_oz_retile<<<unsigned(std::max<int64_t>(blocks, 1)), 256, 0, s>>>(
-      static_cast<const __nv_bfloat16*>(from.tiles), from.rt, from.kst, static_cast<__nv_bfloat16*>(to.tiles), to.rt,
-      to.kst, to.S, from.rows, rows_pad, to.nkt);
-  cudaMemcpyAsync(to.exps, from.exps, size_t(to.rows) * sizeof(int), cudaMemcpyDeviceToDevice, s);
-  count_launches(1);
-}
-
 void oz_slice_ex(const double* src, int64_t sr, int64_t sk, const int* ridx, OzOperand& op, int64_t kg0, int64_t kg1,
                  bool exps_ready, cudaStream_t s) {
   if (op.rows <= 0 || kg1 <= kg0) return;
@@ -1421,6 +1401,7 @@ void oz_gemm(const OzOperand& A, const OzOperand& B, double* C, int64_t ldc, int
   P.nkt = A.nkt;
   P.akst = A.kst > 0 ? A.kst : A.nkt;
   P.bkst = B.kst > 0 ? B.kst : B.nkt;
+  P.bgroups = B.rt == oz_bn(B.S) ? 0 : B.nrt * (kBM / 8);
   P.tri = tri;
   P.sym = sym;
   P.splits = splits < 1 ? 1 : splits;
@@ -1432,7 +1413,7 @@ void oz_gemm(const OzOperand& A, const OzOperand& B, double* C, int64_t ldc, int
   P.err = err;
   P.wait_ns = oz_wait_limit();
   P.ntm = A.nrt;
-  P.ntn = B.nrt;
+  P.ntn = (B.rows + oz_bn(B.S) - 1) / oz_bn(B.S);
   // Persistent CTAs pay off where a tile's epilogue is long against its main
   // loop (it then runs under the next tile's): with 5 digits, and with the exact
   // epilogues over short K (131072 x 48 x 512, 8 digits: 291 -> 213 us); long,
@@ -1523,7 +1504,8 @@ void oz_columns(const OzColumnJob* jobs, int nlev, const int* scount, int* err, 
 // The one free launch parameter of a product shape is its split-K factor
 // (how many CTAs share one output tile's k range).  On the first product of
 // a shape (rows of A, rows of B, k tiles, digits, symmetric or not) outside
-// any graph capture, every admissible candidate runs on the real operands
+// any graph capture (products of more than 0.3 ms follow a rule instead, see
+// oz_tuned_splits), every admissible candidate runs on the real operands
 // (one warm-up run, then one timed run per candidate, CUDA events on the
 // product's stream) and the fastest is cached for the process; the heuristic's choice
 // is among the candidates, and the chosen one runs last so C holds its
@@ -1550,6 +1532,35 @@ int oz_tuned_splits(Plan* p, const OzOperand& A, const OzOperand& B, double* C, 
     if (it != g_tune.end()) return it->second.first;
   }
   if ((p && p->capturing) || std::getenv("ISDF_NO_AUTOTUNE")) return heuristic;
+  // Products of more than 0.3 ms: waves of CTAs decide, which needs no
+  // measurement.  A wave takes its share of k at the measured tensor rate and one
+  // epilogue, the last one is three quarters idle on average, and the partial
+  // results are written and read once.  (Timing the Coulomb matrix of the 2x2x2
+  // diamond cell with every split took 0.7 s of its first pass.  1657 x 1657 x
+  // 903168, 7 digits, symmetric: 64.9 ms with one split, 56.5 with 3, 56.4 with 8,
+  // 55.6 with 16, the rule's choice, 54.6 with 32.)
+  {
+    const int bn = oz_bn(A.S) * (A.S == 5 ? 2 : 1);
+    const int64_t mt = (A.rows + kBM - 1) / kBM, nt = (B.rows + bn - 1) / bn;
+    int64_t tiles = mt * nt;
+    if (sym) {
+      tiles = 0;
+      for (int64_t i = 0; i < mt; ++i) tiles += std::min(nt, (i * kBM + kBM - 1) / bn + 1);
+    }
+    const double step = 2.0 * kBM * bn * kBK * (A.S * (A.S + 1) / 2) / (1.7e15 / 152.0);  // one k tile, seconds
+    if (double(tiles) * double(A.nkt) * step / 152.0 > 3e-4 && !win) {
+      int best = 1;
+      double best_t = 1e30;
+      for (int c : {1, 2, 4, 8, 16, 32, 64}) {
+        if (c > A.nkt) break;
+        const double waves = std::max(1.0, double(tiles) * c / 152.0 + 0.75);
+        const double t = waves * (double((A.nkt + c - 1) / c) * step + 4e-6) +
+                         (c > 1 ? 16.0 * c * double(A.rows) * double(B.rows) / 6e12 : 0.0);
+        if (t < 0.99 * best_t) best_t = t, best = c;
+      }
+      return best;
+    }
+  }
   std::vector<int> cand;
   for (int c : {1, 2, 4, 8, 16, 32, 64})
     if (c <= std::max<int64_t>(1, A.nkt)) cand.push_back(c);
