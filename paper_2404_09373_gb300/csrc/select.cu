@@ -1,15 +1,16 @@
 // Interpolation-point selection (kernel family (b)): greedy pivoted Cholesky on
 // the block-diagonal matrix (+)_l w_l M_l (Section II.A, Eq. 2).
 //
-// The loop stays on the device: each step is four kernels that read and write
+// The loop stays on the device: each step is two kernels that read and write
 // a small state record, so the pivot index never travels to the host.
-//   k_sel_max    d_max = max residual (atomicMax on the bit pattern, d >= 0)
-//   k_sel_first  tie rule: smallest global index with d >= thr (atomicMin)
-//   k_sel_pick   one thread: records the pivot, advances counters, checks the
-//                stop rules and the device-clock time budget
+//   k_sel_first  stop rules; tie rule: smallest global index with d >= thr
+//                (atomicMin); the last block to contribute records the pivot,
+//                advances counters and checks the device-clock time budget
 //   k_sel_col    new factor column on the pivot's level and residual update:
 //                L[g,k] = (w M(g,p) - sum_j L[g,j] L[p,j]) / sqrt(d_p),
-//                d(g) -= L[g,k]^2,  L[p,k] = sqrt(d_p), d(p) = 0
+//                d(g) -= L[g,k]^2,  L[p,k] = sqrt(d_p), d(p) = 0;
+//                and the level's largest residual (atomicMax on the bit
+//                pattern, d >= 0), which k_sel_max finds before the first step
 // Steps are captured once into a CUDA graph and replayed.  No kernel waits on
 // another; there is no spin anywhere.
 //
@@ -33,8 +34,9 @@ namespace isdf {
 namespace {
 
 struct SelState {
-  unsigned long long dmax_bits;
+  unsigned long long lmax[ISDF_MAX_LEVELS];  // largest residual of every level (bits; >= 0)
   unsigned long long first;
+  unsigned int arrived;  // blocks of k_sel_first that have contributed
   double d0;
   double dp;
   long long gp;  // grid index of this step's pivot
@@ -175,20 +177,77 @@ __global__ void k_gather_diag(const double* __restrict__ d0, const int* __restri
   if (t < nc) d[t] = d0[cidx ? cidx[t] : t];
 }
 
+// Largest residual of every level, before the first step; from then on k_sel_col
+// keeps its level's.  blockIdx.y: the level.
 __global__ void k_sel_max(SelParams P, SelState* st) {
   if (st->done) return;
   __shared__ double sh[32];
+  const int l = blockIdx.y;
   double m = 0.0;
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < P.ntot; i += int64_t(gridDim.x) * blockDim.x)
+  for (int64_t i = P.coff[l] + int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < P.coff[l + 1];
+       i += int64_t(gridDim.x) * blockDim.x)
     m = fmax(m, P.d[i]);
   m = block_reduce(m, MaxOp(), sh);
-  if (threadIdx.x == 0) atomicMax(&st->dmax_bits, (unsigned long long)__double_as_longlong(m));
+  if (threadIdx.x == 0 && m > 0.0) atomicMax(&st->lmax[l], (unsigned long long)__double_as_longlong(m));
 }
 
+__device__ __forceinline__ double sel_dmax(const SelState* st) {
+  unsigned long long m = 0ull;
+#pragma unroll
+  for (int l = 0; l < ISDF_MAX_LEVELS; ++l) m = max(m, st->lmax[l]);
+  return __longlong_as_double((long long)m);
+}
+
+// The pivot of the step whose smallest qualifying index is known; one thread.
+__device__ __forceinline__ void sel_pick(const SelParams& P, SelState* st, unsigned long long idx, double dmax) {
+  if (idx == ULLONG_MAX) {  // nothing qualified (cannot happen with dmax > 0)
+    st->done = 1;
+    st->skip = 1;
+    return;
+  }
+  int l = 0;
+  while (l + 1 < P.nlev && (long long)idx >= P.coff[l + 1]) ++l;
+  const long long t = (long long)idx - P.coff[l];
+  const long long g = P.cidx[l] ? P.cidx[l][t] : t;
+  const double dp = P.d[idx];
+  const int k = st->k;
+  if (k == 0) st->d0 = dmax;
+  st->lev = l;
+  st->gp = g;
+  st->tp = t;
+  st->dp = dp;
+  st->col = st->kl[l];
+  P.piv[k] = ((long long)l << kPivShift) | g;
+  P.dval[k] = dp;
+  st->kl[l] += 1;
+  st->k = k + 1;
+  st->skip = 0;
+  st->lmax[l] = 0ull;  // k_sel_col puts the level's new one here
+  if (P.timeout_ns) {
+    const unsigned long long now = globaltimer();
+    if (k == 0) {
+      st->t0 = now;
+    } else if (now - st->t0 > P.timeout_ns) {
+      st->err = ISDF_ERR_TIMEOUT;
+      st->done = 1;  // this step's column is still computed
+    }
+  }
+}
+
+// Blocks of the passes over all residuals: one value a thread as far as four blocks an SM go
+unsigned sel_blocks(int64_t ntot, int nsm) {
+  return unsigned(std::max<int64_t>(1, std::min<int64_t>(int64_t(nsm) * 4, (ntot + 255) / 256)));
+}
+
+// The step's pivot: smallest index within the tie window of the largest
+// residual; the last block to contribute records it.  Launches of a few
+// microseconds bound a step of a small cell: with max, first, pick and column as
+// four of them, one cell on a 24^3 grid took 13.9 ms for 312 steps and its fit,
+// now 10.9 ms.
 __global__ void k_sel_first(SelParams P, SelState* st) {
   if (st->done) return;
   __shared__ unsigned long long sh[32];
-  const double dmax = __longlong_as_double((long long)st->dmax_bits);
+  const double dmax = sel_dmax(st);
   const int k = st->k;
   const double d0 = (k == 0) ? dmax : st->d0;
   const bool stop = (k >= P.nip) || !(dmax > 0.0) || (dmax < P.tol * d0);
@@ -210,45 +269,15 @@ __global__ void k_sel_first(SelParams P, SelState* st) {
     }
   }
   best = block_reduce(best, MinOp(), sh);
-  if (threadIdx.x == 0 && best != ULLONG_MAX) atomicMin(&st->first, best);
-}
-
-__global__ void k_sel_pick(SelParams P, SelState* st) {
-  if (threadIdx.x != 0 || st->done) return;
-  const unsigned long long idx = st->first;
-  if (idx == ULLONG_MAX) {  // nothing qualified (cannot happen with dmax > 0)
-    st->done = 1;
-    st->skip = 1;
-    return;
-  }
-  int l = 0;
-  while (l + 1 < P.nlev && (long long)idx >= P.coff[l + 1]) ++l;
-  const long long t = (long long)idx - P.coff[l];
-  const long long g = P.cidx[l] ? P.cidx[l][t] : t;
-  const double dp = P.d[idx];
-  const int k = st->k;
-  if (k == 0) st->d0 = __longlong_as_double((long long)st->dmax_bits);
-  st->lev = l;
-  st->gp = g;
-  st->tp = t;
-  st->dp = dp;
-  st->col = st->kl[l];
-  P.piv[k] = ((long long)l << kPivShift) | g;
-  P.dval[k] = dp;
-  st->kl[l] += 1;
-  st->k = k + 1;
-  st->skip = 0;
-  st->dmax_bits = 0ull;
-  st->first = ULLONG_MAX;
-  if (P.timeout_ns) {
-    const unsigned long long now = globaltimer();
-    if (k == 0) {
-      st->t0 = now;
-    } else if (now - st->t0 > P.timeout_ns) {
-      st->err = ISDF_ERR_TIMEOUT;
-      st->done = 1;  // this step's column is still computed
-    }
-  }
+  if (threadIdx.x != 0) return;
+  if (best != ULLONG_MAX) atomicMin(&st->first, best);
+  __threadfence();
+  if (atomicAdd(&st->arrived, 1u) + 1u < gridDim.x) return;
+  // every other block has read the state and left its index
+  __threadfence();
+  const unsigned long long idx = atomicExch(&st->first, ULLONG_MAX);
+  st->arrived = 0u;
+  sel_pick(P, st, idx, dmax);
 }
 
 // One block works on 32 candidate points at a time (one point per lane, so
@@ -257,7 +286,7 @@ __global__ void k_sel_pick(SelParams P, SelState* st) {
 // in shared memory in a fixed order.  Grid-striding over 32-point groups keeps
 // every SM equally busy whatever the number of candidates.
 constexpr int kColWarps = 8;
-__global__ __launch_bounds__(32 * kColWarps) void k_sel_col(SelParams P, const SelState* st) {
+__global__ __launch_bounds__(32 * kColWarps) void k_sel_col(SelParams P, SelState* st) {
   if (st->skip) return;
   extern __shared__ double sm[];
   const int l = st->lev;
@@ -278,6 +307,7 @@ __global__ __launch_bounds__(32 * kColWarps) void k_sel_col(SelParams P, const S
   const double w = P.w[l];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t ngroups = (nc + 31) / 32;
+  double dmax = 0.0;  // of this lane's candidates, warp 0
   for (int64_t grp = blockIdx.x; grp < ngroups; grp += gridDim.x) {
     const int64_t t = grp * 32 + lane;
     const bool valid = t < nc;
@@ -328,9 +358,15 @@ __global__ __launch_bounds__(32 * kColWarps) void k_sel_col(SelParams P, const S
       double v = (m - s) / sq;
       if (t == tp) v = sq;
       fac[int64_t(col) * nc + t] = v;
-      d[t] = (t == tp) ? 0.0 : d[t] - v * v;
+      const double left = (t == tp) ? 0.0 : d[t] - v * v;
+      d[t] = left;
+      dmax = fmax(dmax, left);
     }
     __syncthreads();
+  }
+  if (warp == 0) {
+    for (int o = 16; o > 0; o >>= 1) dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
+    if (lane == 0 && dmax > 0.0) atomicMax(&st->lmax[l], (unsigned long long)__double_as_longlong(dmax));
   }
 }
 
@@ -617,8 +653,9 @@ __global__ void k_step_begin(SelState* st) {
   if (threadIdx.x != 0) return;
   st->done = st->final_ ? 1 : 0;
   st->skip = 1;
-  st->dmax_bits = 0ull;
+  for (int l = 0; l < ISDF_MAX_LEVELS; ++l) st->lmax[l] = 0ull;
   st->first = ULLONG_MAX;
+  st->arrived = 0u;
 }
 
 // Largest of a warp's 64-bit keys: two 32-bit warp reductions.
@@ -975,7 +1012,6 @@ isdf_status select_loop(Plan* p, int nip, double tol, const double* d0full, int*
   P.tie_abs = p->opt.tie_abs;
   P.timeout_ns = (unsigned long long)p->opt.timeout_ms * 1000000ull;
   SelState h{};
-  h.dmax_bits = 0;
   h.first = ULLONG_MAX;
   h.skip = 1;
   if ((st = cuda_check(p, cudaMemcpyAsync(p->d_selstate, &h, sizeof(h), cudaMemcpyHostToDevice, s), "state init")))
@@ -992,18 +1028,18 @@ isdf_status select_loop(Plan* p, int nip, double tol, const double* d0full, int*
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sel_col, 32 * kColWarps, smem);
-  const unsigned red_blocks = unsigned(nsm) * 4;
+  const unsigned red_blocks = sel_blocks(P.ntot, nsm);
   const unsigned col_blocks = per_sm > 0 ? unsigned(per_sm * nsm) : kColBlocks;
+  k_sel_max<<<dim3(red_blocks, unsigned(P.nlev)), 256, 0, s>>>(P, dst);
+  count_launches(1);
   auto one_step = [&]() {
-    k_sel_max<<<red_blocks, 256, 0, s>>>(P, dst);
     k_sel_first<<<red_blocks, 256, 0, s>>>(P, dst);
-    k_sel_pick<<<1, 32, 0, s>>>(P, dst);
     k_sel_col<<<col_blocks, 256, smem, s>>>(P, dst);
   };
   // Capture a chunk of steps into a graph (not possible on the legacy stream).
   const int chunk = 32;
   bool graphed = false;
-  Prof* loop_prof = new Prof(p, "select_loop", 0.0, "flop", 4ll * nip);
+  Prof* loop_prof = new Prof(p, "select_loop", 0.0, "flop", 2ll * nip);
   if (s != nullptr && nip >= chunk) {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -1240,7 +1276,6 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
   TopSOut O{sidx, sg, stp, scount};
 
   SelState h{};
-  h.dmax_bits = 0;
   h.first = ULLONG_MAX;
   h.skip = 1;
   if ((st = cuda_check(p, cudaMemcpyAsync(p->d_selstate, &h, sizeof(h), cudaMemcpyHostToDevice, s), "state init")))
@@ -1255,7 +1290,7 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sel_col, 32 * kColWarps, smem);
-  const unsigned red_blocks = unsigned(nsm) * 4;
+  const unsigned red_blocks = sel_blocks(P.ntot, nsm);
   const unsigned col_blocks = per_sm > 0 ? unsigned(per_sm * nsm) : kColBlocks;
   // ---- exact compaction of the candidates below tau (see above)
   int64_t since_compact = 0;
@@ -1522,13 +1557,12 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
     }
     if (taken == 0) {
       // the greedy pivot was not in S: one ordinary step
-      Prof pr(p, "select_loop", 0.0, "flop", 4);
+      Prof pr(p, "select_loop", 0.0, "flop", 3);
       k_step_begin<<<1, 32, 0, s>>>(dst);
-      k_sel_max<<<red_blocks, 256, 0, s>>>(P, dst);
+      k_sel_max<<<dim3(red_blocks, unsigned(P.nlev)), 256, 0, s>>>(P, dst);
       k_sel_first<<<red_blocks, 256, 0, s>>>(P, dst);
-      k_sel_pick<<<1, 32, 0, s>>>(P, dst);
       k_sel_col<<<col_blocks, 256, smem, s>>>(P, dst);
-      count_launches(5);
+      count_launches(4);
       ++nplain;
       cudaMemcpyAsync(&h, dst, sizeof(h), cudaMemcpyDeviceToHost, s);
       if ((st = cuda_check(p, cudaStreamSynchronize(s), "plain step"))) return bail(st);
