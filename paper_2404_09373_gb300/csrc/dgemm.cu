@@ -349,8 +349,8 @@ void dgemm(const GemmArgs& g, cudaStream_t s) {
   const int64_t tm = (g.M + BT - 1) / BT, tn = (g.N + BT - 1) / BT;
   // Few tiles over a long k (the V blocks and exchange projections of a small
   // cell) leave most SMs idle: share the k range over enough CTAs for about four
-  // per SM, at least 128 k values each.  140 x 140 x 15000: 9 CTAs, 6.9 ms ->
-  // 0.14 ms.
+  // per SM, at least 128 k values each.  The Coulomb block of a cell's 24^3 grid (about
+  // 150 x 150 x 14976) has 25 tiles: 0.61 ms as 1025 CTAs.
   const int64_t tiles = g.sym ? tm * (tm + 1) / 2 : tm * tn;
   const int64_t splits = std::max<int64_t>(1, std::min<int64_t>({(608 + tiles - 1) / tiles, g.K / 128, 64}));
   double* work = nullptr;

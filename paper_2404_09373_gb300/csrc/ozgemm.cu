@@ -970,10 +970,12 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, 1) k_oz_gemm(OzGemmPara
 // ten launches a block (three per level and the combination), each too short to
 // fill the chip on a small cell (18 us of fill and epilogue), and moved every
 // result through memory four more times: columns of a block on one cell 290 ->
-// 163 us, on 2x2x2 2.01 -> 1.76 ms, and one launch instead of up to 21 for the
-// digits of the set's rows.
-// Bound: the candidates' digit stream (16 bytes a value) from HBM; persistent
-// CTAs, one per SM, the levels in order (the longest k ranges first).
+// 163 us, on 2x2x2 2.01 -> 1.76 ms (99 us and 1.57 ms with integer sums and two
+// issuing warps), and one launch instead of up to 21 for the digits of the set's
+// rows.
+// Bound: the tensor cores (0.75 of their measured rate for two N tiles a level)
+// and the candidates' digit stream (16 bytes a value) from HBM; persistent CTAs,
+// one per SM, the levels in order (the longest k ranges first).
 struct OzColSeg {
   const __nv_bfloat16 *A, *B;
   const int *ea, *eb;

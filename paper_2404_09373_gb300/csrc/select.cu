@@ -389,8 +389,8 @@ __global__ __launch_bounds__(32 * kColWarps) void k_sel_col(SelParams P, SelStat
 // candidates' residuals with the same tie rule; k_blk_commit takes them over.
 // No step waits for the whole chip: three launches serve up to s steps, where
 // a cooperative launch with two grid barriers per step took 13 us a step on one
-// cell and 20 us on the 2x2x2 workload.  Per block: one cell 182 -> 75 us, 2x2x2
-// 860 -> 400 us, the digits of the new columns included.
+// cell and 20 us on the 2x2x2 workload.  Per block: one cell 182 -> 94 us, 2x2x2
+// 860 -> 434 us, the digits of the new columns included.
 
 constexpr int kMaxSet = 256;  // options.select_block's limit
 
