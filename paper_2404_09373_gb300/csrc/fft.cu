@@ -26,7 +26,7 @@
 // 12), 22 of them per complex addition.  The former passes (four in-place stages
 // of radix 4, 4, 2, 3 through shared memory) spent as many again on addresses, and
 // their conversions sent zeros and tiny values through the FP64 unit (60 % of
-// its time in the x pass).  96 vectors of 96^3: 4.00 -> 1.77 ms a call (0.62 ms
+// its time in the x pass).  96 vectors of 96^3: 4.00 -> 1.79 ms a call (0.62 ms
 // is the memory traffic of three passes at the copy rate); the Coulomb matrices
 // of a 1 x 1 x 2 cell with three grids: 3.5 -> 1.95 ms of transforms.
 #include <cmath>
