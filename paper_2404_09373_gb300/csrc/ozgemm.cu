@@ -121,6 +121,13 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t phase, const i
   return __all_sync(0xffffffffu, mbar_wait(bar, phase, err, wait_ns)) != 0;
 }
 
+// The CTA's abort flag, one answer for the whole warp: lanes that read it at
+// different times would part, and some of them then sit without a limit in a
+// warp-wide instruction (tcgen05.ld, __syncwarp) that the others never reach.
+__device__ __forceinline__ bool warp_aborted(const int* flag) {
+  return __any_sync(0xffffffffu, *(volatile const int*)flag) != 0;
+}
+
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
@@ -850,7 +857,7 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, 1) k_oz_gemm(OzGemmPara
             stop = true;
             break;
           }
-          if (__any_sync(0xffffffffu, *(volatile int*)abort_flag)) {
+          if (warp_aborted(abort_flag)) {
             stop = true;
             break;
           }
@@ -876,7 +883,7 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, 1) k_oz_gemm(OzGemmPara
     const int row = quarter * 32 + lane;
     constexpr int HC = BN / (Cfg::epi / 4);  // columns per thread
     int64_t h = 0;  // accumulator chunks taken over (all tiles)
-    for (int64_t t = blockIdx.x; t < ntiles && !*(volatile int*)abort_flag; t += gridDim.x) {
+    for (int64_t t = blockIdx.x; t < ntiles && !warp_aborted(abort_flag); t += gridDim.x) {
       const Tile T = tile_at(t);
       if (T.skip) continue;
       const int64_t nchunks = (T.nk + Cfg::kc - 1) / Cfg::kc;
@@ -885,7 +892,7 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, 1) k_oz_gemm(OzGemmPara
 #pragma unroll
       for (int b = 0; b < Cfg::pair; ++b) sums[b].clear();
       for (int64_t c = 0; c < nchunks; ++c) {
-        if (!mbar_wait(acc_full, uint32_t(h & 1), P.err, P.wait_ns)) {
+        if (!warp_wait(acc_full, uint32_t(h & 1), P.err, P.wait_ns)) {
           set_err(P.err, 14);
           *(volatile int*)abort_flag = 1;
           break;
@@ -900,7 +907,7 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, 1) k_oz_gemm(OzGemmPara
         __syncwarp();
         if (lane == 0) mbar_arrive(acc_empty);
       }
-      if (*(volatile int*)abort_flag) break;
+      if (warp_aborted(abort_flag)) break;
       // rows beyond M and columns beyond N hold padding (scales of padding rows
       // are not written: only live ones may be used)
       const int ea = m < P.M ? P.ea[m] : 0;
@@ -1121,7 +1128,7 @@ __global__ void __launch_bounds__(OzColCfg::threads, 1) k_oz_columns(const __gri
               stop = true;
             }
             if (stop) *(volatile int*)abort_flag = 1;
-            if (stop || __any_sync(0xffffffffu, *(volatile int*)abort_flag)) {
+            if (stop || warp_aborted(abort_flag)) {
               stop = true;
               break;
             }
@@ -1148,7 +1155,7 @@ __global__ void __launch_bounds__(OzColCfg::threads, 1) k_oz_columns(const __gri
     const uint32_t tbase = tmem + (uint32_t(quarter * 32) << 16) + uint32_t(part * HC);
     double* mine = stash + part * HC * kBM + row;
     int64_t h = 0;  // accumulator chunks taken over (all tiles)
-    for (int64_t t = blockIdx.x; t < ntiles && !*(volatile int*)abort_flag; t += gridDim.x) {
+    for (int64_t t = blockIdx.x; t < ntiles && !warp_aborted(abort_flag); t += gridDim.x) {
       const Tile T = tile_at(t);
       const OzColLevel& L = P.l[T.l];
       const int64_t m = T.mt * kBM + row;
@@ -1168,7 +1175,7 @@ __global__ void __launch_bounds__(OzColCfg::threads, 1) k_oz_columns(const __gri
         OzSums<S, HC> sums;
         sums.clear();
         for (int c = 0; c < nchunks; ++c) {
-          if (!mbar_wait(acc_full, uint32_t(h & 1), P.err, P.wait_ns)) {
+          if (!warp_wait(acc_full, uint32_t(h & 1), P.err, P.wait_ns)) {
             set_err(P.err, 14);
             *(volatile int*)abort_flag = 1;
             break;
@@ -1180,7 +1187,7 @@ __global__ void __launch_bounds__(OzColCfg::threads, 1) k_oz_columns(const __gri
           __syncwarp();
           if (lane == 0) mbar_arrive(acc_empty);
         }
-        if (*(volatile int*)abort_flag) break;
+        if (warp_aborted(abort_flag)) break;
         const int ea = live && nchunks ? Q.ea[m] : 0;
         const int* ebp = Q.eb + n0;
         const int cols = nchunks ? T.members - n0 : 0;  // live ones among this thread's (the others' scales are unset)
