@@ -610,8 +610,10 @@ __device__ __forceinline__ void mma_stage(int part, uint32_t el, uint32_t tmem, 
 //     below 2^24, paired in 32 bits (L0 2^7 + L1 and so on, below 2^31); levels
 //     6 and 7 lie below 2^-42, where FP32 rounding is harmless.
 //   6 digits: 14 bits in rem.  5 digits: 7 bits, four columns to a word.  Every
-//     level's FP32 sum is an integer; levels 0 and 1 are exact for 1024 k, the
-//     deeper ones unless adversarial digits push them past 2^24.
+//     level's FP32 sum is an integer; levels 0 and 1 are exact for 1024 k.  The
+//     deeper ones reach 20480 to 32768 a k value (2^24.3 to 2^25 a chunk) where the
+//     operands hardly change along k: FP32 then rounds them, and times 128 they
+//     need 64 bits.
 // Integer sums take 2 or 3 operations per level where double-float ones took 8,
 // and leave one value to round at the end.
 template <int S, int HC>
@@ -648,11 +650,11 @@ struct OzSums {
           th[c] += (long long)p01 * (1 << 14) + (long long)p23 + (lo >> 28) + (long long)(f >> 28);
           rem[c] = f & 0x0FFFFFFFu;
         } else {
-          th[c] += (long long)L[0] * (1 << 21) + (long long)L[1] * (1 << 14) + (long long)(L[2] * 128);
+          th[c] += (long long)L[0] * (1 << 21) + (long long)L[1] * (1 << 14) + (long long)L[2] * 128;
           if constexpr (S == 6) {
-            const int lo = L[4] * 128 + L[5];
+            const long long lo = (long long)L[4] * 128 + L[5];
             const uint32_t f = rem[c] + (uint32_t(lo) & 0x3FFFu);
-            th[c] += (long long)(L[3] + (lo >> 14) + int(f >> 14));
+            th[c] += (long long)L[3] + (lo >> 14) + (long long)(f >> 14);
             rem[c] = f & 0x3FFFu;
           } else {
             const int sh = 8 * (c & 3);
