@@ -1462,7 +1462,10 @@ isdf_status isdf_rfft3(const double* f, int nx, int ny, int nz, int64_t batch, d
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   isdf_status st = rfft3_df(nullptr, f, nx, ny, nz, batch, reinterpret_cast<double2*>(S), s);
   const cudaError_t e = cudaStreamSynchronize(s);
-  if (!st && e != cudaSuccess) {
+  if (st) {
+    g_plan_error = st == ISDF_ERR_OOM ? "isdf_rfft3: no memory for the twiddle tables"
+                                      : "isdf_rfft3: a transform pass could not be started";
+  } else if (e != cudaSuccess) {
     g_plan_error = std::string("isdf_rfft3: ") + cudaGetErrorString(e);
     st = ISDF_ERR_CUDA;
   }

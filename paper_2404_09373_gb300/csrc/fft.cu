@@ -228,8 +228,8 @@ __device__ __forceinline__ RealPair real_pair(const FftPass& P, int64_t c) {
 
 // shared memory of a line: value n2 of transform k1 at k1 * row + n2, lines ld apart (both odd: the
 // 16-byte accesses of eight neighbouring threads fall in different banks either way)
-__host__ __device__ inline int fft_row(int r2) { return r2 | 1; }
-__host__ __device__ inline int fft_ld(int r1, int r2) { return (r1 * fft_row(r2)) | 1; }
+__host__ __device__ constexpr int fft_row(int r2) { return r2 | 1; }
+__host__ __device__ constexpr int fft_ld(int r1, int r2) { return (r1 * fft_row(r2)) | 1; }
 
 // First half: thread tasks (line, n2)
 template <int R1>
@@ -362,13 +362,25 @@ __global__ void __launch_bounds__(kFftThreads, BIG ? 2 : 4) k_fft_pass(FftPass P
 }
 
 // n = r1 r2 with halves of at most 9 and 12 points (16 and 8 for 128)
+constexpr int kAxes[][3] = {{1, 1, 1},  {2, 1, 2},  {3, 1, 3},  {4, 2, 2},  {6, 2, 3},  {8, 2, 4},  {9, 3, 3},   {12, 3, 4},
+                            {16, 4, 4}, {18, 3, 6}, {24, 4, 6}, {27, 3, 9}, {32, 4, 8}, {36, 6, 6}, {48, 6, 8},  {54, 6, 9},
+                            {64, 8, 8}, {72, 8, 9}, {81, 9, 9}, {96, 8, 12}, {108, 9, 12}, {128, 16, 8}};
 bool split_axis(int n, int* r1, int* r2) {
-  static const int sizes[][3] = {{1, 1, 1},  {2, 1, 2},  {3, 1, 3},  {4, 2, 2},  {6, 2, 3},  {8, 2, 4},  {9, 3, 3},   {12, 3, 4},
-                                 {16, 4, 4}, {18, 3, 6}, {24, 4, 6}, {27, 3, 9}, {32, 4, 8}, {36, 6, 6}, {48, 6, 8},  {54, 6, 9},
-                                 {64, 8, 8}, {72, 8, 9}, {81, 9, 9}, {96, 8, 12}, {108, 9, 12}, {128, 16, 8}};
-  for (const auto& t : sizes)
+  for (const auto& t : kAxes)
     if (t[0] == n) return *r1 = t[1], *r2 = t[2], true;
   return false;
+}
+
+// Lines per block: whole rounds of the 128 threads in both halves for the usual
+// sizes, and at most about 64 KB
+constexpr int fft_lines(int n) { return n >= 48 ? 32 : n >= 24 ? 64 : 128; }
+constexpr int fft_smem(int n, int r1, int r2) { return fft_lines(n) * fft_ld(r1, r2) * int(sizeof(float4)); }
+// the most that any axis of a kernel's needs
+constexpr int fft_max_smem(bool big) {
+  int m = 0;
+  for (const auto& t : kAxes)
+    if ((t[1] == 16) == big && fft_smem(t[0], t[1], t[2]) > m) m = fft_smem(t[0], t[1], t[2]);
+  return m;
 }
 
 }  // namespace
@@ -419,16 +431,25 @@ isdf_status rfft3_df(Plan* p, const double* f, int nx, int ny, int nz, int64_t b
   }
   float4* io = reinterpret_cast<float4*>(S);
   const int64_t nq = int64_t(nz) * ny * nxh;
+  cudaError_t failed = cudaSuccess;  // the first launch that was refused: its pass is missing
   auto launch = [&](FftPass P) {
+    if (failed != cudaSuccess) return;
     split_axis(P.n, &P.r1, &P.r2);
-    // lines per block: whole rounds of the 128 threads in both halves for the
-    // usual sizes, and at most about 64 KB
-    P.lpb = P.n >= 48 ? 32 : P.n >= 24 ? 64 : 128;
+    P.lpb = fft_lines(P.n);
     const int64_t blocks = (P.nlines + P.lpb - 1) / P.lpb;
-    const size_t smem = size_t(P.lpb) * fft_ld(P.r1, P.r2) * sizeof(float4);
-    auto kernel = P.r1 == 16 ? k_fft_pass<true> : k_fft_pass<false>;
-    if (smem > 40 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    kernel<<<unsigned(blocks), kFftThreads, smem, s>>>(P);
+    const bool big = P.r1 == 16;
+    auto kernel = big ? k_fft_pass<true> : k_fft_pass<false>;
+    // the limit belongs to the kernel, not to this call: every caller sets the
+    // same value, so that no thread lowers it under another's launch
+    failed = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  big ? fft_max_smem(true) : fft_max_smem(false));
+    if (failed != cudaSuccess) return;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(unsigned(blocks));
+    cfg.blockDim = dim3(kFftThreads);
+    cfg.dynamicSmemBytes = size_t(fft_smem(P.n, P.r1, P.r2));
+    cfg.stream = s;
+    failed = cudaLaunchKernelEx(&cfg, kernel, P);
     count_launches(1);
   };
   // x: lines (v, z, y), contiguous
@@ -471,7 +492,8 @@ isdf_status rfft3_df(Plan* p, const double* f, int nx, int ny, int nz, int64_t b
   R.out64 = S;
   launch(R);
   release();
-  return ISDF_OK;
+  if (failed != cudaSuccess) cudaGetLastError();  // reported here
+  return cuda_check(p, failed, "double-float transform");
 }
 
 }  // namespace isdf
