@@ -965,6 +965,12 @@ namespace {
 
 constexpr unsigned kColBlocks = 152 * 6;  // fallback grid if the occupancy query fails
 
+// Limits of dynamic shared memory.  They belong to the kernel, not to a plan:
+// every selection sets the same value, so that no thread lowers it under
+// another's launches.
+constexpr size_t kColSmem = 227 * 1024;     // k_sel_col, when a plan needs more than 48 KB
+constexpr size_t kGreedySmem = 216 * 1024;  // k_blk_greedy; more members than fit work in global memory
+
 // One greedy run over the given candidates (cidx[l] == nullptr: all points).
 isdf_status select_loop(Plan* p, int nip, double tol, const double* d0full, int* const* cidx, const int64_t* nc,
                         int* nfound, int* kl_out) {
@@ -1019,7 +1025,7 @@ isdf_status select_loop(Plan* p, int nip, double tol, const double* d0full, int*
   SelState* dst = static_cast<SelState*>(p->d_selstate);
   const size_t smem = sizeof(double) * (size_t((nGmax + 1) & ~1) + 3 * kColWarps * 32);
   if (smem > 48 * 1024) {
-    if ((st = cuda_check(p, cudaFuncSetAttribute(k_sel_col, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)),
+    if ((st = cuda_check(p, cudaFuncSetAttribute(k_sel_col, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kColSmem)),
                          "smem attribute")))
       return st;
   }
@@ -1247,10 +1253,10 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
   P.tie_abs = p->opt.tie_abs;
   P.timeout_ns = (unsigned long long)p->opt.timeout_ms * 1000000ull;
   const int64_t nbk = (P.ntot + kCompactBlock - 1) / kCompactBlock;
-  // B and the members' columns during the greedy steps: shared memory up to 112 members, else global
+  // B and the members' columns during the greedy steps: shared memory up to 108 members, else global
   const int gthreads = ((smax + 31) / 32) * 32;
   const size_t gsmem = 2 * sizeof(double) * size_t(gthreads) * smax;
-  const bool gshared = gsmem <= 216 * 1024;
+  const bool gshared = gsmem <= kGreedySmem;
   if ((st = dalloc_t(p, &counts, size_t(std::max<int64_t>(nbk, 1)), "block counts")) ||
       (st = dalloc_t(p, &nlist, 1, "list size")) ||
       (st = dalloc_t(p, &list, size_t(std::max<int64_t>(P.ntot, 1)), "local maxima")) ||
@@ -1260,8 +1266,8 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
       (st = dalloc_t(p, &round, 1, "block round")) ||
       (!gshared && (st = dalloc_t(p, &gcols, size_t(gthreads) * smax, "block columns"))))
     return bail(st);
-  if (gshared && gsmem > 40 * 1024 &&
-      (st = cuda_check(p, cudaFuncSetAttribute(k_blk_greedy, cudaFuncAttributeMaxDynamicSharedMemorySize, int(gsmem)),
+  if (gshared &&
+      (st = cuda_check(p, cudaFuncSetAttribute(k_blk_greedy, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kGreedySmem)),
                        "smem attribute")))
     return bail(st);
   BlkParams BP{};
@@ -1283,7 +1289,7 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
   SelState* dst = static_cast<SelState*>(p->d_selstate);
   const size_t smem = sizeof(double) * (size_t((nGmax + 1) & ~1) + 3 * kColWarps * 32);
   if (smem > 48 * 1024 &&
-      (st = cuda_check(p, cudaFuncSetAttribute(k_sel_col, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)),
+      (st = cuda_check(p, cudaFuncSetAttribute(k_sel_col, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kColSmem)),
                        "smem attribute")))
     return bail(st);
   int dev = 0, nsm = 152, per_sm = 0;
@@ -1525,6 +1531,8 @@ isdf_status select_loop_blocked(Plan* p, int nip, double tol, const double* d0fu
         }
         const unsigned nblk = unsigned(std::max<int64_t>(BP.boff[nlev], 1));
         k_blk_greedy<<<1, gthreads, gshared ? gsmem : 0, s>>>(BP, dst, round, m, smax, gcols);
+        // the next two kernels index by what this one has written
+        if ((st = cuda_check(p, cudaGetLastError(), "selection steps"))) return bail(st);
         k_blk_apply<<<nblk, kApply, 0, s>>>(BP, dst, round);
         k_blk_commit<<<nblk, kApply, 0, s>>>(BP, round, dst);
       }
