@@ -47,6 +47,7 @@
 
 #include "digits.cuh"
 #include "internal.cuh"
+#include "rules.h"
 
 namespace isdf {
 namespace {
@@ -619,6 +620,7 @@ __device__ __forceinline__ void mma_stage(int part, uint32_t el, uint32_t tmem, 
 template <int S, int HC>
 struct OzSums {
   static constexpr int NR = S == 5 ? HC / 4 : HC;
+  static constexpr int64_t wide = oz_wide_k(S);  // 5 and 6 digits
   long long th[HC];
   uint32_t rem[NR];
   __device__ __forceinline__ void clear() {
@@ -672,12 +674,13 @@ struct OzSums {
     else if constexpr (S == 6) return rem[c] << 14;
     else return ((rem[c / 4] >> (8 * (c & 3))) & 0x7Fu) << 21;
   }
-  // every column's value times 2^(ea + eb(c)), rounded once; wide: a 5- or
-  // 6-digit sum may not fit 64 bits.  Straight-line code (the rare cases
-  // afterwards, out of line), so that the columns' conversions overlap, and no
-  // FP64 instruction: each holds its scheduler for over 100 cycles.
+  // every column's value times 2^(ea + eb(c)), rounded once; k: values summed (a
+  // 5- or 6-digit sum of many may not fit 64 bits with its fraction).  Straight-line
+  // code (the rare cases afterwards, out of line), so that the columns'
+  // conversions overlap, and no FP64 instruction: each holds its scheduler for
+  // over 100 cycles.
   template <class E>
-  __device__ __forceinline__ void values(int ea, E eb, bool wide, double (&v)[HC]) const {
+  __device__ __forceinline__ void values(int ea, E eb, int64_t k, double (&v)[HC]) const {
     constexpr int FB = 7 * (S - 4);  // bits of the fraction (S < 7)
     int m = 0;
 #pragma unroll
@@ -687,7 +690,9 @@ struct OzSums {
       if constexpr (S >= 7) v[c] = fixed_to_double(th[c], rem[c], en);
       else v[c] = ll_to_double(th[c] * (1 << FB) + (long long)(frac(c) >> (28 - FB)), en - FB);
     }
-    if (m > kNearExp - 64 || (S < 7 && wide))
+    bool far = m > kNearExp - 64;
+    if constexpr (S < 7) far = far || k >= wide;
+    if (far)
 #pragma unroll
       for (int c = 0; c < HC; ++c) v[c] = far_double(th[c], frac(c), ea + eb(c) - 35);
   }
@@ -926,7 +931,7 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, 1) k_oz_gemm(OzGemmPara
         auto eb = [&](int j) { return j < live ? __ldg(ebp + j) : 0; };
         double* out = (part ? P.work + int64_t(T.z) * P.M * P.N : P.C) + mrow * sm + nb * sn;
         double v[HC];
-        sums[b].values(ea, eb, T.nk * kBK >= (int64_t(1) << (35 - 14 * (S - 4))), v);
+        sums[b].values(ea, eb, T.nk * kBK, v);
         if (scale) {
 #pragma unroll
           for (int j = 0; j < HC; ++j) v[j] *= P.alpha;
@@ -1195,7 +1200,7 @@ __global__ void __launch_bounds__(OzColCfg::threads, 1) k_oz_columns(const __gri
         const int cols = nchunks ? T.members - n0 : 0;  // live ones among this thread's (the others' scales are unset)
         auto eb = [&](int j) { return j < cols ? __ldg(ebp + j) : 0; };
         double v[HC];
-        sums.values(ea, eb, false, v);
+        sums.values(ea, eb, int64_t(Q.nkt) * kBK, v);
         if (sg == 1) {
 #pragma unroll
           for (int j = 0; j < HC; ++j) {
