@@ -54,8 +54,9 @@ namespace {
 
 constexpr int kMaxDevices = 64;  // per-device launch set-up and scratch addresses
 
-constexpr int kBM = 128;  // A rows per CTA = TMEM lanes
-constexpr int kBK = kOzBK;  // k values per tile / pipeline stage
+constexpr int kBM = kOzTileM;  // A rows per CTA = TMEM lanes
+constexpr int kBK = kOzTileK;  // k values per tile / pipeline stage
+static_assert(kBK == kOzBK, "digit tiles");
 constexpr int kKcTiles = 1024 / kBK;  // 1024 k values per exact chunk
 constexpr long long kWaitLimit = 1ll << 30;
 constexpr unsigned long long kWaitNs = 2000000000ull;  // 2 s of device time per wait
@@ -1401,8 +1402,7 @@ static unsigned long long oz_wait_limit() {
   return (fault && std::strcmp(fault, "oz_wait") == 0) ? 0ull : kWaitNs;
 }
 
-// S levels x BN columns of tensor memory: 5 x 48 (two tiles), 6 x 64, 7 x 48, 8 x 48
-int oz_bn(int S) { return S == 6 ? 64 : 48; }
+int oz_bn(int S) { return oz_tile_n(S); }
 
 void oz_gemm(const OzOperand& A, const OzOperand& B, double* C, int64_t ldc, int trans, double alpha, int tri, int sym,
              int splits, double* work, int* err, cudaStream_t s, const OzWindows* win) {
@@ -1520,8 +1520,8 @@ void oz_columns(const OzColumnJob* jobs, int nlev, const int* scount, int* err, 
 // The one free launch parameter of a product shape is its split-K factor
 // (how many CTAs share one output tile's k range).  On the first product of
 // a shape (rows of A, rows of B, k tiles, digits, symmetric or not) outside
-// any graph capture (products of more than 0.3 ms follow a rule instead, see
-// oz_tuned_splits), every admissible candidate runs on the real operands
+// any graph capture (products of more than 0.3 ms follow oz_rule_splits
+// instead), every admissible candidate runs on the real operands
 // (one warm-up run, then one timed run per candidate, CUDA events on the
 // product's stream) and the fastest is cached for the process; the heuristic's choice
 // is among the candidates, and the chosen one runs last so C holds its
@@ -1548,35 +1548,8 @@ int oz_tuned_splits(Plan* p, const OzOperand& A, const OzOperand& B, double* C, 
     if (it != g_tune.end()) return it->second.first;
   }
   if ((p && p->capturing) || std::getenv("ISDF_NO_AUTOTUNE")) return heuristic;
-  // Products of more than 0.3 ms: waves of CTAs decide, which needs no
-  // measurement.  A wave takes its share of k at the measured tensor rate and one
-  // epilogue, the last one is three quarters idle on average, and the partial
-  // results are written and read once.  (Timing the Coulomb matrix of the 2x2x2
-  // diamond cell with every split took 0.7 s of its first pass.  1657 x 1657 x
-  // 903168, 7 digits, symmetric: 64.9 ms with one split, 56.5 with 3, 56.4 with 8,
-  // 55.6 with 16, the rule's choice, 54.6 with 32.)
-  {
-    const int bn = oz_bn(A.S) * (A.S == 5 ? 2 : 1);
-    const int64_t mt = (A.rows + kBM - 1) / kBM, nt = (B.rows + bn - 1) / bn;
-    int64_t tiles = mt * nt;
-    if (sym) {
-      tiles = 0;
-      for (int64_t i = 0; i < mt; ++i) tiles += std::min(nt, (i * kBM + kBM - 1) / bn + 1);
-    }
-    const double step = 2.0 * kBM * bn * kBK * (A.S * (A.S + 1) / 2) / (1.7e15 / 152.0);  // one k tile, seconds
-    if (double(tiles) * double(A.nkt) * step / 152.0 > 3e-4 && !win) {
-      int best = 1;
-      double best_t = 1e30;
-      for (int c : {1, 2, 4, 8, 16, 32, 64}) {
-        if (c > A.nkt) break;
-        const double waves = std::max(1.0, double(tiles) * c / 152.0 + 0.75);
-        const double t = waves * (double((A.nkt + c - 1) / c) * step + 4e-6) +
-                         (c > 1 ? 16.0 * c * double(A.rows) * double(B.rows) / 6e12 : 0.0);
-        if (t < 0.99 * best_t) best_t = t, best = c;
-      }
-      return best;
-    }
-  }
+  if (!win)
+    if (const int c = oz_rule_splits(A.rows, B.rows, A.nkt, A.S, sym != 0)) return c;
   std::vector<int> cand;
   for (int c : {1, 2, 4, 8, 16, 32, 64})
     if (c <= std::max<int64_t>(1, A.nkt)) cand.push_back(c);
@@ -1589,8 +1562,8 @@ int oz_tuned_splits(Plan* p, const OzOperand& A, const OzOperand& B, double* C, 
   float best_ms = 1e30f;
   for (int c : cand) {
     double* work = nullptr;
+    if (!oz_splits_fit(c, A.rows, B.rows)) continue;
     const size_t wbytes = c > 1 ? sizeof(double) * size_t(c) * A.rows * B.rows : 0;
-    if (wbytes > (size_t(2) << 30)) continue;
     if (wbytes && cudaMallocAsync(reinterpret_cast<void**>(&work), wbytes, s) != cudaSuccess) {
       cudaGetLastError();
       continue;
