@@ -7,6 +7,8 @@
 // vector ready for the FFT), pick CC^T out of its pivot columns, factor it
 // with an FP64 Cholesky R R^T, invert R, and apply Xi^T = R^-T (R^-1 ZC^T^T)
 // as two triangular GEMMs.
+#include <algorithm>
+
 #include "internal.cuh"
 
 namespace isdf {
@@ -163,7 +165,10 @@ isdf_status fit_run(Plan* p) {
   struct LevelBuf {
     double *phiP = nullptr, *y = nullptr, *cc = nullptr, *li = nullptr, *scr = nullptr;
   } buf[ISDF_MAX_LEVELS];
+  double* y = nullptr;  // FP64 solve
   auto cleanup = [&]() {
+    dfree(y);
+    y = nullptr;
     for (LevelBuf& b : buf) {
       for (double* q : {b.phiP, b.y, b.cc, b.li, b.scr}) dfree(q);
       b = LevelBuf();
@@ -207,7 +212,8 @@ isdf_status fit_run(Plan* p) {
     if ((st = dalloc_t(p, &zct, size_t(k) * ng, "ZC^T / Xi"))) return cleanup(), st;
     (factored ? lv.zct : lv.xiT) = zct;
     if ((st = dalloc_t(p, &b.phiP, size_t(lv.nG) * k, "phi at pivots")) ||
-        (st = dalloc_t(p, &b.y, size_t(k) * ng, "fit scratch")) || (st = dalloc_t(p, &b.cc, size_t(k) * k, "CC^T")) ||
+        (factored && (st = dalloc_t(p, &b.y, size_t(k) * ng, "fit scratch"))) ||
+        (st = dalloc_t(p, &b.cc, size_t(k) * k, "CC^T")) ||
         (st = dalloc_t(p, &b.li, size_t(k) * k, "R^-1")) ||
         (st = dalloc_t(p, &b.scr, size_t(k / 2 + 64) * k + 64, "trtri scratch")))
       return cleanup(), st;
@@ -266,7 +272,11 @@ isdf_status fit_run(Plan* p) {
     cleanup();
     return st ? st : gather_pivot_factors(p);
   }
-  // ---- the solve and the residual statistics of every level
+  // ---- the solve and the residual statistics of every level, one after the
+  // other in scratch as large as the largest level's vectors
+  size_t ysize = 0;
+  for (int i = 0; i < njobs; ++i) ysize = std::max(ysize, size_t(p->lev[job_level[i]].k) * p->lev[job_level[i]].ng);
+  if (ysize && (st = dalloc_t(p, &y, ysize, "fit scratch"))) return cleanup(), st;
   for (int i = 0; i < njobs; ++i) {
     const int l = job_level[i];
     Level& lv = p->lev[l];
@@ -283,7 +293,7 @@ isdf_status fit_run(Plan* p) {
       g1.lda = k;
       g1.B = lv.xiT;
       g1.ldb = ng;
-      g1.C = b.y;
+      g1.C = y;
       g1.ldc = ng;
       g1.tri = 1;
       dgemm(g1, s);
@@ -294,7 +304,7 @@ isdf_status fit_run(Plan* p) {
       g2.K = k;
       g2.A = b.li;
       g2.lda = k;
-      g2.B = b.y;
+      g2.B = y;
       g2.ldb = ng;
       g2.C = lv.xiT;
       g2.ldc = ng;
@@ -303,7 +313,7 @@ isdf_status fit_run(Plan* p) {
     }
     // y still holds R^-1 (ZC^T)^T: residual statistics of this level
     cudaMemsetAsync(b.scr, 0, 2 * sizeof(double), s);
-    k_fit_residual<<<152 * 4, 256, 0, s>>>(lv.phi, ng, lv.nL, lv.nG, lv.w, b.y, k,
+    k_fit_residual<<<152 * 4, 256, 0, s>>>(lv.phi, ng, lv.nL, lv.nG, lv.w, y, k,
                                            reinterpret_cast<unsigned long long*>(b.scr), b.scr + 1, lv.resid);
     count_launches(1);
     cudaMemcpyAsync(&p->fit_resid[2 * l], b.scr, 2 * sizeof(double), cudaMemcpyDeviceToHost, s);
