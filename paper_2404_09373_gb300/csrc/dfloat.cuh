@@ -87,15 +87,24 @@ __device__ __forceinline__ double f32_to_f64(float f) {
 }
 __device__ __forceinline__ double df_to_double(DF x) { return f32_to_f64(x.hi) + f32_to_f64(x.lo); }
 
-// 1 / sqrt(d) for finite d > 0: FP32 estimate of the significand's root and one
-// step of the third-order iteration r (1 + e/2 + 3 e^2 / 8), e = 1 - d r^2 (the
-// Taylor series of (1 - e)^-1/2): from 2^-22 to rounding error in four dependent
-// FP64 operations instead of the forty of a square root and a division.
-__device__ __forceinline__ double rsqrt64(double d) {
+// r = 1 / sqrt(d) and s = sqrt(d) for finite d > 0.  r: FP32 estimate of the
+// significand's root and one step of the third-order iteration r (1 + e/2 + 3 e^2 /
+// 8), e = 1 - d r^2 (the Taylor series of (1 - e)^-1/2): from 2^-22 to rounding error
+// in four dependent FP64 operations instead of the forty of a square root and a
+// division.  s: d r and one correction by its residual.  Both on the significand,
+// scaled back by its exponent, so that no residual of a tiny d runs into the
+// subnormal numbers.
+struct Root64 {
+  double r, s;
+};
+__device__ __forceinline__ Root64 root64(double d) {
   const long long b = __double_as_longlong(d);
-  int E = int((b >> 52) & 0x7FF);
-  if (E == 0) return 1.0 / sqrt(d);  // subnormal
-  const int h = (E - 1023) >> 1;     // d = m 4^h, m in [1, 4)
+  const int E = int((b >> 52) & 0x7FF);
+  if (E == 0) {  // subnormal
+    const double s = sqrt(d);
+    return {1.0 / s, s};
+  }
+  const int h = (E - 1023) >> 1;  // d = m 4^h, m in [1, 4)
   const double m = __longlong_as_double(b - ((long long)(2 * h) << 52));
   const int odd = (E - 1023) & 1;
   const float mf = __int_as_float(((127 + odd) << 23) | int((b >> 29) & 0x7FFFFF));
@@ -103,35 +112,43 @@ __device__ __forceinline__ double rsqrt64(double d) {
   const double t = m * r0;
   const double e = fma(-t, r0, 1.0);
   const double r = fma(r0 * e, fma(0.375, e, 0.5), r0);
-  return __longlong_as_double(__double_as_longlong(r) - ((long long)h << 52));
+  const double s0 = m * r, s = fma(fma(-s0, s0, m), 0.5 * r, s0);
+  const long long hs = (long long)h << 52;
+  return {__longlong_as_double(__double_as_longlong(r) - hs), __longlong_as_double(__double_as_longlong(s) + hs)};
 }
 
-// 1 / sqrt(d) as a double-float, FP32 operations only: the same iteration with
-// the residual e = 1 - m r0^2 and its correction carried as pairs.
+// 1 / sqrt(d) as a double-float, FP32 operations only: the same iteration.  Its
+// residual e = 1 - m r^2 is kept to 2^-70 or so: m's 53 bits in three parts, every
+// product of two parts above 2^-50 with its rounding error, so that the result
+// carries little more than a double-float's own rounding: 2^-49.0 at most over
+// [1, 4) (1 / sqrt(d) in FP64 rounded to a pair: 2^-48.9; with the residual in one
+// pair: 2^-47.1).
 __device__ __forceinline__ DF df_rsqrt(double d) {
   const long long b = __double_as_longlong(d);
   const int E = int((b >> 52) & 0x7FF);
   const int h = (E - 1023) >> 1;  // d = m 4^h, m in [1, 4)
   if (E == 0 || h < -120 || h > 120) return df_from_double(1.0 / sqrt(d));
   const DF m = df_from_double(__longlong_as_double(b - ((long long)(2 * h) << 52)));
+  // what m.lo leaves of the low 29 bits (below 2^-48)
+  const int m29 = int(uint32_t(b) & 0x1FFFFFFFu), i29 = m29 - ((m29 >> 28) << 29);
+  const float rest = __int2float_rn(i29 - __float2int_rn(__int2float_rn(i29))) * ((E - 1023) & 1 ? 0x1p-51f : 0x1p-52f);
   const float r = rsqrtf(m.hi);
-  const float p = __fmul_rn(m.hi, r);
-  const float pe = __fmaf_rn(m.lo, r, __fmaf_rn(m.hi, r, -p));
-  const float q = __fmul_rn(p, r);
-  const float qe = __fmaf_rn(pe, r, __fmaf_rn(p, r, -q));
-  const DF e = two_sum(__fsub_rn(1.0f, q), -qe);  // 1 - q is exact
+  // m r = p + (u.hi + u.lo + te)
+  const float p = __fmul_rn(m.hi, r), pe = __fmaf_rn(m.hi, r, -p);
+  const float t = __fmul_rn(m.lo, r), te = __fmaf_rn(rest, r, __fmaf_rn(m.lo, r, -t));
+  const DF u = two_sum(pe, t);
+  // m r^2 = q + qe + v + ve
+  const float q = __fmul_rn(p, r), qe = __fmaf_rn(p, r, -q);
+  const float v = __fmul_rn(u.hi, r), ve = __fmaf_rn(__fadd_rn(u.lo, te), r, __fmaf_rn(u.hi, r, -v));
+  const DF e1 = two_sum(__fsub_rn(1.0f, q), -qe);  // 1 - q is exact
+  DF e = two_sum(e1.hi, -v);
+  e.lo = __fadd_rn(e.lo, __fsub_rn(e1.lo, ve));
   const float hr = 0.5f * r, c = __fmul_rn(hr, e.hi);
   const float cl = __fmaf_rn(hr, e.hi, -c) + __fmaf_rn(hr, e.lo, hr * (0.75f * e.hi * e.hi));
   const DF s = two_sum(r, c);
   const DF x = quick_two_sum(s.hi, __fadd_rn(s.lo, cl));
   const float sc = __int_as_float((127 - h) << 23);
   return {x.hi * sc, x.lo * sc};
-}
-
-// sqrt(d) from r = rsqrt64(d)
-__device__ __forceinline__ double sqrt_from(double d, double r) {
-  const double s = d * r;
-  return fma(fma(-s, s, d), 0.5 * r, s);
 }
 
 }  // namespace

@@ -192,7 +192,8 @@ __device__ void chol_diag(const CholLevel& P, int kb, DiagSmem& S) {
         if (tid == 0) atomicMin(P.err, kb + j);
         d = 1.0;
       }
-      const double r = rsqrt64(d);
+      const Root64 q = root64(d);
+      const double r = q.r;
       // the column below the diagonal, two rows a lane (rows at or above j stay)
       const int i0 = tid, i1 = tid + 32;
       const double x0 = S.s[i0][j], x1 = S.s[i1][j];
@@ -201,7 +202,7 @@ __device__ void chol_diag(const CholLevel& P, int kb, DiagSmem& S) {
       if (i1 > j) S.s[i1][j] = x1 * r;
       if (tid == 0) {
         S.r[j] = r;
-        S.s[j][j] = sqrt_from(d, r);
+        S.s[j][j] = q.s;
       }
     }
     __syncthreads();

@@ -849,7 +849,7 @@ __global__ void __launch_bounds__(kApply) k_blk_apply(BlkParams B, const SelStat
     pos_s[k] = r.pos;
     t_s[k] = r.t;
     inv_s[k] = df_rsqrt(r.dp);
-    sq_s[k] = sqrt_from(r.dp, rsqrt64(r.dp));
+    sq_s[k] = root64(r.dp).s;
   }
   auto stage = [&](int k) {  // lp of the level's step k
     for (int i = tid; i < q0 + k; i += kApply) {
