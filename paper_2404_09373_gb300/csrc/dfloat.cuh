@@ -46,9 +46,9 @@ __device__ __forceinline__ DF df_half(DF x) { return {__fmul_rn(0.5f, x.hi), __f
 // that they stay off the narrow FP64 unit.  hi is x's significand rounded to 24
 // bits (the round bit added into the exponent|significand field carries
 // correctly); lo = x - hi is the signed remainder of the low 29 bits, exact in
-// FP64 and rounded once to FP32.  Below 2^-73 lo, and below 2^-126 hi, run
-// into FP32's subnormals (both reached through a second power of two); only
-// values above 2^125 take the FP64 route.
+// FP64 and rounded once to FP32.  Below 2^-73 lo runs into FP32's subnormals
+// (reached through a second power of two), below 2^-126 hi does and nothing is
+// left for lo; only values above 2^125 take the FP64 route.
 __device__ __forceinline__ DF df_from_double(double x) {
   const uint64_t b = uint64_t(__double_as_longlong(x));
   const int E = int((b >> 52) & 0x7FF);
@@ -58,9 +58,13 @@ __device__ __forceinline__ DF df_from_double(double x) {
   }
   const uint32_t sign = uint32_t(b >> 32) & 0x80000000u;
   if (E < 897) {  // |x| < 2^-126
-    const float m = __uint_as_float(0x3F800000u | (uint32_t(b >> 29) & 0x7FFFFFu));
-    const float hi = E > 860 ? __fmul_rn(__fmul_rn(m, 0x1p-100f), __uint_as_float(uint32_t(E - 796) << 23)) : 0.0f;
-    return {__uint_as_float(__float_as_uint(hi) | sign), 0.0f};
+    uint32_t q = 0u;  // |x| in units of 2^-149, to the nearest (ties to even)
+    if (E > 872) {
+      const uint64_t m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+      const int r = 926 - E;
+      q = uint32_t((m + ((1ull << (r - 1)) - 1ull) + ((m >> r) & 1ull)) >> r);
+    }
+    return {__uint_as_float(q | sign), 0.0f};
   }
   const uint32_t m29 = uint32_t(b) & 0x1FFFFFFFu;
   const uint32_t up = m29 >> 28;

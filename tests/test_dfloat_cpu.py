@@ -51,6 +51,13 @@ void t_rsqrt(const double* d, int n, int ulps, float* hi, float* lo, double* r, 
     r[i] = q.r, s[i] = q.s;
   }
 }
+void t_pair(const double* x, int n, float* hi, float* lo, double* back) {
+  for (int i = 0; i < n; ++i) {
+    const DF p = df_from_double(x[i]);
+    hi[i] = p.hi, lo[i] = p.lo;
+    back[i] = df_to_double(p);
+  }
+}
 }
 """
 
@@ -94,3 +101,29 @@ def test_reciprocal_roots(lib, ulps, lo, hi):
     assert np.max(np.abs(s / root - 1.0)[normal]) <= 2.0 ** -53 + 2.0 ** -62
     if not np.all(normal):  # FP64's own square root and division
         assert np.max(np.abs(r * root - 1.0)[~normal]) <= 2.0 ** -52 + 2.0 ** -62
+
+
+def test_conversions(lib):
+    """FP64 to a pair: hi is a nearest FP32 number (subnormal ones, where nothing is left for lo, ties to even), lo the
+    nearest to what is left; and back.  Every exponent up to 2^126, significands at the edges of the rounding."""
+    rng = np.random.default_rng(7)
+    e = np.arange(-1074, 126)
+    frac = np.concatenate([[1.0, 1.5, 2.0 - 2.0 ** -52], 1.0 + 2.0 ** -rng.integers(1, 53, 40).astype(float),
+                           1.0 + 2.0 ** -24 + np.array([-1, 0, 1]) * 2.0 ** -52, 1.0 + 3 * 2.0 ** -24 + np.array([-1, 0, 1]) * 2.0 ** -52,
+                           rng.uniform(1.0, 2.0, 200)])
+    x = np.ldexp(frac[None, :], e[:, None]).ravel()
+    x = np.concatenate([x, -x, [0.0, -0.0]])
+    n = x.size
+    hi, lo, back = np.empty(n, np.float32), np.empty(n, np.float32), np.empty(n)
+    lib.t_pair(_ptr(x), n, _ptr(hi), _ptr(lo), _ptr(back))
+    near = x.astype(np.float32).astype(np.float64)
+    hi64 = hi.astype(np.float64)
+    np.testing.assert_array_equal(np.abs(x - hi64), np.abs(x - near))  # a tie may go either way: lo makes it good
+    tiny = np.abs(x) < 2.0 ** -126
+    np.testing.assert_array_equal(hi64[tiny], near[tiny])
+    np.testing.assert_array_equal(np.signbit(hi64), np.signbit(near))
+    rest, lo64 = x - hi64, lo.astype(np.float64)
+    sub = np.abs(rest) < 2.0 ** -126  # to 24 bits first, then to units of 2^-149: 3/4 of one
+    np.testing.assert_array_equal(lo64[~sub], rest.astype(np.float32)[~sub])
+    assert np.max(np.abs(rest - lo64)[sub]) <= 0.75 * 2.0 ** -149
+    np.testing.assert_array_equal(back, hi64 + lo64)
