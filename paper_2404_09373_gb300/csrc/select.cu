@@ -200,9 +200,10 @@ __device__ __forceinline__ double sel_dmax(const SelState* st) {
 
 // The pivot of the step whose smallest qualifying index is known; one thread.
 __device__ __forceinline__ void sel_pick(const SelParams& P, SelState* st, unsigned long long idx, double dmax) {
-  if (idx == ULLONG_MAX) {  // nothing qualified (cannot happen with dmax > 0)
+  if (idx == ULLONG_MAX) {  // nothing qualifies: the largest residual is infinite, its tie threshold not a number
     st->done = 1;
     st->skip = 1;
+    st->final_ = 1;
     return;
   }
   int l = 0;
@@ -738,6 +739,7 @@ __global__ void __launch_bounds__(kMaxSet) k_blk_greedy(BlkParams B, SelState* s
     const int k = B.k + j;
     // no further pivot: the next block's set, or an ordinary step, decides what that means
     if (k >= P.nip || mk == 0ull) break;
+    if ((mk >> 52) == 0x7FFull) break;  // infinite: no threshold, so no member would be found below
     if (P.tol > 0.0 && k > 0 && dmax < P.tol * d0) break;
     if (k == 0) {
       d0 = dmax;
