@@ -439,27 +439,31 @@ isdf_status isdf_propose_residual(isdf_plan_t plan, const int64_t* quota, int64_
  *   C[m*ldc + n] = alpha * sum_k A[m*lda + k] * B[n*ldb + k]
  * A, B, C are DEVICE pointers (row-major FP64).  Each operand row is scaled
  * by a power of two and split into `slices` BF16 digit planes (5 to 8,
- * about 7 bits each).  With 5 or 6, digit-pair products accumulate in FP32
- * tensor memory per 1024-wide k chunk and are summed in double-float
- * registers; the error is below 2^-(7*slices-2) * K * max_k|A[m,k]| *
- * max_k|B[n,k]| per element.  With 7 or 8, the six leading digit levels are
- * summed exactly (512-wide chunks, integer accumulation) and the rest, below
- * 2^-42 of the result, in FP32: with 7 the error is below 2^-47 * K *
- * max_k|A[m,k]| * max_k|B[n,k]|, with 8 (FP64-grade) below 2^-52 * K *
- * max_k|A[m,k]| * max_k|B[n,k]| + 2^-53 |C[m,n]|.
+ * about 7 bits each).  Digit-pair products accumulate in FP32 tensor memory
+ * per k chunk (1024 wide with 5 or 6 digits, 512 with 7 or 8) and the chunks
+ * are summed as integers.  With a_m and b_n the powers of two above the rows'
+ * largest magnitudes, the error per element is below 2^-(7*slices-2) * K *
+ * a_m * b_n with 5, 6 or 7 digits, and with 8 (FP64-grade) below 2^-52 * K *
+ * max_k|A[m,k]| * max_k|B[n,k]| + 2^-53 |C[m,n]|.  With 5 or 6, operands that
+ * hardly change along k can push a chunk's FP32 sums past 2^24, whose rounding
+ * then adds at most 2^-31 * K * a_m * b_n.
  * splits > 1 divides K over that many CTAs (needs splits*M*N*8 bytes of
- * scratch, allocated by the call).  Enqueued on `stream`; returns after the
- * stream is idle.  A pipeline wait that exceeds its bound returns
- * ISDF_ERR_TIMEOUT (no fault or trap). */
+ * scratch).  Scratch -- the digit planes, about 2*slices*(M + N)*K bytes, and
+ * the partial results -- comes from a private stream-ordered pool, one per
+ * device, shared with isdf_rfft3 by all threads and streams.  The pool keeps up
+ * to 4 GiB from call to call, which no other allocator of the process can use;
+ * it is emptied when a plan of this library runs out of memory and by
+ * isdf_plan_batch.  A capturing stream is refused with ISDF_ERR_CUDA.
+ * Enqueued on `stream`; returns after the stream is idle.  A pipeline wait
+ * that exceeds its bound returns ISDF_ERR_TIMEOUT (no fault or trap). */
 isdf_status isdf_gemm_f64(const double* A, const double* B, double* C, int64_t M, int64_t N, int64_t K, int64_t lda,
                           int64_t ldb, int64_t ldc, double alpha, int slices, int splits, void* stream);
 
 /* The same product as isdf_gemm_f64 for callers that cannot allocate device
  * memory: code inside a framework whose caching allocator owns the device's
- * memory (a cudaMalloc there can fail or fragment the pool), and paths that
- * cannot take the implicit device synchronisation of cudaMalloc/cudaFree
- * (a solver loop that must not stall other streams).  (The paper has no
- * counterpart; this is an interface of this library only.)
+ * memory (an allocation there can fail, and what isdf_gemm_f64's pool keeps is
+ * lost to it).  (The paper has no counterpart; this is an interface of this
+ * library only.)
  * All scratch -- the BF16 digit planes of both operands, their row scales and
  * an error word -- lives in one static device array of
  * isdf_gemm_f64_noalloc_capacity() bytes (32 MiB), which every GPU that loads
@@ -507,6 +511,7 @@ isdf_status isdf_grids_for_threshold(const isdf_system* sys, double eps_K, int* 
  * pipes.  f: batch x nz x ny x nx FP64; S: batch x nz x ny x (nx/2+1) complex
  * FP64 (interleaved re, im); DEVICE pointers, S must not overlap f.  Every axis
  * must be 2^a 3^b <= 128, else ISDF_ERR_ARG (isdf_coulomb then uses cuFFT).
+ * The twiddle tables (16 (nx + ny + nz) bytes) come from isdf_gemm_f64's pool.
  * Enqueued on `stream`; returns after the stream is idle. */
 isdf_status isdf_rfft3(const double* f, int nx, int ny, int nz, int64_t batch, double* S, void* stream);
 

@@ -234,7 +234,7 @@ isdf_status dpotrf_lower(Plan* p, const FactorJob* jobs, int count, cudaStream_t
 void dtrtri_lower(Plan* p, const FactorJob* jobs, int count, bool tensor, cudaStream_t s);
 
 // FP64-accurate GEMM from sliced BF16 products on tcgen05 (ozgemm.cu).
-// An operand is rows x K, pre-sliced into S BF16 digit planes (S = 5 or 6)
+// An operand is rows x K, pre-sliced into S BF16 digit planes (S = 5 to 8)
 // and pre-tiled for the tensor cores; A operands use row tiles of 128, B
 // operands row tiles of oz_bn(S).
 constexpr int kOzBK = 32;  // k values per digit tile (two K = 16 tcgen05.mma steps, one pipeline stage)

@@ -9,8 +9,9 @@
 //     (A B^T)_mn = 2^{e_m + f_n - 14} sum_q 2^{-7q} L_q,  L_q = sum_k sum_{s+t=q} d_s b_t.
 // Each level has its own FP32 accumulator in tensor memory.  Digit products
 // are integers below 2^14, so levels 0 and 1 summed over a chunk of 1024 k
-// values stay below 2^24 and are exact in FP32; deeper levels are scaled by
-// 2^-14 or less, where FP32 rounding is harmless.  After every chunk the
+// values stay below 2^24 and are exact in FP32; deeper levels are too unless the
+// operands hardly change along k (their FP32 rounding then adds at most 2^-31 K of
+// the rows' scales: 77 units of 2^-28 in a chunk's level 2).  After every chunk the
 // epilogue warps read the levels out (tcgen05.ld) and add them as integers
 // (OzSums); the result is rounded once.  With S = 7 or 8 (FP64-grade: 49 or 56
 // fraction bits per operand) the chunk is 512 k, so that levels 0..5 are exact:

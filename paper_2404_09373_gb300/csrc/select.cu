@@ -52,7 +52,6 @@ struct SelState {
   // speculative blocks
   int final_;                // a stop rule ended the selection
   int bsteps;                // steps accepted in the current round of a block
-  int btried;                // steps the round tried
   int members[ISDF_MAX_LEVELS];  // the block's set, per level
 };
 
@@ -928,7 +927,6 @@ __global__ void __launch_bounds__(kApply) k_blk_commit(BlkParams B, BlkRound* R,
     }
     if (tid == 0) {
       st->bsteps = js;
-      st->btried = R->nsteps;
       for (int a = 0; a < P.nlev; ++a) st->members[a] = B.scount[a];
       st->k = B.k + js;
       for (int a = 0; a < P.nlev; ++a) {
@@ -1118,10 +1116,11 @@ __global__ void k_gather_cols(const double* __restrict__ fo, int64_t no, const i
 constexpr int kSlices = 8;  // FP64-grade sliced products for the selection
 
 // Speculative-block form of select_loop (same result: every pivot is the
-// greedy one).  Per block: S from the residual's local maxima, three
-// tensor-core products per level for the columns of S, then up to s greedy
-// steps replayed from a CUDA graph; a step whose pivot lies outside S ends the
-// block (if it was the block's first step, one ordinary step is taken).
+// greedy one).  Per block: S from the residual's local maxima, the columns of S
+// at every candidate in one tensor-core launch, then rounds of greedy steps among
+// the members of S (k_blk_greedy), verified at every candidate (k_blk_apply) and
+// taken over up to the first step that failed (k_blk_commit).  A round that
+// loses a step ends the block; if it accepted none, one ordinary step is taken.
 // tau > 0: the candidates are the points with initial residual >= tau (the
 // exact prefilter).  Residuals only shrink, so a candidate whose residual
 // falls below tau can never be picked while every pivot value stays above
