@@ -154,6 +154,13 @@ __global__ __launch_bounds__(NT) void k_zc(int64_t k, int64_t ng, int nL, int nG
 // so the serial part, the 64 dependent columns, is hidden wherever the update is
 // longer.  The inverted diagonal blocks are those of R^-1, where
 // dtrtri_lower starts.
+//
+// A product with the inverted block leaves an error of eps cond(R_kk) |A| in a
+// block column where a substitution leaves eps |A|.  Residual |A - R R^T| / |A|
+// emulated for CC^T of one cell at 6 points a function (cond(CC^T) up to 1e6, of
+// the 64 x 64 blocks up to 50 in selection order, 700 in grid order): 1.2 to
+// 2.8e-16 against 1.0 to 2.3e-16 by substitution.  64 neighbouring grid points
+// first (block 7e5, CC^T 1e14): 1.2e-15 against 1.1e-16.
 constexpr int CB = 64;
 
 struct CholLevel {
@@ -192,8 +199,7 @@ __device__ void chol_diag(const CholLevel& P, int kb, DiagSmem& S) {
         if (tid == 0) atomicMin(P.err, kb + j);
         d = 1.0;
       }
-      const Root64 q = root64(d);
-      const double r = q.r;
+      const double r = root64(d).r;
       // the column below the diagonal, two rows a lane (rows at or above j stay)
       const int i0 = tid, i1 = tid + 32;
       const double x0 = S.s[i0][j], x1 = S.s[i1][j];
@@ -202,7 +208,7 @@ __device__ void chol_diag(const CholLevel& P, int kb, DiagSmem& S) {
       if (i1 > j) S.s[i1][j] = x1 * r;
       if (tid == 0) {
         S.r[j] = r;
-        S.s[j][j] = q.s;
+        S.s[j][j] = d;  // no later column reads it: the roots are taken together below
       }
     }
     __syncthreads();
@@ -215,7 +221,10 @@ __device__ void chol_diag(const CholLevel& P, int kb, DiagSmem& S) {
     __syncthreads();
   }
   // inverse by doubling: [A 0; C B]^-1 = [A^-1 0; -B^-1 C A^-1  B^-1]
-  for (int i = tid; i < CB; i += NT) S.v[i][i] = i < b ? S.r[i] : 1.0;
+  for (int i = tid; i < CB; i += NT) {
+    if (i < b) S.s[i][i] = root64(S.s[i][i]).s;
+    S.v[i][i] = i < b ? S.r[i] : 1.0;
+  }
   __syncthreads();
   for (int h = 1; h < CB; h *= 2) {
     const int per = h * h, tot = (CB / (2 * h)) * per;  // <= 32 * 64 / 2
