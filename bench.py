@@ -379,11 +379,10 @@ def gpu_config(args, workload, world):
 # DRAM traffic of a kernel family per unit of its algorithmic work, from one
 # ncu capture of the same kernel (dram__bytes_read.sum + dram__bytes_write.sum
 # over the algorithmic bytes of the captured launches); absent where no capture
-# of the current kernel exists.  select_gemm: the 8-digit product with the
-# selection's launch shape on a probe of 262144 x 48 x 832 (3.51 GB read +
-# 0.11 GB written for 1.745 GB of FP64 operands: the 16-byte digit planes
-# read once).
-TRAFFIC_PER_WORK = {"select_gemm": 2.075}
+# of the current kernel exists.  select_gemm: k_oz_columns, all 108 launches of a
+# timed step of the 2x2x2 diamond workload (853.96 GB read + 13.26 GB written for
+# 475.99 GB: 16-byte digit planes read once, the coarse levels' partly from L2).
+TRAFFIC_PER_WORK = {"select_gemm": 1.822}
 
 
 # BF16 digit-pair products per FP64-equivalent flop: 5 digits (s + t <= 4) in

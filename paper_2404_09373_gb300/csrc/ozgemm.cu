@@ -989,8 +989,9 @@ __global__ void __launch_bounds__(OzCfg<S, BN>::threads, 1) k_oz_gemm(OzGemmPara
 // 163 us, on 2x2x2 2.01 -> 1.76 ms (99 us and 1.57 ms with integer sums and two
 // issuing warps), and one launch instead of up to 21 for the digits of the set's
 // rows.
-// Bound: the tensor cores (0.75 of their measured rate for two N tiles a level)
-// and the candidates' digit stream (16 bytes a value) from HBM; persistent CTAs,
+// Bound: the tensor cores (0.7 of their measured rate on 2x2x2, the padding of the
+// N tiles counted) and the candidates' digit stream (16 bytes a value) from HBM
+// (0.76 of the copy rate); persistent CTAs,
 // one per SM, the levels in order (the longest k ranges first).
 struct OzColSeg {
   const __nv_bfloat16 *A, *B;
